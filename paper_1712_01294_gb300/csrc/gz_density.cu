@@ -1,0 +1,758 @@
+// Density pass (steps O4, O3): the support radius H of every particle, its
+// number density and its neighbour list.
+//
+// A group of kLanes lanes shares one particle.  The lanes take the cells of
+// the search window in rounds, test their cell's candidates into a bit mask,
+// place the hits by a prefix sum over the group (so the cache holds them in
+// scan order: cells in row order, ascending index within a cell) and keep
+// their share of the cached distances in registers for the iteration.  What
+// bounds the pass is the chain of dependent loads (cell range, then
+// candidates) and the instructions per candidate; a group shortens the chain
+// by its lanes, keeps 4 to 8 times fewer particles' caches per block in
+// shared memory, and loses less to lanes whose cells hold more particles
+// than their neighbours' (an evolved state).
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
+#include "gz_device.cuh"
+#include "gz_launch.cuh"
+
+namespace gz {
+
+namespace {
+
+inline int blocks(int n, int t) { return (n + t - 1) / t; }
+
+constexpr int kDensBlock = 128;
+constexpr int kDensCache = 64;  // candidates within 1.05 H a group can hold
+constexpr int kLanes = 4;       // lanes of a group (8 measured slower from 32^3 particles on)
+
+// FP32 launches of this many particles or more fill the chip with one thread
+// each (k_density_one), which then takes fewer instructions a particle.
+// Measured, group / thread, us a launch, first steps (late in the run): Sod
+// 32^3 38 / 44 (52 / 68), KH 41^3 72 / 72 (81 / 74), Sedov 64^3 179 / 117
+// (342 / 524), turbulence 128^3 1483 / 921 (1808 / 1325).
+constexpr int kThreadMin = 100000;
+
+// Radius of the candidate cache for a support Ht: 5% headroom so that small
+// growth of H during the iteration needs no rescan, never past h_lim.
+template <typename T>
+__device__ __forceinline__ T dens_cache_radius(T Ht, const KParams& p) {
+    T R = Ht * T(1.05);
+    if (!(R < (T)p.h_lim)) R = max(Ht, (T)p.h_lim);
+    return R;
+}
+
+// The two terms of the density sum at q = r/H, from t = max(1 - q, 0) and
+// v = max(1/2 - q, 0):  W/2 = t^3 - 4 v^3,  -q W'/6 = q (t^2 - 4 v^2)
+// (both vanish beyond the support, so no distance test is needed).  The
+// second is returned as two factors x y, summed by explicit multiply-adds, so
+// that every kernel rounds the sums alike.
+__device__ __forceinline__ void dens_terms2(float q, float& w, float& x, float& y) {
+    const float t = __saturatef(1.f - q), v = __saturatef(0.5f - q);
+    const float t2 = t * t, v2 = v * v;
+    w = fmaf(-4.f * v2, v, t2 * t);
+    x = q;
+    y = fmaf(-4.f, v2, t2);
+}
+__device__ __forceinline__ void dens_terms2(double q, double& w, double& x1, double& d) {
+    // one cubic in x = q (inside) or 1 - q (outside), coefficients selected;
+    // the pieces decided on the high word (no FP64 comparison)
+    const bool in = __double2hiint(q) < 0x3FE00000;
+    const bool out = __double2hiint(q) >= 0x3FF00000;
+    const double x = in ? q : 1.0 - q;
+    const double x2 = x * x;
+    const double a = fma(fma(in ? 3.0 : 1.0, x, in ? -3.0 : 0.0), x2, in ? 0.5 : 0.0);
+    const double b = fma(in ? -3.0 : -1.0, x, in ? 2.0 : 1.0) * x2;
+    w = out ? 0.0 : a;
+    x1 = 1.0;
+    d = out ? 0.0 : b;
+}
+
+// r from r^2 for the iteration.
+__device__ __forceinline__ float dist(float r2) {
+    const float m = fmaxf(r2, 1e-37f);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(m));
+    return m * y;
+}
+__device__ __forceinline__ double dist(double r2) { return sqrt(r2); }
+
+// Compensated partial sums combined over the lanes of a group (every lane
+// gets the same bits: the two-sum's error is exact in either order).
+template <int G>
+__device__ __forceinline__ float group_sum(unsigned gm, Acc<float> a) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) {
+        const float b = __shfl_xor_sync(gm, a.s, o), cb = __shfl_xor_sync(gm, a.c, o);
+        const float s = __fadd_rn(a.s, b);
+        const float bb = __fsub_rn(s, a.s);
+        const float e = __fadd_rn(__fsub_rn(a.s, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+        a.s = s;
+        a.c = __fsub_rn(__fadd_rn(a.c, cb), e);
+    }
+    return a.fvalue();
+}
+template <int G>
+__device__ __forceinline__ double group_sum(unsigned gm, Acc<double> a) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) a.s += __shfl_xor_sync(gm, a.s, o);
+    return a.s;
+}
+template <int G, typename T>
+__device__ __forceinline__ T group_add(unsigned gm, T v) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) v += __shfl_xor_sync(gm, v, o);
+    return v;
+}
+
+// Result of one evaluation: f's sign decides the bracket, and the next H.
+template <typename T>
+struct HIter {
+    T lo = T(0), hi = T(0);
+    bool has_lo = false, has_hi = false, clamped = false;
+};
+
+// One step of the bracketed Newton iteration on
+// f(H) = (32/3)(1 + S) - N_ngb, f' = (32/3) sd / H, S = sum w, sd = sum -w' q.
+// Returns true when |f| is within the tolerance, else sets H to the next
+// trial.  FP32: f, the quotient and the bracket are FP32 numbers, and so is
+// the next trial's rounding H - f/f' (the FP64 difference of two FP32 numbers
+// rounded to FP32 is their FP32 difference), so the FP64 update needs no FP64
+// arithmetic except near h_lim.
+__device__ __forceinline__ bool h_step(HIter<float>& b, float& H, float S, float sd, const KParams& p, bool last) {
+    const float C = 32.f / 3.f;
+    const float f = C * __fadd_rn(1.f, S) - (float)p.ngb;
+    if (fabsf(f) <= p.ftol) return true;
+    if (last) return false;
+    if (f < 0.f) {
+        b.lo = H;
+        b.has_lo = true;
+    } else {
+        b.hi = H;
+        b.has_hi = true;
+    }
+    const float lo = b.has_lo ? b.lo : 0.5f * H, hi = b.has_hi ? b.hi : 2.f * H;
+    const float fp = C * sd / H;
+    float Hn = 0.f;
+    bool ok = false;
+    if (fp > 0.f) {
+        Hn = __fsub_rn(H, f / fp);
+        ok = Hn > lo && Hn < hi;
+    }
+    if (!ok) Hn = (b.has_lo && b.has_hi) ? 0.5f * __fadd_rn(b.lo, b.hi) : (f < 0.f ? 2.f * H : 0.5f * H);
+    if (Hn >= p.hlimf) {
+        Hn = (float)(0.5 * ((double)H + p.h_lim));
+        b.clamped = true;
+    }
+    H = Hn;
+    return false;
+}
+__device__ __forceinline__ bool h_step(HIter<double>& b, double& H, double S, double sd, const KParams& p, bool last) {
+    const double C = 32.0 / 3.0;
+    const double f = C * (1.0 + S) - p.ngb;
+    if (fabs(f) <= p.dtol) return true;
+    if (last) return false;
+    if (f < 0.0) {
+        b.lo = H;
+        b.has_lo = true;
+    } else {
+        b.hi = H;
+        b.has_hi = true;
+    }
+    const double lo = b.has_lo ? b.lo : 0.5 * H, hi = b.has_hi ? b.hi : 2.0 * H;
+    const double fp = C * sd / H;
+    double Hn = 0.0;
+    bool ok = false;
+    if (fp > 0.0) {
+        Hn = H - f / fp;
+        ok = Hn > lo && Hn < hi;
+    }
+    if (!ok) Hn = (b.has_lo && b.has_hi) ? 0.5 * (b.lo + b.hi) : (f < 0.0 ? 2.0 * H : 0.5 * H);
+    if (Hn >= p.h_lim) {
+        Hn = 0.5 * (H + p.h_lim);
+        b.clamped = true;
+    }
+    H = Hn;
+    return false;
+}
+
+// Whether a support spans so many cells that scanning its window is left to a
+// warp from the start (a blast's emptied centre: up to thousands of mostly
+// empty cells, which one thread or a group of four would walk while the rest
+// of the block waits).
+template <typename T>
+__device__ __forceinline__ bool wide(T R, int nc) {
+    return (float)R * (float)nc > 2.1f;
+}
+
+// Starting H of particle i: its guess, or (flagged by the caller) the box's
+// mean when the guess is unusable.
+template <typename T>
+__device__ __forceinline__ T h_start(T h, const BoxInfo& bx, const KParams& p, bool& bad) {
+    bad = !((double)h > 0.0) || !((double)h < p.h_lim);
+    if (!bad) return h;
+    double H = cbrt(3.0 * p.ngb / (4.0 * kPi * (double)bx.count));
+    if (!(H < p.h_lim)) H = 0.5 * p.h_lim;
+    return (T)H;
+}
+
+__device__ __forceinline__ float n_of(float S, float H) {
+    return 8.f * __fadd_rn(1.f, S) / ((float)kPi * H * H * H);
+}
+__device__ __forceinline__ double n_of(double S, double H) { return 8.0 * (1.0 + S) / (kPi * H * H * H); }
+
+template <typename T>
+__global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
+    k_density(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr, int* __restrict__ ncount,
+              int* __restrict__ iters, DevStatus* st, const int* __restrict__ list,
+              const int* __restrict__ nlist, int* __restrict__ defer, int* __restrict__ ndefer, int ccap) {
+    constexpr int G = kLanes, P = kDensBlock / G, E = kDensCache / G;
+    constexpr int S = kDensCache + G;  // (the groups of a warp start on different banks)
+    __shared__ T c_r2[P][S];
+    __shared__ unsigned c_j[P][S];
+    const int gl = threadIdx.x % G, gp = threadIdx.x / G;
+    const unsigned gm = group_mask<G>();
+    int i = blockIdx.x * P + gp;
+    if (list) {  // the particles of an index list only (hierarchical steps)
+        if (i >= *nlist) return;
+        i = list[i];
+    } else if (i >= N) {
+        return;
+    }
+    const BoxInfo bx = g.boxes[s.box[i]];
+    const P4<T> me = s.pos[i];
+    bool bad;
+    T H = h_start<T>(s.h[i], bx, p, bad);
+    if (bad && gl == 0) set_status(st, GZ_S_NONFINITE, GZ_C_NONFINITE, s.id[i]);
+    T Rc = T(-1), Hev = H, Sv = T(0), sdv = T(0);
+    T r[E];
+    int ncache = 0, it;
+    HIter<T> b;
+    bool conv = false;
+    for (it = 1; it <= p.max_iter; ++it) {
+        if (!(H <= Rc)) {  // first evaluation, or grown past the cache radius
+            Rc = dens_cache_radius<T>(H, p);
+            __syncwarp(gm);
+            ncache = wide(Rc, bx.nc) ? ccap + 1 : group_scan<T, G>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, gl, gm, ccap,
+                                            [&](int k, int j) {
+                                                if (k < kDensCache) c_j[gp][k] = (unsigned)j;
+                                            });
+            if (ncache > ccap) {
+                // more candidates than the cache holds (a support spanning
+                // many cells): left to k_density_warp
+                if (gl == 0) defer[atomicAdd(ndefer, 1)] = i;
+                return;
+            }
+            __syncwarp(gm);
+#pragma unroll
+            for (int u = 0; u < E; ++u) {
+                const int k = u * G + gl;
+                r[u] = T(8);  // (past every support)
+                if (k < ncache) {
+                    const P4<T> q = s.pos[c_j[gp][k]];
+                    const T r2 = sep2(mi_diff(q.x, me.x, me.x - T(1)), mi_diff(q.y, me.y, me.y - T(1)),
+                                      mi_diff(q.z, me.z, me.z - T(1)));
+                    c_r2[gp][k] = r2;
+                    r[u] = dist(r2);
+                }
+            }
+        }
+        const T iH = T(1) / H;
+        Acc<T> sw;
+        T sd = T(0);
+#pragma unroll
+        for (int u = 0; u < E; ++u) {
+            if (u * G >= ncache) break;
+            T w, x, y;
+            dens_terms2(r[u] * iH, w, x, y);
+            sw.add(w);
+            sd = fma(x, y, sd);
+        }
+        Sv = T(2) * group_sum<G>(gm, sw);
+        sdv = T(6) * group_add<G>(gm, sd);
+        Hev = H;
+        if (h_step(b, H, Sv, sdv, p, it == p.max_iter)) {
+            conv = true;
+            break;
+        }
+    }
+    if (it > p.max_iter) it = p.max_iter;
+    const T H2 = Hev * Hev;
+    int cnt = 0;
+    for (int k0 = 0; k0 < ncache; k0 += G) {  // list of the returned H, in scan order
+        const int k = k0 + gl;
+        const bool in = k < ncache && c_r2[gp][k] < H2;
+        const unsigned m = (__ballot_sync(gm, in) & gm) >> (threadIdx.x & 31 & ~(G - 1));
+        const int slot = cnt + __popc(m & ((1u << gl) - 1u));
+        if (in && slot < p.cap) store_slot(nbr + lslot(slot, i, N), c_j[gp][k]);
+        cnt += __popc(m);
+    }
+    if (gl != 0) return;
+    s.h[i] = Hev;
+    s.n[i] = n_of(Sv, Hev);
+    if (s.sd) s.sd[i] = sdv;  // (absent in the allocation-free density call)
+    iters[i] = it;
+    ncount[i] = cnt;
+    if (!conv) {
+        set_status(st, GZ_S_HCONV, GZ_C_HCONV, s.id[i]);
+        if (b.clamped) atomicOr(&st->bits, GZ_S_HLIM);
+    }
+    if (cnt > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
+}
+
+// FP32, one thread per particle: the form for launches that fill the chip
+// (k_density is faster below kThreadMin particles).  The first scan keeps
+// (r^2, j) of the candidates within 1.05 H in the thread's column of shared
+// memory.  Entry k adds to partial sum k mod 4, as lane k mod 4 of a group of
+// four does, and the four are combined as the group combines them, so both
+// forms give the same bits.  Held to 96 registers (10 blocks of 64 per SM).
+constexpr int kOneBlock = 64;
+template <int kCache>
+__device__ __noinline__ int dens_fill(const Grid& g, const BoxInfo& bx, const P4<float>* __restrict__ pos, int i,
+                                      float xi, float yi, float zi, float R, float (*c_r2)[kOneBlock],
+                                      unsigned (*c_j)[kOneBlock], int t) {
+    const float R2 = R * R;
+    int n = 0;
+    for_candidates<float>(g, bx, pos, i, xi, yi, zi, R, [&](int j, float, float, float, float r2) {
+        if (r2 < R2) {
+            if (n < kCache) {
+                c_r2[n][t] = r2;
+                c_j[n][t] = (unsigned)j;
+            }
+            ++n;
+        }
+    });
+    return n;
+}
+
+__device__ __forceinline__ Acc<float> combine(Acc<float> a, const Acc<float>& b) {
+    const float s = __fadd_rn(a.s, b.s);
+    const float bb = __fsub_rn(s, a.s);
+    const float e = __fadd_rn(__fsub_rn(a.s, __fsub_rn(s, bb)), __fsub_rn(b.s, bb));
+    a.s = s;
+    a.c = __fsub_rn(__fadd_rn(a.c, b.c), e);
+    return a;
+}
+
+template <int kCache>
+__global__ void __launch_bounds__(kOneBlock, 10)
+    k_density_one(int N, Sorted<float> s, Grid g, KParams p, unsigned* __restrict__ nbr,
+                  int* __restrict__ ncount, int* __restrict__ iters, DevStatus* st,
+                  const int* __restrict__ list, const int* __restrict__ nlist, int* __restrict__ defer,
+                  int* __restrict__ ndefer) {
+    __shared__ float c_r2[kCache][kOneBlock];
+    __shared__ unsigned c_j[kCache][kOneBlock];
+    const int t = threadIdx.x;
+    int i = blockIdx.x * kOneBlock + t;
+    if (list) {  // the particles of an index list only (hierarchical steps)
+        if (i >= *nlist) return;
+        i = list[i];
+    } else if (i >= N) {
+        return;
+    }
+    const BoxInfo bx = g.boxes[s.box[i]];
+    const P4<float> me = s.pos[i];
+    bool bad;
+    float H = h_start<float>(s.h[i], bx, p, bad);
+    if (bad) set_status(st, GZ_S_NONFINITE, GZ_C_NONFINITE, s.id[i]);
+    float Rc = dens_cache_radius<float>(H, p);
+    int ncache = 0;
+    if (wide(Rc, bx.nc)) {
+        ncache = kCache + 1;
+    } else {  // the cache of the starting H, scanned before the iteration (few live values here)
+        const float R2 = Rc * Rc;
+        for_candidates<float>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, [&](int j, float, float, float, float r2) {
+            if (r2 < R2) {
+                if (ncache < kCache) {
+                    c_r2[ncache][t] = r2;
+                    c_j[ncache][t] = (unsigned)j;
+                }
+                ++ncache;
+            }
+        });
+    }
+    float Hev = H, Sv = 0.f, sdv = 0.f;
+    HIter<float> b;
+    bool conv = false;
+    int it;
+    for (it = 1; it <= p.max_iter; ++it) {
+        if (H > Rc) {  // grown past the cache radius: rescan
+            Rc = dens_cache_radius<float>(H, p);
+            ncache = wide(Rc, bx.nc) ? kCache + 1 : dens_fill<kCache>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, c_r2, c_j, t);
+        }
+        if (ncache > kCache) {  // left to k_density_warp
+            defer[atomicAdd(ndefer, 1)] = i;
+            return;
+        }
+        const float iH = 1.f / H;
+        Acc<float> sw[4];
+        float sd[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int k0 = 0; k0 < ncache; k0 += 4) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                float r = 8.f;  // (past every support)
+                if (k0 + u < ncache) r = dist(c_r2[k0 + u][t]);
+                float w, x, y;
+                dens_terms2(r * iH, w, x, y);
+                sw[u].add(w);
+                sd[u] = fmaf(x, y, sd[u]);
+            }
+        }
+        Sv = 2.f * combine(combine(sw[0], sw[1]), combine(sw[2], sw[3])).fvalue();
+        sdv = 6.f * ((sd[0] + sd[1]) + (sd[2] + sd[3]));
+        Hev = H;
+        if (h_step(b, H, Sv, sdv, p, it == p.max_iter)) {
+            conv = true;
+            break;
+        }
+    }
+    if (it > p.max_iter) it = p.max_iter;
+    const float H2 = Hev * Hev;
+    int cnt = 0;
+    for (int k = 0; k < ncache; ++k) {  // list of the returned H, in scan order
+        if (c_r2[k][t] < H2) {
+            if (cnt < p.cap) store_slot(nbr + lslot(cnt, i, N), c_j[k][t]);
+            ++cnt;
+        }
+    }
+    s.h[i] = Hev;
+    s.n[i] = n_of(Sv, Hev);
+    if (s.sd) s.sd[i] = sdv;
+    iters[i] = it;
+    ncount[i] = cnt;
+    if (!conv) {
+        set_status(st, GZ_S_HCONV, GZ_C_HCONV, s.id[i]);
+        if (b.clamped) atomicOr(&st->bits, GZ_S_HLIM);
+    }
+    if (cnt > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
+}
+
+// The particles k_density deferred (more candidates within 1.05 H than its
+// cache holds): one warp per particle, the same iteration.  The candidates
+// within 1.05 H are gathered once into a warp's cache of kWarpCache entries
+// (in scan order); later evaluations and the list read only that.  A particle
+// with more of them scans the cells at every evaluation.  Grid-stride over
+// the deferred list, whose length only the device knows.
+// The sums run as in k_density: the lanes form the entries' terms, then lane
+// c = 0..3 adds those of entries k mod 4 = c in order, so which kernel
+// iterates a particle does not change its bits.
+constexpr int kWarpDensBlock = 64;
+constexpr int kWarpCache = 512;
+
+template <typename T>
+__global__ void __launch_bounds__(kWarpDensBlock)
+    k_density_warp(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
+                   int* __restrict__ ncount, int* __restrict__ iters, DevStatus* st,
+                   const int* __restrict__ defer, const int* __restrict__ ndefer) {
+    constexpr unsigned full = 0xffffffffu;
+    __shared__ T w_r2[kWarpDensBlock / 32][kWarpCache];
+    __shared__ unsigned w_j[kWarpDensBlock / 32][kWarpCache];
+    __shared__ T w_t[kWarpDensBlock / 32][3][kWarpCache];
+    const int lane = threadIdx.x & 31;
+    T *t_w = w_t[threadIdx.x >> 5][0], *t_x = w_t[threadIdx.x >> 5][1], *t_y = w_t[threadIdx.x >> 5][2];
+    T* c_r2 = w_r2[threadIdx.x >> 5];
+    unsigned* c_j = w_j[threadIdx.x >> 5];
+    const int warps = gridDim.x * (kWarpDensBlock / 32);
+    const int nd = *ndefer;
+    for (int w = blockIdx.x * (kWarpDensBlock / 32) + (threadIdx.x >> 5); w < nd; w += warps) {
+        const int i = defer[w];
+        const BoxInfo bx = g.boxes[s.box[i]];
+        const P4<T> me = s.pos[i];
+        bool bad;  // (flagged by k_density)
+        T H = h_start<T>(s.h[i], bx, p, bad);
+        T Rc = T(-1), Hev = H, Sv = T(0), sdv = T(0);
+        int ncache = 0, it;
+        HIter<T> b;
+        bool conv = false;
+        for (it = 1; it <= p.max_iter; ++it) {
+            if (!(H <= Rc)) {
+                Rc = dens_cache_radius<T>(H, p);
+                __syncwarp();
+                ncache = for_hits_lanes_ordered<T>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, Rc * Rc, lane,
+                                                   [&](int k, int j, T r2) {
+                                                       if (k < kWarpCache) {
+                                                           c_r2[k] = r2;
+                                                           c_j[k] = (unsigned)j;
+                                                       }
+                                                   });
+                __syncwarp();
+            }
+            const T iH = T(1) / H;
+            Acc<T> sw;
+            T sd = T(0);
+            if (ncache <= kWarpCache) {
+                const int n4 = (ncache + 3) & ~3;
+                for (int k = lane; k < n4; k += 32) {
+                    T wv = T(0), x = T(0), y = T(0);
+                    if (k < ncache) dens_terms2(dist(c_r2[k]) * iH, wv, x, y);
+                    t_w[k] = wv;
+                    t_x[k] = x;
+                    t_y[k] = y;
+                }
+                __syncwarp();
+                if (lane < 4) {
+#pragma unroll 4
+                    for (int k = lane; k < n4; k += 4) {
+                        sw.add(t_w[k]);
+                        sd = fma(t_x[k], t_y[k], sd);
+                    }
+                }
+                const T S = group_sum<4>(full, sw), D = group_add<4>(full, sd);
+                Sv = T(2) * __shfl_sync(full, S, 0);
+                sdv = T(6) * __shfl_sync(full, D, 0);
+            } else {
+                const T H2 = H * H;
+                for_candidates_lanes<T>(g, bx, s.pos, i, me.x, me.y, me.z, H, lane, [&](int, T, T, T, T r2) {
+                    if (r2 < H2) {
+                        T wv, x, y;
+                        dens_terms2(dist(r2) * iH, wv, x, y);
+                        sw.add(wv);
+                        sd = fma(x, y, sd);
+                    }
+                });
+                __syncwarp();
+                Sv = T(2) * group_sum<32>(full, sw);
+                sdv = T(6) * group_add<32>(full, sd);
+            }
+            Hev = H;
+            if (h_step(b, H, Sv, sdv, p, it == p.max_iter)) {
+                conv = true;
+                break;
+            }
+        }
+        if (it > p.max_iter) it = p.max_iter;
+        // list of the returned H, in the order a thread's scan writes it
+        const T H2 = Hev * Hev;
+        int cnt = 0;
+        if (ncache <= kWarpCache) {
+            for (int k0 = 0; k0 < ncache; k0 += 32) {
+                const int k = k0 + lane;
+                const bool in = k < ncache && c_r2[k] < H2;
+                const unsigned m = __ballot_sync(full, in);
+                const int slot = cnt + __popc(m & ((1u << lane) - 1u));
+                if (in && slot < p.cap) store_slot(nbr + lslot(slot, i, N), c_j[k]);
+                cnt += __popc(m);
+            }
+        } else {
+            cnt = for_hits_lanes_ordered<T>(g, bx, s.pos, i, me.x, me.y, me.z, Hev, H2, lane, [&](int k, int j, T) {
+                if (k < p.cap) store_slot(nbr + lslot(k, i, N), (unsigned)j);
+            });
+        }
+        if (lane == 0) {
+            s.h[i] = Hev;
+            s.n[i] = n_of(Sv, Hev);
+            if (s.sd) s.sd[i] = sdv;
+            iters[i] = it;
+            ncount[i] = cnt;
+            if (!conv) {
+                set_status(st, GZ_S_HCONV, GZ_C_HCONV, s.id[i]);
+                if (b.clamped) atomicOr(&st->bits, GZ_S_HLIM);
+            }
+            if (cnt > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
+        }
+        __syncwarp();
+    }
+}
+
+// Neighbour lists N_i = {j : r_ij < H_i} for given H (O3).  only_over > 0:
+// only the particles whose count exceeds it (lists a checkpoint kept up to
+// that many slots; the others are restored from it).
+template <typename T>
+__global__ void __launch_bounds__(128)
+    k_lists(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
+            int* __restrict__ ncount, DevStatus* st, int only_over) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    if (only_over > 0 && ncount[i] <= only_over) return;
+    const BoxInfo bx = g.boxes[s.box[i]];
+    const T Hi = s.h[i];
+    const T H2 = Hi * Hi;
+    int c = 0;
+    const P4<T> me = s.pos[i];
+    for_candidates<T>(g, bx, s.pos, i, me.x, me.y, me.z, Hi,
+                      [&](int j, T, T, T, T r2) {
+                          if (r2 < H2) {
+                              if (c < p.cap) store_slot(nbr + lslot(c, i, N), (unsigned)j);
+                              ++c;
+                          }
+                      });
+    ncount[i] = c;
+    if (c > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
+}
+
+// Density pass for a known converged H (a step checkpoint's): the neighbour
+// list of H, n and the sum of -w'(q) q in one cell scan of radius H.  The
+// candidates inside H come in the h-iteration's scan order and are summed the
+// same way, so n and the sums equal the h-iteration's last evaluation bit
+// for bit.
+template <typename T>
+__global__ void __launch_bounds__(128)
+    k_dens_given(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
+                 int* __restrict__ ncount, DevStatus* st) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    const BoxInfo bx = g.boxes[s.box[i]];
+    const T Ht = s.h[i];
+    const T H2 = Ht * Ht;
+    const T iH = T(1) / Ht;
+    const P4<T> me = s.pos[i];
+    Acc<T> sw;
+    T sd = T(0);
+    int c = 0;
+    for_candidates<T>(g, bx, s.pos, i, me.x, me.y, me.z, Ht,
+                      [&](int j, T, T, T, T r2) {
+                          if (r2 < H2) {
+                              const T q = psqrt(r2) * iH;
+                              T w, qdw;
+                              dens_terms(q, w, qdw);
+                              sw.add(w);
+                              sd += qdw;
+                              if (c < p.cap) store_slot(nbr + lslot(c, i, N), (unsigned)j);
+                              ++c;
+                          }
+                      });
+    double S;
+    if constexpr (std::is_same<T, float>::value)
+        S = (double)sw.fvalue();  // as the h-iteration forms it
+    else
+        S = sw.value();
+    const double Hev = (double)Ht;
+    if (std::is_same<T, float>::value) {
+        const float Hf = (float)Hev;
+        s.n[i] = (T)(8.f * (float)(1.0 + S) / ((float)kPi * Hf * Hf * Hf));
+    } else {
+        s.n[i] = (T)(8.0 * (1.0 + S) / (kPi * Hev * Hev * Hev));
+    }
+    s.sd[i] = sd;
+    ncount[i] = c;
+    if (c > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
+}
+
+// Work of the cell scan at the converged H: per particle, the candidates a
+// scan of radius 1.05 H (the density cache's) tests, those inside 1.05 H and
+// those inside H; summed over the particles (out[0..2]).
+template <typename T>
+__global__ void __launch_bounds__(128)
+    k_scan_stats(int N, Sorted<T> s, Grid g, KParams p, unsigned long long* __restrict__ out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned long long v[3] = {0, 0, 0};
+    if (i < N) {
+        const BoxInfo bx = g.boxes[s.box[i]];
+        const P4<T> me = s.pos[i];
+        const T Ht = s.h[i];
+        const T R = dens_cache_radius<T>(Ht, p);
+        const T R2 = R * R, H2 = Ht * Ht;
+        for_candidates<T>(g, bx, s.pos, i, me.x, me.y, me.z, R, [&](int, T, T, T, T r2) {
+            if (r2 < T(1e29)) ++v[0];  // (slots past a cell's range read a far point)
+            if (r2 < R2) ++v[1];
+            if (r2 < H2) ++v[2];
+        });
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        unsigned long long x = v[k];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if ((threadIdx.x & 31) == 0 && x) atomicAdd(out + k, x);
+    }
+}
+
+}  // namespace
+
+static Grid grid_of(const Ctx& c) {
+    Grid g;
+    g.boxes = c.boxes;
+    g.cells = c.cells;
+    return g;
+}
+
+template <typename T>
+cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
+    if (!list) n = c.N;
+    if (n < 1) return cudaSuccess;
+    constexpr int P = kDensBlock / kLanes;
+    const Sorted<T> sv = sorted_view<T>(c);
+    // particles with more candidates within 1.05 H than their cache holds are
+    // iterated by a warp each.  k_density_one: 40 entries (the largest count
+    // seen on the workloads with N_ngb = 32) for boxes of 32^3 particles or
+    // more, 48 for smaller ones, whose strong contrasts overflow 40 more often
+    long long min_count = c.N;
+    for (const BoxInfo& b : c.hboxes) min_count = std::min(min_count, (long long)b.count);
+    const int asked = c.params.density_cache, ccap = asked > 0 ? asked : kDensCache;
+    const int tcap = asked > 0 ? asked : (min_count >= 32 * 32 * 32 ? 40 : 48);
+    c.launches += 2;
+    cudaMemsetAsync(c.ndefer, 0, sizeof(int), c.stream);
+    auto one = [&](auto kernel) {
+        kernel<<<blocks(n, kOneBlock), kOneBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
+                                                                 c.iters, c.status, list, nlist, c.defer,
+                                                                 c.ndefer);
+    };
+    bool done = false;
+    if constexpr (std::is_same<T, float>::value) {
+        if (n >= kThreadMin) {
+            if (tcap == 40)
+                one(k_density_one<40>);
+            else
+                one(k_density_one<48>);
+            done = true;
+        }
+    }
+    if (!done)
+        k_density<T><<<blocks(n, P), kDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
+                                                                 c.iters, c.status, list, nlist, c.defer,
+                                                                 c.ndefer, ccap);
+    const int wb = std::max(1, std::min(blocks(n, kWarpDensBlock / 32), 152 * 4));
+    k_density_warp<T><<<wb, kWarpDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
+                                                            c.iters, c.status, c.defer, c.ndefer);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t run_density_given(Ctx& c) {
+    c.launches += 1;
+    k_dens_given<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
+                                                             c.nbr, c.ncount, c.status);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t run_build_lists(Ctx& c) {
+    c.launches += 1;
+    k_lists<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
+                                                        c.nbr, c.ncount, c.status, 0);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t run_lists_over(Ctx& c, int kept) {
+    c.launches += 1;
+    k_lists<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
+                                                        c.nbr, c.ncount, c.status, kept);
+    return cudaGetLastError();
+}
+
+
+template <typename T>
+cudaError_t run_scan_stats(Ctx& c, long long* out_dev) {
+    c.launches += 1;
+    cudaError_t e = cudaMemsetAsync(out_dev, 0, 3 * sizeof(long long), c.stream);
+    if (e != cudaSuccess) return e;
+    k_scan_stats<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
+                                                             (unsigned long long*)out_dev);
+    return cudaGetLastError();
+}
+template cudaError_t run_scan_stats<float>(Ctx&, long long*);
+template cudaError_t run_scan_stats<double>(Ctx&, long long*);
+
+
+#define GZ_INST(T)                                                            \
+    template cudaError_t run_density<T>(Ctx&, const int*, const int*, int);   \
+    template cudaError_t run_density_given<T>(Ctx&);                          \
+    template cudaError_t run_build_lists<T>(Ctx&);                            \
+    template cudaError_t run_lists_over<T>(Ctx&, int);
+GZ_INST(float)
+GZ_INST(double)
+#undef GZ_INST
+
+}  // namespace gz

@@ -5,6 +5,8 @@
 // pair is either symmetric in its operands or evaluated in one fixed order of
 // the pair (pair_order), so both particles get bitwise-opposite
 // contributions (no atomics on rates).
+#include <math.h>
+
 #include <algorithm>
 #include <type_traits>
 
@@ -16,457 +18,6 @@ namespace gz {
 namespace {
 
 inline int blocks(int n, int t) { return (n + t - 1) / t; }
-
-// --------------------------------------------------------------- O4 / O5
-// Bracketed Newton iteration on f(H) = (4 pi/3) H^3 n(H) - N_ngb, written as
-// (32/3)(1 + sum_j w(q_j)) - N_ngb with f' = (32/3) sum_j (-w'(q_j)) q_j / H.
-// The first evaluation scans the cells once with radius Rc = 1.05 H and keeps
-// (r^2, j) of the candidates inside Rc in shared memory; later evaluations
-// read only that cache (rebuilt if H grows past Rc).  A particle with more
-// than kDensCache candidates falls back to scanning the cells at every
-// evaluation.  The neighbour list of the returned H is written at the end.
-constexpr int kDensBlock = 64;
-// Cache entries per thread: 40 (the largest count within 1.05 H seen on the
-// workloads with N_ngb = 32) for boxes of 32^3 particles or more, where the
-// smaller cache buys occupancy; 48 for smaller boxes, whose strong contrasts
-// (blasts in a few thousand particles) overflow 40 more often.
-constexpr int kDensCacheLarge = 40, kDensCacheSmall = 48;
-
-// Radius of the candidate cache for a support Ht: 5% headroom so that small
-// growth of H during the iteration needs no rescan, never past h_lim.
-template <typename T>
-__device__ __forceinline__ T dens_cache_radius(T Ht, const KParams& p) {
-    T R = Ht * T(1.05);
-    if (!(R < (T)p.h_lim)) R = max(Ht, (T)p.h_lim);
-    return R;
-}
-
-// Rescan into the thread's shared-memory cache (the support grew past the
-// cache radius): kept out of line so that the iteration loop holds no scan
-// state; returns the number of candidates within R.
-template <typename T, int kDensCache>
-__device__ __noinline__ int dens_fill(const Grid& g, const BoxInfo& bx, const P4<T>* __restrict__ pos, int i,
-                                      T xi, T yi, T zi, T R, T (*c_r2)[kDensBlock],
-                                      unsigned (*c_j)[kDensBlock], int t) {
-    const T R2 = R * R;
-    int n = 0;
-    for_candidates<T>(g, bx, pos, i, xi, yi, zi, R, [&](int j, T, T, T, T r2) {
-        if (r2 < R2) {
-            if (n < kDensCache) {
-                c_r2[n][t] = r2;
-                c_j[n][t] = (unsigned)j;
-            }
-            ++n;
-        }
-    });
-    return n;
-}
-
-// One evaluation straight from the cells (more candidates than the cache
-// holds and no deferral): the sums and the neighbour list of Ht.
-template <typename T>
-__device__ __noinline__ void dens_eval_cells(const Grid& g, const BoxInfo& bx, const P4<T>* __restrict__ pos,
-                                             int i, T xi, T yi, T zi, T Ht, unsigned* __restrict__ col, int cap,
-                                             int N, Acc<T>& sw, T& sd, int& c) {
-    const T H2 = Ht * Ht;
-    const T iH = T(1) / Ht;
-    for_candidates<T>(g, bx, pos, i, xi, yi, zi, Ht, [&](int j, T, T, T, T r2) {
-        if (r2 < H2) {
-            const T q = psqrt(r2) * iH;
-            T w, qdw;
-            dens_terms(q, w, qdw);
-            sw.add(w);
-            sd += qdw;
-            if (c < cap) store_slot(col + lcol(c, N), (unsigned)j);
-            ++c;
-        }
-    });
-}
-
-// FP32: held to 96 registers (10 blocks of 64 per SM; the cache of 40 allows
-// 10 to 11), which measured faster than 119 unspilled registers at 8 blocks.
-template <typename T, int kDensCache>
-__global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 10 : 1)
-    k_density(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
-              int* __restrict__ ncount, int* __restrict__ iters, DevStatus* st,
-              const int* __restrict__ list, const int* __restrict__ nlist, int* __restrict__ defer,
-              int* __restrict__ ndefer) {
-    __shared__ T c_r2[kDensCache][kDensBlock];
-    __shared__ unsigned c_j[kDensCache][kDensBlock];
-    const int t = threadIdx.x;
-    int i = blockIdx.x * kDensBlock + t;
-    if (list) {  // the particles of an index list only (hierarchical steps)
-        if (i >= *nlist) return;
-        i = list[i];
-    } else if (i >= N) {
-        return;
-    }
-    const BoxInfo bx = g.boxes[s.box[i]];
-    const P4<T> me = s.pos[i];
-    const T xi = me.x, yi = me.y, zi = me.z;
-    double H = (double)s.h[i];
-    if (!(H > 0.0) || !(H < p.h_lim)) {
-        set_status(st, GZ_S_NONFINITE, GZ_C_NONFINITE, s.id[i]);
-        H = cbrt(3.0 * p.ngb / (4.0 * kPi * (double)bx.count));
-        if (!(H < p.h_lim)) H = 0.5 * p.h_lim;
-    }
-    // the cache of the starting H, scanned before the iteration (few live
-    // values here, the iteration's FP64 state not yet among them)
-    T Rc;
-    int ncache;
-    bool cached;
-    {
-        Rc = dens_cache_radius<T>((T)H, p);
-        const T R2 = Rc * Rc;
-        int n = 0;
-        for_candidates<T>(g, bx, s.pos, i, xi, yi, zi, Rc, [&](int j, T, T, T, T r2) {
-            if (r2 < R2) {
-                if (n < kDensCache) {
-                    c_r2[n][t] = r2;
-                    c_j[n][t] = (unsigned)j;
-                }
-                ++n;
-            }
-        });
-        ncache = n;
-        cached = n <= kDensCache;
-        if (!cached && defer) {
-            // more candidates than the cache holds (a support spanning many
-            // cells): left to k_density_warp, where a whole warp scans for
-            // it and runs the iteration from the starting H
-            defer[atomicAdd(ndefer, 1)] = i;
-            return;
-        }
-    }
-    const double C = 32.0 / 3.0;
-    double lo = 0.0, hi = 0.0, S = 0.0, Hev = H;
-    bool has_lo = false, has_hi = false, conv = false, clamped = false;
-    T sd_last = T(0);
-    int it, cnt = 0;
-    for (it = 1; it <= p.max_iter; ++it) {
-        const T Ht = (T)H;
-        const T H2 = Ht * Ht;
-        const T iH = T(1) / Ht;
-        if (!cached || Ht > Rc) {  // grew past the cache radius: rescan
-            Rc = dens_cache_radius<T>(Ht, p);
-            ncache = dens_fill<T, kDensCache>(g, bx, s.pos, i, xi, yi, zi, Rc, c_r2, c_j, t);
-            cached = ncache <= kDensCache;
-            if (!cached && defer) {
-                defer[atomicAdd(ndefer, 1)] = i;
-                return;
-            }
-        }
-        Acc<T> sw;
-        T sd = T(0);
-        int c = 0;
-        if (cached) {
-            for (int k = 0; k < ncache; ++k) {
-                const T r2 = c_r2[k][t];
-                if (r2 < H2) {
-                    const T q = psqrt(r2) * iH;
-                    T w, qdw;
-                    dens_terms(q, w, qdw);
-                    sw.add(w);
-                    sd += qdw;
-                    ++c;
-                }
-            }
-        } else {
-            dens_eval_cells<T>(g, bx, s.pos, i, xi, yi, zi, Ht, nbr + 4 * (size_t)i, p.cap, N, sw, sd, c);
-        }
-        cnt = c;
-        sd_last = sd;
-        Hev = (double)Ht;
-        // f = (32/3)(1 + S) - N_ngb.  FP32 path: in FP32 (its rounding, about
-        // 4e-6, is well inside the stop tolerance 1e-6 N_ngb); H, the bracket
-        // and the update below stay FP64
-        double f;
-        if constexpr (std::is_same<T, float>::value) {
-            const float Sf = sw.fvalue();
-            S = (double)Sf;
-            f = (double)((32.f / 3.f) * (1.f + Sf) - (float)p.ngb);
-        } else {
-            S = sw.value();
-            f = C * (1.0 + S) - p.ngb;
-        }
-        if (fabs(f) <= p.tol * p.ngb) {
-            conv = true;
-            break;
-        }
-        if (it == p.max_iter) break;
-        if (f < 0.0) {
-            lo = Hev;
-            has_lo = true;
-        } else {
-            hi = Hev;
-            has_hi = true;
-        }
-        const double lo_eff = has_lo ? lo : 0.5 * Hev;
-        const double hi_eff = has_hi ? hi : 2.0 * Hev;
-        double Hn = 0.0;
-        bool ok = false;
-        // Newton step H - f / f' with f' = C sd / H.  H and the update stay
-        // FP64; on the FP32 path the quotient f / f' (only its leading digits
-        // matter to the step) is formed in FP32, sparing two FP64 divisions
-        // an iteration on a part whose FP64 rate is 1/64 of FP32.
-        if (std::is_same<T, float>::value) {
-            const float fpf = (float)C * (float)sd / Ht;
-            if (fpf > 0.f) {
-                Hn = Hev - (double)((float)f / fpf);
-                ok = (Hn > lo_eff) && (Hn < hi_eff);
-            }
-        } else {
-            const double fp = C * (double)sd / Hev;
-            if (fp > 0.0) {
-                Hn = Hev - f / fp;
-                ok = (Hn > lo_eff) && (Hn < hi_eff);
-            }
-        }
-        if (!ok) Hn = (has_lo && has_hi) ? 0.5 * (lo + hi) : (f < 0.0 ? 2.0 * Hev : 0.5 * Hev);
-        if (Hn >= p.h_lim) {
-            Hn = 0.5 * (Hev + p.h_lim);
-            clamped = true;
-        }
-        H = Hn;
-    }
-    if (it > p.max_iter) it = p.max_iter;
-    if (cached) {  // list of the returned H, in scan order
-        const T Ht = (T)Hev;
-        const T H2 = Ht * Ht;
-        int c = 0;
-        for (int k = 0; k < ncache; ++k) {
-            if (c_r2[k][t] < H2) {
-                if (c < p.cap) store_slot(nbr + lslot(c, i, N), c_j[k][t]);
-                ++c;
-            }
-        }
-    }
-    s.h[i] = (T)Hev;
-    if (std::is_same<T, float>::value) {  // FP32 path: no FP64 division per particle
-        const float Hf = (float)Hev;
-        s.n[i] = (T)(8.f * (float)(1.0 + S) / ((float)kPi * Hf * Hf * Hf));
-    } else {
-        s.n[i] = (T)(8.0 * (1.0 + S) / (kPi * Hev * Hev * Hev));
-    }
-    if (s.sd) s.sd[i] = sd_last;  // (absent in the allocation-free density call)
-    iters[i] = it;
-    ncount[i] = cnt;
-    if (!conv) {
-        set_status(st, GZ_S_HCONV, GZ_C_HCONV, s.id[i]);
-        if (clamped) atomicOr(&st->bits, GZ_S_HLIM);
-    }
-    if (cnt > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
-}
-
-// The particles k_density deferred (more candidates within 1.05 H than its
-// cache holds): one warp per particle, the same bracketed Newton iteration,
-// each evaluation a warp-cooperative scan (for_candidates_lanes; sums reduced
-// across the warp in FP64, so every lane holds the same totals and takes the
-// same steps); the neighbour list of the returned H lane by lane.  Grid-stride over the deferred
-// list, whose length only the device knows.
-constexpr int kWarpDensBlock = 128;
-
-template <typename T>
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kWarpDensBlock)
-    k_density_warp(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
-                   int* __restrict__ ncount, int* __restrict__ iters, DevStatus* st,
-                   const int* __restrict__ defer, const int* __restrict__ ndefer) {
-    const int lane = threadIdx.x & 31;
-    const int warps = gridDim.x * (kWarpDensBlock / 32);
-    const int nd = *ndefer;
-    for (int w = blockIdx.x * (kWarpDensBlock / 32) + (threadIdx.x >> 5); w < nd; w += warps) {
-        const int i = defer[w];
-        const BoxInfo bx = g.boxes[s.box[i]];
-        const P4<T> me = s.pos[i];
-        const T xi = me.x, yi = me.y, zi = me.z;
-        double H = (double)s.h[i];
-        if (!(H > 0.0) || !(H < p.h_lim)) {  // (flagged by k_density)
-            H = cbrt(3.0 * p.ngb / (4.0 * kPi * (double)bx.count));
-            if (!(H < p.h_lim)) H = 0.5 * p.h_lim;
-        }
-        const double C = 32.0 / 3.0;
-        double lo = 0.0, hi = 0.0, S = 0.0, Hev = H;
-        bool has_lo = false, has_hi = false, conv = false, clamped = false;
-        T sd_last = T(0);
-        int it, cnt = 0;
-        for (it = 1; it <= p.max_iter; ++it) {
-            const T Ht = (T)H;
-            const T H2 = Ht * Ht;
-            const T iH = T(1) / Ht;
-            Acc<T> sw;
-            T sd = T(0);
-            int c = 0;
-            for_candidates_lanes<T>(g, bx, s.pos, i, xi, yi, zi, Ht, lane, [&](int, T, T, T, T r2) {
-                if (r2 < H2) {
-                    const T q = psqrt(r2) * iH;
-                    T w, qdw;
-                    dens_terms(q, w, qdw);
-                    sw.add(w);
-                    sd += qdw;
-                    ++c;
-                }
-            });
-            const double Sw = warp_sum<T>(sw.value());
-            const T sdw = (T)warp_sum<T>((double)sd);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-            cnt = c;
-            sd_last = sdw;
-            Hev = (double)Ht;
-            double f;
-            if constexpr (std::is_same<T, float>::value) {
-                const float Sf = (float)Sw;
-                S = (double)Sf;
-                f = (double)((32.f / 3.f) * (1.f + Sf) - (float)p.ngb);
-            } else {
-                S = Sw;
-                f = C * (1.0 + S) - p.ngb;
-            }
-            if (fabs(f) <= p.tol * p.ngb) {
-                conv = true;
-                break;
-            }
-            if (it == p.max_iter) break;
-            if (f < 0.0) {
-                lo = Hev;
-                has_lo = true;
-            } else {
-                hi = Hev;
-                has_hi = true;
-            }
-            const double lo_eff = has_lo ? lo : 0.5 * Hev;
-            const double hi_eff = has_hi ? hi : 2.0 * Hev;
-            double Hn = 0.0;
-            bool ok = false;
-            if (std::is_same<T, float>::value) {
-                const float fpf = (float)C * (float)sdw / Ht;
-                if (fpf > 0.f) {
-                    Hn = Hev - (double)((float)f / fpf);
-                    ok = (Hn > lo_eff) && (Hn < hi_eff);
-                }
-            } else {
-                const double fp = C * (double)sdw / Hev;
-                if (fp > 0.0) {
-                    Hn = Hev - f / fp;
-                    ok = (Hn > lo_eff) && (Hn < hi_eff);
-                }
-            }
-            if (!ok) Hn = (has_lo && has_hi) ? 0.5 * (lo + hi) : (f < 0.0 ? 2.0 * Hev : 0.5 * Hev);
-            if (Hn >= p.h_lim) {
-                Hn = 0.5 * (Hev + p.h_lim);
-                clamped = true;
-            }
-            H = Hn;
-        }
-        if (it > p.max_iter) it = p.max_iter;
-        {  // list of the returned H, in the order a thread's scan writes it (the
-           // order of k_density, k_dens_given and k_lists)
-            const T Ht = (T)Hev;
-            for_hits_lanes_ordered<T>(g, bx, s.pos, i, xi, yi, zi, Ht, Ht * Ht, lane, [&](int k, int j) {
-                if (k < p.cap) store_slot(nbr + lslot(k, i, N), (unsigned)j);
-            });
-        }
-        if (lane == 0) {
-            s.h[i] = (T)Hev;
-            if (std::is_same<T, float>::value) {
-                const float Hf = (float)Hev;
-                s.n[i] = (T)(8.f * (float)(1.0 + S) / ((float)kPi * Hf * Hf * Hf));
-            } else {
-                s.n[i] = (T)(8.0 * (1.0 + S) / (kPi * Hev * Hev * Hev));
-            }
-            if (s.sd) s.sd[i] = sd_last;
-            iters[i] = it;
-            ncount[i] = cnt;
-            if (!conv) {
-                set_status(st, GZ_S_HCONV, GZ_C_HCONV, s.id[i]);
-                if (clamped) atomicOr(&st->bits, GZ_S_HLIM);
-            }
-            if (cnt > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
-        }
-        __syncwarp();
-    }
-}
-
-// Neighbour lists N_i = {j : r_ij < H_i} for given H (O3).  only_over > 0:
-// only the particles whose count exceeds it (lists a checkpoint kept up to
-// that many slots; the others are restored from it).
-template <typename T>
-__global__ void __launch_bounds__(128)
-    k_lists(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
-            int* __restrict__ ncount, DevStatus* st, int only_over) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    if (only_over > 0 && ncount[i] <= only_over) return;
-    const BoxInfo bx = g.boxes[s.box[i]];
-    const T Hi = s.h[i];
-    const T H2 = Hi * Hi;
-    int c = 0;
-    const P4<T> me = s.pos[i];
-    for_candidates<T>(g, bx, s.pos, i, me.x, me.y, me.z, Hi,
-                      [&](int j, T, T, T, T r2) {
-                          if (r2 < H2) {
-                              if (c < p.cap) store_slot(nbr + lslot(c, i, N), (unsigned)j);
-                              ++c;
-                          }
-                      });
-    ncount[i] = c;
-    if (c > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
-}
-
-// Density pass for a known converged H (a step checkpoint's): the neighbour
-// list of H, n and the sum of -w'(q) q in one cell scan of radius H.  The
-// candidates inside H come in the h-iteration's scan order and are summed the
-// same way, so n and the sums equal the h-iteration's last evaluation bit
-// for bit.
-template <typename T>
-__global__ void __launch_bounds__(128)
-    k_dens_given(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
-                 int* __restrict__ ncount, DevStatus* st) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const BoxInfo bx = g.boxes[s.box[i]];
-    const T Ht = s.h[i];
-    const T H2 = Ht * Ht;
-    const T iH = T(1) / Ht;
-    const P4<T> me = s.pos[i];
-    Acc<T> sw;
-    T sd = T(0);
-    int c = 0;
-    for_candidates<T>(g, bx, s.pos, i, me.x, me.y, me.z, Ht,
-                      [&](int j, T, T, T, T r2) {
-                          if (r2 < H2) {
-                              const T q = psqrt(r2) * iH;
-                              T w, qdw;
-                              dens_terms(q, w, qdw);
-                              sw.add(w);
-                              sd += qdw;
-                              if (c < p.cap) store_slot(nbr + lslot(c, i, N), (unsigned)j);
-                              ++c;
-                          }
-                      });
-    double S;
-    if constexpr (std::is_same<T, float>::value)
-        S = (double)sw.fvalue();  // as the h-iteration forms it
-    else
-        S = sw.value();
-    const double Hev = (double)Ht;
-    if (std::is_same<T, float>::value) {
-        const float Hf = (float)Hev;
-        s.n[i] = (T)(8.f * (float)(1.0 + S) / ((float)kPi * Hf * Hf * Hf));
-    } else {
-        s.n[i] = (T)(8.0 * (1.0 + S) / (kPi * Hev * Hev * Hev));
-    }
-    s.sd[i] = sd;
-    ncount[i] = c;
-    if (c > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
-}
 
 // Reverse pairs (O10): j in N_i with r_ij >= H_j is appended to j's list.
 // Reads the packed positions, whose w component is the converged H.
@@ -1155,34 +706,6 @@ __global__ void k_pairs(int N, const int* __restrict__ ncount, const int* __rest
     if ((threadIdx.x & 31) == 0) atomicAdd((unsigned long long*)out, (unsigned long long)v);
 }
 
-// Work of the cell scan at the converged H: per particle, the candidates a
-// scan of radius 1.05 H (the density cache's) tests, those inside 1.05 H and
-// those inside H; summed over the particles (out[0..2]).
-template <typename T>
-__global__ void __launch_bounds__(128)
-    k_scan_stats(int N, Sorted<T> s, Grid g, KParams p, unsigned long long* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long v[3] = {0, 0, 0};
-    if (i < N) {
-        const BoxInfo bx = g.boxes[s.box[i]];
-        const P4<T> me = s.pos[i];
-        const T Ht = s.h[i];
-        const T R = dens_cache_radius<T>(Ht, p);
-        const T R2 = R * R, H2 = Ht * Ht;
-        for_candidates<T>(g, bx, s.pos, i, me.x, me.y, me.z, R, [&](int, T, T, T, T r2) {
-            if (r2 < T(1e29)) ++v[0];  // (slots past a cell's range read a far point)
-            if (r2 < R2) ++v[1];
-            if (r2 < H2) ++v[2];
-        });
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        unsigned long long x = v[k];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if ((threadIdx.x & 31) == 0 && x) atomicAdd(out + k, x);
-    }
-}
-
 }  // namespace
 
 cudaError_t run_pair_count(Ctx& c, long long* out_dev) {
@@ -1205,80 +728,15 @@ KParams kparams(const Ctx& c) {
     k.hancock = c.params.hancock;
     k.scheme = c.params.scheme;
     k.max_iter = c.params.max_iter;
+    const double tn = c.params.tol * c.params.ngb;
+    k.dtol = tn;
+    k.ftol = (float)tn;
+    if ((double)k.ftol > tn) k.ftol = nextafterf(k.ftol, 0.f);
+    k.hlimf = (float)c.params.h_lim;
+    if ((double)k.hlimf < c.params.h_lim) k.hlimf = nextafterf(k.hlimf, 1.f);
     k.cap = c.cap;
     k.rcap = c.rcap;
     return k;
-}
-
-static Grid grid_of(const Ctx& c) {
-    Grid g;
-    g.boxes = c.boxes;
-    g.cells = c.cells;
-    return g;
-}
-
-template <typename T>
-cudaError_t run_scan_stats(Ctx& c, long long* out_dev) {
-    c.launches += 1;
-    cudaError_t e = cudaMemsetAsync(out_dev, 0, 3 * sizeof(long long), c.stream);
-    if (e != cudaSuccess) return e;
-    k_scan_stats<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
-                                                             (unsigned long long*)out_dev);
-    return cudaGetLastError();
-}
-template cudaError_t run_scan_stats<float>(Ctx&, long long*);
-template cudaError_t run_scan_stats<double>(Ctx&, long long*);
-
-template <typename T>
-cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
-    if (!list) n = c.N;
-    if (n < 1) return cudaSuccess;
-    long long min_count = c.N;
-    for (const BoxInfo& b : c.hboxes) min_count = std::min(min_count, (long long)b.count);
-    if (c.grid_count > 0) min_count = c.grid_count;  // a subdomain: as the whole box
-    if (c.params.density_cache == kDensCacheLarge) min_count = 32 * 32 * 32;
-    if (c.params.density_cache == kDensCacheSmall) min_count = 0;
-    const Sorted<T> sv = sorted_view<T>(c);
-    c.launches += c.defer ? 2 : 1;
-    if (c.defer) cudaMemsetAsync(c.ndefer, 0, sizeof(int), c.stream);
-    if (min_count >= 32 * 32 * 32)
-        k_density<T, kDensCacheLarge><<<blocks(n, kDensBlock), kDensBlock, 0, c.stream>>>(
-            c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount, c.iters, c.status, list, nlist, c.defer,
-            c.ndefer);
-    else
-        k_density<T, kDensCacheSmall><<<blocks(n, kDensBlock), kDensBlock, 0, c.stream>>>(
-            c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount, c.iters, c.status, list, nlist, c.defer,
-            c.ndefer);
-    if (c.defer) {
-        const int wb = std::max(1, std::min(blocks(n, kWarpDensBlock / 32), 152 * 4));
-        k_density_warp<T><<<wb, kWarpDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
-                                                                c.iters, c.status, c.defer, c.ndefer);
-    }
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t run_density_given(Ctx& c) {
-    c.launches += 1;
-    k_dens_given<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
-                                                             c.nbr, c.ncount, c.status);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t run_build_lists(Ctx& c) {
-    c.launches += 1;
-    k_lists<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
-                                                        c.nbr, c.ncount, c.status, 0);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t run_lists_over(Ctx& c, int kept) {
-    c.launches += 1;
-    k_lists<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
-                                                        c.nbr, c.ncount, c.status, kept);
-    return cudaGetLastError();
 }
 
 template <typename T>
@@ -1455,10 +913,6 @@ cudaError_t run_get_neighbours(Ctx& c, int32_t* count_out, int64_t* ids_out, int
 }
 
 #define GZ_INST(T)                                                   \
-    template cudaError_t run_density<T>(Ctx&, const int*, const int*, int);                    \
-    template cudaError_t run_density_given<T>(Ctx&);                                            \
-    template cudaError_t run_build_lists<T>(Ctx&);                                              \
-    template cudaError_t run_lists_over<T>(Ctx&, int);                                          \
     template cudaError_t run_reverse<T>(Ctx&);                                                  \
     template cudaError_t run_prim<T>(Ctx&);                                                     \
     template cudaError_t run_gradients<T>(Ctx&, bool, bool, const int*, const int*, int);      \

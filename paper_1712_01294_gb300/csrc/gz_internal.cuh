@@ -39,6 +39,8 @@ struct BoxInfo {
 // Scalar parameters passed by value to kernels.
 struct KParams {
     double gamma, ngb, tol, cfl, kappa_max, beta, u_floor_frac, h_lim;
+    double dtol;        // tol * ngb
+    float ftol, hlimf;  // tol * ngb rounded down, h_lim rounded up (the same tests on FP32 numbers)
     int hancock, max_iter, cap, rcap, scheme;
 };
 
@@ -186,13 +188,19 @@ __device__ __forceinline__ void set_status(DevStatus* st, unsigned bit, int coun
 }
 
 // --------------------------------------------------------- O1 min image
-// FP64: exactly the oracle's expression (difference, then shift by one).
+// FP64: exactly the oracle's expression (difference, then shift by one where
+// d >= 1/2 or d < -1/2).  The two comparisons are made on d's words: the FP64
+// pipe runs at 1/64 of the FP32 rate and is what bounds every FP64 pass, and
+// most pairs then cost it the one subtraction.
 __device__ __forceinline__ double mi_diff(double xj, double xi, double /*xim1*/) {
     double d = xj - xi;
-    if (d >= 0.5)
-        d = d - 1.0;
-    else if (d < -0.5)
-        d = d + 1.0;
+    const unsigned h = (unsigned)__double2hiint(d);
+    if ((h & 0x7fffffffu) >= 0x3FE00000u) {  // |d| >= 1/2 (or NaN)
+        if ((int)h >= 0)
+            d = d - 1.0;
+        else if (h > 0xBFE00000u || __double2loint(d) != 0)
+            d = d + 1.0;
+    }
     return d;
 }
 // FP32: shift the operand near 1 first (x - 1 is exact for x in [1/2, 1)),
@@ -479,96 +487,285 @@ __device__ __forceinline__ void for_candidates_lanes(const Grid& g, const BoxInf
     }
 }
 
+// The FP32 number below a position x in [0, 1] (its leading 24 bits), formed
+// from its words: a conversion would go through the FP64 pipe, whose rate is
+// 1/64 of FP32's.  (Numbers below 2^-126 give 0 or a denormal.)
+__device__ __forceinline__ float chop(double x) {
+    const int h = max(__double2hiint(x), 0x38000000);
+    return __int_as_float(((h - 0x38000000) << 3) | (int)((unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ float chop(float x) { return x; }
+
+// Search window of a particle: the cells overlapping [x - R, x + R] (periodic),
+// their offsets and the tests for_candidates applies to them, with the cells
+// numbered in its loop order.
+template <typename T>
+struct Window {
+    int lo[3], ex, exy, ncube, nc;
+    float R2m, cl, rex, rexy;
+    bool wraps_all, percell;
+    __device__ __forceinline__ Window(int nc_, T xi, T yi, T zi, T R) : nc(nc_) {
+        ncube = 0;
+        // positions outside [0, 1] (flagged by the binning pass) see no candidates
+        if (!(xi >= T(0) && xi <= T(1) && yi >= T(0) && yi <= T(1) && zi >= T(0) && zi <= T(1) && R >= T(0))) return;
+        const bool full = !(R < T(0.5));  // (also catches non-finite R)
+        const T c3[3] = {xi, yi, zi};
+        int n[3];
+        wraps_all = full;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = full ? 0 : (int)floor((c3[a] - R) * (T)nc - T(1e-3));
+            int hi = full ? nc - 1 : (int)floor((c3[a] + R) * (T)nc + T(1e-3));
+            if (hi - lo[a] + 1 >= nc) {
+                lo[a] = 0;
+                hi = nc - 1;
+                wraps_all = true;
+            }
+            n[a] = hi - lo[a] + 1;
+        }
+        ex = n[0];
+        exy = n[0] * n[1];
+        ncube = exy * n[2];
+        rex = __frcp_rn((float)ex);
+        rexy = __frcp_rn((float)exy);
+        cl = 1.f / (float)nc;
+        const float Rf = (float)R + (sizeof(T) == 8 ? 4e-7f : 0.f);
+        R2m = Rf * Rf * 1.0001f;
+        percell = sizeof(T) == 4 && !wraps_all && (2.f * Rf + 2.f * cl < 0.5f);
+    }
+    // Coordinates of cell f of the window (x fastest), unwrapped.  The float
+    // quotients are off by at most one, corrected after.
+    __device__ __forceinline__ void coords(int f, int& cx, int& cy, int& cz) const {
+        int z = (int)(((float)f + 0.5f) * rexy);
+        int rem = f - z * exy;
+        if (rem < 0) {
+            --z;
+            rem += exy;
+        } else if (rem >= exy) {
+            ++z;
+            rem -= exy;
+        }
+        int y = (int)(((float)rem + 0.5f) * rex);
+        int x = rem - y * ex;
+        if (x < 0) {
+            --y;
+            x += ex;
+        } else if (x >= ex) {
+            ++y;
+            x -= ex;
+        }
+        cx = lo[0] + x;
+        cy = lo[1] + y;
+        cz = lo[2] + z;
+    }
+    // Candidates of cell (cx, cy, cz): none when its nearest point lies beyond R.
+    // In FP32 for both precisions: the margin on R^2 covers the rounding of the
+    // cell bounds and of the FP32 copies of x and R.
+    __device__ __forceinline__ int2 range(const int2* __restrict__ cells, int cx, int cy, int cz, float xi, float yi,
+                                          float zi) const {
+        auto gap = [&](int c, float v) {
+            return wraps_all ? 0.f : max(max((float)c * cl - v, v - (float)(c + 1) * cl), 0.f);
+        };
+        const float gx = gap(cx, xi), gy = gap(cy, yi), gz = gap(cz, zi);
+        if ((gz * gz + gy * gy) + gx * gx > R2m) return make_int2(0, 0);
+        const int wx = cx < 0 ? cx + nc : (cx >= nc ? cx - nc : cx);
+        const int wy = cy < 0 ? cy + nc : (cy >= nc ? cy - nc : cy);
+        const int wz = cz < 0 ? cz + nc : (cz >= nc ? cz - nc : cz);
+        return cells[(wz * nc + wy) * nc + wx];
+    }
+};
+
+template <int G>
+__device__ __forceinline__ unsigned group_mask() {
+    static_assert(G >= 2 && G <= 32 && (G & (G - 1)) == 0, "a group is a power of two of lanes");
+    return (0xffffffffu >> (32 - G)) << (threadIdx.x & 31 & ~(G - 1));
+}
+
+// Squared distance of two chopped positions in FP32 and the bound below which
+// every pair with r < R falls: chop and the subtraction put at most 1.8e-7 on
+// an axis (3.2e-7 on r), the squares and sums 3 rounding errors.
+__device__ __forceinline__ float r2_chop(double xj, double yj, double zj, float xi, float yi, float zi) {
+    float dx = chop(xj) - xi, dy = chop(yj) - yi, dz = chop(zj) - zi;
+    dx -= rintf(dx);
+    dy -= rintf(dy);
+    dz -= rintf(dz);
+    return fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+}
+__device__ __forceinline__ float r2_chop_bound(double R) {
+    const float r = ((float)R + 4e-7f) * (1.f + 1e-6f);
+    return r * r;
+}
+
+// Scan of one particle's search window by the G lanes of its group (all of
+// them pass the same particle): the candidates j != self with r^2 < R^2,
+// handed to emit(k, j) with k = 0, 1, ... in for_candidates' order (cells in
+// its loop order, j ascending within a cell), each by one lane of the group.
+// A round takes G cells, one a lane: the lane tests its cell's candidates
+// into a bit mask, a prefix sum over the group numbers the hits, and the lane
+// hands its set bits over (a few instructions each: lanes have unequal hits,
+// so what is done per hit is left to the caller's pass over the numbered
+// hits, where every lane is busy).  Returns the number of hits (the same for
+// every lane); stops early once there are more than `most`.
+// FP64: the mask comes from FP32 distances with a margin, so the FP64 pipe
+// sees only the hits; candidates up to 5e-7 outside R are handed over too.
+template <typename T, int G, typename E>
+__device__ __forceinline__ int group_scan(const Grid& g, const BoxInfo& bx, const P4<T>* __restrict__ pos,
+                                          int self, T xi, T yi, T zi, T R, int gl, unsigned gm, int most,
+                                          E&& emit) {
+    const Window<T> w(bx.nc, xi, yi, zi, R);
+    const int2* __restrict__ cells = g.cells + bx.cell_off;
+    const T xim1 = xi - T(1), yim1 = yi - T(1), zim1 = zi - T(1);
+    const T R2 = R * R;
+    const float xf = chop(xi), yf = chop(yi), zf = chop(zi);
+    const float R2f = sizeof(T) == 8 ? r2_chop_bound((double)R) : 0.f;
+    int base = 0;
+    for (int f0 = 0; f0 < w.ncube; f0 += G) {
+        int2 se = make_int2(0, 0);
+        // FP32 well inside half the box: the periodic shift of the cell,
+        // (x_j + a) - b, the same correctly rounded offsets mi_diff gives
+        T ax = T(0), ay = T(0), az = T(0), bxx = xi, byy = yi, bzz = zi;
+        if (f0 + gl < w.ncube) {
+            int cx, cy, cz;
+            w.coords(f0 + gl, cx, cy, cz);
+            se = w.range(cells, cx, cy, cz, xf, yf, zf);
+            if (sizeof(T) == 4 && w.percell) {
+                ax = cx < 0 ? T(-1) : T(0);
+                ay = cy < 0 ? T(-1) : T(0);
+                az = cz < 0 ? T(-1) : T(0);
+                bxx = cx >= w.nc ? xim1 : xi;
+                byy = cy >= w.nc ? yim1 : yi;
+                bzz = cz >= w.nc ? zim1 : zi;
+            }
+        }
+        auto near = [&](const P4<T>& q) {
+            if constexpr (sizeof(T) == 8) return r2_chop(q.x, q.y, q.z, xf, yf, zf) < R2f;
+            if (w.percell) return sep2((q.x + ax) - bxx, (q.y + ay) - byy, (q.z + az) - bzz) < R2;
+            return sep2(mi_diff(q.x, xi, xim1), mi_diff(q.y, yi, yim1), mi_diff(q.z, zi, zim1)) < R2;
+        };
+        unsigned m = 0;  // hits among the cell's first 32 candidates
+        const int end = min(se.y, se.x + 32), last = se.y - 1;
+        auto test4 = [&](auto hit) {
+            for (int j0 = se.x; j0 < end; j0 += 4) {
+                P4<T> q[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) q[u] = pos[min(j0 + u, last)];
+                unsigned n4 = 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (hit(q[u])) n4 |= 1u << u;
+                m |= n4 << (j0 - se.x);
+            }
+        };
+        if constexpr (sizeof(T) == 8)
+            test4(near);
+        else if (w.percell)
+            test4([&](const P4<T>& q) { return sep2((q.x + ax) - bxx, (q.y + ay) - byy, (q.z + az) - bzz) < R2; });
+        else
+            test4(near);
+        const int nj = se.y - se.x;
+        if (nj < 32) m &= (1u << nj) - 1u;  // (the last group of four repeats the last candidate)
+        if (self >= se.x && self < end) m &= ~(1u << (self - se.x));
+        int more = 0;  // hits past the cell's first 32 candidates
+        for (int j = se.x + 32; j < se.y; ++j)
+            if (j != self && near(pos[j])) ++more;
+        const int cnt = __popc(m) + more;
+        int pre = cnt;
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) {
+            const int y = __shfl_up_sync(gm, pre, o, G);
+            if (gl >= o) pre += y;
+        }
+        const int total = __shfl_sync(gm, pre, G - 1, G);
+        int k = base + pre - cnt;
+        while (m) {
+            emit(k++, se.x + __ffs(m) - 1);
+            m &= m - 1;
+        }
+        if (more)
+            for (int j = se.x + 32; j < se.y; ++j)
+                if (j != self && near(pos[j])) emit(k++, j);
+        base += total;
+        if (base > most) break;
+    }
+    return base;
+}
+
 // The candidates j != self with r^2 < R2 in the cells overlapping
 // [x - R, x + R] (every lane passes the same particle), handed to
-// emit(k, j) with k = 0, 1, ... in the order for_candidates visits them
+// emit(k, j, r2) with k = 0, 1, ... in the order for_candidates visits them
 // (cells in its loop order, j ascending within a cell), so a list written
 // by a warp equals the one a thread's scan writes.  Cells are taken as
 // for_candidates_lanes takes them: small ranges candidate by candidate (a
 // ballot per 32 candidates places the hits), large ones 32 cells at a time
 // (each lane counts its cell's hits, an exclusive prefix across the warp
-// places them, the lane writes them).  Returns the number of hits.
+// places them, the lane writes them), with the ranges of four such rounds
+// loaded together: a wide support's cells are mostly empty, and the scan
+// waits on those loads.  Returns the number of hits.
+constexpr int kAhead = 4;
 template <typename T, typename E>
 __device__ __forceinline__ int for_hits_lanes_ordered(const Grid& g, const BoxInfo& bx,
                                                       const P4<T>* __restrict__ pos, int self, T xi, T yi,
                                                       T zi, T R, T R2, int lane, E&& emit) {
-    const int nc = bx.nc;
+    const Window<T> w(bx.nc, xi, yi, zi, R);
     const int2* __restrict__ cells = g.cells + bx.cell_off;
-    if (!(xi >= T(0) && xi <= T(1) && yi >= T(0) && yi <= T(1) && zi >= T(0) && zi <= T(1) &&
-          R >= T(0)))
-        return 0;
-    const bool full = !(R < T(0.5));
-    const T c3[3] = {xi, yi, zi};
-    int lo[3], hi[3];
-    bool wraps_all = full;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        lo[a] = full ? 0 : (int)floor((c3[a] - R) * (T)nc - T(1e-3));
-        hi[a] = full ? nc - 1 : (int)floor((c3[a] + R) * (T)nc + T(1e-3));
-        if (hi[a] - lo[a] + 1 >= nc) {
-            lo[a] = 0;
-            hi[a] = nc - 1;
-            wraps_all = true;
-        }
-    }
     const T xim1 = xi - T(1), yim1 = yi - T(1), zim1 = zi - T(1);
-    const T cl = T(1) / (T)nc, R2m = R * R * T(1.0001);
-    auto gap = [&](int c, T v) { return wraps_all ? T(0) : max(max((T)c * cl - v, v - (T)(c + 1) * cl), T(0)); };
-    auto cell_range = [&](int cx, int cy, int cz, int2& se) {
-        const T gx = gap(cx, xi), gy = gap(cy, yi), gz = gap(cz, zi);
-        if (gx * gx + gy * gy + gz * gz > R2m) return false;
-        const int wx = cx < 0 ? cx + nc : (cx >= nc ? cx - nc : cx);
-        const int wy = cy < 0 ? cy + nc : (cy >= nc ? cy - nc : cy);
-        const int wz = cz < 0 ? cz + nc : (cz >= nc ? cz - nc : cz);
-        se = cells[(wz * nc + wy) * nc + wx];
-        return true;
-    };
-    auto hit = [&](int j) {
+    const float xf = chop(xi), yf = chop(yi), zf = chop(zi);
+    auto r2_of = [&](int j) {
         const P4<T> q = pos[j];
-        const T dx = mi_diff(q.x, xi, xim1), dy = mi_diff(q.y, yi, yim1), dz = mi_diff(q.z, zi, zim1);
-        return sep2(dx, dy, dz) < R2;
+        return sep2(mi_diff(q.x, xi, xim1), mi_diff(q.y, yi, yim1), mi_diff(q.z, zi, zim1));
     };
     const unsigned full_mask = 0xffffffffu;
     int base = 0;
-    const int ex = hi[0] - lo[0] + 1, ey = hi[1] - lo[1] + 1, ez = hi[2] - lo[2] + 1;
-    const int ncube = ex * ey * ez;
-    if (ncube >= kLaneCells) {
-        for (int f0 = 0; f0 < ncube; f0 += 32) {
-            const int f = f0 + lane;
-            int2 se = make_int2(0, 0);
-            bool ok = false;
-            if (f < ncube) ok = cell_range(lo[0] + f % ex, lo[1] + (f / ex) % ey, lo[2] + f / (ex * ey), se);
-            int cnt = 0;
-            if (ok)
-                for (int j = se.x; j < se.y; ++j)
-                    if (j != self && hit(j)) ++cnt;
-            int pre = cnt;
+    if (w.ncube >= kLaneCells) {
+        for (int f0 = 0; f0 < w.ncube; f0 += 32 * kAhead) {
+            int2 ses[kAhead];
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(full_mask, pre, o);
-                if (lane >= o) pre += y;
+            for (int u = 0; u < kAhead; ++u) {
+                const int f = f0 + 32 * u + lane;
+                ses[u] = make_int2(0, 0);
+                if (f < w.ncube) {
+                    int cx, cy, cz;
+                    w.coords(f, cx, cy, cz);
+                    ses[u] = w.range(cells, cx, cy, cz, xf, yf, zf);
+                }
             }
-            const int total = __shfl_sync(full_mask, pre, 31);
-            int k = base + pre - cnt;
-            if (ok)
+#pragma unroll 1
+            for (int u = 0; u < kAhead; ++u) {
+                const int2 se = u == 0 ? ses[0] : (u == 1 ? ses[1] : (u == 2 ? ses[2] : ses[3]));
+                if (!__any_sync(full_mask, se.y > se.x)) continue;
+                int cnt = 0;
                 for (int j = se.x; j < se.y; ++j)
-                    if (j != self && hit(j)) emit(k++, j);
-            base += total;
+                    if (j != self && r2_of(j) < R2) ++cnt;
+                int pre = cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(full_mask, pre, o);
+                    if (lane >= o) pre += y;
+                }
+                const int total = __shfl_sync(full_mask, pre, 31);
+                int k = base + pre - cnt;
+                if (cnt)
+                    for (int j = se.x; j < se.y; ++j) {
+                        const T r2 = r2_of(j);
+                        if (j != self && r2 < R2) emit(k++, j, r2);
+                    }
+                base += total;
+            }
         }
     } else {
-        for (int cz = lo[2]; cz <= hi[2]; ++cz)
-            for (int cy = lo[1]; cy <= hi[1]; ++cy)
-                for (int cx = lo[0]; cx <= hi[0]; ++cx) {
-                    int2 se;
-                    if (!cell_range(cx, cy, cz, se)) continue;  // (the same for every lane)
-                    for (int j0 = se.x; j0 < se.y; j0 += 32) {
-                        const int j = j0 + lane;
-                        const bool h = j < se.y && j != self && hit(j);
-                        const unsigned m = __ballot_sync(full_mask, h);
-                        if (h) emit(base + __popc(m & ((1u << lane) - 1u)), j);
-                        base += __popc(m);
-                    }
-                }
+        for (int f = 0; f < w.ncube; ++f) {
+            int cx, cy, cz;
+            w.coords(f, cx, cy, cz);
+            const int2 se = w.range(cells, cx, cy, cz, xf, yf, zf);  // (the same for every lane)
+            for (int j0 = se.x; j0 < se.y; j0 += 32) {
+                const int j = j0 + lane;
+                const T r2 = j < se.y ? r2_of(j) : T(0);
+                const bool h = j < se.y && j != self && r2 < R2;
+                const unsigned m = __ballot_sync(full_mask, h);
+                if (h) emit(base + __popc(m & ((1u << lane) - 1u)), j, r2);
+                base += __popc(m);
+            }
+        }
     }
     return base;
 }
