@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 1)
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     T a[kRecord];
-    load_rec(rec + (size_t)i * kRecord, a);
+    load_rec(rec, i, a);
     const long long idi = sid[i];
     const T hdt = (T)(0.5 * dt_use[sbox[i]]);
     const T gam = (T)p.gamma;
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 1)
         for (int k = 0; k < cnt; ++k) {
             const int j = (int)L[lcol(k, N)];
             T b[kRecord];
-            load_rec(rec + (size_t)j * kRecord, b);
+            load_rec(rec, j, b);
             T wj[4];
             load4(wgt + 4 * (size_t)j, wj);
             const T wp[3] = {wi[0] - wj[0], wi[1] - wj[1], wi[2] - wj[2]};
@@ -473,13 +473,13 @@ __global__ void __launch_bounds__(128)
     T* sd = seeds + (size_t)i * kSeed;
     unsigned long long bloom = 0ull;
     const T* G = ginfo + (size_t)i * kGInfo;
-    const T* R = rec + (size_t)i * kRecord;
     const P4<T> me = s.pos[i];
     const T xi = me.x, yi = me.y, zi = me.z, Hi = me.w;
     const T xim1 = xi - T(1), yim1 = yi - T(1), zim1 = zi - T(1);
     const P4<T> pm = s.prim[i];
     const T Wi[5] = {pm.x, pm.y, pm.z, pm.w, s.prim2[i].x};
-    const T Bs[6] = {R[26], R[27], R[28], R[29], R[30], R[31]};
+    const T Bs[6] = {rec[rec_at<T>(i, 26)], rec[rec_at<T>(i, 27)], rec[rec_at<T>(i, 28)],
+                     rec[rec_at<T>(i, 29)], rec[rec_at<T>(i, 30)], rec[rec_at<T>(i, 31)]};
     T fbi[5] = {0, 0, 0, 0, 0};
     T xbi[3] = {0, 0, 0};
     T Hbi = T(0.0), nbi = T(0.0);

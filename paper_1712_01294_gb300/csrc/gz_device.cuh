@@ -40,6 +40,82 @@ __device__ __forceinline__ double pdiv(double a, double b) { return a / b; }
 __device__ __forceinline__ float psqrt(float x) { return x > 0.f ? x * rsqrtf(x) : 0.f; }
 __device__ __forceinline__ double psqrt(double x) { return sqrt(x); }
 
+// Reciprocal and reciprocal square root of the flux pass, for normal positive
+// arguments.  FP32: the hardware approximations (2 ulp), without the range
+// scaling the library forms add around them.  FP64: the hardware's 20-bit
+// start and one step of third order, y (1 + e + e^2) with e = 1 - x y, and
+// y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 (the binomial series of 1/(1 - e)
+// and (1 - e)^(-1/2)): 3 and 5 FP64 operations, to the last place or two.
+__device__ __forceinline__ float rcp_(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rsq_(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ double rcp_(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double rsq_(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+// min and max of two numbers.  FP64: compared as integers (a negative number's
+// magnitude bits flipped), which leaves the FP64 pipe alone.
+__device__ __forceinline__ float min_(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ float max_(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ long long order_(double a) {
+    const long long i = __double_as_longlong(a);
+    return i ^ ((i >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double min_(double a, double b) { return order_(a) < order_(b) ? a : b; }
+__device__ __forceinline__ double max_(double a, double b) { return order_(a) < order_(b) ? b : a; }
+__device__ __forceinline__ bool pos_(float a) { return a > 0.f; }
+__device__ __forceinline__ bool pos_(double a) {  // a > 0 (false for NaN)
+    const long long i = __double_as_longlong(a);
+    return i > 0 && i <= 0x7ff0000000000000ll;
+}
+// Smallest squares the pair geometry takes (below them rsq_ has no normal
+// argument): a face this small (area 3e-19) carries nothing.
+template <typename T>
+struct Tiny;
+template <>
+struct Tiny<float> {
+    static constexpr float sq = 1e-37f;
+};
+template <>
+struct Tiny<double> {
+    static constexpr double sq = 1e-300;
+};
+// W(q)/2 = t^3 - 4 v^3, t = max(1 - q, 0), v = max(1/2 - q, 0): the kernel
+// shape of both pieces without a test (0 beyond the support).
+__device__ __forceinline__ float kern_half(float r, float iH) {
+    const float t = __saturatef(fmaf(-r, iH, 1.f)), v = __saturatef(fmaf(-r, iH, 0.5f));
+    return fmaf(-4.f * (v * v), v, t * t * t);
+}
+__device__ __forceinline__ double kern_half(double r, double iH) {
+    const double q = __dmul_rn(r, iH);
+    const int h = __double2hiint(q);
+    const bool in = h < 0x3FE00000;
+    const double x = in ? q : 1.0 - q;
+    const double w = fma(fma(in ? 3.0 : 1.0, x, in ? -3.0 : 0.0), x * x, in ? 0.5 : 0.0);
+    return h >= 0x3FF00000 ? 0.0 : w;
+}
+
+// x . y, fused the same way wherever it is formed.
+template <typename T>
+__device__ __forceinline__ T dot3(T x0, T x1, T x2, T y0, T y1, T y2) {
+    return fma(x2, y2, fma(x1, y1, mul_rn(x0, y0)));
+}
+
 // Symmetric 3x3 inverse by adjugate; kappa = |E|_F |B|_F / 3.
 template <typename A>
 __device__ __forceinline__ void invert_sym(const A E[6], A B[6], A& det, A& kap) {
@@ -62,23 +138,31 @@ __device__ __forceinline__ void invert_sym(const A E[6], A B[6], A& det, A& kap)
 
 // ---------------------------------------------------------- O10-O12
 // A flux record is one 128-byte line (FP32) or two (FP64), read with 32-byte
-// vector loads (sm_100+ ld.global.v8.f32 / v4.f64): a warp gathering 32
-// records from scattered lines then moves whole sectors per L1 wavefront
-// instead of half sectors.  Records start on 128-byte boundaries.
-__device__ __forceinline__ void load_rec(const float* __restrict__ p, float (&v)[kRecord]) {
+// vector loads (sm_100+ ld.global.v8.f32 / v4.f64).  Its 32-byte sectors are
+// stored rotated by the record's index: a warp gathering one sector of 32
+// records would otherwise find them all in the same quarter of the L1 data
+// banks (records start on 128-byte lines) and take one pass a lane (31
+// measured for 28 lanes); rotated, adjacent records' sectors lie in different
+// quarters.
+template <typename T>
+__device__ __forceinline__ size_t rec_at(int i, int q) {  // place of value q of record i
+    constexpr int per = 32 / sizeof(T), ns = kRecord / per;
+    return (size_t)i * kRecord + (((q / per + i) & (ns - 1)) * per + q % per);
+}
+__device__ __forceinline__ void load_rec(const float* __restrict__ rec, int i, float (&v)[kRecord]) {
 #pragma unroll
     for (int k = 0; k < kRecord / 8; ++k)
         asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
             : "=f"(v[8 * k]), "=f"(v[8 * k + 1]), "=f"(v[8 * k + 2]), "=f"(v[8 * k + 3]), "=f"(v[8 * k + 4]),
               "=f"(v[8 * k + 5]), "=f"(v[8 * k + 6]), "=f"(v[8 * k + 7])
-            : "l"(p + 8 * k));
+            : "l"(rec + rec_at<float>(i, 8 * k)));
 }
-__device__ __forceinline__ void load_rec(const double* __restrict__ p, double (&v)[kRecord]) {
+__device__ __forceinline__ void load_rec(const double* __restrict__ rec, int i, double (&v)[kRecord]) {
 #pragma unroll
     for (int k = 0; k < kRecord / 4; ++k)
         asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
             : "=d"(v[4 * k]), "=d"(v[4 * k + 1]), "=d"(v[4 * k + 2]), "=d"(v[4 * k + 3])
-            : "l"(p + 4 * k));
+            : "l"(rec + rec_at<double>(i, 4 * k)));
 }
 
 // Face state of particle a toward the face at a + s o (o = offset to the
@@ -164,6 +248,13 @@ __device__ __forceinline__ void store_row32(double* p, const double* v) {
                      : "memory");
 }
 
+template <typename T>
+__device__ __forceinline__ void store_rec(T* rec, int i, const T (&v)[kRecord]) {
+    constexpr int per = 32 / sizeof(T);
+#pragma unroll
+    for (int k = 0; k < kRecord; k += per) store_row32<per>(rec + rec_at<T>(i, k), v + k);
+}
+
 // Four values to / from 16-byte-aligned memory.
 __device__ __forceinline__ void store4(float* dst, float a, float b, float c, float d) {
     *reinterpret_cast<float4*>(dst) = make_float4(a, b, c, d);
@@ -215,27 +306,28 @@ __device__ __forceinline__ void mfv_flux(const T (&FL)[5], const T (&FR)[5], T u
     const T wx = (left ? FL[1] : FR[1]) - vfx;
     const T wy = (left ? FL[2] : FR[2]) - vfy;
     const T wz = (left ? FL[3] : FR[3]) - vfz;
-    const T E = pdiv(P, gam - T(1)) + T(0.5) * rho * ((wx * wx + wy * wy) + wz * wz);
-    const T ru = rho * un;
+    const T E = fma(T(0.5) * rho, dot3(wx, wy, wz, wx, wy, wz), pdiv(P, gam - T(1)));
+    const T ru = mul_rn(rho, un);
     T fr = ru;
-    T fx = ru * wx + P * nx, fy = ru * wy + P * ny, fz = ru * wz + P * nz;
-    T fe = un * (E + P);
+    T fx = fma(ru, wx, mul_rn(P, nx)), fy = fma(ru, wy, mul_rn(P, ny)), fz = fma(ru, wz, mul_rn(P, nz));
+    T fe = mul_rn(un, E + P);
     if (star) {
         const T SK = left ? SL : SR;
         const T q = pdiv(T(1), SK - ss);
-        const T g = rho * q, f = g * (SK - un);
-        const T k = SK * (ss - un);
-        fr += k * g;
-        fx += k * (g * wx + f * nx);
-        fy += k * (g * wy + f * ny);
-        fz += k * (g * wz + f * nz);
-        fe += k * (q * (E + P) + f * ss);
+        const T g = mul_rn(rho, q), f = mul_rn(g, SK - un);
+        const T k = mul_rn(SK, ss - un);
+        fr = fma(k, g, fr);
+        fx = fma(k, fma(g, wx, mul_rn(f, nx)), fx);
+        fy = fma(k, fma(g, wy, mul_rn(f, ny)), fy);
+        fz = fma(k, fma(g, wz, mul_rn(f, nz)), fz);
+        fe = fma(k, fma(q, E + P, mul_rn(f, ss)), fe);
     }
+    // (explicit multiply-adds: every kernel that forms the flux gets the same bits)
     Fm = fr;
-    Fp[0] = fx + vfx * fr;
-    Fp[1] = fy + vfy * fr;
-    Fp[2] = fz + vfz * fr;
-    FE = (fe + ((vfx * fx + vfy * fy) + vfz * fz)) + T(0.5) * ((vfx * vfx + vfy * vfy) + vfz * vfz) * fr;
+    Fp[0] = fma(vfx, fr, fx);
+    Fp[1] = fma(vfy, fr, fy);
+    Fp[2] = fma(vfz, fr, fz);
+    FE = fma(T(0.5) * dot3(vfx, vfy, vfz, vfx, vfy, vfz), fr, fe + dot3(vfx, vfy, vfz, fx, fy, fz));
 }
 
 // x^y for x > 0: FP32 as 2^(y log2 x) from the hardware base-2 logarithm
@@ -348,120 +440,325 @@ __device__ __forceinline__ bool pair_order(int i, int j, long long idi, const lo
         return i < j;
 }
 
+// Primitives of a record (rho, v, P) at the half step: W plus the Hancock
+// increments of O11, (dt/2)(-rho div v, -grad P / rho, -gamma P div v); hdt = 0
+// without them.  Both particles of a pair form a particle's values with these
+// same operations.
+template <typename T>
+__device__ __forceinline__ void half_state(const T (&a)[kRecord], T hdt, T gam, T (&W)[5]) {
+    const T div = (a[11 + 3] + a[11 + 7]) + a[11 + 11];
+    const T e = -hdt * div;
+    const T k = -hdt * rcp_(a[6]);
+    W[0] = fma(e, a[6], a[6]);
+    W[1] = fma(k, a[11 + 12], a[8]);
+    W[2] = fma(k, a[11 + 13], a[9]);
+    W[3] = fma(k, a[11 + 14], a[10]);
+    W[4] = fma(gam * e, a[7], a[7]);
+}
+
 // Contribution of the pair (a, b) to particle a's rates: dp (3), dE and,
-// under MFV (O15), dm.  kRiem: the MFM face's star from HLLC (0), the exact
-// solver (1), or HLLC with the exact star where HLLC's P* < 0 (2).  Returns
-// false when the face area vanishes.  flags: 1 fallback, 2 P* < 0 (or vacuum).
+// under MFV (O15), dm.  Wh: half_state of a.  kRiem: the MFM face's star from
+// HLLC (0), the exact solver (1), or HLLC with the exact star where HLLC's
+// P* < 0 (2).  Returns false when the face area vanishes.  flags: 1 fallback,
+// 2 P* < 0 (or vacuum).
+//
+// Every quantity is symmetric or changes sign under a <-> b, d -> -d, down to
+// the bits, so the two particles of a pair get opposite contributions.  For
+// the HLLC star that holds by the form it is written in: with
+// du = (v_b - v_a).n of the face states, m_a = rho_a min(-c_a, du - c_b) and
+// m_b = rho_b max(c_b, c_a - du) (the Davis speeds relative to the face
+// states; their exchange is -m_b, -m_a),
+//   P* = (m_a P_b - m_b P_a - m_a m_b du) / (m_a - m_b),
+//   S* = ((v_a + v_b).n + (2 (P_b - P_a) - (m_a + m_b) du) / (m_a - m_b)) / 2,
+// the contact speed in the lab frame, S*_face + v_f.n whatever v_f is.  Only
+// velocity differences enter P*, so nothing cancels at high Mach number.
 template <typename T, bool kMFV, int kRiem>
-__device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[kRecord], bool aL,
-                                           T hdt, T gam, bool hancock, const T (&inca)[5], T (&dp)[3],
-                                           T& dE, T& dm, int& fl) {
+__device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[kRecord], const T (&Wh)[5], bool aL,
+                                           T hdt, T gam, T (&dp)[3], T& dE, T& dm, int& fl) {
     const T dx = mi_diff(b[0], a[0], a[0] - T(1));
     const T dy = mi_diff(b[1], a[1], a[1] - T(1));
     const T dz = mi_diff(b[2], a[2], a[2] - T(1));
-    const T r2 = sep2(dx, dy, dz);
-    const T r = psqrt(r2);
-    const T ca = r2 < a[3] * a[3] ? a[5] * kern_w(r * a[4]) : T(0);
-    const T cb = r2 < b[3] * b[3] ? b[5] * kern_w(r * b[4]) : T(0);
-    const T Bax = (a[26] * dx + a[27] * dy) + a[28] * dz;
-    const T Bay = (a[27] * dx + a[29] * dy) + a[30] * dz;
-    const T Baz = (a[28] * dx + a[30] * dy) + a[31] * dz;
-    const T Bbx = (b[26] * dx + b[27] * dy) + b[28] * dz;
-    const T Bby = (b[27] * dx + b[29] * dy) + b[30] * dz;
-    const T Bbz = (b[28] * dx + b[30] * dy) + b[31] * dz;
+    const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
+    const T r = mul_rn(r2, rsq_(r2));
+    const T ca = a[5] * kern_half(r, a[4]);  // (half of V psi; doubled in A)
+    const T cb = b[5] * kern_half(r, b[4]);
+    const T Bax = dot3(a[26], a[27], a[28], dx, dy, dz), Bay = dot3(a[27], a[29], a[30], dx, dy, dz),
+            Baz = dot3(a[28], a[30], a[31], dx, dy, dz);
+    const T Bbx = dot3(b[26], b[27], b[28], dx, dy, dz), Bby = dot3(b[27], b[29], b[30], dx, dy, dz),
+            Bbz = dot3(b[28], b[30], b[31], dx, dy, dz);
     const T A0 = add_rn(mul_rn(ca, Bax), mul_rn(cb, Bbx));
     const T A1 = add_rn(mul_rn(ca, Bay), mul_rn(cb, Bby));
     const T A2 = add_rn(mul_rn(ca, Baz), mul_rn(cb, Bbz));
     const T Aq = sep2(A0, A1, A2);
-    if (!(Aq > T(0))) return false;
-    const T Am = psqrt(Aq);
-    const T iA = pdiv(T(1), Am);
+    if (!pos_(Aq - Tiny<T>::sq)) return false;
+    const T iA = rsq_(Aq);
     const T n0 = A0 * iA, n1 = A1 * iA, n2 = A2 * iA;
-    const T Hs = a[3] + b[3];
-    const T sa = pdiv(a[3], Hs), sb = pdiv(b[3], Hs);
-    T Fa[5], Fb[5];
-    T incb[5];
-    hancock_inc(b, hdt, gam, hancock, incb);
-    face_state(a, sa, dx, dy, dz, inca, Fa);
-    face_state(b, sb, -dx, -dy, -dz, incb, Fb);
-    const T Wa[5] = {a[6], a[8], a[9], a[10], a[7]};
-    const T Wb[5] = {b[6], b[8], b[9], b[10], b[7]};
+    const T iH = rcp_(a[3] + b[3]);
+    const T sa = a[3] * iH, sb = b[3] * iH;
+    // face states: half-step primitives + g . (s d), clamped between the
+    // particles' primitives
+    T Fa[5], Fb[5], Wb[5];
+    half_state(b, hdt, gam, Wb);
+    const T Wa0[5] = {a[6], a[8], a[9], a[10], a[7]};
+    const T Wb0[5] = {b[6], b[8], b[9], b[10], b[7]};
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
-        const T lo = min(Wa[f], Wb[f]), hi = max(Wa[f], Wb[f]);
-        Fa[f] = min(max(Fa[f], lo), hi);
-        Fb[f] = min(max(Fb[f], lo), hi);
+        const T ga = dot3(a[11 + 3 * f], a[12 + 3 * f], a[13 + 3 * f], dx, dy, dz);
+        const T gb = dot3(b[11 + 3 * f], b[12 + 3 * f], b[13 + 3 * f], dx, dy, dz);
+        const T lo = min_(Wa0[f], Wb0[f]), hi = max_(Wa0[f], Wb0[f]);
+        Fa[f] = min_(max_(fma(sa, ga, Wh[f]), lo), hi);
+        Fb[f] = min_(max_(fma(-sb, gb, Wb[f]), lo), hi);
     }
-    if (!(Fa[0] > T(0) && Fa[4] > T(0) && Fb[0] > T(0) && Fb[4] > T(0))) {
+    if (!(pos_(Fa[0]) && pos_(Fa[4]) && pos_(Fb[0]) && pos_(Fb[4]))) {
 #pragma unroll
         for (int f = 0; f < 5; ++f) {
-            Fa[f] = Wa[f];
-            Fb[f] = Wb[f];
+            Fa[f] = Wa0[f];
+            Fb[f] = Wb0[f];
         }
         fl |= 1;
     }
-    // canonical order: L = a when aL (pair_order)
-    T FL[5], FR[5];
-#pragma unroll
-    for (int f = 0; f < 5; ++f) {
-        FL[f] = aL ? Fa[f] : Fb[f];
-        FR[f] = aL ? Fb[f] : Fa[f];
-    }
-    const T vLx = aL ? Wa[1] : Wb[1], vLy = aL ? Wa[2] : Wb[2], vLz = aL ? Wa[3] : Wb[3];
-    const T vRx = aL ? Wb[1] : Wa[1], vRy = aL ? Wb[2] : Wa[2], vRz = aL ? Wb[3] : Wa[3];
-    const T sL = aL ? sa : sb;
-    const T nx = aL ? n0 : -n0, ny = aL ? n1 : -n1, nz = aL ? n2 : -n2;
-    const T vfx = vLx + sL * (vRx - vLx), vfy = vLy + sL * (vRy - vLy), vfz = vLz + sL * (vRz - vLz);
-    const T vfn = (vfx * nx + vfy * ny) + vfz * nz;
-    const T uL = ((FL[1] - vfx) * nx + (FL[2] - vfy) * ny) + (FL[3] - vfz) * nz;
-    const T uR = ((FR[1] - vfx) * nx + (FR[2] - vfy) * ny) + (FR[3] - vfz) * nz;
-    // O12 HLLC with Davis wave speeds
-    const T rL = FL[0], PL = FL[4], rR = FR[0], PR = FR[4];
-    const T cL = psqrt(pdiv(gam * PL, rL)), cR = psqrt(pdiv(gam * PR, rR));
-    const T SL = min(uL - cL, uR - cR), SR = max(uL + cL, uR + cR);
-    const T num = ((PR - PL) + rL * uL * (SL - uL)) - rR * uR * (SR - uR);
-    const T den = rL * (SL - uL) - rR * (SR - uR);
-    const T ss = pdiv(num, den);
-    T ps = PL + rL * (SL - uL) * (ss - uL);
-    T sm = ss;  // contact speed of the MFM energy rate
+    // O12 star state from the face states
+    const T qa = gam * Fa[4] * rcp_(Fa[0]), qb = gam * Fb[4] * rcp_(Fb[0]);
+    const T cca = mul_rn(qa, rsq_(max_(qa, Tiny<T>::sq))), ccb = mul_rn(qb, rsq_(max_(qb, Tiny<T>::sq)));
+    const T du = dot3(Fb[1] - Fa[1], Fb[2] - Fa[2], Fb[3] - Fa[3], n0, n1, n2);
+    const T ma = mul_rn(Fa[0], min_(-cca, du - ccb)), mb = mul_rn(Fb[0], max_(ccb, cca - du));
+    const T iden = rcp_(ma - mb);
+    T ps = fma(-(ma * mb), du, add_rn(mul_rn(ma, Fb[4]), -mul_rn(mb, Fa[4]))) * iden;
     bool neg = ps < T(0);
-    if constexpr (!kMFV && kRiem != 0) {
-        if (kRiem == 1 || neg) {
-            T pe, ue;
-            if (exact_star(rL, uL, PL, rR, uR, PR, gam, pe, ue)) {
-                ps = pe;
-                sm = ue;
-                if (kRiem == 1) neg = false;
+    const T Am = T(2) * (Aq * iA);
+    if constexpr (!kMFV && kRiem == 0) {
+        if (neg) {
+            fl |= 2;
+            ps = T(0);
+        }
+        const T us = dot3(Fa[1] + Fb[1], Fa[2] + Fb[2], Fa[3] + Fb[3], n0, n1, n2);
+        const T ss = add_rn(us, mul_rn(fma(-(ma + mb), du, T(2) * (Fb[4] - Fa[4])), iden));
+        const T p2 = T(-2) * ps;
+        dp[0] = mul_rn(p2, A0);  // (rounded here: every caller adds the same bits)
+        dp[1] = mul_rn(p2, A1);
+        dp[2] = mul_rn(p2, A2);
+        dE = mul_rn(T(-0.5) * ps, ss * Am);
+        dm = T(0);
+        return true;
+    } else {
+        // canonical order: L = a when aL (pair_order); face frame v_f
+        T FL[5], FR[5];
+#pragma unroll
+        for (int f = 0; f < 5; ++f) {
+            FL[f] = aL ? Fa[f] : Fb[f];
+            FR[f] = aL ? Fb[f] : Fa[f];
+        }
+        const T vLx = aL ? a[8] : b[8], vLy = aL ? a[9] : b[9], vLz = aL ? a[10] : b[10];
+        const T vRx = aL ? b[8] : a[8], vRy = aL ? b[9] : a[9], vRz = aL ? b[10] : a[10];
+        const T sL = aL ? sa : sb;
+        const T nx = aL ? n0 : -n0, ny = aL ? n1 : -n1, nz = aL ? n2 : -n2;
+        const T vfx = fma(sL, vRx - vLx, vLx), vfy = fma(sL, vRy - vLy, vLy), vfz = fma(sL, vRz - vLz, vLz);
+        const T uL = dot3(FL[1] - vfx, FL[2] - vfy, FL[3] - vfz, nx, ny, nz);
+        const T uR = dot3(FR[1] - vfx, FR[2] - vfy, FR[3] - vfz, nx, ny, nz);
+        const T mL = aL ? ma : -mb, mR = aL ? mb : -ma;
+        const T s0 = mul_rn(fma(-mR, uR, fma(mL, uL, FR[4] - FL[4])), iden);  // S* in the face frame
+        if constexpr (kMFV) {
+            // both particles of the pair form the same canonical flux bits; L
+            // loses what R gains
+            if (neg) fl |= 2;
+            const T cL = aL ? cca : ccb, cR = aL ? ccb : cca;
+            const T SL = min(uL - cL, uR - cR), SR = max(uL + cL, uR + cR);
+            T Fm, Fp[3], FE;
+            mfv_flux(FL, FR, uL, uR, SL, SR, s0, vfx, vfy, vfz, nx, ny, nz, gam, Fm, Fp, FE);
+            const T m = mul_rn(Fm, Am), px = mul_rn(Fp[0], Am), py = mul_rn(Fp[1], Am),
+                    pz = mul_rn(Fp[2], Am), e = mul_rn(FE, Am);
+            dm = aL ? -m : m;
+            dp[0] = aL ? -px : px;
+            dp[1] = aL ? -py : py;
+            dp[2] = aL ? -pz : pz;
+            dE = aL ? -e : e;
+            return true;
+        } else {
+            const T vfn = dot3(vfx, vfy, vfz, nx, ny, nz);
+            T sm = s0;  // contact speed of the energy rate
+            if (kRiem == 1 || neg) {
+                T pe, ue;
+                if (exact_star(FL[0], uL, FL[4], FR[0], uR, FR[4], gam, pe, ue)) {
+                    ps = pe;
+                    sm = ue;
+                    if (kRiem == 1) neg = false;
+                } else {
+                    ps = T(0);
+                    sm = T(0);
+                    neg = true;
+                }
+            }
+            if (neg) fl |= 2;
+            if (ps < T(0)) ps = T(0);
+            dm = T(0);
+            const T p2 = T(-2) * ps;
+            dp[0] = mul_rn(p2, A0);
+            dp[1] = mul_rn(p2, A1);
+            dp[2] = mul_rn(p2, A2);
+            const T ef = mul_rn(ps * (sm + vfn), Am);
+            dE = aL ? -ef : ef;
+            return true;
+        }
+    }
+}
+
+// Sums of one particle's pair contributions, shared by the flux pass and the
+// hierarchical exchange: over N_i then R_i, in the working precision over runs
+// of 8 list slots, the runs added up in FP64 in list order.  One thread forms
+// the runs one after another (sum_runs), or the block's four warps, which then
+// hold the same 32 particles, form four of them at a time (sum_runs_split):
+// the same bits.
+template <int nq>
+struct Totals {
+    double v[nq];
+};
+template <typename T, bool kMFV, int kRiem>
+constexpr bool kLoadAhead = sizeof(T) == 4 && !kMFV && kRiem == 0;
+
+// pair(rec, j, dst) adds the pair with record rec of partner j to dst[nq].
+// kAhead: the next partner's record is loaded while the current pair is
+// evaluated (two record buffers, so the loop is written for two pairs at a
+// time; 165 registers, 12 warps an SM).  The pass waits on its gathers: FP32
+// MFM at 128^3 856 us without, 803 with.  The forms with more arithmetic a
+// pair (MFV, the exact solver, FP64) need the registers themselves.
+template <typename T, int nq, bool kAhead, typename P>
+__device__ __forceinline__ Totals<nq> sum_runs(int i, int N, const T* __restrict__ rec,
+                                               const unsigned* __restrict__ nbr, int cnt,
+                                               const unsigned* __restrict__ rnbr, int rcnt, P&& pair) {
+    Totals<nq> t;
+#pragma unroll
+    for (int q = 0; q < nq; ++q) t.v[q] = 0.0;
+    T A[kRecord], B[kRecord];
+#pragma unroll 1
+    for (int list = 0; list < 2; ++list) {
+        const unsigned* L = (list == 0 ? nbr : rnbr) + 4 * (size_t)i;
+        const int n = list == 0 ? cnt : rcnt;
+        if (n < 1) continue;
+        uint4 jj = col4_once(L, 0, N);
+        if constexpr (kAhead) load_rec(rec, (int)jj.x, A);
+        T run[nq];
+#pragma unroll 1
+        for (int k0 = 0; k0 < n; k0 += 4) {
+            if (!(k0 & 4)) {
+#pragma unroll
+                for (int q = 0; q < nq; ++q) run[q] = T(0);
+            }
+            uint4 nn = jj;
+            if (k0 + 4 < n) nn = col4_once(L, k0 + 4, N);
+            if constexpr (kAhead) {
+                if (k0 + 1 < n) load_rec(rec, (int)jj.y, B);
+                pair(A, (int)jj.x, run);
+                if (k0 + 1 < n) {
+                    if (k0 + 2 < n) load_rec(rec, (int)jj.z, A);
+                    pair(B, (int)jj.y, run);
+                    if (k0 + 2 < n) {
+                        if (k0 + 3 < n) load_rec(rec, (int)jj.w, B);
+                        pair(A, (int)jj.z, run);
+                        if (k0 + 3 < n) {
+                            if (k0 + 4 < n) load_rec(rec, (int)nn.x, A);
+                            pair(B, (int)jj.w, run);
+                        }
+                    }
+                }
             } else {
-                ps = T(0);
-                sm = T(0);
-                neg = true;
+                const unsigned js[4] = {jj.x, jj.y, jj.z, jj.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (k0 + u >= n) break;
+                    load_rec(rec, (int)js[u], A);
+                    pair(A, (int)js[u], run);
+                }
+            }
+            jj = nn;
+            if ((k0 & 4) || k0 + 4 >= n) {
+#pragma unroll
+                for (int q = 0; q < nq; ++q) t.v[q] += (double)run[q];
             }
         }
     }
-    if (neg) fl |= 2;
-    if (ps < T(0)) ps = T(0);
-    if constexpr (kMFV) {
-        // both particles of the pair form the same canonical flux bits; L
-        // loses what R gains
-        T Fm, Fp[3], FE;
-        mfv_flux(FL, FR, uL, uR, SL, SR, ss, vfx, vfy, vfz, nx, ny, nz, gam, Fm, Fp, FE);
-        const T m = mul_rn(Fm, Am), px = mul_rn(Fp[0], Am), py = mul_rn(Fp[1], Am),
-                pz = mul_rn(Fp[2], Am), e = mul_rn(FE, Am);
-        dm = aL ? -m : m;
-        dp[0] = aL ? -px : px;
-        dp[1] = aL ? -py : py;
-        dp[2] = aL ? -pz : pz;
-        dE = aL ? -e : e;
-        return true;
+    return t;
+}
+
+// Four warps: warp c forms runs c, c + 4, ...; v[0] becomes quantity c's total
+// (v[1], in warp 0, the fifth's).  Every thread of the block must get here.
+template <typename T, int nq, typename P>
+__device__ __forceinline__ Totals<2> sum_runs_split(int i, int N, const T* __restrict__ rec,
+                                                    const unsigned* __restrict__ nbr, int cnt,
+                                                    const unsigned* __restrict__ rnbr, int rcnt, P&& pair) {
+    __shared__ T sh[4][nq][32];
+    const int c = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const int runs = (cnt + 7) / 8, all = runs + (rcnt + 7) / 8;
+    Totals<2> t;
+    t.v[0] = t.v[1] = 0.0;
+    for (int r0 = 0; __syncthreads_or(r0 < all); r0 += 4) {
+        const int r = r0 + c;
+        T run[nq];
+#pragma unroll
+        for (int q = 0; q < nq; ++q) run[q] = T(0);
+        if (r < all) {
+            const unsigned* L = (r < runs ? nbr : rnbr) + 4 * (size_t)i;
+            const int n = r < runs ? cnt : rcnt, k1 = 8 * (r < runs ? r : r - runs);
+#pragma unroll 1
+            for (int k0 = k1; k0 < min(n, k1 + 8); k0 += 4) {
+                const uint4 jj = col4_once(L, k0, N);
+                const unsigned js[4] = {jj.x, jj.y, jj.z, jj.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (k0 + u >= n) break;
+                    T b[kRecord];
+                    load_rec(rec, (int)js[u], b);
+                    pair(b, (int)js[u], run);
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < nq; ++q) sh[c][q][l] = run[q];
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            if (r0 + w >= all) break;
+            t.v[0] += (double)sh[w][c][l];
+            if constexpr (nq == 5) t.v[1] += (double)sh[w][4][l];
+        }
     }
-    dm = T(0);
-    dp[0] = -mul_rn(ps, A0);
-    dp[1] = -mul_rn(ps, A1);
-    dp[2] = -mul_rn(ps, A2);
-    const T ef = ps * (sm + vfn) * Am;
-    dE = aL ? -ef : ef;
-    return true;
+    return t;
+}
+
+// Particle of a flux thread (or its position in an index list).
+template <bool kSplit>
+__device__ __forceinline__ int flux_item() {
+    return kSplit ? blockIdx.x * 32 + (threadIdx.x & 31) : blockIdx.x * blockDim.x + threadIdx.x;
+}
+// The rates of a thread's particle: all of them, or (four warps) quantity c.
+template <int nq>
+__device__ __forceinline__ void store_rates(const double (&v)[nq], int i, int N, double* __restrict__ dpdt,
+                                            double* __restrict__ dEdt, double* __restrict__ dmdt) {
+    dpdt[i] = v[0];
+    dpdt[(size_t)N + i] = v[1];
+    dpdt[2 * (size_t)N + i] = v[2];
+    dEdt[i] = v[3];
+    if constexpr (nq == 5) dmdt[i] = v[4];
+}
+template <int nq>
+__device__ __forceinline__ void store_rates_split(const double (&v)[2], int i, int N, double* __restrict__ dpdt,
+                                                  double* __restrict__ dEdt, double* __restrict__ dmdt) {
+    const int c = threadIdx.x >> 5;
+    if (c < 3)
+        dpdt[(size_t)c * N + i] = v[0];
+    else
+        dEdt[i] = v[0];
+    if constexpr (nq == 5)
+        if (c == 0) dmdt[i] = v[1];
+}
+__device__ __forceinline__ void count_flags(DevStatus* st, int nfall, int nneg) {
+    if (nfall) {
+        atomicOr(&st->bits, GZ_S_FALLBACK);
+        atomicAdd(&st->counters[GZ_C_FALLBACK], (unsigned long long)nfall);
+    }
+    if (nneg) {
+        atomicOr(&st->bits, GZ_S_PSTAR_NEG);
+        atomicAdd(&st->counters[GZ_C_PSTAR_NEG], (unsigned long long)nneg);
+    }
 }
 
 // ----------------------------------------------------------------- O14

@@ -331,8 +331,11 @@ __global__ void k_h_persist(int N, const int* __restrict__ alist, const int* __r
     if (t >= *nA) return;
     const int i = alist[t];
     const unsigned o = s.orig[i];
-    const T* R = rec + (size_t)i * kRecord;
+    T R[kRecord];
+    load_rec(rec, i, R);
+#pragma unroll
     for (int q = 0; q < 15; ++q) hgrad[(size_t)q * N + o] = R[11 + q];
+#pragma unroll
     for (int q = 0; q < 6; ++q) hB[(size_t)q * N + o] = R[26 + q];
     hn[o] = s.n[i];
     ((T*)p.h)[o] = s.h[i];
@@ -402,10 +405,9 @@ constexpr int kXBlock = 128;
 // Touched particle i over its pair lists (an active particle: N_i then its
 // r >= H_i pairs; an inactive one: its active partners): the pair's face
 // fluxes with the Hancock half step of dt_ij, scaled by 2^(k_i - k_ij),
-// summed like the flux pass (working precision over runs of 8 pairs, then
-// FP64).  kRiem: the MFM face's Riemann solver; kMFV: the MFV fluxes, whose
+// summed like the flux pass (sum_runs).  kRiem: the MFM face's Riemann solver; kMFV: the MFV fluxes, whose
 // mass share is summed too (pair_rates).
-template <typename T, int kRiem, bool kMFV>
+template <typename T, int kRiem, bool kMFV, bool kSplit>
 __global__ void __launch_bounds__(kXBlock)
     k_h_exchange(const int* __restrict__ tlist, const int* __restrict__ nT, const T* __restrict__ rec,
                  const long long* __restrict__ sid, const int* __restrict__ sbox,
@@ -415,74 +417,44 @@ __global__ void __launch_bounds__(kXBlock)
                  double* __restrict__ dpdt, double* __restrict__ dEdt, double* __restrict__ dmdt, int N,
                  DevStatus* st) {
     constexpr int nq = kMFV ? 5 : 4;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= *nT) return;
-    const int i = tlist[t];
+    const int t = flux_item<kSplit>(), n = *nT;
+    if (kSplit ? (int)blockIdx.x * 32 >= n : t >= n) return;
+    const int i = tlist[min(t, n - 1)];  // (kSplit: spare threads repeat a particle, with no pairs)
     T a[kRecord];
-    load_rec(rec + (size_t)i * kRecord, a);
+    load_rec(rec, i, a);
     const long long idi = kMFV ? sid[i] : 0;  // (MFV pairs are oriented by id)
     const int ka = sbin[i];
     const double Db = D[sbox[i]];
     const T gam = (T)p.gamma;
-    const bool hancock = p.hancock != 0;
-    T part[nq];
-    double acc[nq];
-#pragma unroll
-    for (int q = 0; q < nq; ++q) {
-        part[q] = T(0);
-        acc[q] = 0.0;
-    }
-    int np = 0, nfall = 0, nneg = 0;
-#pragma unroll 1
-    for (int list = 0; list < 2; ++list) {
-        const unsigned* L = list == 0 ? nbr + 4 * (size_t)i : rnbr + 4 * (size_t)i;
-        const int cnt = list == 0 ? min(ncount[i], p.cap) : min(rcount[i], p.rcap);
-        for (int k = 0; k < cnt; ++k) {
-            const int j = (int)L[lcol(k, N)];
-            T b[kRecord];
-            load_rec(rec + (size_t)j * kRecord, b);
-            const int kab = max(ka, sbin[j]);
-            const T hdt = (T)(0.5 * ldexp(Db, -kab));
-            T inca[5];
-            hancock_inc(a, hdt, gam, hancock, inca);
-            T dp[3], dE, dm;
-            int fl = 0;
-            const bool aL = pair_order<kMFV>(i, j, idi, sid);
-            if (pair_rates<T, kMFV, kRiem>(a, b, aL, hdt, gam, hancock, inca, dp, dE, dm, fl)) {
-                const T sc = (T)ldexp(1.0, ka - kab);
-                part[0] += dp[0] * sc;
-                part[1] += dp[1] * sc;
-                part[2] += dp[2] * sc;
-                part[3] += dE * sc;
-                if constexpr (kMFV) part[4] += dm * sc;
-            }
-            nfall += fl & 1;
-            nneg += (fl >> 1) & 1;
-            if (++np == 8) {
-#pragma unroll
-                for (int q = 0; q < nq; ++q) {
-                    acc[q] += (double)part[q];
-                    part[q] = T(0);
-                }
-                np = 0;
-            }
+    const int cnt = t < n ? min(ncount[i], p.cap) : 0, rcnt = t < n ? min(rcount[i], p.rcap) : 0;
+    int nfall = 0, nneg = 0;
+    auto pair = [&](const T(&b)[kRecord], int j, T(&run)[nq]) {
+        const int kab = max(ka, sbin[j]);
+        const T hdt = p.hancock ? (T)(0.5 * ldexp(Db, -kab)) : T(0);
+        T Wh[5];
+        half_state(a, hdt, gam, Wh);
+        T dp[3], dE, dm;
+        int fl = 0;
+        const bool aL = pair_order<kMFV>(i, j, idi, sid);
+        if (pair_rates<T, kMFV, kRiem>(a, b, Wh, aL, hdt, gam, dp, dE, dm, fl)) {
+            const T sc = (T)ldexp(1.0, ka - kab);
+            run[0] += dp[0] * sc;
+            run[1] += dp[1] * sc;
+            run[2] += dp[2] * sc;
+            run[3] += dE * sc;
+            if constexpr (kMFV) run[4] += dm * sc;
         }
+        nfall += fl & 1;
+        nneg += (fl >> 1) & 1;
+    };
+    if constexpr (kSplit) {
+        const Totals<2> s = sum_runs_split<T, nq>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
+        if (t < n) store_rates_split<nq>(s.v, i, N, dpdt, dEdt, dmdt);
+    } else {
+        const Totals<nq> s = sum_runs<T, nq, false>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
+        store_rates<nq>(s.v, i, N, dpdt, dEdt, dmdt);
     }
-#pragma unroll
-    for (int q = 0; q < nq; ++q) acc[q] += (double)part[q];
-    dpdt[i] = acc[0];
-    dpdt[(size_t)N + i] = acc[1];
-    dpdt[2 * (size_t)N + i] = acc[2];
-    dEdt[i] = acc[3];
-    if constexpr (kMFV) dmdt[i] = acc[4];
-    if (nfall) {
-        atomicOr(&st->bits, GZ_S_FALLBACK);
-        atomicAdd(&st->counters[GZ_C_FALLBACK], (unsigned long long)nfall);
-    }
-    if (nneg) {
-        atomicOr(&st->bits, GZ_S_PSTAR_NEG);
-        atomicAdd(&st->counters[GZ_C_PSTAR_NEG], (unsigned long long)nneg);
-    }
+    count_flags(st, nfall, nneg);
 }
 
 // Kick of a touched particle by dt_i times its scaled sums: the O14 momentum
@@ -563,21 +535,23 @@ __global__ void k_h_finalize(int N, int s, int K, gz_particles p, T* __restrict_
 }
 
 template <typename T>
-void launch_exchange(Ctx& c, const KParams& kp, int N) {
+void launch_exchange(Ctx& c, const KParams& kp, int N, int nA) {
     const int r = c.params.riemann;
-    auto go = [&](auto kernel) {
-        kernel<<<nblk(N, kXBlock), kXBlock, 0, c.stream>>>(c.tlist, c.hcount + 2, (const T*)c.rec, c.sid, c.sbox,
+    const bool split = nA < kFluxSplit;
+    auto go = [&](auto one, auto four) {
+        auto kernel = split ? four : one;
+        kernel<<<nblk(N, split ? 32 : kXBlock), kXBlock, 0, c.stream>>>(c.tlist, c.hcount + 2, (const T*)c.rec, c.sid, c.sbox,
                                                            c.sbin, c.nbr, c.ncount, c.rnbr, c.rcount, kp, c.dt_use,
                                                            c.dpdt, c.dEdt, c.dmdt, N, c.status);
     };
     if (c.params.scheme == GZ_MFV)
-        go(k_h_exchange<T, GZ_RIEMANN_HLLC, true>);
+        go(k_h_exchange<T, GZ_RIEMANN_HLLC, true, false>, k_h_exchange<T, GZ_RIEMANN_HLLC, true, true>);
     else if (r == GZ_RIEMANN_EXACT)
-        go(k_h_exchange<T, GZ_RIEMANN_EXACT, false>);
+        go(k_h_exchange<T, GZ_RIEMANN_EXACT, false, false>, k_h_exchange<T, GZ_RIEMANN_EXACT, false, true>);
     else if (r == GZ_RIEMANN_FALLBACK)
-        go(k_h_exchange<T, GZ_RIEMANN_FALLBACK, false>);
+        go(k_h_exchange<T, GZ_RIEMANN_FALLBACK, false, false>, k_h_exchange<T, GZ_RIEMANN_FALLBACK, false, true>);
     else
-        go(k_h_exchange<T, GZ_RIEMANN_HLLC, false>);
+        go(k_h_exchange<T, GZ_RIEMANN_HLLC, false, false>, k_h_exchange<T, GZ_RIEMANN_HLLC, false, true>);
 }
 
 }  // namespace
@@ -713,7 +687,7 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             timer.end(GZ_PASS_GRAD);
             timer.begin(GZ_PASS_FLUX);
             c.launches += 1;
-            launch_exchange<T>(c, kp, N);
+            launch_exchange<T>(c, kp, N, nA);
             timer.end(GZ_PASS_FLUX);
             timer.begin(GZ_PASS_UPDATE);
             cudaMemsetAsync(c.box_hits, 0, sizeof(int) * (size_t)c.nboxes, st);

@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1)
         for (int q = 0; q < 15; ++q) R[11 + q] = al[q / 3] * gt[q];
 #pragma unroll
         for (int q = 0; q < 6; ++q) R[26 + q] = B[q];
-        store_row32<kRecord>(rec + (size_t)i * kRecord, R);
+        store_rec(rec, i, R);
     }
     if (want_dt) {
         // warp-level minimum per box, one atomic per warp when the warp is in one box;
@@ -418,7 +418,7 @@ __global__ void k_pack_given(int N, Sorted<T> s, const T* __restrict__ grad, con
     const unsigned o = s.orig[i];
     const T Hi = s.h[i], ni = s.n[i];
     const T iH = T(1) / Hi;
-    T* R = rec + (size_t)i * kRecord;
+    T R[kRecord];
     R[0] = s.x[i];
     R[1] = s.y[i];
     R[2] = s.z[i];
@@ -430,8 +430,11 @@ __global__ void k_pack_given(int N, Sorted<T> s, const T* __restrict__ grad, con
     R[8] = s.vx[i];
     R[9] = s.vy[i];
     R[10] = s.vz[i];
+#pragma unroll
     for (int q = 0; q < 15; ++q) R[11 + q] = grad[(size_t)q * N + o];
+#pragma unroll
     for (int q = 0; q < 6; ++q) R[26 + q] = B[(size_t)q * N + o];
+    store_rec(rec, i, R);
 }
 
 template <typename T>
@@ -440,22 +443,25 @@ __global__ void k_grad_out(int N, const unsigned* __restrict__ orig, const T* __
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const unsigned o = orig[i];
-    const T* R = rec + (size_t)i * kRecord;
+    T R[kRecord];
+    load_rec(rec, i, R);
     if (grad)
+#pragma unroll
         for (int q = 0; q < 15; ++q) grad[(size_t)q * N + o] = R[11 + q];
     if (B)
+#pragma unroll
         for (int q = 0; q < 6; ++q) B[(size_t)q * N + o] = R[26 + q];
 }
 
-// One thread per particle over its pairs N_i then R_i (both contiguous
-// lists, read four indices per 16-byte load).  Contributions are summed in
-// the working precision over runs of 8 pairs and each run is added to FP64
-// accumulators.  kMFV: the MFV fluxes (O15), which add dm/dt.  kRiem: the
-// MFM face's Riemann solver (pair_rates).
+// Rates of a particle over its pairs N_i then R_i (sum_runs: one thread, or
+// kSplit four warps per 32 particles; either reads one list group of adjacent
+// particles at a time, so that a warp's partners lie close together).  kMFV:
+// the MFV fluxes (O15), which add dm/dt.  kRiem: the MFM face's Riemann solver
+// (pair_rates).
 constexpr int kFluxBlock = 128;
 
-template <typename T, bool kMFV, int kRiem>
-__global__ void __launch_bounds__(kFluxBlock)
+template <typename T, bool kMFV, int kRiem, bool kSplit>
+__global__ void __launch_bounds__(kFluxBlock, kLoadAhead<T, kMFV, kRiem> ? 3 : 1)
     k_fluxes(int N, const T* __restrict__ rec, const long long* __restrict__ sid,
              const int* __restrict__ sbox, const unsigned* __restrict__ nbr,
              const int* __restrict__ ncount, const unsigned* __restrict__ rnbr,
@@ -463,75 +469,39 @@ __global__ void __launch_bounds__(kFluxBlock)
              double* __restrict__ dpdt, double* __restrict__ dEdt, double* __restrict__ dmdt,
              DevStatus* st) {
     constexpr int nq = kMFV ? 5 : 4;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
+    const int it = flux_item<kSplit>();
+    if (!kSplit && it >= N) return;
+    const int i = min(it, N - 1);  // (kSplit: the last block's spare threads repeat a particle, with no pairs)
     T a[kRecord];
-    load_rec(rec + (size_t)i * kRecord, a);
+    load_rec(rec, i, a);
     const long long idi = kMFV ? sid[i] : 0;  // (MFV pairs are oriented by id)
-    const T hdt = (T)(0.5 * dt_use[sbox[i]]);
+    const T hdt = p.hancock ? (T)(0.5 * dt_use[sbox[i]]) : T(0);
     const T gam = (T)p.gamma;
-    const bool hancock = p.hancock != 0;
-    T inca[5];
-    hancock_inc(a, hdt, gam, hancock, inca);
-    T part[nq];
-    double acc[nq];
-#pragma unroll
-    for (int q = 0; q < nq; ++q) {
-        part[q] = T(0);
-        acc[q] = 0.0;
-    }
-    int np = 0, nfall = 0, nneg = 0;
-#pragma unroll 1
-    for (int list = 0; list < 2; ++list) {
-        const unsigned* L = list == 0 ? nbr + 4 * (size_t)i : rnbr + 4 * (size_t)i;
-        const int cnt = list == 0 ? min(ncount[i], p.cap) : min(rcount[i], p.rcap);
-        for (int k0 = 0; k0 < cnt; k0 += 4) {
-            const uint4 jj = col4_once(L, k0, N);
-            const unsigned js[4] = {jj.x, jj.y, jj.z, jj.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (k0 + u >= cnt) break;
-                const int j = (int)js[u];
-                T b[kRecord];
-                load_rec(rec + (size_t)j * kRecord, b);
-                T dp[3], dE, dm;
-                int fl = 0;
-                if (pair_rates<T, kMFV, kRiem>(a, b, pair_order<kMFV>(i, j, idi, sid), hdt, gam, hancock, inca,
-                                               dp, dE, dm, fl)) {
-                    part[0] += dp[0];
-                    part[1] += dp[1];
-                    part[2] += dp[2];
-                    part[3] += dE;
-                    if constexpr (kMFV) part[4] += dm;
-                }
-                nfall += fl & 1;
-                nneg += (fl >> 1) & 1;
-                if (++np == 8) {
-#pragma unroll
-                    for (int q = 0; q < nq; ++q) {
-                        acc[q] += (double)part[q];
-                        part[q] = T(0);
-                    }
-                    np = 0;
-                }
-            }
+    T Wh[5];
+    half_state(a, hdt, gam, Wh);
+    const int cnt = it < N ? min(ncount[i], p.cap) : 0, rcnt = it < N ? min(rcount[i], p.rcap) : 0;
+    int nfall = 0, nneg = 0;
+    auto pair = [&](const T(&b)[kRecord], int j, T(&run)[nq]) {
+        T dp[3], dE, dm;
+        int fl = 0;
+        if (pair_rates<T, kMFV, kRiem>(a, b, Wh, pair_order<kMFV>(i, j, idi, sid), hdt, gam, dp, dE, dm, fl)) {
+            run[0] += dp[0];
+            run[1] += dp[1];
+            run[2] += dp[2];
+            run[3] += dE;
+            if constexpr (kMFV) run[4] += dm;
         }
+        nfall += fl & 1;
+        nneg += (fl >> 1) & 1;
+    };
+    if constexpr (kSplit) {
+        const Totals<2> t = sum_runs_split<T, nq>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
+        if (it < N) store_rates_split<nq>(t.v, i, N, dpdt, dEdt, dmdt);
+    } else {
+        const Totals<nq> t = sum_runs<T, nq, kLoadAhead<T, kMFV, kRiem>>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
+        store_rates<nq>(t.v, i, N, dpdt, dEdt, dmdt);
     }
-#pragma unroll
-    for (int q = 0; q < nq; ++q) acc[q] += (double)part[q];
-    dpdt[i] = acc[0];
-    dpdt[(size_t)N + i] = acc[1];
-    dpdt[2 * (size_t)N + i] = acc[2];
-    dEdt[i] = acc[3];
-    if constexpr (kMFV) dmdt[i] = acc[4];
-    if (nfall) {
-        atomicOr(&st->bits, GZ_S_FALLBACK);
-        atomicAdd(&st->counters[GZ_C_FALLBACK], (unsigned long long)nfall);
-    }
-    if (nneg) {
-        atomicOr(&st->bits, GZ_S_PSTAR_NEG);
-        atomicAdd(&st->counters[GZ_C_PSTAR_NEG], (unsigned long long)nneg);
-    }
+    count_flags(st, nfall, nneg);
 }
 
 // dmdt (MFV, O15) non-null: the mass advances too and is written back.
@@ -792,9 +762,15 @@ cudaError_t run_grad_out(Ctx& c, T* grad, T* B) {
 
 template <typename T, bool kMFV, int kRiem>
 static void launch_fluxes(Ctx& c) {
-    k_fluxes<T, kMFV, kRiem><<<blocks(c.N, kFluxBlock), kFluxBlock, 0, c.stream>>>(
-        c.N, (const T*)c.rec, c.sid, c.sbox, c.nbr, c.ncount, c.rnbr, c.rcount, kparams(c), c.dt_use,
-        c.dpdt, c.dEdt, kMFV ? c.dmdt : nullptr, c.status);
+    auto go = [&](auto kernel, int items) {
+        kernel<<<blocks(c.N, items), kFluxBlock, 0, c.stream>>>(c.N, (const T*)c.rec, c.sid, c.sbox, c.nbr, c.ncount,
+                                                                c.rnbr, c.rcount, kparams(c), c.dt_use, c.dpdt,
+                                                                c.dEdt, kMFV ? c.dmdt : nullptr, c.status);
+    };
+    if (c.N < kFluxSplit)
+        go(k_fluxes<T, kMFV, kRiem, true>, 32);
+    else
+        go(k_fluxes<T, kMFV, kRiem, false>, kFluxBlock);
 }
 
 template <typename T>

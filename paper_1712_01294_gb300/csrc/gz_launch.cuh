@@ -24,6 +24,11 @@ cudaError_t unpermute_T(Ctx& c, const T* src, T* dst, int rows);
 cudaError_t unpermute_d(Ctx& c, const double* src, double* dst, int rows);
 cudaError_t unpermute_i(Ctx& c, const int* src, int* dst);
 
+// Flux launches of fewer particles than this give each particle's pairs to four
+// warps (k_fluxes, kSplit).  FP32, four warps / one thread, us: Sod 16^3 15 / 31,
+// Sod 32^3 28 / 26, Sedov 64^3 150 / 110.
+constexpr int kFluxSplit = 30000;
+
 // Hydro passes (sorted order).
 // list (device, sorted indices) and nlist (device count, at most n): run on
 // those particles only.
