@@ -1,7 +1,8 @@
 // Density pass (steps O4, O3): the support radius H of every particle, its
 // number density and its neighbour list.
 //
-// A group of kLanes lanes shares one particle.  The lanes take the cells of
+// A group of lanes shares one particle (launches that fill the chip: one
+// thread a particle, k_density_one).  The lanes take the cells of
 // the search window in rounds, test their cell's candidates into a bit mask,
 // place the hits by a prefix sum over the group (so the cache holds them in
 // scan order: cells in row order, ascending index within a cell) and keep
@@ -26,14 +27,18 @@ inline int blocks(int n, int t) { return (n + t - 1) / t; }
 
 constexpr int kDensBlock = 128;
 constexpr int kDensCache = 64;  // candidates within 1.05 H a group can hold
-constexpr int kLanes = 4;       // lanes of a group (8 measured slower from 32^3 particles on)
+constexpr int kLanes = 4;       // lanes of a group ...
+constexpr int kWideLanes = 16;  // ... and in FP32 launches too small for those
 
-// FP32 launches of this many particles or more fill the chip with one thread
-// each (k_density_one), which then takes fewer instructions a particle.
-// Measured, group / thread, us a launch, first steps (late in the run): Sod
-// 32^3 38 / 44 (52 / 68), KH 41^3 72 / 72 (81 / 74), Sedov 64^3 179 / 117
-// (342 / 524), turbulence 128^3 1483 / 921 (1808 / 1325).
-constexpr int kThreadMin = 100000;
+// FP32 launches: below kWideMax particles sixteen lanes each, below kThreadMin
+// four, and from there on one thread each (k_density_one), which fills the
+// chip with fewer instructions a particle.  Measured, us a launch on the first
+// steps (late in the run): Sod 16^3 sixteen lanes 24 (27), eight 28 (35), four
+// 40 (53); Sod 32^3 sixteen 69 (81), eight 58 (68), four 50 (67), one 51 (93);
+// KH 41^3 four 105 (99), one 76 (77); Sedov 64^3 one 121 (532); 128^3 one 984
+// (1397).  FP64 keeps four: its sums are the lanes' sums.
+constexpr int kWideMax = 12000;
+constexpr int kThreadMin = 45000;
 
 // Radius of the candidate cache for a support Ht: 5% headroom so that small
 // growth of H during the iteration needs no rescan, never past h_lim.
@@ -44,21 +49,21 @@ __device__ __forceinline__ T dens_cache_radius(T Ht, const KParams& p) {
     return R;
 }
 
-// The two terms of the density sum at q = r/H, from t = max(1 - q, 0) and
-// v = max(1/2 - q, 0):  W/2 = t^3 - 4 v^3,  -q W'/6 = q (t^2 - 4 v^2)
-// (both vanish beyond the support, so no distance test is needed).  The
-// second is returned as two factors x y, summed by explicit multiply-adds, so
-// that every kernel rounds the sums alike.
+// The two terms of the density sum at q = r/H: W(q) and -q W'(q) = x y.  One
+// cubic in q (q <= 1/2) or 1 - q (beyond) with selected coefficients,
+// W = 1 - 6x^2 + 6x^3 | 2x^3, -q W' = (12 - 18x) x^2 | (6 - 6x) x^2.  FP32: the
+// second as two factors, summed by explicit multiply-adds, so that every form
+// of the pass rounds its sums alike; callers add the entries with r < H.  FP64
+// (halved and divided by 6; the pieces decided on the high word, no FP64
+// comparison) vanishes beyond the support.
 __device__ __forceinline__ void dens_terms2(float q, float& w, float& x, float& y) {
-    const float t = __saturatef(1.f - q), v = __saturatef(0.5f - q);
-    const float t2 = t * t, v2 = v * v;
-    w = fmaf(-4.f * v2, v, t2 * t);
-    x = q;
-    y = fmaf(-4.f, v2, t2);
+    const bool in = q <= 0.5f;
+    const float t = in ? q : 1.f - q;
+    x = t * t;
+    w = fmaf(fmaf(in ? 6.f : 2.f, t, in ? -6.f : 0.f), x, in ? 1.f : 0.f);
+    y = fmaf(in ? -18.f : -6.f, t, in ? 12.f : 6.f);
 }
-__device__ __forceinline__ void dens_terms2(double q, double& w, double& x1, double& d) {
-    // one cubic in x = q (inside) or 1 - q (outside), coefficients selected;
-    // the pieces decided on the high word (no FP64 comparison)
+__device__ __forceinline__ void dens_terms2(double q, double& w, double& d) {
     const bool in = __double2hiint(q) < 0x3FE00000;
     const bool out = __double2hiint(q) >= 0x3FF00000;
     const double x = in ? q : 1.0 - q;
@@ -66,7 +71,6 @@ __device__ __forceinline__ void dens_terms2(double q, double& w, double& x1, dou
     const double a = fma(fma(in ? 3.0 : 1.0, x, in ? -3.0 : 0.0), x2, in ? 0.5 : 0.0);
     const double b = fma(in ? -3.0 : -1.0, x, in ? 2.0 : 1.0) * x2;
     w = out ? 0.0 : a;
-    x1 = 1.0;
     d = out ? 0.0 : b;
 }
 
@@ -79,32 +83,61 @@ __device__ __forceinline__ float dist(float r2) {
 }
 __device__ __forceinline__ double dist(double r2) { return sqrt(r2); }
 
-// Compensated partial sums combined over the lanes of a group (every lane
-// gets the same bits: the two-sum's error is exact in either order).
-template <int G>
-__device__ __forceinline__ float group_sum(unsigned gm, Acc<float> a) {
-#pragma unroll
-    for (int o = 1; o < G; o <<= 1) {
-        const float b = __shfl_xor_sync(gm, a.s, o), cb = __shfl_xor_sync(gm, a.c, o);
-        const float s = __fadd_rn(a.s, b);
-        const float bb = __fsub_rn(s, a.s);
-        const float e = __fadd_rn(__fsub_rn(a.s, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-        a.s = s;
-        a.c = __fsub_rn(__fadd_rn(a.c, cb), e);
-    }
-    return a.fvalue();
-}
-template <int G>
-__device__ __forceinline__ double group_sum(unsigned gm, Acc<double> a) {
-#pragma unroll
-    for (int o = 1; o < G; o <<= 1) a.s += __shfl_xor_sync(gm, a.s, o);
-    return a.s;
-}
 template <int G, typename T>
 __device__ __forceinline__ T group_add(unsigned gm, T v) {
 #pragma unroll
     for (int o = 1; o < G; o <<= 1) v += __shfl_xor_sync(gm, v, o);
     return v;
+}
+
+// One evaluation of the sums S = sum W and sd = sum -q W' over the entries with
+// r < H among the n cached ones (scan order; lane l of a group of G holds
+// entries l, l + G, ...: distance r[u] and r^2 at r2[u G + l]).
+// FP32: a compensated sum over the entries in scan order, whichever form of
+// the pass holds them (the support's last bits, and with them which pairs just
+// reach each other, then do not depend on the form): the lanes form the terms
+// of G entries and every lane adds all of them in order.
+template <int G, int E>
+__device__ __forceinline__ void group_eval(unsigned gm, int gl, int n, const float (&r)[E], const float* r2, float H,
+                                           float& S, float& sd) {
+    const float H2 = H * H, iH = 1.f / H;
+    Acc<float> sw;
+    sd = 0.f;
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+        if (u * G >= n) break;
+        const int k = u * G + gl;
+        const bool in = k < n && r2[k] < H2;
+        float w, x, y;
+        dens_terms2(r[u] * iH, w, x, y);
+        const unsigned m = __ballot_sync(gm, in) >> (threadIdx.x & 31 & ~(G - 1));
+#pragma unroll
+        for (int s = 0; s < G; ++s) {
+            const float ws = __shfl_sync(gm, w, s, G), xs = __shfl_sync(gm, x, s, G), ys = __shfl_sync(gm, y, s, G);
+            if (m >> s & 1u) {
+                sw.add(ws);
+                sd = fmaf(ys, xs, sd);
+            }
+        }
+    }
+    S = sw.fvalue();
+}
+// FP64: the lanes' sums added up.
+template <int G, int E>
+__device__ __forceinline__ void group_eval(unsigned gm, int, int n, const double (&r)[E], const double*, double H,
+                                           double& S, double& sd) {
+    const double iH = 1.0 / H;
+    double a = 0.0, b = 0.0;
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+        if (u * G >= n) break;
+        double w, d;
+        dens_terms2(r[u] * iH, w, d);
+        a += w;
+        b += d;
+    }
+    S = 2.0 * group_add<G>(gm, a);
+    sd = 6.0 * group_add<G>(gm, b);
 }
 
 // Result of one evaluation: f's sign decides the bracket, and the next H.
@@ -203,12 +236,12 @@ __device__ __forceinline__ float n_of(float S, float H) {
 }
 __device__ __forceinline__ double n_of(double S, double H) { return 8.0 * (1.0 + S) / (kPi * H * H * H); }
 
-template <typename T>
+template <typename T, int G>
 __global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
     k_density(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr, int* __restrict__ ncount,
               int* __restrict__ iters, DevStatus* st, const int* __restrict__ list,
               const int* __restrict__ nlist, int* __restrict__ defer, int* __restrict__ ndefer, int ccap) {
-    constexpr int G = kLanes, P = kDensBlock / G, E = kDensCache / G;
+    constexpr int P = kDensBlock / G, E = kDensCache / G;
     constexpr int S = kDensCache + G;  // (the groups of a warp start on different banks)
     __shared__ T c_r2[P][S];
     __shared__ unsigned c_j[P][S];
@@ -259,19 +292,7 @@ __global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
                 }
             }
         }
-        const T iH = T(1) / H;
-        Acc<T> sw;
-        T sd = T(0);
-#pragma unroll
-        for (int u = 0; u < E; ++u) {
-            if (u * G >= ncache) break;
-            T w, x, y;
-            dens_terms2(r[u] * iH, w, x, y);
-            sw.add(w);
-            sd = fma(x, y, sd);
-        }
-        Sv = T(2) * group_sum<G>(gm, sw);
-        sdv = T(6) * group_add<G>(gm, sd);
+        group_eval<G>(gm, gl, ncache, r, c_r2[gp], H, Sv, sdv);
         Hev = H;
         if (h_step(b, H, Sv, sdv, p, it == p.max_iter)) {
             conv = true;
@@ -305,9 +326,7 @@ __global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
 // FP32, one thread per particle: the form for launches that fill the chip
 // (k_density is faster below kThreadMin particles).  The first scan keeps
 // (r^2, j) of the candidates within 1.05 H in the thread's column of shared
-// memory.  Entry k adds to partial sum k mod 4, as lane k mod 4 of a group of
-// four does, and the four are combined as the group combines them, so both
-// forms give the same bits.  Held to 96 registers (10 blocks of 64 per SM).
+// memory.  Held to 96 registers (10 blocks of 64 per SM).
 constexpr int kOneBlock = 64;
 template <int kCache>
 __device__ __noinline__ int dens_fill(const Grid& g, const BoxInfo& bx, const P4<float>* __restrict__ pos, int i,
@@ -325,15 +344,6 @@ __device__ __noinline__ int dens_fill(const Grid& g, const BoxInfo& bx, const P4
         }
     });
     return n;
-}
-
-__device__ __forceinline__ Acc<float> combine(Acc<float> a, const Acc<float>& b) {
-    const float s = __fadd_rn(a.s, b.s);
-    const float bb = __fsub_rn(s, a.s);
-    const float e = __fadd_rn(__fsub_rn(a.s, __fsub_rn(s, bb)), __fsub_rn(b.s, bb));
-    a.s = s;
-    a.c = __fsub_rn(__fadd_rn(a.c, b.c), e);
-    return a;
 }
 
 template <int kCache>
@@ -386,22 +396,25 @@ __global__ void __launch_bounds__(kOneBlock, 10)
             defer[atomicAdd(ndefer, 1)] = i;
             return;
         }
-        const float iH = 1.f / H;
-        Acc<float> sw[4];
-        float sd[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int k0 = 0; k0 < ncache; k0 += 4) {
+        const float H2 = H * H, iH = 1.f / H;
+        Acc<float> sw;
+        sdv = 0.f;
+        for (int k0 = 0; k0 < ncache; k0 += 4) {  // four entries' terms at a time, added in order
+            float r2[4], w[4], x[4], y[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                float r = 8.f;  // (past every support)
-                if (k0 + u < ncache) r = dist(c_r2[k0 + u][t]);
-                float w, x, y;
-                dens_terms2(r * iH, w, x, y);
-                sw[u].add(w);
-                sd[u] = fmaf(x, y, sd[u]);
+                r2[u] = k0 + u < ncache ? c_r2[k0 + u][t] : 1e30f;
+                dens_terms2(dist(r2[u]) * iH, w[u], x[u], y[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (r2[u] < H2) {
+                    sw.add(w[u]);
+                    sdv = fmaf(y[u], x[u], sdv);
+                }
             }
         }
-        Sv = 2.f * combine(combine(sw[0], sw[1]), combine(sw[2], sw[3])).fvalue();
-        sdv = 6.f * ((sd[0] + sd[1]) + (sd[2] + sd[3]));
+        Sv = sw.fvalue();
         Hev = H;
         if (h_step(b, H, Sv, sdv, p, it == p.max_iter)) {
             conv = true;
@@ -435,11 +448,81 @@ __global__ void __launch_bounds__(kOneBlock, 10)
 // (in scan order); later evaluations and the list read only that.  A particle
 // with more of them scans the cells at every evaluation.  Grid-stride over
 // the deferred list, whose length only the device knows.
-// The sums run as in k_density: the lanes form the entries' terms, then lane
-// c = 0..3 adds those of entries k mod 4 = c in order, so which kernel
-// iterates a particle does not change its bits.
+// The sums run as in group_eval (FP32: the lanes form the terms of 32 entries,
+// then every lane adds those with r < H in order), so which form iterates a
+// particle does not change its bits.
 constexpr int kWarpDensBlock = 64;
 constexpr int kWarpCache = 512;
+
+__device__ __forceinline__ void warp_eval(int lane, int n, const float* r2, float* tw, float* tx, float* ty, float H,
+                                          float& S, float& sd) {
+    const float H2 = H * H, iH = 1.f / H;
+    Acc<float> sw;
+    sd = 0.f;
+    for (int k0 = 0; k0 < n; k0 += 32) {
+        const int k = k0 + lane;
+        const float q = k < n ? r2[k] : 1e30f;
+        const bool in = q < H2;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (in) {  // the hits of these 32, close together in order
+            const int at = __popc(m & ((1u << lane) - 1u));
+            dens_terms2(dist(q) * iH, tw[at], tx[at], ty[at]);
+        }
+        __syncwarp();
+        const int hits = __popc(m);
+#pragma unroll 4
+        for (int s = 0; s < hits; ++s) {
+            sw.add(tw[s]);
+            sd = fmaf(ty[s], tx[s], sd);
+        }
+        __syncwarp();
+    }
+    S = sw.fvalue();
+}
+__device__ __forceinline__ void warp_eval(int lane, int n, const double* r2, double*, double*, double*, double H,
+                                          double& S, double& sd) {
+    // (lane l's four-entry stride as in group_eval: lanes 4 m + c add class c)
+    const double iH = 1.0 / H;
+    double a = 0.0, b = 0.0;
+    if (lane < kLanes) {
+        for (int k = lane; k < n; k += kLanes) {
+            double w, d;
+            dens_terms2(sqrt(r2[k]) * iH, w, d);
+            a += w;
+            b += d;
+        }
+    }
+    a = group_add<kLanes>(0xffffffffu, a);
+    b = group_add<kLanes>(0xffffffffu, b);
+    S = 2.0 * __shfl_sync(0xffffffffu, a, 0);
+    sd = 6.0 * __shfl_sync(0xffffffffu, b, 0);
+}
+
+// An evaluation straight from the cells (more candidates than the warp's cache
+// holds), the lanes' sums added up.
+template <typename T>
+__device__ __noinline__ void warp_eval_cells(const Grid& g, const BoxInfo& bx, const P4<T>* __restrict__ pos, int i,
+                                             const P4<T>& me, int lane, T H, T& S, T& sd) {
+    const T H2 = H * H, iH = T(1) / H;
+    double a = 0.0, b = 0.0;
+    for_candidates_lanes<T>(g, bx, pos, i, me.x, me.y, me.z, H, lane, [&](int, T, T, T, T r2) {
+        if (r2 < H2) {
+            if constexpr (sizeof(T) == 4) {
+                float w, x, y;
+                dens_terms2(dist(r2) * iH, w, x, y);
+                a += (double)w;
+                b += (double)(x * y);
+            } else {
+                double w, d;
+                dens_terms2(sqrt(r2) * iH, w, d);
+                a += 2.0 * w;
+                b += 6.0 * d;
+            }
+        }
+    });
+    S = (T)group_add<32>(0xffffffffu, a);
+    sd = (T)group_add<32>(0xffffffffu, b);
+}
 
 template <typename T>
 __global__ void __launch_bounds__(kWarpDensBlock)
@@ -449,7 +532,7 @@ __global__ void __launch_bounds__(kWarpDensBlock)
     constexpr unsigned full = 0xffffffffu;
     __shared__ T w_r2[kWarpDensBlock / 32][kWarpCache];
     __shared__ unsigned w_j[kWarpDensBlock / 32][kWarpCache];
-    __shared__ T w_t[kWarpDensBlock / 32][3][kWarpCache];
+    __shared__ T w_t[kWarpDensBlock / 32][3][32];
     const int lane = threadIdx.x & 31;
     T *t_w = w_t[threadIdx.x >> 5][0], *t_x = w_t[threadIdx.x >> 5][1], *t_y = w_t[threadIdx.x >> 5][2];
     T* c_r2 = w_r2[threadIdx.x >> 5];
@@ -479,43 +562,10 @@ __global__ void __launch_bounds__(kWarpDensBlock)
                                                    });
                 __syncwarp();
             }
-            const T iH = T(1) / H;
-            Acc<T> sw;
-            T sd = T(0);
-            if (ncache <= kWarpCache) {
-                const int n4 = (ncache + 3) & ~3;
-                for (int k = lane; k < n4; k += 32) {
-                    T wv = T(0), x = T(0), y = T(0);
-                    if (k < ncache) dens_terms2(dist(c_r2[k]) * iH, wv, x, y);
-                    t_w[k] = wv;
-                    t_x[k] = x;
-                    t_y[k] = y;
-                }
-                __syncwarp();
-                if (lane < 4) {
-#pragma unroll 4
-                    for (int k = lane; k < n4; k += 4) {
-                        sw.add(t_w[k]);
-                        sd = fma(t_x[k], t_y[k], sd);
-                    }
-                }
-                const T S = group_sum<4>(full, sw), D = group_add<4>(full, sd);
-                Sv = T(2) * __shfl_sync(full, S, 0);
-                sdv = T(6) * __shfl_sync(full, D, 0);
-            } else {
-                const T H2 = H * H;
-                for_candidates_lanes<T>(g, bx, s.pos, i, me.x, me.y, me.z, H, lane, [&](int, T, T, T, T r2) {
-                    if (r2 < H2) {
-                        T wv, x, y;
-                        dens_terms2(dist(r2) * iH, wv, x, y);
-                        sw.add(wv);
-                        sd = fma(x, y, sd);
-                    }
-                });
-                __syncwarp();
-                Sv = T(2) * group_sum<32>(full, sw);
-                sdv = T(6) * group_add<32>(full, sd);
-            }
+            if (ncache <= kWarpCache)
+                warp_eval(lane, ncache, c_r2, t_w, t_x, t_y, H, Sv, sdv);
+            else
+                warp_eval_cells(g, bx, s.pos, i, me, lane, H, Sv, sdv);
             Hev = H;
             if (h_step(b, H, Sv, sdv, p, it == p.max_iter)) {
                 conv = true;
@@ -671,7 +721,6 @@ template <typename T>
 cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
     if (!list) n = c.N;
     if (n < 1) return cudaSuccess;
-    constexpr int P = kDensBlock / kLanes;
     const Sorted<T> sv = sorted_view<T>(c);
     // particles with more candidates within 1.05 H than their cache holds are
     // iterated by a warp each.  k_density_one: 40 entries (the largest count
@@ -698,10 +747,18 @@ cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
             done = true;
         }
     }
-    if (!done)
-        k_density<T><<<blocks(n, P), kDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
-                                                                 c.iters, c.status, list, nlist, c.defer,
-                                                                 c.ndefer, ccap);
+    auto group = [&](auto kernel, int lanes) {
+        kernel<<<blocks(n, kDensBlock / lanes), kDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr,
+                                                                           c.ncount, c.iters, c.status, list, nlist,
+                                                                           c.defer, c.ndefer, ccap);
+    };
+    if constexpr (std::is_same<T, float>::value) {
+        if (!done && n < kWideMax) {
+            group(k_density<T, kWideLanes>, kWideLanes);
+            done = true;
+        }
+    }
+    if (!done) group(k_density<T, kLanes>, kLanes);
     const int wb = std::max(1, std::min(blocks(n, kWarpDensBlock / 32), 152 * 4));
     k_density_warp<T><<<wb, kWarpDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
                                                             c.iters, c.status, c.defer, c.ndefer);

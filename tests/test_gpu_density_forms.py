@@ -1,4 +1,4 @@
-"""The density pass's forms (one thread, a group of four lanes or a warp per
+"""The density pass's forms (one thread, four or sixteen lanes, or a warp per
 particle) give the same bits, so which one a launch or a particle takes never
 shows; and the FP32 prefilter of the FP64 scan drops no neighbour."""
 import numpy as np
@@ -48,8 +48,10 @@ def test_forms_give_the_same_bits(name, make, prec):
     for kw in ({"density_cache": 40}, {"density_cache": 48}):  # more particles left to the warp form
         for a, b in zip(ref, _run(m, [q.N], q, prec, **kw)):
             assert np.array_equal(a, b), (name, kw)
-    copies = -(-100000 // q.N)  # enough boxes for the one-thread form
-    if prec == 1 and copies <= 70:
+    # enough boxes for the four-lane and the one-thread form
+    for copies in (-(-13000 // q.N), -(-100000 // q.N)):
+        if prec == 0 or copies > 70:
+            continue
         big = _run(m, [q.N], q, prec, copies)
         for a, b in zip(ref[:4], big[:4]):
             assert np.array_equal(np.tile(a, copies), b), name
