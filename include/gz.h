@@ -431,7 +431,7 @@ gz_status gz_profile_read(gz_ctx* ctx, double* ms, int64_t* calls, int32_t reset
  * NULL) receives this call's device status bits (GZ_S_*: positions outside
  * the box, non-convergence, ...; never GZ_S_NBR_OVERFLOW, as no list is
  * kept) when the stream reaches the end of the call.
- * Scratch: a fixed array inside the library (about 8.3 MB, held on every GPU
+ * Scratch: a fixed array inside the library (about 8.5 MB, held on every GPU
  * that loads the library until exit).  Limits: 1 <= n <= 32768 and a cell
  * grid of at most 32^3 cells (cell_factor * H0 >= 1/32), else GZ_E_INVAL.
  * The first call on a device looks up the array's device address (once per

@@ -606,7 +606,7 @@ gz_status create_ctx(const gz_params* params, int32_t nboxes, const int64_t* cou
     c.rcap = std::max(32, c.cap / 2 / 4 * 4);
     // per-box cell grids: cell length ~ cell_factor * H0 of the box
     int maxnc = 1;
-    long long cells = 0;
+    long long cells = 0, keys = 0;
     int first = 0;
     c.hboxes.resize(nboxes);
     for (int b = 0; b < nboxes; ++b) {
@@ -618,8 +618,10 @@ gz_status create_ctx(const gz_params* params, int32_t nboxes, const int64_t* cou
         c.hboxes[b].cell_off = (int)cells;
         c.hboxes[b].first = first;
         c.hboxes[b].count = (int)counts[b];
+        c.hboxes[b].key_off = (unsigned)keys;
         first += (int)counts[b];
         cells += (long long)nc * nc * nc;
+        keys += 1ll << (3 * ceil_log2(nc));
         maxnc = std::max(maxnc, nc);
     }
     if (cells >= (1ll << 30)) {
@@ -627,17 +629,15 @@ gz_status create_ctx(const gz_params* params, int32_t nboxes, const int64_t* cou
         return GZ_E_INVAL;
     }
     c.total_cells = (int)cells;
-    c.cbits = ceil_log2(maxnc);
-    c.box_bits = ceil_log2(nboxes);
-    if (3 * c.cbits + c.box_bits > 32) {
+    if (3 * ceil_log2(maxnc) + ceil_log2(nboxes) > 32) {  // (keys have 32 bits)
         delete ctx;
         return GZ_E_INVAL;
     }
+    c.total_keys = keys;
+    const bool counted = counting_sort_fits(N, keys);
     // one arena for all scratch
     const size_t Nz = (size_t)N;
     const size_t sz = params->precision == GZ_FP64 ? 8 : 4;
-    const int nblk = (int)((N + 4095) / 4096);
-    c.hist_len = 1024 * nblk + 1024;  // per-block counts of up to 1024 digits, then the digit totals
     struct Item {
         void** ptr;
         size_t bytes;
@@ -645,7 +645,9 @@ gz_status create_ctx(const gz_params* params, int32_t nboxes, const int64_t* cou
     std::vector<Item> items = {
         {(void**)&c.keys, 4 * Nz},        {(void**)&c.keys_alt, 4 * Nz},
         {(void**)&c.vals, 4 * Nz},        {(void**)&c.vals_alt, 4 * Nz},
-        {(void**)&c.hist, 4 * (size_t)c.hist_len},
+        {(void**)&c.hist, 4 * sort_sums_len(N, keys, counted)},
+        {(void**)&c.kcount, counted ? 4 * (size_t)keys : 0},
+        {(void**)&c.kstart, counted ? 4 * (size_t)keys : 0},
         {(void**)&c.box_of, 4 * Nz},      {(void**)&c.boxes, sizeof(BoxInfo) * (size_t)nboxes},
         {(void**)&c.cells, sizeof(int2) * (size_t)cells},
         {(void**)&c.sx, sz * Nz},         {(void**)&c.sy, sz * Nz},

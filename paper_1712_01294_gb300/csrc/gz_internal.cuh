@@ -34,6 +34,7 @@ struct BoxInfo {
     int cell_off;    // first cell of this box in the cell array
     int first;       // first particle (sorted order == caller order per box)
     int count;       // particles in the box
+    unsigned key_off;  // first sort key of this box (keys: Morton index of the cell + key_off)
 };
 
 // Scalar parameters passed by value to kernels.
@@ -81,8 +82,7 @@ struct Ctx {
     std::vector<int64_t> counts;
     std::vector<BoxInfo> hboxes;
     int total_cells;
-    int cbits;     // bits per axis of a cell coordinate
-    int box_bits;  // bits of the box index in a key
+    long long total_keys;  // sort keys of all boxes (per box 8^b, 2^b >= cells per axis)
     cudaStream_t stream;
     // a second stream for the step checkpoint's list copies, which overlap
     // the pair passes (created on the first checkpointing step)
@@ -96,8 +96,8 @@ struct Ctx {
     BoxInfo* boxes;
     int2* cells;
     unsigned *keys, *keys_alt, *vals, *vals_alt;
-    unsigned* hist;
-    int hist_len;
+    unsigned *kcount, *kstart;  // particles per key and their first sorted index (counting sort), else null
+    unsigned* hist;             // partial sums of the sort
     int* box_of;  // caller order
     // sorted state (working precision) and derived per-particle data
     void *sx, *sy, *sz, *svx, *svy, *svz, *sm, *su, *sh, *sn, *srho, *sP, *sc, *ssd;

@@ -8,12 +8,21 @@ namespace gz {
 template <typename T>
 Sorted<T> sorted_view(Ctx& c);
 
-// Binning + radix sort + permutation into the context's sorted arrays, and
+// Keys per particle up to which the counting sort is taken: its scan of the
+// keys then costs less than the radix sort's passes over the particles (a grid
+// of one support radius a cell has 0.13 to 1.05; a grid much finer than the
+// particles has more).
+constexpr long long kKeysPerParticle = 8;
+inline bool counting_sort_fits(long long N, long long keys) { return keys <= kKeysPerParticle * N + 65536; }
+// Partial sums (32-bit words) the sort needs.
+size_t sort_sums_len(long long N, long long keys, bool counted);
+
+// Binning + sort + permutation into the context's sorted arrays, and
 // cell ranges.  n_in (caller order, may be null) is permuted into the sorted
 // n array as well.  Returns a CUDA error code.
 template <typename T>
 cudaError_t sort_and_bin(Ctx& c, const gz_particles& p, const void* n_in);
-// The part of sort_and_bin after the radix sort, from c.keys and c.vals as a
+// The part of sort_and_bin after the sort, from c.keys and c.vals as a
 // sort left them (a checkpoint's copy of them: the same start state).
 template <typename T>
 cudaError_t permute_and_bin(Ctx& c, const gz_particles& p, const void* n_in);

@@ -24,11 +24,12 @@ constexpr int kCap = 32;          // neighbour-list slots (lists are not returne
 constexpr int kMaxDevices = 64;
 
 constexpr size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
-constexpr size_t kHistLen = 1024 * ((kMaxN + 4095) / 4096) + 1024;  // counts + digit totals
+constexpr size_t kMaxKeys = 32768;  // sort keys of a grid of at most 32^3 cells
+constexpr size_t kSumsLen = 64;     // partial sums of the counting sort's scan
 // Worst case (FP64) of every slice the density pass touches.
 constexpr size_t kScratchBytes =
     4 * al(4 * (size_t)kMaxN)                          // keys, keys_alt, vals, vals_alt
-    + al(4 * kHistLen)                                 // radix histogram
+    + al(4 * kSumsLen) + 2 * al(4 * kMaxKeys)          // counting sort
     + al(4 * (size_t)kMaxN)                            // box of each particle
     + al(sizeof(BoxInfo))                              // box table
     + al(sizeof(int2) * (size_t)kMaxCells)             // cell ranges
@@ -41,7 +42,7 @@ constexpr size_t kScratchBytes =
     + al(sizeof(DevStatus));
 
 // The scratch itself: every GPU that loads the library holds these bytes
-// (8,295,168 B, about 8.3 MB) until the process exits.  All calls share it.
+// (8,520,704 B, about 8.5 MB) until the process exits.  All calls share it.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 std::mutex g_mu;
@@ -68,7 +69,7 @@ cudaError_t scratch_on_current_device(void** out) {
 // The one-box table, written on the device from values passed by value (no
 // host buffer is referenced by the enqueued work).
 __global__ void k_noalloc_box(BoxInfo* boxes, int nc, int count) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) boxes[0] = BoxInfo{nc, 0, 0, count};
+    if (threadIdx.x == 0 && blockIdx.x == 0) boxes[0] = BoxInfo{nc, 0, 0, count, 0u};
 }
 
 // Copies the status bits of this call to the caller's word.  The lists are
@@ -104,11 +105,9 @@ gz_status run(const gz_params* prm, int N, gz_particles* p, void* n_out, int32_t
     c.cap = kCap;
     c.rcap = 0;
     c.total_cells = nc * nc * nc;
-    c.cbits = ceil_log2i(nc);
-    c.box_bits = 0;
+    c.total_keys = 1ll << (3 * ceil_log2i(nc));
     c.launches = 0;
     c.prof = 0;
-    c.hist_len = (int)kHistLen;
     char* q = (char*)base;
     auto take = [&](size_t bytes) {
         void* r = q;
@@ -120,7 +119,9 @@ gz_status run(const gz_params* prm, int N, gz_particles* p, void* n_out, int32_t
     c.keys_alt = (unsigned*)take(4 * Nz);
     c.vals = (unsigned*)take(4 * Nz);
     c.vals_alt = (unsigned*)take(4 * Nz);
-    c.hist = (unsigned*)take(4 * kHistLen);
+    c.hist = (unsigned*)take(4 * kSumsLen);
+    c.kcount = (unsigned*)take(4 * kMaxKeys);
+    c.kstart = (unsigned*)take(4 * kMaxKeys);
     c.box_of = (int*)take(4 * Nz);
     c.boxes = (BoxInfo*)take(sizeof(BoxInfo));
     c.cells = (int2*)take(sizeof(int2) * (size_t)kMaxCells);

@@ -1,6 +1,8 @@
-// Binning, device LSD radix sort and permutation (step S1: particles are
-// Morton-sorted into a uniform cell grid per box; cell ranges are derived
-// from the sorted keys).
+// Binning, sort and permutation (step S1: particles are Morton-sorted into a
+// uniform cell grid per box, in caller order within a cell, and the cells'
+// ranges formed).  A counting sort over the keys where there are at most
+// kKeysPerParticle keys a particle (every grid of about one support radius a
+// cell), else a device LSD radix sort; both are stable and give one order.
 #include <algorithm>
 
 #include "gz_launch.cuh"
@@ -8,6 +10,8 @@
 namespace gz {
 
 namespace {
+
+inline int blocks(int n, int t) { return (n + t - 1) / t; }
 
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
@@ -44,24 +48,148 @@ __device__ __forceinline__ int cell_coord(T v, int nc) {
     return (int)s;
 }
 
+// Sort key of a particle: its box's first key + the Morton index of its cell.
+template <typename T>
+__device__ __forceinline__ unsigned key_of(const BoxInfo& bx, T x, T y, T z) {
+    return bx.key_off + (spread3(cell_coord(x, bx.nc)) | (spread3(cell_coord(y, bx.nc)) << 1) |
+                         (spread3(cell_coord(z, bx.nc)) << 2));
+}
+template <typename T>
+__device__ __forceinline__ bool inside(T x, T y, T z) {
+    return x >= T(0) && x < T(1) && y >= T(0) && y < T(1) && z >= T(0) && z < T(1);
+}
+
 template <typename T>
 __global__ void k_keys(int N, const T* __restrict__ x, const T* __restrict__ y,
                        const T* __restrict__ z, const int64_t* __restrict__ id,
-                       const int* __restrict__ box_of, const BoxInfo* __restrict__ boxes, int cbits,
+                       const int* __restrict__ box_of, const BoxInfo* __restrict__ boxes,
                        unsigned* __restrict__ keys, unsigned* __restrict__ vals, DevStatus* st) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    const int b = box_of[i];
-    const int nc = boxes[b].nc;
     const T xv = x[i], yv = y[i], zv = z[i];
-    const bool ok = xv >= T(0) && xv < T(1) && yv >= T(0) && yv < T(1) && zv >= T(0) && zv < T(1);
-    if (!ok) set_status(st, GZ_S_NONFINITE, GZ_C_NONFINITE, id[i]);
-    unsigned mort = spread3(cell_coord(xv, nc)) | (spread3(cell_coord(yv, nc)) << 1) |
-                    (spread3(cell_coord(zv, nc)) << 2);
-    keys[i] = (cbits * 3 >= 32 ? 0u : ((unsigned)b << (3 * cbits))) | mort;
+    if (!inside(xv, yv, zv)) set_status(st, GZ_S_NONFINITE, GZ_C_NONFINITE, id[i]);
+    keys[i] = key_of(boxes[box_of[i]], xv, yv, zv);
     vals[i] = (unsigned)i;
 }
 
+// ------------------------------------------------------- counting sort
+// Key of every particle and its arrival number in its key's count (any order:
+// k_permute puts the particles of a cell in caller order).
+template <typename T>
+__global__ void k_cs_count(int N, const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z,
+                           const int64_t* __restrict__ id, const int* __restrict__ box_of,
+                           const BoxInfo* __restrict__ boxes, unsigned* __restrict__ count,
+                           unsigned* __restrict__ key, unsigned* __restrict__ slot, DevStatus* st) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    const T xv = x[i], yv = y[i], zv = z[i];
+    if (!inside(xv, yv, zv)) set_status(st, GZ_S_NONFINITE, GZ_C_NONFINITE, id[i]);
+    const unsigned k = key_of(boxes[box_of[i]], xv, yv, zv);
+    key[i] = k;
+    slot[i] = atomicAdd(&count[k], 1u);
+}
+
+constexpr int kScanThreads = 1024;
+constexpr int kScanTile = 4 * kScanThreads;
+constexpr int kScanDirect = 8;  // up to this many tiles, a block sums the counts before its own itself
+
+__device__ __forceinline__ uint4 count4(const unsigned* __restrict__ count, long long k, long long K) {
+    if (k + 3 < K) return *reinterpret_cast<const uint4*>(count + k);
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (k < K) v.x = count[k];
+    if (k + 1 < K) v.y = count[k + 1];
+    if (k + 2 < K) v.z = count[k + 2];
+    return v;
+}
+// Sum over the block (every thread gets it).
+__device__ __forceinline__ unsigned block_sum(unsigned v, unsigned* sh) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    unsigned t = 0;
+#pragma unroll
+    for (int w = 0; w < kScanThreads / 32; ++w) t += sh[w];
+    __syncthreads();
+    return t;
+}
+
+__global__ void __launch_bounds__(kScanThreads)
+    k_cs_sums(long long K, const unsigned* __restrict__ count, unsigned* __restrict__ sums) {
+    __shared__ unsigned sh[kScanThreads / 32];
+    const uint4 v = count4(count, (long long)blockIdx.x * kScanTile + 4 * threadIdx.x, K);
+    const unsigned t = block_sum(v.x + v.y + v.z + v.w, sh);
+    if (threadIdx.x == 0) sums[blockIdx.x] = t;
+}
+
+// First sorted index of every key, and the range of every cell (empty ones
+// included).  sums: the tiles' sums, or null when every block adds the counts
+// before its tile itself.
+__global__ void __launch_bounds__(kScanThreads)
+    k_cs_scan(long long K, const unsigned* __restrict__ count, const unsigned* __restrict__ sums,
+              const BoxInfo* __restrict__ boxes, int nboxes, unsigned* __restrict__ start,
+              int2* __restrict__ cells) {
+    __shared__ unsigned sh[kScanThreads / 32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    unsigned before = 0;
+    if (sums) {
+        for (int b = t; b < (int)blockIdx.x; b += kScanThreads) before += sums[b];
+    } else {
+        for (int b = 0; b < (int)blockIdx.x; ++b) {
+            const uint4 v = *reinterpret_cast<const uint4*>(count + (size_t)b * kScanTile + 4 * t);
+            before += v.x + v.y + v.z + v.w;
+        }
+    }
+    unsigned base = blockIdx.x ? block_sum(before, sh) : 0u;
+    const long long k0 = (long long)blockIdx.x * kScanTile + 4 * t;
+    const uint4 v = count4(count, k0, K);
+    const unsigned c[4] = {v.x, v.y, v.z, v.w};
+    const unsigned mine = (c[0] + c[1]) + (c[2] + c[3]);
+    unsigned x = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) sh[warp] = x;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) base += sh[w];
+    unsigned s = base + x - mine;
+    if (k0 >= K) return;
+    int b = 0;  // box of the key: the last with key_off <= k0
+    for (int hi = nboxes - 1; b < hi;) {
+        const int mid = (b + hi + 1) >> 1;
+        if (boxes[mid].key_off <= (unsigned)k0)
+            b = mid;
+        else
+            hi = mid - 1;
+    }
+    BoxInfo bx = boxes[b];
+    unsigned next = b + 1 < nboxes ? boxes[b + 1].key_off : 0xffffffffu;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const long long k = k0 + u;
+        if (k >= K) break;
+        while (b + 1 < nboxes && (unsigned)k >= next) {
+            bx = boxes[++b];
+            next = b + 1 < nboxes ? boxes[b + 1].key_off : 0xffffffffu;
+        }
+        start[k] = s;
+        const unsigned mort = (unsigned)k - bx.key_off;
+        const int cx = compact3(mort), cy = compact3(mort >> 1), cz = compact3(mort >> 2);
+        if (cx < bx.nc && cy < bx.nc && cz < bx.nc)
+            cells[bx.cell_off + (cz * bx.nc + cy) * bx.nc + cx] = make_int2((int)s, (int)(s + c[u]));
+        s += c[u];
+    }
+}
+
+__global__ void k_cs_place(int N, const unsigned* __restrict__ key, const unsigned* __restrict__ slot,
+                           const unsigned* __restrict__ start, unsigned* __restrict__ order) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N) order[start[key[i]] + slot[i]] = (unsigned)i;
+}
+
+// ----------------------------------------------------------- radix sort
 // Digit counts of one tile (nd = 2^bits digits, mask = nd - 1).
 __global__ void k_rs_hist(const unsigned* __restrict__ keys, int N, int shift, unsigned mask, int nd,
                           unsigned* __restrict__ hist, int nblk) {
@@ -190,38 +318,59 @@ __global__ void k_rs_scatter(const unsigned* __restrict__ kin, const unsigned* _
     }
 }
 
-template <typename T>
-__global__ void k_permute(int N, const unsigned* __restrict__ skeys,
-                          const unsigned* __restrict__ svals, gz_particles p,
+// The state in sorted order.  kCounted: p walks k_cs_place's order, a cell's
+// particles in any order; a particle's place is its cell's start plus the
+// number of the cell's particles before it in caller order (a loop over the
+// cell, fewer steps than the density pass's scan of it), and the sorted keys
+// and indices are written.  Else they are given, and the cells' ranges
+// are written from the keys' boundaries (cells zeroed before).
+template <typename T, bool kCounted>
+__global__ void k_permute(int N, unsigned* __restrict__ skeys, unsigned* __restrict__ svals,
+                          const unsigned* __restrict__ order, const unsigned* __restrict__ key_in,
+                          const unsigned* __restrict__ count, const unsigned* __restrict__ start, gz_particles p,
                           const void* __restrict__ n_in, const int* __restrict__ box_of,
-                          const BoxInfo* __restrict__ boxes, int cbits, Sorted<T> s,
-                          int2* __restrict__ cells) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const unsigned src = svals[i];
-    s.x[i] = ((const T*)p.x)[src];
-    s.y[i] = ((const T*)p.y)[src];
-    s.z[i] = ((const T*)p.z)[src];
+                          const BoxInfo* __restrict__ boxes, Sorted<T> s, int2* __restrict__ cells) {
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= N) return;
+    unsigned src, key;
+    int i = q;
+    if constexpr (kCounted) {
+        src = order[q];
+        key = key_in[src];
+        const int a = (int)start[key], e = a + (int)count[key];
+        i = a;
+        for (int k = a; k < e; ++k) i += order[k] < src;
+        skeys[i] = key;
+        svals[i] = src;
+    } else {
+        src = svals[q];
+        key = skeys[q];
+    }
+    const T x = ((const T*)p.x)[src], y = ((const T*)p.y)[src], z = ((const T*)p.z)[src], h = ((const T*)p.h)[src];
+    s.x[i] = x;
+    s.y[i] = y;
+    s.z[i] = z;
     // velocities, mass and energy are optional (the density pass reads none)
     if (p.vx) s.vx[i] = ((const T*)p.vx)[src];
     if (p.vy) s.vy[i] = ((const T*)p.vy)[src];
     if (p.vz) s.vz[i] = ((const T*)p.vz)[src];
     if (p.m) s.m[i] = ((const T*)p.m)[src];
     if (p.u) s.u[i] = ((const T*)p.u)[src];
-    s.h[i] = ((const T*)p.h)[src];
-    s.pos[i] = P4<T>{s.x[i], s.y[i], s.z[i], s.h[i]};
+    s.h[i] = h;
+    s.pos[i] = P4<T>{x, y, z, h};
     s.id[i] = (long long)p.id[src];
     if (n_in) s.n[i] = ((const T*)n_in)[src];
     s.orig[i] = src;
     const int b = box_of[src];
     s.box[i] = b;
-    const unsigned key = skeys[i];
-    const unsigned mort = cbits * 3 >= 32 ? key : (key & ((1u << (3 * cbits)) - 1u));
-    const int nc = boxes[b].nc;
-    const int cx = compact3(mort), cy = compact3(mort >> 1), cz = compact3(mort >> 2);
-    const int lin = boxes[b].cell_off + (cz * nc + cy) * nc + cx;
-    if (i == 0 || skeys[i - 1] != key) cells[lin].x = i;
-    if (i == N - 1 || skeys[i + 1] != key) cells[lin].y = i + 1;
+    if constexpr (!kCounted) {
+        const BoxInfo bx = boxes[b];
+        const unsigned mort = key - bx.key_off;
+        const int cx = compact3(mort), cy = compact3(mort >> 1), cz = compact3(mort >> 2);
+        const int lin = bx.cell_off + (cz * bx.nc + cy) * bx.nc + cx;
+        if (i == 0 || skeys[i - 1] != key) cells[lin].x = i;
+        if (i == N - 1 || skeys[i + 1] != key) cells[lin].y = i + 1;
+    }
 }
 
 template <typename T>
@@ -232,8 +381,6 @@ __global__ void k_unpermute(int N, int rows, const unsigned* __restrict__ orig,
     const unsigned o = orig[i];
     for (int r = 0; r < rows; ++r) dst[(size_t)r * N + o] = src[(size_t)r * N + i];
 }
-
-inline int blocks(int n, int t) { return (n + t - 1) / t; }
 
 }  // namespace
 
@@ -265,16 +412,44 @@ Sorted<T> sorted_view(Ctx& c) {
 template Sorted<float> sorted_view<float>(Ctx&);
 template Sorted<double> sorted_view<double>(Ctx&);
 
+size_t sort_sums_len(long long N, long long keys, bool counted) {
+    if (counted) return (size_t)((keys + kScanTile - 1) / kScanTile);
+    const size_t nblk = (size_t)((N + kSortTile - 1) / kSortTile);
+    return kMaxDigits * nblk + kMaxDigits;  // per-block counts of up to 1024 digits, then the digit totals
+}
+
+template <typename T>
+static cudaError_t counting_sort(Ctx& c, const gz_particles& p, const void* n_in) {
+    const int N = c.N;
+    const long long K = c.total_keys;
+    cudaStream_t st = c.stream;
+    unsigned* order = (unsigned*)c.defer;  // (free until the density pass)
+    cudaMemsetAsync(c.kcount, 0, 4 * (size_t)K, st);
+    k_cs_count<T><<<blocks(N, 256), 256, 0, st>>>(N, (const T*)p.x, (const T*)p.y, (const T*)p.z, p.id, c.box_of,
+                                                   c.boxes, c.kcount, c.keys_alt, c.vals_alt, c.status);
+    const int tiles = (int)((K + kScanTile - 1) / kScanTile);
+    const bool direct = tiles <= kScanDirect;
+    if (!direct) k_cs_sums<<<tiles, kScanThreads, 0, st>>>(K, c.kcount, c.hist);
+    k_cs_scan<<<tiles, kScanThreads, 0, st>>>(K, c.kcount, direct ? nullptr : c.hist, c.boxes, c.nboxes, c.kstart,
+                                              c.cells);
+    k_cs_place<<<blocks(N, 256), 256, 0, st>>>(N, c.keys_alt, c.vals_alt, c.kstart, order);
+    k_permute<T, true><<<blocks(N, 256), 256, 0, st>>>(N, c.keys, c.vals, order, c.keys_alt, c.kcount, c.kstart, p,
+                                                        n_in, c.box_of, c.boxes, sorted_view<T>(c), c.cells);
+    c.launches += direct ? 4 : 5;
+    return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t sort_and_bin(Ctx& c, const gz_particles& p, const void* n_in) {
     c.last_lim = nullptr;  // a new sort: earlier sorted-order indices no longer apply
+    if (c.kcount) return counting_sort<T>(c, p, n_in);
     const int N = c.N;
     cudaStream_t st = c.stream;
     k_keys<T><<<blocks(N, 256), 256, 0, st>>>(N, (const T*)p.x, (const T*)p.y, (const T*)p.z, p.id,
-                                               c.box_of, c.boxes, c.cbits, c.keys, c.vals,
-                                               c.status);
+                                               c.box_of, c.boxes, c.keys, c.vals, c.status);
     const int nblk = blocks(N, kSortTile);
-    const int total_bits = 3 * c.cbits + c.box_bits;
+    int total_bits = 0;
+    while ((1ll << total_bits) < c.total_keys) ++total_bits;
     // the fewest passes of at most kMaxDigitBits bits, the bits spread evenly
     const int npass = (total_bits + kMaxDigitBits - 1) / kMaxDigitBits;
     const int bits = npass ? (total_bits + npass - 1) / npass : 0;
@@ -309,9 +484,8 @@ cudaError_t permute_and_bin(Ctx& c, const gz_particles& p, const void* n_in) {
     cudaStream_t st = c.stream;
     c.launches += 1;
     cudaMemsetAsync(c.cells, 0, sizeof(int2) * (size_t)c.total_cells, st);
-    Sorted<T> s = sorted_view<T>(c);
-    k_permute<T><<<blocks(N, 256), 256, 0, st>>>(N, c.keys, c.vals, p, n_in, c.box_of, c.boxes,
-                                                  c.cbits, s, c.cells);
+    k_permute<T, false><<<blocks(N, 256), 256, 0, st>>>(N, c.keys, c.vals, nullptr, nullptr, nullptr, nullptr, p,
+                                                         n_in, c.box_of, c.boxes, sorted_view<T>(c), c.cells);
     return cudaGetLastError();
 }
 template cudaError_t sort_and_bin<float>(Ctx&, const gz_particles&, const void*);
