@@ -71,17 +71,13 @@ __device__ __forceinline__ T vbar(T va, T v, T dvs) {
         return 0.5 * (va + v);
 }
 
-// Predicted positions of every particle at substep s (caller order) and the
-// number of particles active there.
+// Predicted positions of every particle at substep s (caller order).
 template <typename T>
 __global__ void k_h_predict(int N, int s, int K, gz_particles p, const T* __restrict__ hva,
                             const T* __restrict__ hdvs, const int* __restrict__ hsa,
-                            const int* __restrict__ hbin, const int* __restrict__ box_of,
-                            const double* __restrict__ D, T* __restrict__ xp, int* __restrict__ count) {
+                            const int* __restrict__ box_of, const double* __restrict__ D, T* __restrict__ xp) {
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    bool act = false;
     if (o < N) {
-        act = s % (1 << (K - hbin[o])) == 0;
         const int steps = s - hsa[o];
         const T* X[3] = {(const T*)p.x, (const T*)p.y, (const T*)p.z};
         const T* V[3] = {(const T*)p.vx, (const T*)p.vy, (const T*)p.vz};
@@ -97,30 +93,37 @@ __global__ void k_h_predict(int N, int s, int K, gz_particles p, const T* __rest
             }
         }
     }
-    const int c = __syncthreads_count(act);
+}
+
+// Number of particles active at substep s, once the bins up to it are final.
+__global__ void k_h_count(int N, int s, int K, const int* __restrict__ hbin, int* __restrict__ count) {
+    const int o = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = __syncthreads_count(o < N && s % (1 << (K - hbin[o])) == 0);
     if (threadIdx.x == 0 && c) atomicAdd(count, c);
 }
 
-// Sorted bins and active flags.
-__global__ void k_h_flags(int N, int s, int K, const unsigned* __restrict__ orig,
-                          const int* __restrict__ hbin, int* __restrict__ sbin,
-                          unsigned char* __restrict__ aflag) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const int b = hbin[orig[i]];
-    sbin[i] = b;
-    aflag[i] = (unsigned char)(s % (1 << (K - b)) == 0);
+// Sorted bins and active flags, and the flags' counts per compaction block.
+__global__ void __launch_bounds__(kCmpBlock)
+    k_h_flags(int N, int s, int K, const unsigned* __restrict__ orig, const int* __restrict__ hbin,
+              int* __restrict__ sbin, unsigned char* __restrict__ aflag, int* __restrict__ bcount) {
+    const int i = blockIdx.x * kCmpBlock + threadIdx.x;
+    bool act = false;
+    if (i < N) {
+        const int b = hbin[orig[i]];
+        sbin[i] = b;
+        act = s % (1 << (K - b)) == 0;
+        aflag[i] = (unsigned char)act;
+    }
+    const int c = __syncthreads_count(act);
+    if (threadIdx.x == 0) bcount[blockIdx.x] = c;
 }
 
 // ------------------------------------------- ordered stream compaction
-// flag -> list of the flagged indices in increasing order: per-block counts,
-// one block scanning them, per-block writes (warp ballots within a block).
-__global__ void __launch_bounds__(kCmpBlock)
-    k_cmp_count(int N, const unsigned char* __restrict__ flag, int* __restrict__ bcount) {
-    const int i = blockIdx.x * kCmpBlock + threadIdx.x;
-    const int c = __syncthreads_count(i < N && flag[i]);
-    if (threadIdx.x == 0) bcount[blockIdx.x] = c;
-}
+// flag -> list of the flagged indices in increasing order: per-block counts
+// (by the kernel that sets the flags), their scan (by every writing block for
+// itself up to kCmpDirect blocks, else by one block), per-block writes (warp
+// ballots within a block).
+constexpr int kCmpDirect = 4096;
 
 __global__ void __launch_bounds__(kCmpBlock) k_cmp_scan(int nb, int* __restrict__ bcount, int* __restrict__ total) {
     __shared__ int part[kCmpBlock];
@@ -146,10 +149,25 @@ __global__ void __launch_bounds__(kCmpBlock) k_cmp_scan(int nb, int* __restrict_
     if (t == kCmpBlock - 1) *total = part[t];
 }
 
+// total non-null: boff holds the counts, and the last block writes their sum.
 __global__ void __launch_bounds__(kCmpBlock)
     k_cmp_write(int N, const unsigned char* __restrict__ flag, const int* __restrict__ boff,
-                int* __restrict__ list) {
+                int* __restrict__ list, int* __restrict__ total) {
     __shared__ int wsum[kCmpBlock / 32];
+    int base = 0;
+    if (total) {
+        int v = 0;
+        for (int b = threadIdx.x; b < (int)blockIdx.x; b += kCmpBlock) v += boff[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v;
+        __syncthreads();
+        for (int w2 = 0; w2 < kCmpBlock / 32; ++w2) base += wsum[w2];
+        __syncthreads();
+        if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = base + boff[blockIdx.x];
+    } else {
+        base = boff[blockIdx.x];
+    }
     const int i = blockIdx.x * kCmpBlock + threadIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const bool f = i < N && flag[i];
@@ -167,27 +185,35 @@ __global__ void __launch_bounds__(kCmpBlock)
         wsum[lane] = x - v;
     }
     __syncthreads();
-    if (f) list[boff[blockIdx.x] + wsum[w] + __popc(ball & ((1u << lane) - 1u))] = i;
+    if (f) list[base + wsum[w] + __popc(ball & ((1u << lane) - 1u))] = i;
 }
 
 // --------------------------------------------------------- pair lists
-// Cells holding at least one active particle (sorted ranges).
-__global__ void k_h_cellact(int ncells, const int2* __restrict__ cells, const unsigned char* __restrict__ aflag,
-                            unsigned char* __restrict__ cellact) {
+// Smallest support radius among every cell's active particles (+inf without
+// any), rounded down.
+template <typename T>
+__global__ void k_h_cellmin(int ncells, const int2* __restrict__ cells, const unsigned char* __restrict__ aflag,
+                            const P4<T>* __restrict__ pos, float* __restrict__ cellmin) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncells) return;
     const int2 se = cells[c];
-    unsigned char any = 0;
-    for (int i = se.x; i < se.y && !any; ++i) any = aflag[i];
-    cellact[c] = any;
+    float h = INFINITY;
+    for (int i = se.x; i < se.y; ++i)
+        if (aflag[i]) {
+            if constexpr (sizeof(T) == 8)
+                h = fminf(h, __double2float_rd(pos[i].w));
+            else
+                h = fminf(h, pos[i].w);
+        }
+    cellmin[c] = h;
 }
 
 // Cells within two cells (per axis, periodic) of a cell holding an active
 // particle, marked by the active cells themselves (near must start zeroed).
 __global__ void k_h_dilate(int ncells, const BoxInfo* __restrict__ boxes, int nboxes,
-                           const unsigned char* __restrict__ cellact, unsigned char* __restrict__ near) {
+                           const float* __restrict__ cellmin, unsigned char* __restrict__ near) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncells || !cellact[c]) return;
+    if (c >= ncells || cellmin[c] == INFINITY) return;
     int lo = 0, hi = nboxes - 1;  // box of the cell: last box with cell_off <= c
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -220,17 +246,23 @@ __device__ __forceinline__ int cell_of(T v, int nc) {
 }
 
 // The flux pairs of active i with r >= H_i (so r < H_j, O10), found from the
-// partner's side: every particle j scans its own support (cells without an
-// active particle skipped) and appends itself to the list of each active i
-// there with r >= H_i; the lists are put in index order by k_h_sort.  r^2 is
-// the bit pattern the density pass forms for the pair, so these lists and
-// N_i split the flux pairs exactly.
+// partner's side: every particle j scans its own support and appends itself to
+// the list of each active i there with r >= H_i; the lists are put in index
+// order by k_h_sort.  r^2 is the bit pattern the density pass forms for the
+// pair, so these lists and N_i split the flux pairs exactly.  Cells whose
+// active particles all have H >= H_j hold no such pair and are skipped.  Sixteen
+// lanes share a particle's cells: a blast's emptied centre spans up to
+// thousands of them, and with one thread each the launch waited for those
+// (Sedov 64^3, an interval's lists of 16 substeps, late in the run: one thread
+// 9.6 ms, 4 lanes 6.2, 8 lanes 5.1, 16 lanes 4.7).
+constexpr int kScatterLanes = 16;
 template <typename T>
 __global__ void __launch_bounds__(128)
     k_h_rscatter(int N, Sorted<T> s, Grid g, KParams p, const unsigned char* __restrict__ aflag,
-                 const unsigned char* __restrict__ cellact, const unsigned char* __restrict__ near,
+                 const float* __restrict__ cellmin, const unsigned char* __restrict__ near,
                  unsigned* __restrict__ rnbr, int* __restrict__ rcount, DevStatus* st) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const int gl = threadIdx.x % kScatterLanes;
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) / kScatterLanes;
     if (j >= N) return;
     const BoxInfo bx = g.boxes[s.box[j]];
     const P4<T> me = s.pos[j];
@@ -243,25 +275,43 @@ __global__ void __launch_bounds__(128)
         if (!near[bx.cell_off + (cell_of(me.z, nc) * nc + cell_of(me.y, nc)) * nc + cell_of(me.x, nc)]) return;
     }
     const T H2 = Hj * Hj;
-    const unsigned char* ca = cellact + bx.cell_off;
-    for_candidates<T>(
-        g, bx, s.pos, j, me.x, me.y, me.z, Hj,
-        [&](int i, T, T, T, T r2) {
-            if (r2 < H2 && aflag[i]) {
-                const T Hi = s.pos[i].w;
-                if (!(r2 < Hi * Hi)) {
-                    const int slot = atomicAdd(&rcount[i], 1);
-                    if (slot < p.rcap)
-                        rnbr[lslot(slot, i, N)] = (unsigned)j;
-                    else
-                        set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
-                }
+    const float Hf = (float)Hj * (1.f + 1e-6f);  // (not below H_j)
+    const T xm1 = me.x - T(1), ym1 = me.y - T(1), zm1 = me.z - T(1);
+    const float xf = chop(me.x), yf = chop(me.y), zf = chop(me.z);
+    const Window<T> w(bx.nc, me.x, me.y, me.z, Hj);
+    for (int f = gl; f < w.ncube; f += kScatterLanes) {
+        int cx, cy, cz;
+        w.coords(f, cx, cy, cz);
+        const int lc = w.wrapped(cx, cy, cz);
+        if (!(cellmin[bx.cell_off + lc] < Hf)) continue;
+        const int2 se = w.range(g.cells + bx.cell_off, cx, cy, cz, xf, yf, zf);
+        for (int i0 = se.x; i0 < se.y; i0 += 4) {  // four candidates' loads in flight at a time
+            P4<T> q[4];
+            unsigned char act[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = min(i0 + u, se.y - 1);
+                q[u] = s.pos[i];
+                act[u] = aflag[i];
             }
-        },
-        [&](int lc) { return ca[lc] != 0; });
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = i0 + u;
+                const T r2 = sep2(mi_diff(q[u].x, me.x, xm1), mi_diff(q[u].y, me.y, ym1), mi_diff(q[u].z, me.z, zm1));
+                if (i >= se.y || i == j || !act[u] || !(r2 < H2) || r2 < q[u].w * q[u].w) continue;
+                const int slot = atomicAdd(&rcount[i], 1);
+                if (slot < p.rcap)
+                    rnbr[lslot(slot, i, N)] = (unsigned)j;
+                else
+                    set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
+            }
+        }
+    }
 }
 
-// Active i appends itself to the list of each inactive partner.
+// Active i appends itself to the list of each inactive partner: thread (t, y)
+// takes list groups y, y + kInGroups, ... (four slots each) of active particle t.
+constexpr int kInGroups = 8;
 __global__ void k_h_inlist(const int* __restrict__ alist, const int* __restrict__ nA,
                            const unsigned char* __restrict__ aflag, unsigned* __restrict__ nbr,
                            int* __restrict__ ncount, const unsigned* __restrict__ rnbr,
@@ -273,24 +323,33 @@ __global__ void k_h_inlist(const int* __restrict__ alist, const int* __restrict_
     for (int list = 0; list < 2; ++list) {
         const unsigned* L = list == 0 ? nbr + 4 * (size_t)i : rnbr + 4 * (size_t)i;
         const int n = list == 0 ? min(ncount[i], cap) : min(rcount[i], rcap);
-        for (int k = 0; k < n; ++k) {
-            const int j = (int)L[lcol(k, N)];
-            if (aflag[j]) continue;
-            const int slot = atomicAdd(&ncount[j], 1);
-            if (slot < cap)
-                nbr[lslot(slot, j, N)] = (unsigned)i;
-            else
-                set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, sid[j]);
+        for (int k0 = 4 * threadIdx.y; k0 < n; k0 += 4 * kInGroups) {
+            const uint4 jj = col4(L, k0, N);
+            const unsigned js[4] = {jj.x, jj.y, jj.z, jj.w};
+            bool in[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) in[u] = k0 + u < n && !aflag[js[u]];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (!in[u]) continue;
+                const int j = (int)js[u];
+                const int slot = atomicAdd(&ncount[j], 1);
+                if (slot < cap)
+                    nbr[lslot(slot, j, N)] = (unsigned)i;
+                else
+                    set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, sid[j]);
+            }
         }
     }
 }
 
 // Index order for the lists written by other threads: the inactive
 // particles' partner lists and the active particles' r >= H_i pairs.
-__global__ void k_h_sort(int N, const unsigned char* __restrict__ aflag, int* __restrict__ ncount,
-                         unsigned* __restrict__ nbr, int cap, const int* __restrict__ rcount,
-                         unsigned* __restrict__ rnbr, int rcap) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kListBlock)
+    k_h_sort(int N, const unsigned char* __restrict__ aflag, int* __restrict__ ncount,
+             unsigned* __restrict__ nbr, int cap, const int* __restrict__ rcount,
+             unsigned* __restrict__ rnbr, int rcap) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / kListLanes;
     if (i >= N) return;
     unsigned* L;
     int n;
@@ -299,25 +358,22 @@ __global__ void k_h_sort(int N, const unsigned char* __restrict__ aflag, int* __
         n = min(rcount[i], rcap);
     } else {
         n = min(ncount[i], cap);
-        ncount[i] = n;
         L = nbr + 4 * (size_t)i;
     }
-    for (int a = 1; a < n; ++a) {
-        const unsigned v = L[lcol(a, N)];
-        int b = a - 1;
-        while (b >= 0 && L[lcol(b, N)] > v) {
-            L[lcol(b + 1, N)] = L[lcol(b, N)];
-            --b;
-        }
-        L[lcol(b + 1, N)] = v;
-    }
+    sort_list(L, n, N);
+    if (!aflag[i] && threadIdx.x % kListLanes == 0) ncount[i] = n;
 }
 
-__global__ void k_h_tflags(int N, const unsigned char* __restrict__ aflag, const int* __restrict__ ncount,
-                           unsigned char* __restrict__ tflag) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    tflag[i] = (unsigned char)(aflag[i] || ncount[i] > 0);
+// Touched particles (active, or with an active partner), and their counts per
+// compaction block.
+__global__ void __launch_bounds__(kCmpBlock)
+    k_h_tflags(int N, const unsigned char* __restrict__ aflag, const int* __restrict__ ncount,
+               unsigned char* __restrict__ tflag, int* __restrict__ bcount) {
+    const int i = blockIdx.x * kCmpBlock + threadIdx.x;
+    const bool t = i < N && (aflag[i] || ncount[i] > 0);
+    if (i < N) tflag[i] = (unsigned char)t;
+    const int c = __syncthreads_count(t);
+    if (threadIdx.x == 0) bcount[blockIdx.x] = c;
 }
 
 // ----------------------------------------------- per-particle bookkeeping
@@ -570,7 +626,7 @@ cudaError_t ensure_hier_scratch(Ctx& c) {
         {(void**)&c.hsa, 4 * Nz},      {(void**)&c.hbin, 4 * Nz},    {(void**)&c.sbin, 4 * Nz},
         {(void**)&c.alist, 4 * Nz},    {(void**)&c.tlist, 4 * Nz},   {(void**)&c.hcount, 4 * 4},
         {(void**)&c.bcount, 4 * nb},   {(void**)&c.aflag, Nz},       {(void**)&c.tflag, Nz},
-        {(void**)&c.cellact, (size_t)c.total_cells}, {(void**)&c.cellnear, (size_t)c.total_cells},
+        {(void**)&c.cellmin, 4 * (size_t)c.total_cells}, {(void**)&c.cellnear, (size_t)c.total_cells},
         {(void**)&c.dtmax, 8 * (size_t)c.nboxes},
     };
     size_t total = 0;
@@ -579,6 +635,13 @@ cudaError_t ensure_hier_scratch(Ctx& c) {
     cudaError_t e = cudaMalloc(&base, total);
     if (e != cudaSuccess) return e;
     e = cudaMallocHost((void**)&c.hcount_host, 4 * sizeof(int));
+    if (e == cudaSuccess && !c.hier_counted) {
+        e = cudaEventCreateWithFlags(&c.hier_counted, cudaEventDisableTiming);
+        if (e != cudaSuccess) {
+            cudaFreeHost(c.hcount_host);
+            c.hcount_host = nullptr;
+        }
+    }
     if (e != cudaSuccess) {
         cudaFree(base);
         return e;
@@ -592,12 +655,13 @@ cudaError_t ensure_hier_scratch(Ctx& c) {
     return cudaSuccess;
 }
 
+// The list of the flagged particles, from the flags' block counts in c.bcount.
 static cudaError_t compact(Ctx& c, const unsigned char* flag, int* list, int* count) {
     const int nb = nblk(c.N, kCmpBlock);
-    c.launches += 3;
-    k_cmp_count<<<nb, kCmpBlock, 0, c.stream>>>(c.N, flag, c.bcount);
-    k_cmp_scan<<<1, kCmpBlock, 0, c.stream>>>(nb, c.bcount, count);
-    k_cmp_write<<<nb, kCmpBlock, 0, c.stream>>>(c.N, flag, c.bcount, list);
+    const bool direct = nb <= kCmpDirect;
+    c.launches += direct ? 1 : 2;
+    if (!direct) k_cmp_scan<<<1, kCmpBlock, 0, c.stream>>>(nb, c.bcount, count);
+    k_cmp_write<<<nb, kCmpBlock, 0, c.stream>>>(c.N, flag, c.bcount, list, direct ? count : nullptr);
     return cudaGetLastError();
 }
 
@@ -621,22 +685,23 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
     k_h_init<T><<<nblk(N, 256), 256, 0, st>>>(N, p, (T*)c.hva, (T*)c.hdvs, c.hsa, c.hbin);
     long long active = 0;
     const int S = 1 << K;
+    int nA = N;  // (substep 0: every particle)
     for (int s = 0; s < S && e == cudaSuccess; ++s) {
-        cudaMemsetAsync(c.hcount, 0, 4 * sizeof(int), st);
+        if (s > 0) {  // the count of this substep's active particles, formed after the last one's bins
+            e = cudaEventSynchronize(c.hier_counted);
+            if (e != cudaSuccess) break;
+            nA = c.hcount_host[s & 1];
+        }
         c.launches += 1;
         k_h_predict<T><<<nblk(N, 256), 256, 0, st>>>(N, s, K, p, (const T*)c.hva, (const T*)c.hdvs, c.hsa,
-                                                      c.hbin, c.box_of, c.dt_use, hxp, c.hcount);
-        cudaMemcpyAsync(c.hcount_host, c.hcount, sizeof(int), cudaMemcpyDeviceToHost, st);
-        e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) break;
-        const int nA = c.hcount_host[0];
+                                                      c.box_of, c.dt_use, hxp);
         active += nA;
         if (nA > 0) {
             Sorted<T> sv = sorted_view<T>(c);
             timer.begin(GZ_PASS_SORT);
             e = sort_and_bin<T>(c, pp, c.hn);
             c.launches += 1;
-            k_h_flags<<<nblk(N, 256), 256, 0, st>>>(N, s, K, c.vals, c.hbin, c.sbin, c.aflag);
+            k_h_flags<<<nblk(N, kCmpBlock), kCmpBlock, 0, st>>>(N, s, K, c.vals, c.hbin, c.sbin, c.aflag, c.bcount);
             if (e == cudaSuccess) e = compact(c, c.aflag, c.alist, c.hcount + 1);
             timer.end(GZ_PASS_SORT);
             cudaMemsetAsync(c.ncount, 0, sizeof(int) * (size_t)N, st);
@@ -650,17 +715,19 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             timer.begin(GZ_PASS_REVERSE);
             c.launches += 6;
             c.launches += 1;
-            k_h_cellact<<<nblk(c.total_cells, 256), 256, 0, st>>>(c.total_cells, c.cells, c.aflag, c.cellact);
+            k_h_cellmin<T><<<nblk(c.total_cells, 256), 256, 0, st>>>(c.total_cells, c.cells, c.aflag, sv.pos,
+                                                                      c.cellmin);
             cudaMemsetAsync(c.cellnear, 0, (size_t)c.total_cells, st);
-            k_h_dilate<<<nblk(c.total_cells, 256), 256, 0, st>>>(c.total_cells, c.boxes, c.nboxes, c.cellact,
+            k_h_dilate<<<nblk(c.total_cells, 256), 256, 0, st>>>(c.total_cells, c.boxes, c.nboxes, c.cellmin,
                                                                   c.cellnear);
-            k_h_rscatter<T><<<nblk(N, 128), 128, 0, st>>>(N, sv, g, kp, c.aflag, c.cellact, c.cellnear, c.rnbr,
-                                                           c.rcount, c.status);
-            k_h_inlist<<<nblk(nA, 128), 128, 0, st>>>(c.alist, c.hcount + 1, c.aflag, c.nbr, c.ncount, c.rnbr,
-                                                       c.rcount, c.cap, c.rcap, c.sid, c.N, c.status);
-            k_h_sort<<<nblk(N, 128), 128, 0, st>>>(N, c.aflag, c.ncount, c.nbr, c.cap, c.rcount, c.rnbr,
-                                                    c.rcap);
-            k_h_tflags<<<nblk(N, 256), 256, 0, st>>>(N, c.aflag, c.ncount, c.tflag);
+            k_h_rscatter<T><<<nblk(N, 128 / kScatterLanes), 128, 0, st>>>(N, sv, g, kp, c.aflag, c.cellmin, c.cellnear,
+                                                                           c.rnbr, c.rcount, c.status);
+            k_h_inlist<<<nblk(nA, 32), dim3(32, kInGroups), 0, st>>>(c.alist, c.hcount + 1, c.aflag, c.nbr, c.ncount,
+                                                                     c.rnbr, c.rcount, c.cap, c.rcap, c.sid, c.N,
+                                                                     c.status);
+            k_h_sort<<<nblk(N, kListBlock / kListLanes), kListBlock, 0, st>>>(N, c.aflag, c.ncount, c.nbr, c.cap,
+                                                                              c.rcount, c.rnbr, c.rcap);
+            k_h_tflags<<<nblk(N, kCmpBlock), kCmpBlock, 0, st>>>(N, c.aflag, c.ncount, c.tflag, c.bcount);
             if (e == cudaSuccess) e = compact(c, c.tflag, c.tlist, c.hcount + 2);
             timer.end(GZ_PASS_REVERSE);
             timer.begin(GZ_PASS_GRAD);
@@ -685,6 +752,18 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             k_h_bins<<<nblk(nA, 256), 256, 0, st>>>(c.alist, c.hcount + 1, c.vals, c.sbox, c.dti, c.dt_use,
                                                      c.params.cfl, K, s == 0 ? 1 : 0, c.hbin, c.sbin);
             timer.end(GZ_PASS_GRAD);
+        }
+        if (s + 1 < S) {
+            // the bins are final: the next substep's count goes to the host
+            // while the exchange runs
+            c.launches += 1;
+            cudaMemsetAsync(c.hcount + 3, 0, sizeof(int), st);
+            k_h_count<<<nblk(N, 256), 256, 0, st>>>(N, s + 1, K, c.hbin, c.hcount + 3);
+            cudaMemcpyAsync(c.hcount_host + ((s + 1) & 1), c.hcount + 3, sizeof(int), cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaEventRecord(c.hier_counted, st);
+        }
+        if (nA > 0) {
+            Sorted<T> sv = sorted_view<T>(c);
             timer.begin(GZ_PASS_FLUX);
             c.launches += 1;
             launch_exchange<T>(c, kp, N, nA);
@@ -721,6 +800,8 @@ template cudaError_t run_step_hier<double>(Ctx&, gz_particles&, int, double, dou
 void free_hier_scratch(Ctx& c) {
     if (c.hier_arena) cudaFree(c.hier_arena);
     if (c.hcount_host) cudaFreeHost(c.hcount_host);
+    if (c.hier_counted) cudaEventDestroy(c.hier_counted);
+    c.hier_counted = nullptr;
     c.hier_arena = nullptr;
     c.hcount_host = nullptr;
 }

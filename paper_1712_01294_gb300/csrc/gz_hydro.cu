@@ -53,22 +53,32 @@ __global__ void k_reverse(int N, Sorted<T> s, KParams p, const unsigned* __restr
     }
 }
 
-// Orders each reverse list by sorted index so the flux sums are deterministic.
+// Orders each reverse list by sorted index so the flux sums are deterministic:
+// up to eight entries (most lists) in registers, each placed by the number of
+// smaller ones; longer ones by insertion.
 __global__ void k_sort_rev(int N, const int* __restrict__ rcount, unsigned* __restrict__ rnbr,
                            int rcap) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const int n = min(rcount[i], rcap);
+    if (n < 2) return;
     unsigned* L = rnbr + 4 * (size_t)i;
-    for (int a = 1; a < n; ++a) {
-        const unsigned v = L[lcol(a, N)];
-        int b = a - 1;
-        while (b >= 0 && L[lcol(b, N)] > v) {
-            L[lcol(b + 1, N)] = L[lcol(b, N)];
-            --b;
+    if (n <= 8) {
+        const uint4 a = *reinterpret_cast<const uint4*>(L);
+        uint4 b = make_uint4(0, 0, 0, 0);
+        if (n > 4) b = *reinterpret_cast<const uint4*>(L + lcol(4, N));
+        const unsigned v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (k >= n) break;
+            int at = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) at += q < n && v[q] < v[k];
+            L[lcol(at, N)] = v[k];
         }
-        L[lcol(b + 1, N)] = v;
+        return;
     }
+    insert_sort(L, n, N);
 }
 
 // O5 primitives: rho = m n, P = (gamma - 1) rho u, c = sqrt(gamma P / rho).

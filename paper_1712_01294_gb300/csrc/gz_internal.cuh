@@ -160,14 +160,15 @@ struct Ctx {
     int* sbin = nullptr;      // [N] bin (sorted order)
     int* alist = nullptr;     // [N] active particles (sorted indices)
     int* tlist = nullptr;     // [N] particles with an exchange this substep
-    int* hcount = nullptr;    // [4] device counters (predicted actives, |alist|, |tlist|)
+    int* hcount = nullptr;    // [4] device counters (1: |alist|, 2: |tlist|, 3: next substep's actives)
     int* bcount = nullptr;    // per-block counts of the list compaction
     unsigned char* aflag = nullptr;  // [N] active (sorted order)
     unsigned char* tflag = nullptr;  // [N] touched (sorted order)
-    unsigned char* cellact = nullptr;     // [cells] cell holds an active particle
+    float* cellmin = nullptr;             // [cells] smallest H of the cell's active particles
     unsigned char* cellnear = nullptr;    // [cells] an active cell lies within two cells
     unsigned long long* dtmax = nullptr;  // [nboxes] largest finite criterion (bits)
-    int* hcount_host = nullptr;           // pinned copy of hcount
+    int* hcount_host = nullptr;           // pinned: active particles of the next substep (two slots)
+    cudaEvent_t hier_counted = nullptr;   // its copy done
     // subdomain of a decomposed box (gz_create_subdomain): the particles held
     // are the owned ones and ghost copies completing their neighbourhoods
     unsigned char* owned = nullptr;  // [capacity] 1 = owned (caller order); null: all owned
@@ -568,10 +569,14 @@ struct Window {
         };
         const float gx = gap(cx, xi), gy = gap(cy, yi), gz = gap(cz, zi);
         if ((gz * gz + gy * gy) + gx * gx > R2m) return make_int2(0, 0);
+        return cells[wrapped(cx, cy, cz)];
+    }
+    // Index of cell (cx, cy, cz) within its box.
+    __device__ __forceinline__ int wrapped(int cx, int cy, int cz) const {
         const int wx = cx < 0 ? cx + nc : (cx >= nc ? cx - nc : cx);
         const int wy = cy < 0 ? cy + nc : (cy >= nc ? cy - nc : cy);
         const int wz = cz < 0 ? cz + nc : (cz >= nc ? cz - nc : cz);
-        return cells[(wz * nc + wy) * nc + wx];
+        return (wz * nc + wy) * nc + wx;
     }
 };
 
@@ -594,6 +599,45 @@ __device__ __forceinline__ float r2_chop(double xj, double yj, double zj, float 
 __device__ __forceinline__ float r2_chop_bound(double R) {
     const float r = ((float)R + 4e-7f) * (1.f + 1e-6f);
     return r * r;
+}
+
+// The n entries of the list column L put in increasing order by insertion.
+__device__ __forceinline__ void insert_sort(unsigned* __restrict__ L, int n, int N) {
+    for (int a = 1; a < n; ++a) {
+        const unsigned x = L[lcol(a, N)];
+        int b = a - 1;
+        while (b >= 0 && L[lcol(b, N)] > x) {
+            L[lcol(b + 1, N)] = L[lcol(b, N)];
+            --b;
+        }
+        L[lcol(b + 1, N)] = x;
+    }
+}
+
+// The same by kListLanes lanes (the entries are distinct; blocks of kListBlock
+// threads): each lane places its entries by the number of smaller ones; lists
+// longer than kListMax by insertion.  For lists of a few dozen entries: one
+// thread's insertion through global memory is a chain of dependent accesses
+// (hierarchical Sedov 64^3: 26 us a substep, 15 so).
+constexpr int kListLanes = 8, kListBlock = 128, kListMax = 64;
+__device__ __forceinline__ void sort_list(unsigned* __restrict__ L, int n, int N) {
+    __shared__ unsigned sh[kListBlock / kListLanes][kListMax + kListLanes];
+    if (n < 2) return;
+    const int gl = threadIdx.x % kListLanes;
+    const unsigned gm = group_mask<kListLanes>();
+    unsigned* v = sh[threadIdx.x / kListLanes];
+    if (n <= kListMax) {
+        for (int k = gl; k < n; k += kListLanes) v[k] = L[lcol(k, N)];
+        __syncwarp(gm);
+        for (int k = gl; k < n; k += kListLanes) {
+            const unsigned x = v[k];
+            int at = 0;
+            for (int q = 0; q < n; ++q) at += v[q] < x;
+            L[lcol(at, N)] = x;
+        }
+    } else if (gl == 0) {
+        insert_sort(L, n, N);
+    }
 }
 
 // Scan of one particle's search window by the G lanes of its group (all of

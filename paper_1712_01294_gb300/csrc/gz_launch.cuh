@@ -107,8 +107,8 @@ struct PassTimer {
 };
 
 // Hierarchical timesteps: one sync interval of 2^K substeps in place on p
-// (one host synchronisation per substep to read the number of active
-// particles).  active_out (host) receives the active particle-substeps.
+// (one host wait per substep for the number of active particles, formed while
+// the substep before still runs).  active_out (host) receives the active particle-substeps.
 cudaError_t ensure_hier_scratch(Ctx& c);
 void free_hier_scratch(Ctx& c);
 template <typename T>
