@@ -116,6 +116,38 @@ __device__ __forceinline__ T dot3(T x0, T x1, T x2, T y0, T y1, T y2) {
     return fma(x2, y2, fma(x1, y1, mul_rn(x0, y0)));
 }
 
+// Minimum-image offsets of four positions from (x, y, z) (xm1 = x - 1, ...).
+// FP32: plain differences, which are mi_diff's wherever no |d| reaches 1/2, and
+// one test for the four; FP64: mi_diff (its test is on words).
+__device__ __forceinline__ void offsets4(const P4<float> (&q)[4], float x, float y, float z, float xm1, float ym1,
+                                         float zm1, float (&dx)[4], float (&dy)[4], float (&dz)[4]) {
+    float m = 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        dx[u] = q[u].x - x;
+        dy[u] = q[u].y - y;
+        dz[u] = q[u].z - z;
+        m = fmaxf(fmaxf(m, fabsf(dx[u])), fmaxf(fabsf(dy[u]), fabsf(dz[u])));
+    }
+    if (m >= 0.5f) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            dx[u] = mi_diff(q[u].x, x, xm1);
+            dy[u] = mi_diff(q[u].y, y, ym1);
+            dz[u] = mi_diff(q[u].z, z, zm1);
+        }
+    }
+}
+__device__ __forceinline__ void offsets4(const P4<double> (&q)[4], double x, double y, double z, double, double,
+                                         double, double (&dx)[4], double (&dy)[4], double (&dz)[4]) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        dx[u] = mi_diff(q[u].x, x, 0.0);
+        dy[u] = mi_diff(q[u].y, y, 0.0);
+        dz[u] = mi_diff(q[u].z, z, 0.0);
+    }
+}
+
 // Symmetric 3x3 inverse by adjugate; kappa = |E|_F |B|_F / 3.
 template <typename A>
 __device__ __forceinline__ void invert_sym(const A E[6], A B[6], A& det, A& kap) {

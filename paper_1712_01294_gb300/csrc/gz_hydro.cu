@@ -106,14 +106,19 @@ __global__ void k_prim(int N, Sorted<T> s, KParams p, DevStatus* st) {
 // signal-speed step (over N_i and the reverse list) and its per-box minimum.
 // Record (32 values): x y z H | 1/H knorm rho P | vx vy vz g0 | g1..g14 | B0..B5
 // with knorm = 8/(pi H^3 n^2) so that V_i psi_j(x_i) = knorm * w(r/H).
-// Neighbours are read four at a time (one 16-byte load of indices, then the
-// packed records of all four) so their loads are in flight together.
+// Neighbours are read four at a time (one 16-byte load of indices, a group
+// ahead, then the packed records of all four) so their loads are in flight
+// together.  The pass waits on them half the time and issues the other half;
+// instructions a neighbour (one boundary test for four offsets, the kernel
+// without its two pieces, the pair weight's constant applied after the loop,
+// min/max as such) took it from 624 to 488 us at 128^3, FP64 at 48^3 894 to
+// 627.  Held to 128 registers (4 blocks per SM); at 5 blocks it spills (570 us),
+// and with the next group's records loaded ahead (162 registers) it took 598.
 // kInfo: also track which particles the limiter's bounds came from and write
 // what the adjoint reads (ginfo, lim); without it (a plain forward step) that
-// bookkeeping takes no registers or instructions (3 % faster; capped at 5
-// blocks per SM the FP32 kernel spills and gains nothing more).
+// bookkeeping takes no registers or instructions.
 template <typename T, bool kInfo>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
     k_gradients(int N, Sorted<T> s, const unsigned* __restrict__ nbr, const int* __restrict__ ncount,
                 const unsigned* __restrict__ rnbr, const int* __restrict__ rcount, KParams p,
                 T* __restrict__ rec, double* __restrict__ dti, unsigned long long* __restrict__ dtmin,
@@ -156,28 +161,33 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1)
         bool any = false;
         const int cnt = min(ncount[i], p.cap);
         const unsigned* L = nbr + 4 * (size_t)i;
+        uint4 jj = make_uint4(0, 0, 0, 0);
+        if (cnt > 0) jj = col4(L, 0, N);
         for (int k0 = 0; k0 < cnt; k0 += 4) {
-            const uint4 jj = col4(L, k0, N);
             const unsigned js[4] = {jj.x, jj.y, jj.z, jj.w};
+            if (k0 + 4 < cnt) jj = col4(L, k0 + 4, N);
             P4<T> q[4], w[4];
             P2<T> w2[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
+                q[u] = me;
                 if (k0 + u < cnt) {
                     q[u] = s.pos[js[u]];
                     w[u] = s.prim[js[u]];
                     w2[u] = s.prim2[js[u]];
                 }
             }
+            T dx4[4], dy4[4], dz4[4];
+            offsets4(q, xi, yi, zi, xim1, yim1, zim1, dx4, dy4, dz4);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (k0 + u >= cnt) break;
-                const T dx = mi_diff(q[u].x, xi, xim1), dy = mi_diff(q[u].y, yi, yim1),
-                        dz = mi_diff(q[u].z, zi, zim1);
-                const T r2 = sep2(dx, dy, dz);
-                const T r = psqrt(r2);
-                const T psi = norm * kern_w(r * iH);
-                const T pdx = psi * dx, pdy = psi * dy, pdz = psi * dz;
+                const T dx = dx4[u], dy = dy4[u], dz = dz4[u];
+                const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
+                const T ir = rsq_(r2);
+                // (half of W(r/H); the pair's weight is psi = norm W, applied after the loop)
+                const T kh = kern_half(mul_rn(r2, ir), iH);
+                const T pdx = kh * dx, pdy = kh * dy, pdz = kh * dz;
                 E[0] += pdx * dx;
                 E[1] += pdx * dy;
                 E[2] += pdx * dz;
@@ -185,29 +195,39 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1)
                 E[4] += pdy * dz;
                 E[5] += pdz * dz;
                 const T Wj[5] = {w[u].x, w[u].y, w[u].z, w[u].w, w2[u].x};
+                T df[5];
 #pragma unroll
                 for (int f = 0; f < 5; ++f) {
-                    const T df = Wj[f] - Wi[f];
-                    Sg[3 * f] += df * pdx;
-                    Sg[3 * f + 1] += df * pdy;
-                    Sg[3 * f + 2] += df * pdz;
-                    if (Wj[f] > fmax[f]) {
-                        fmax[f] = Wj[f];
-                        if constexpr (kInfo) kmax[f] = (int)js[u];
-                    }
-                    if (Wj[f] < fmin[f]) {
-                        fmin[f] = Wj[f];
-                        if constexpr (kInfo) kmin[f] = (int)js[u];
+                    df[f] = Wj[f] - Wi[f];
+                    Sg[3 * f] += df[f] * pdx;
+                    Sg[3 * f + 1] += df[f] * pdy;
+                    Sg[3 * f + 2] += df[f] * pdz;
+                    if constexpr (kInfo) {
+                        if (Wj[f] > fmax[f]) {
+                            fmax[f] = Wj[f];
+                            kmax[f] = (int)js[u];
+                        }
+                        if (Wj[f] < fmin[f]) {
+                            fmin[f] = Wj[f];
+                            kmin[f] = (int)js[u];
+                        }
+                    } else {
+                        fmax[f] = max_(fmax[f], Wj[f]);
+                        fmin[f] = min_(fmin[f], Wj[f]);
                     }
                 }
                 if (want_dt) {
-                    const T vd = ((Wj[1] - Wi[1]) * dx + (Wj[2] - Wi[2]) * dy) + (Wj[3] - Wi[3]) * dz;
-                    const T vs = ci + w2[u].y - min(pdiv(vd, r), T(0));
-                    vmax = any ? max(vmax, vs) : vs;
+                    const T vd = dot3(df[1], df[2], df[3], dx, dy, dz);
+                    const T vs = ci + w2[u].y - min_(vd * ir, T(0));
+                    vmax = any ? max_(vmax, vs) : vs;
                     any = true;
                 }
             }
         }
+#pragma unroll
+        for (int q = 0; q < 6; ++q) E[q] *= T(2) * norm;
+#pragma unroll
+        for (int q = 0; q < 15; ++q) Sg[q] *= T(2) * norm;
         // O7: B = E^-1; FP64 re-do of E and its inverse when kappa > kappa_max
         T B[6], det, kap;
         invert_sym<T>(E, B, det, kap);
@@ -270,30 +290,37 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1)
         T Dpos[5] = {T(0), T(0), T(0), T(0), T(0)}, Dneg[5] = {T(0), T(0), T(0), T(0), T(0)};
         int jpos[5] = {-1, -1, -1, -1, -1}, jneg[5] = {-1, -1, -1, -1, -1};
         const T beta = (T)p.beta;
+        if (cnt > 0) jj = col4(L, 0, N);
         for (int k0 = 0; k0 < cnt; k0 += 4) {
-            const uint4 jj = col4(L, k0, N);
             const unsigned js[4] = {jj.x, jj.y, jj.z, jj.w};
+            if (k0 + 4 < cnt) jj = col4(L, k0 + 4, N);
             P4<T> q[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < 4; ++u) {
+                q[u] = me;  // (a spare slot: D = 0, no constraint)
                 if (k0 + u < cnt) q[u] = s.pos[js[u]];
+            }
+            T dx4[4], dy4[4], dz4[4];
+            offsets4(q, xi, yi, zi, xim1, yim1, zim1, dx4, dy4, dz4);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (k0 + u >= cnt) break;
-                const T dx = mi_diff(q[u].x, xi, xim1), dy = mi_diff(q[u].y, yi, yim1),
-                        dz = mi_diff(q[u].z, zi, zim1);
-                const T sij = pdiv(Hi, Hi + q[u].w);
-                const T ox = sij * dx, oy = sij * dy, oz = sij * dz;
+                const T sij = Hi * rcp_(Hi + q[u].w);
+                const T ox = sij * dx4[u], oy = sij * dy4[u], oz = sij * dz4[u];
 #pragma unroll
                 for (int f = 0; f < 5; ++f) {
-                    const T D = (gt[3 * f] * ox + gt[3 * f + 1] * oy) + gt[3 * f + 2] * oz;
-                    if (D > Dpos[f]) {
-                        Dpos[f] = D;
-                        if constexpr (kInfo) jpos[f] = (int)js[u];
-                    }
-                    if (D < Dneg[f]) {
-                        Dneg[f] = D;
-                        if constexpr (kInfo) jneg[f] = (int)js[u];
+                    const T D = dot3(gt[3 * f], gt[3 * f + 1], gt[3 * f + 2], ox, oy, oz);
+                    if constexpr (kInfo) {
+                        if (D > Dpos[f]) {
+                            Dpos[f] = D;
+                            jpos[f] = (int)js[u];
+                        }
+                        if (D < Dneg[f]) {
+                            Dneg[f] = D;
+                            jneg[f] = (int)js[u];
+                        }
+                    } else {
+                        Dpos[f] = max_(Dpos[f], D);
+                        Dneg[f] = min_(Dneg[f], D);
                     }
                 }
             }
@@ -336,10 +363,10 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1)
                 const P4<T> w = s.prim[j];
                 const T dx = mi_diff(q.x, xi, xim1), dy = mi_diff(q.y, yi, yim1),
                         dz = mi_diff(q.z, zi, zim1);
-                const T r = psqrt(sep2(dx, dy, dz));
-                const T vd = ((w.y - Wi[1]) * dx + (w.z - Wi[2]) * dy) + (w.w - Wi[3]) * dz;
-                const T vs = ci + s.prim2[j].y - min(pdiv(vd, r), T(0));
-                vmax = any ? max(vmax, vs) : vs;
+                const T ir = rsq_(max_(sep2(dx, dy, dz), Tiny<T>::sq));
+                const T vd = dot3(w.y - Wi[1], w.z - Wi[2], w.w - Wi[3], dx, dy, dz);
+                const T vs = ci + s.prim2[j].y - min_(vd * ir, T(0));
+                vmax = any ? max_(vmax, vs) : vs;
                 any = true;
             }
             if (std::is_same<T, float>::value)  // FP32 path: no FP64 cbrt / division per particle
