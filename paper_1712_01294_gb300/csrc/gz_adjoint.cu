@@ -25,199 +25,148 @@ inline int blocks(int n, int t) { return (n + t - 1) / t; }
 
 enum : int { AX = 0, AV = 3, AU = 6, AM = 7, AH = 8, AN = 9, ARHO = 10, AP = 11, AG = 12, AB = 27 };
 
-// Derivative of the kernel shape (exact, for both precisions).
+// What the pairs of particle a add up to (pair_adjoint); flux_adj_row turns it
+// into a's adjoint row after the last pair, so that nothing that depends on a
+// alone is formed per pair.
 template <typename T>
-__device__ __forceinline__ T dkern(T q) {
-    return kern_dw(q);
-}
+struct AdjSums {
+    T x[3];   // -dJ/dx_a
+    T F[5];   // face value F_a (to the half-step primitives)
+    T W[5];   // primitives of a as clamp bounds or in the first-order fallback
+    T g[15];  // F_a's gradients
+    T B[6];
+    T k;      // knorm_a
+    T q;      // sum of (dJ/dq_a) q_a, q_a = r / H_a
+    T h;      // H_a through the face position
+};
 
 // Adjoint of particle a's share of the pair (a, b).  wp = dpbar_a - dpbar_b
-// and wE = dEbar_a - dEbar_b weight the pair's rate contributions; adj
-// receives dJ/d(a's inputs).  Re-evaluates the forward exactly as
-// pair_rates does so every branch matches.  inv_na = 1/n_a and irho =
-// 1/rho_a are the particle's own reciprocals; every division of the reverse
-// sweep is a product with a reciprocal (pdiv: hardware reciprocal in FP32).
+// and wE = dEbar_a - dEbar_b weight the pair's rate contributions.  The
+// forward is re-evaluated as pair_rates forms it (its symmetric star state,
+// in which v_f drops out), so every branch matches; Wh: half_state of a.
+// Divisions are products with the reciprocals the forward takes anyway: FP64
+// is bound by its pipe (977 operations a pair where the canonical L/R order,
+// v_f and a's own terms were carried through each pair, 3.88 ms at 40^3; 486
+// here, 1.93 ms).
 template <typename T>
-__device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)[kRecord], bool aL,
-                                             T hdt, T gam, bool hancock, T inv_na, T irho, const T* wp,
-                                             T wE, T* adj) {
+__device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)[kRecord], const T (&Wh)[5], bool aL,
+                                             T hdt, T gam, const T* wp, T wE, AdjSums<T>& s) {
     // ---- forward (same operations as pair_rates)
     const T dx = mi_diff(b[0], a[0], a[0] - T(1));
     const T dy = mi_diff(b[1], a[1], a[1] - T(1));
     const T dz = mi_diff(b[2], a[2], a[2] - T(1));
-    const T d[3] = {dx, dy, dz};
-    const T r2 = sep2(dx, dy, dz);
-    const T r = psqrt(r2);
-    const bool ina = r2 < a[3] * a[3], inb = r2 < b[3] * b[3];
-    const T qa = r * a[4], qb = r * b[4];
-    const T wa = kern_w(qa), wb = kern_w(qb);
-    const T ca = ina ? a[5] * wa : T(0);
-    const T cb = inb ? b[5] * wb : T(0);
+    const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
+    const T ir = rsq_(r2);
+    const T r = mul_rn(r2, ir);
+    T wa, wb, da, db;
+    kern_half_d(r, a[4], wa, da);
+    kern_half_d(r, b[4], wb, db);
+    const T ca = a[5] * wa, cb = b[5] * wb;
     const T* Ba = a + 26;
     const T* Bb = b + 26;
-    const T Bda[3] = {(Ba[0] * dx + Ba[1] * dy) + Ba[2] * dz, (Ba[1] * dx + Ba[3] * dy) + Ba[4] * dz,
-                      (Ba[2] * dx + Ba[4] * dy) + Ba[5] * dz};
-    const T Bdb[3] = {(Bb[0] * dx + Bb[1] * dy) + Bb[2] * dz, (Bb[1] * dx + Bb[3] * dy) + Bb[4] * dz,
-                      (Bb[2] * dx + Bb[4] * dy) + Bb[5] * dz};
-    T A[3];
+    const T ua[3] = {dot3(Ba[0], Ba[1], Ba[2], dx, dy, dz), dot3(Ba[1], Ba[3], Ba[4], dx, dy, dz),
+                     dot3(Ba[2], Ba[4], Ba[5], dx, dy, dz)};
+    const T ub[3] = {dot3(Bb[0], Bb[1], Bb[2], dx, dy, dz), dot3(Bb[1], Bb[3], Bb[4], dx, dy, dz),
+                     dot3(Bb[2], Bb[4], Bb[5], dx, dy, dz)};
+    T A[3];  // (half of the face area vector)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) A[k] = add_rn(mul_rn(ca, Bda[k]), mul_rn(cb, Bdb[k]));
+    for (int k = 0; k < 3; ++k) A[k] = add_rn(mul_rn(ca, ua[k]), mul_rn(cb, ub[k]));
     const T Aq = sep2(A[0], A[1], A[2]);
-    if (!(Aq > T(0))) return;
-    const T Am = psqrt(Aq);
-    const T iA = pdiv(T(1), Am);
-    const T nh[3] = {A[0] * iA, A[1] * iA, A[2] * iA};
-    const T Hs = a[3] + b[3];
-    const T sa = pdiv(a[3], Hs), sb = pdiv(b[3], Hs);
-    T Fa[5], Fb[5];
-    T inca[5], incb[5];
-    hancock_inc(a, hdt, gam, hancock, inca);
-    hancock_inc(b, hdt, gam, hancock, incb);
-    face_state(a, sa, dx, dy, dz, inca, Fa);
-    face_state(b, sb, -dx, -dy, -dz, incb, Fb);
-    const T Wa[5] = {a[6], a[8], a[9], a[10], a[7]};
-    const T Wb[5] = {b[6], b[8], b[9], b[10], b[7]};
-    // clamp sides: 0 inside, -1 clamped to the lower bound, +1 to the upper
-    int ka[5], kb[5];
-    T Ca[5], Cb[5];
+    if (!pos_(Aq - Tiny<T>::sq)) return;
+    const T iA = rsq_(Aq);
+    const T n[3] = {A[0] * iA, A[1] * iA, A[2] * iA};
+    const T iHs = rcp_(a[3] + b[3]);
+    const T sa = a[3] * iHs, sb = b[3] * iHs;
+    T Ga[5], Gb[5], Da[5], Db[5], Wb[5];
+    int ka[5], kb[5];  // clamp sides: 0 inside, -1 at the lower bound, +1 at the upper
+    half_state(b, hdt, gam, Wb);
+    const T Wa0[5] = {a[6], a[8], a[9], a[10], a[7]};
+    const T Wb0[5] = {b[6], b[8], b[9], b[10], b[7]};
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
-        const T lo = min(Wa[f], Wb[f]), hi = max(Wa[f], Wb[f]);
-        const T ma = max(Fa[f], lo), mb = max(Fb[f], lo);
-        Ca[f] = min(ma, hi);
-        Cb[f] = min(mb, hi);
-        ka[f] = Fa[f] < lo ? -1 : (ma > hi ? 1 : 0);
-        kb[f] = Fb[f] < lo ? -1 : (mb > hi ? 1 : 0);
+        Da[f] = dot3(a[11 + 3 * f], a[12 + 3 * f], a[13 + 3 * f], dx, dy, dz);
+        Db[f] = dot3(b[11 + 3 * f], b[12 + 3 * f], b[13 + 3 * f], dx, dy, dz);
+        const T lo = min_(Wa0[f], Wb0[f]), hi = max_(Wa0[f], Wb0[f]);
+        const T Fa = fma(sa, Da[f], Wh[f]), Fb = fma(-sb, Db[f], Wb[f]);
+        ka[f] = less_(Fa, lo) ? -1 : (less_(hi, Fa) ? 1 : 0);
+        kb[f] = less_(Fb, lo) ? -1 : (less_(hi, Fb) ? 1 : 0);
+        Ga[f] = ka[f] < 0 ? lo : (ka[f] > 0 ? hi : Fa);
+        Gb[f] = kb[f] < 0 ? lo : (kb[f] > 0 ? hi : Fb);
     }
-    const bool fallback = !(Ca[0] > T(0) && Ca[4] > T(0) && Cb[0] > T(0) && Cb[4] > T(0));
-    T Ga[5], Gb[5];  // face states after clamp / fallback
+    const bool fallback = !(pos_(Ga[0]) && pos_(Ga[4]) && pos_(Gb[0]) && pos_(Gb[4]));
+    if (fallback) {
 #pragma unroll
-    for (int f = 0; f < 5; ++f) {
-        Ga[f] = fallback ? Wa[f] : Ca[f];
-        Gb[f] = fallback ? Wb[f] : Cb[f];
+        for (int f = 0; f < 5; ++f) {
+            Ga[f] = Wa0[f];
+            Gb[f] = Wb0[f];
+        }
     }
-    T FL[5], FR[5];
-#pragma unroll
-    for (int f = 0; f < 5; ++f) {
-        FL[f] = aL ? Ga[f] : Gb[f];
-        FR[f] = aL ? Gb[f] : Ga[f];
-    }
-    const T vL[3] = {aL ? Wa[1] : Wb[1], aL ? Wa[2] : Wb[2], aL ? Wa[3] : Wb[3]};
-    const T vR[3] = {aL ? Wb[1] : Wa[1], aL ? Wb[2] : Wa[2], aL ? Wb[3] : Wa[3]};
-    const T sL = aL ? sa : sb;
-    const T sg = aL ? T(1) : T(-1);
-    const T n[3] = {sg * nh[0], sg * nh[1], sg * nh[2]};
-    const T vf[3] = {vL[0] + sL * (vR[0] - vL[0]), vL[1] + sL * (vR[1] - vL[1]),
-                     vL[2] + sL * (vR[2] - vL[2])};
-    const T vfn = (vf[0] * n[0] + vf[1] * n[1]) + vf[2] * n[2];
-    const T uL = ((FL[1] - vf[0]) * n[0] + (FL[2] - vf[1]) * n[1]) + (FL[3] - vf[2]) * n[2];
-    const T uR = ((FR[1] - vf[0]) * n[0] + (FR[2] - vf[1]) * n[1]) + (FR[3] - vf[2]) * n[2];
-    const T rL = FL[0], PL = FL[4], rR = FR[0], PR = FR[4];
-    const T cL = psqrt(pdiv(gam * PL, rL)), cR = psqrt(pdiv(gam * PR, rR));
-    const T e1 = uL - cL, e2 = uR - cR, e3 = uL + cL, e4 = uR + cR;
-    const T SL = min(e1, e2), SR = max(e3, e4);
-    const T aLv = SL - uL, aRv = SR - uR;
-    const T num = ((PR - PL) + rL * uL * aLv) - rR * uR * aRv;
-    const T den = rL * aLv - rR * aRv;
-    const T ss = pdiv(num, den);
-    const T psr = PL + rL * aLv * (ss - uL);
-    const T ps = psr < T(0) ? T(0) : psr;
-    // ---- reverse, in the working precision
-    const T A_[3] = {A[0], A[1], A[2]};
-    const T wpA = (wp[0] * A_[0] + wp[1] * A_[1]) + wp[2] * A_[2];
-    // J = -ps (wp . A) - sg wE ps (ss + vfn) |A|
-    const T b_ps = -wpA - (T)sg * wE * ((T)ss + vfn) * (T)Am;
-    T bA[3] = {-(T)ps * wp[0], -(T)ps * wp[1], -(T)ps * wp[2]};
-    T b_ss = -(T)sg * wE * (T)ps * (T)Am;
-    const T b_vfn = b_ss;
-    const T b_Am = -(T)sg * wE * (T)ps * ((T)ss + vfn);
-    // ps = max(psr, 0)
-    const T b_psr = psr < T(0) ? T(0) : b_ps;
-    // psr = PL + rL aL (ss - uL)
-    T b_PL = b_psr, b_rL = b_psr * aLv * (ss - uL);
-    T b_aL = b_psr * (T)rL * (ss - uL);
-    b_ss += b_psr * (T)rL * aLv;
-    T b_uL = -b_psr * (T)rL * aLv;
-    T b_PR = T(0), b_rR = T(0), b_uR = T(0), b_aR = T(0);
-    // ss = num / den
-    const T b_num = b_ss * pdiv(T(1), den);
-    const T b_den = -b_num * ss;
-    b_PR += b_num;
-    b_PL -= b_num;
-    b_rL += b_num * (T)uL * aLv;
-    b_uL += b_num * (T)rL * aLv;
-    b_aL += b_num * (T)rL * uL;
-    b_rR -= b_num * (T)uR * aRv;
-    b_uR -= b_num * (T)rR * aRv;
-    b_aR -= b_num * (T)rR * uR;
-    b_rL += b_den * aLv;
-    b_aL += b_den * rL;
-    b_rR -= b_den * aRv;
-    b_aR -= b_den * rR;
-    // aL = SL - uL, aR = SR - uR
-    const T b_SL = b_aL, b_SR = b_aR;
-    b_uL -= b_aL;
-    b_uR -= b_aR;
-    T b_cL = T(0), b_cR = T(0);
-    if (e1 <= e2) {
-        b_uL += b_SL;
-        b_cL -= b_SL;
+    const T ira = rcp_(Ga[0]), irb = rcp_(Gb[0]);
+    const T qa = gam * Ga[4] * ira, qb = gam * Gb[4] * irb;
+    const T ica = rsq_(max_(qa, Tiny<T>::sq)), icb = rsq_(max_(qb, Tiny<T>::sq));
+    const T cca = mul_rn(qa, ica), ccb = mul_rn(qb, icb);
+    const T dv[3] = {Gb[1] - Ga[1], Gb[2] - Ga[2], Gb[3] - Ga[3]};
+    const T sv[3] = {Ga[1] + Gb[1], Ga[2] + Gb[2], Ga[3] + Gb[3]};
+    const T du = dot3(dv[0], dv[1], dv[2], n[0], n[1], n[2]);
+    const T us = dot3(sv[0], sv[1], sv[2], n[0], n[1], n[2]);
+    const T e1 = du - ccb, e2 = cca - du;
+    const T al = min_(-cca, e1), be = max_(ccb, e2);
+    const T ma = mul_rn(Ga[0], al), mb = mul_rn(Gb[0], be);
+    const T iden = rcp_(ma - mb), msum = ma + mb;
+    const T psr = fma(-(ma * mb), du, add_rn(mul_rn(ma, Gb[4]), -mul_rn(mb, Ga[4]))) * iden;
+    const T X = fma(-msum, du, T(2) * (Gb[4] - Ga[4])) * iden;
+    const T S = T(0.5) * (us + X);
+    const bool neg = psr < T(0);
+    const T ps = neg ? T(0) : psr;
+    const T Am = T(2) * (Aq * iA);
+    // ---- reverse: J = -ps (wp . A + wE S |A|)
+    const T wA = T(2) * dot3(wp[0], wp[1], wp[2], A[0], A[1], A[2]);
+    const T wS = wE * S;
+    const T b_psr = neg ? T(0) : -fma(wS, Am, wA);
+    const T b_h = T(-0.5) * (ps * wE) * Am;  // of us and of X
+    // X = num2 iden, psr = num1 iden, iden = 1 / (ma - mb)
+    const T b_2 = b_h * iden, b_1 = b_psr * iden;
+    const T b_den = -fma(b_2, X, b_1 * psr);
+    T b_Pa = -fma(b_1, mb, T(2) * b_2), b_Pb = fma(b_1, ma, T(2) * b_2);
+    const T b_ma = fma(b_1, fma(-mb, du, Gb[4]), fma(-du, b_2, b_den));
+    const T b_mb = -fma(b_1, fma(ma, du, Ga[4]), fma(du, b_2, b_den));
+    T b_du = -fma(msum, b_2, b_1 * (ma * mb));
+    // ma = rho_a min(-c_a, du - c_b), mb = rho_b max(c_b, c_a - du); a tie goes to
+    // the particle that is L (the derivative oracle's rule)
+    T b_ra = b_ma * al, b_rb = b_mb * be;
+    const T b_al = b_ma * Ga[0], b_be = b_mb * Gb[0];
+    T b_ca = T(0), b_cb = T(0);
+    const bool own_a = aL ? !less_(e1, -cca) : less_(-cca, e1);
+    const bool own_b = aL ? less_(e2, ccb) : !less_(ccb, e2);
+    if (own_a) {
+        b_ca -= b_al;
     } else {
-        b_uR += b_SL;
-        b_cR -= b_SL;
+        b_du += b_al;
+        b_cb -= b_al;
     }
-    if (e3 >= e4) {
-        b_uL += b_SR;
-        b_cL += b_SR;
+    if (own_b) {
+        b_cb += b_be;
     } else {
-        b_uR += b_SR;
-        b_cR += b_SR;
+        b_ca += b_be;
+        b_du -= b_be;
     }
     // c = sqrt(gamma P / rho)
-    if (cL > T(0)) {
-        const T h = pdiv(T(0.5), rL);
-        b_PL += b_cL * gam * pdiv(h, cL);
-        b_rL -= b_cL * cL * h;
-    }
-    if (cR > T(0)) {
-        const T h = pdiv(T(0.5), rR);
-        b_PR += b_cR * gam * pdiv(h, cR);
-        b_rR -= b_cR * cR * h;
-    }
-    T bFL[5] = {b_rL, T(0), T(0), T(0), b_PL};
-    T bFR[5] = {b_rR, T(0), T(0), T(0), b_PR};
-    T bvf[3], bn[3];
+    const T ha = T(0.5) * ira * b_ca, hb = T(0.5) * irb * b_cb;
+    b_Pa = fma(ha * gam, ica, b_Pa);
+    b_ra = fma(-ha, cca, b_ra);
+    b_Pb = fma(hb * gam, icb, b_Pb);
+    b_rb = fma(-hb, ccb, b_rb);
+    const T ea = b_h - b_du, eb = b_h + b_du;
+    const T bGa[5] = {b_ra, ea * n[0], ea * n[1], ea * n[2], b_Pa};
+    const T bGb[5] = {b_rb, eb * n[0], eb * n[1], eb * n[2], b_Pb};
+    // A: n = A/|A| and |A| (A here half the area: the factors of 2 cancel in n)
+    const T nn = fma(b_h, us, b_du * du);
+    const T b_Am = -(ps * wS);
+    const T kA = T(-2) * ps, kN = T(2) * b_Am - nn * iA;
+    T bA[3];  // (of the half area vector)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        bFL[1 + k] = b_uL * n[k];
-        bFR[1 + k] = b_uR * n[k];
-        bvf[k] = -(b_uL + b_uR) * n[k] + b_vfn * n[k];
-        bn[k] = b_uL * ((T)FL[1 + k] - vf[k]) + b_uR * ((T)FR[1 + k] - vf[k]) + b_vfn * vf[k];
-    }
-    // vf = vL + sL (vR - vL)
-    T bvL[3], bvR[3], b_sL = T(0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        bvL[k] = bvf[k] * (T(1) - (T)sL);
-        bvR[k] = bvf[k] * (T)sL;
-        b_sL += bvf[k] * ((T)vR[k] - vL[k]);
-    }
-    // back to a / b labels
-    T bGa[5], bGb[5];
-#pragma unroll
-    for (int f = 0; f < 5; ++f) {
-        bGa[f] = aL ? bFL[f] : bFR[f];
-        bGb[f] = aL ? bFR[f] : bFL[f];
-    }
-    T bWa[5] = {0, 0, 0, 0, 0};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) bWa[1 + k] += aL ? bvL[k] : bvR[k];
-    T b_sa = aL ? b_sL : T(0), b_sb = aL ? T(0) : b_sL;
-    // normal n = sg A / |A|, and |A| itself
-    T bnh[3] = {sg * bn[0], sg * bn[1], sg * bn[2]};
-    const T nb_dot = (bnh[0] * nh[0] + bnh[1] * nh[1]) + bnh[2] * nh[2];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) bA[k] += (bnh[k] - nb_dot * nh[k]) * iA + b_Am * nh[k];
+    for (int k = 0; k < 3; ++k)
+        bA[k] = fma(kA, wp[k], fma(kN, n[k], iA * fma(b_h, sv[k], b_du * dv[k])));
     // fallback and clamps; a bound min / max(W_L, W_R) passes its adjoint to
     // L on a tie (the rule the derivative oracle's where() takes), so the two
     // sides of a pair never both claim it
@@ -227,113 +176,57 @@ __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)
         bFa[f] = T(0);
         bFb[f] = T(0);
         if (fallback) {
-            bWa[f] += bGa[f];
+            s.W[f] += bGa[f];
         } else {
-            const bool loA = aL ? (Wa[f] <= Wb[f]) : (Wa[f] < Wb[f]);
-            const bool hiA = aL ? (Wa[f] >= Wb[f]) : (Wa[f] > Wb[f]);
-            // a's face value
-            if (ka[f] == 0)
-                bFa[f] = bGa[f];
-            else
-                bWa[f] += ((ka[f] < 0) ? loA : hiA) ? bGa[f] : T(0);
-            // b's face value (its bounds can be a's values)
-            if (kb[f] == 0)
-                bFb[f] = bGb[f];
-            else
-                bWa[f] += ((kb[f] < 0) ? loA : hiA) ? bGb[f] : T(0);
+            if (ka[f] == 0) bFa[f] = bGa[f];
+            if (kb[f] == 0) bFb[f] = bGb[f];
+            if (ka[f] != 0 || kb[f] != 0) {
+                const bool lt = less_(Wa0[f], Wb0[f]), gt = less_(Wb0[f], Wa0[f]);
+                const bool loA = lt || (aL && !gt), hiA = gt || (aL && !lt);
+                if (ka[f] != 0 && (ka[f] < 0 ? loA : hiA)) s.W[f] += bGa[f];
+                if (kb[f] != 0 && (kb[f] < 0 ? loA : hiA)) s.W[f] += bGb[f];
+            }
         }
     }
-    // face states: F_a = W_a + g_a . (s_a d) + inc_a ; F_b = W_b + g_b . (s_b (-d)) + inc_b
-    T bd[3] = {T(0), T(0), T(0)};
-    T bg[15];
-#pragma unroll
-    for (int q = 0; q < 15; ++q) bg[q] = T(0);
+    // face states: F_a = Wh_a + s_a g_a . d ; F_b = Wh_b - s_b g_b . d
+    T bd[3] = {T(0), T(0), T(0)}, b_sa = T(0), b_sb = T(0);
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
-        bWa[f] += bFa[f];
-        const T g0 = a[11 + 3 * f], g1 = a[12 + 3 * f], g2 = a[13 + 3 * f];
-        bg[3 * f] += bFa[f] * sa * dx;
-        bg[3 * f + 1] += bFa[f] * sa * dy;
-        bg[3 * f + 2] += bFa[f] * sa * dz;
-        b_sa += bFa[f] * ((g0 * dx + g1 * dy) + g2 * dz);
-        bd[0] += bFa[f] * sa * g0;
-        bd[1] += bFa[f] * sa * g1;
-        bd[2] += bFa[f] * sa * g2;
-        const T h0 = b[11 + 3 * f], h1 = b[12 + 3 * f], h2 = b[13 + 3 * f];
-        b_sb -= bFb[f] * ((h0 * dx + h1 * dy) + h2 * dz);
-        bd[0] -= bFb[f] * sb * h0;
-        bd[1] -= bFb[f] * sb * h1;
-        bd[2] -= bFb[f] * sb * h2;
-    }
-    if (hancock) {  // inc_a = (dt/2)(-rho div v, -grad P / rho, -gamma P div v)
-        const T div = (a[11 + 3] + a[11 + 7]) + a[11 + 11];
-        const T rho = a[6], P = a[7];
-        const T b_div = bFa[0] * hdt * (-rho) + bFa[4] * hdt * (-gam * P);
-        bWa[0] += bFa[0] * hdt * (-div);
+        s.F[f] += bFa[f];
+        const T ta = bFa[f] * sa, tb = bFb[f] * sb;
+        s.g[3 * f] = fma(ta, dx, s.g[3 * f]);
+        s.g[3 * f + 1] = fma(ta, dy, s.g[3 * f + 1]);
+        s.g[3 * f + 2] = fma(ta, dz, s.g[3 * f + 2]);
+        b_sa = fma(bFa[f], Da[f], b_sa);
+        b_sb = fma(bFb[f], Db[f], b_sb);  // (its negative)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            bWa[0] += bFa[1 + k] * hdt * a[11 + 12 + k] * irho * irho;
-            bg[12 + k] -= bFa[1 + k] * hdt * irho;
-        }
-        bWa[4] += bFa[4] * hdt * (-gam * div);
-        bg[3] += b_div;
-        bg[7] += b_div;
-        bg[11] += b_div;
+        for (int k = 0; k < 3; ++k) bd[k] = fma(ta, a[11 + 3 * f + k], fma(-tb, b[11 + 3 * f + k], bd[k]));
     }
     // s_a = Ha / Hs, s_b = Hb / Hs
-    const T Hsd = Hs;
-    T bHa = (b_sa - b_sb) * b[3] * pdiv(T(1), Hsd * Hsd);
+    s.h = fma(b_sa + b_sb, b[3] * (iHs * iHs), s.h);
     // A = ca B_a d + cb B_b d
-    const T bca = (bA[0] * Bda[0] + bA[1] * Bda[1]) + bA[2] * Bda[2];
-    const T bcb = (bA[0] * Bdb[0] + bA[1] * Bdb[1]) + bA[2] * Bdb[2];
-    const T bBda[3] = {(T)ca * bA[0], (T)ca * bA[1], (T)ca * bA[2]};
-    const T bBdb[3] = {(T)cb * bA[0], (T)cb * bA[1], (T)cb * bA[2]};
-    T bB[6];
-    bB[0] = bBda[0] * dx;
-    bB[1] = bBda[0] * dy + bBda[1] * dx;
-    bB[2] = bBda[0] * dz + bBda[2] * dx;
-    bB[3] = bBda[1] * dy;
-    bB[4] = bBda[1] * dz + bBda[2] * dy;
-    bB[5] = bBda[2] * dz;
-    bd[0] += (Ba[0] * bBda[0] + Ba[1] * bBda[1]) + Ba[2] * bBda[2];
-    bd[1] += (Ba[1] * bBda[0] + Ba[3] * bBda[1]) + Ba[4] * bBda[2];
-    bd[2] += (Ba[2] * bBda[0] + Ba[4] * bBda[1]) + Ba[5] * bBda[2];
-    bd[0] += (Bb[0] * bBdb[0] + Bb[1] * bBdb[1]) + Bb[2] * bBdb[2];
-    bd[1] += (Bb[1] * bBdb[0] + Bb[3] * bBdb[1]) + Bb[4] * bBdb[2];
-    bd[2] += (Bb[2] * bBdb[0] + Bb[4] * bBdb[1]) + Bb[5] * bBdb[2];
-    // ca = knorm_a w(r / Ha) inside a's support, cb likewise
-    T br = T(0), bka = T(0);
-    if (ina) {
-        bka = bca * wa;
-        const T bq = bca * (T)a[5] * dkern(qa);
-        br += bq * (T)a[4];
-        bHa -= bq * qa * a[4];
-    }
-    if (inb) br += bcb * (T)b[5] * dkern(qb) * (T)b[4];
-    // knorm = 8 / (pi H^3 n^2)
-    bHa += bka * (T(-3) * a[5] * a[4]);
-    const T bna = bka * (-T(2) * a[5] * inv_na);
-    if (r > T(0)) {
-        const T bri = br * pdiv(T(1), r);
-        bd[0] += bri * dx;
-        bd[1] += bri * dy;
-        bd[2] += bri * dz;
-    }
+    const T b_cka = dot3(bA[0], bA[1], bA[2], ua[0], ua[1], ua[2]);
+    const T b_ckb = dot3(bA[0], bA[1], bA[2], ub[0], ub[1], ub[2]);
+    const T va[3] = {ca * bA[0], ca * bA[1], ca * bA[2]};
+    const T vb[3] = {cb * bA[0], cb * bA[1], cb * bA[2]};
+    s.B[0] = fma(va[0], dx, s.B[0]);
+    s.B[1] = fma(va[0], dy, fma(va[1], dx, s.B[1]));
+    s.B[2] = fma(va[0], dz, fma(va[2], dx, s.B[2]));
+    s.B[3] = fma(va[1], dy, s.B[3]);
+    s.B[4] = fma(va[1], dz, fma(va[2], dy, s.B[4]));
+    s.B[5] = fma(va[2], dz, s.B[5]);
+    bd[0] += dot3(Ba[0], Ba[1], Ba[2], va[0], va[1], va[2]) + dot3(Bb[0], Bb[1], Bb[2], vb[0], vb[1], vb[2]);
+    bd[1] += dot3(Ba[1], Ba[3], Ba[4], va[0], va[1], va[2]) + dot3(Bb[1], Bb[3], Bb[4], vb[0], vb[1], vb[2]);
+    bd[2] += dot3(Ba[2], Ba[4], Ba[5], va[0], va[1], va[2]) + dot3(Bb[2], Bb[4], Bb[5], vb[0], vb[1], vb[2]);
+    // ca = knorm_a w(r / Ha), cb likewise
+    s.k = fma(b_cka, wa, s.k);
+    const T b_qa = b_cka * a[5] * da;
+    s.q = fma(b_qa, r, s.q);  // (times 1/H_a after the last pair)
+    const T br = fma(b_qa, a[4], (b_ckb * b[5] * db) * b[4]) * ir;
     // d = x_b - x_a
-    adj[AX] -= bd[0];
-    adj[AX + 1] -= bd[1];
-    adj[AX + 2] -= bd[2];
-    adj[AH] += bHa;
-    adj[AN] += bna;
-    adj[ARHO] += bWa[0];
-    adj[AV] += bWa[1];
-    adj[AV + 1] += bWa[2];
-    adj[AV + 2] += bWa[3];
-    adj[AP] += bWa[4];
-#pragma unroll
-    for (int q = 0; q < 15; ++q) adj[AG + q] += bg[q];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) adj[AB + q] += bB[q];
+    s.x[0] += fma(br, dx, bd[0]);
+    s.x[1] += fma(br, dy, bd[1]);
+    s.x[2] += fma(br, dz, bd[2]);
 }
 
 // Adjoint of the flux pass: per particle over its pairs (N_i then R_i).
@@ -348,18 +241,23 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 1)
     T a[kRecord];
     load_rec(rec, i, a);
     const long long idi = sid[i];
-    const T hdt = (T)(0.5 * dt_use[sbox[i]]);
+    const T hdt = p.hancock ? (T)(0.5 * dt_use[sbox[i]]) : T(0);
     const T gam = (T)p.gamma;
-    const bool hancock = p.hancock != 0;
-    const T inv_na = pdiv(T(1), sn[i]), irho = pdiv(T(1), a[6]);
+    T Wh[5];
+    half_state(a, hdt, gam, Wh);
     T wi[4];
     load4(wgt + 4 * (size_t)i, wi);
-    T acc[kAdj];
-#pragma unroll
-    for (int q = 0; q < kAdj; ++q) acc[q] = T(0);
+    AdjSums<T> s;
+    for (int q = 0; q < 3; ++q) s.x[q] = T(0);
+    for (int q = 0; q < 5; ++q) s.F[q] = s.W[q] = T(0);
+    for (int q = 0; q < 15; ++q) s.g[q] = T(0);
+    for (int q = 0; q < 6; ++q) s.B[q] = T(0);
+    s.k = s.q = s.h = T(0);
+#pragma unroll 1
     for (int list = 0; list < 2; ++list) {
         const unsigned* L = list == 0 ? nbr + 4 * (size_t)i : rnbr + 4 * (size_t)i;
         const int cnt = list == 0 ? min(ncount[i], p.cap) : min(rcount[i], p.rcap);
+#pragma unroll 1
         for (int k = 0; k < cnt; ++k) {
             const int j = (int)L[lcol(k, N)];
             T b[kRecord];
@@ -367,13 +265,46 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 1)
             T wj[4];
             load4(wgt + 4 * (size_t)j, wj);
             const T wp[3] = {wi[0] - wj[0], wi[1] - wj[1], wi[2] - wj[2]};
-            const T wE = wi[3] - wj[3];
-            pair_adjoint(a, b, idi < sid[j], hdt, gam, hancock, inv_na, irho, wp, wE, acc);
+            pair_adjoint(a, b, Wh, idi < sid[j], hdt, gam, wp, wi[3] - wj[3], s);
         }
     }
+    // the half-step primitives: Wh = W + (dt/2)(-rho div v, -grad P/rho, -gamma P div v)
+    const T div = (a[11 + 3] + a[11 + 7]) + a[11 + 11];
+    const T irho = pdiv(T(1), a[6]);
+    const T e = -hdt * div, k = -hdt * irho;
+    T bW[5], bg[15];
+#pragma unroll
+    for (int f = 0; f < 5; ++f) bW[f] = s.F[f] + s.W[f];
+    bW[0] += e * s.F[0];
+    bW[4] += gam * e * s.F[4];
+#pragma unroll
+    for (int q = 0; q < 15; ++q) bg[q] = s.g[q];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        bW[0] -= k * irho * a[11 + 12 + q] * s.F[1 + q];
+        bg[12 + q] += k * s.F[1 + q];
+    }
+    const T b_div = -hdt * (a[6] * s.F[0] + gam * a[7] * s.F[4]);
+    bg[3] += b_div;
+    bg[7] += b_div;
+    bg[11] += b_div;
+    // knorm = 8 / (pi H^3 n^2); q = r / H
+    const T bH = s.h - T(3) * s.k * a[5] * a[4] - s.q * a[4] * a[4];
+    const T bn = T(-2) * s.k * a[5] * pdiv(T(1), sn[i]);
     T* o = adj + (size_t)i * kAdj;
 #pragma unroll
-    for (int q = 0; q < kAdj; ++q) o[q] += acc[q];
+    for (int q = 0; q < 3; ++q) {
+        o[AX + q] -= s.x[q];
+        o[AV + q] += bW[1 + q];
+    }
+    o[AH] += bH;
+    o[AN] += bn;
+    o[ARHO] += bW[0];
+    o[AP] += bW[4];
+#pragma unroll
+    for (int q = 0; q < 15; ++q) o[AG + q] += bg[q];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) o[AB + q] += s.B[q];
 }
 
 // Caller-order adjoint weights of the rates -> sorted [N][4].
@@ -455,6 +386,34 @@ __global__ void k_update_adj(int N, Sorted<T> s, const double* __restrict__ dpdt
 }
 
 // ---------------------------------------------------------- gradients
+// One pair (i, j) of particle i's sums E = sum psi d d^T and
+// S_f = sum psi (f_j - f_i) d, reversed: with psi = 2 norm w (w half the
+// kernel, dw half its derivative, ir = 1/r, iH = 1/H_i), Sb and Eb the sums'
+// adjoints and df the field differences, t[f] = Sb_f . d, and
+//   psib = d^T Eb d + sum_f df_f t_f,   db = psi (2 Eb d + sum_f df_f Sb_f) + psib psi'(r) d / r.
+template <typename T>
+__device__ __forceinline__ void pair_grad_adj(const T* Sb, const T* Eb, T norm2, T w, T dw, T ir, T iH, T dx, T dy,
+                                              T dz, const T (&df)[5], T& psi, T (&t)[5], T& psib, T (&db)[3]) {
+    psi = norm2 * w;
+    const T E0 = T(2) * Eb[0], E3 = T(2) * Eb[3], E5 = T(2) * Eb[5];
+    T v0 = dot3(E0, Eb[1], Eb[2], dx, dy, dz);
+    T v1 = dot3(Eb[1], E3, Eb[4], dx, dy, dz);
+    T v2 = dot3(Eb[2], Eb[4], E5, dx, dy, dz);
+    psib = T(0.5) * dot3(v0, v1, v2, dx, dy, dz);
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+        t[f] = dot3(Sb[3 * f], Sb[3 * f + 1], Sb[3 * f + 2], dx, dy, dz);
+        psib = fma(df[f], t[f], psib);
+        v0 = fma(df[f], Sb[3 * f], v0);
+        v1 = fma(df[f], Sb[3 * f + 1], v1);
+        v2 = fma(df[f], Sb[3 * f + 2], v2);
+    }
+    const T rb = psib * norm2 * dw * iH * ir;
+    db[0] = fma(psi, v0, rb * dx);
+    db[1] = fma(psi, v1, rb * dy);
+    db[2] = fma(psi, v2, rb * dz);
+}
+
 // Seeds of particle i's gradient pass: from the adjoints of its limited
 // gradients and of B, through the limiter (active constraint only), g = B S
 // and B = E^-1.  Adds i's own terms; stores what i's neighbours gather.
@@ -573,7 +532,8 @@ __global__ void __launch_bounds__(128)
         for (int q = 0; q < 28; q += 4) store4(sd + q, r0[q], r0[q + 1], r0[q + 2], r0[q + 3]);
     }
     lbloom[i] = bloom;
-    T normb = T(0.0);
+    T normb = T(0.0), Hq = T(0);  // sums of psib w and of psib w' r (w half the kernel)
+    const T norm2 = T(2) * norm;
     const int cnt = min(ncount[i], p.cap);
     const unsigned* L = nbr + 4 * (size_t)i;
     for (int k0 = 0; k0 < cnt; k0 += 4) {  // four neighbours' loads in flight at a time
@@ -582,53 +542,39 @@ __global__ void __launch_bounds__(128)
       P4<T> qv[4], pv[4];
       T Pv[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < 4; ++u) {
+          qv[u] = me;
           if (k0 + u < cnt) {
               qv[u] = s.pos[js[u]];
               pv[u] = s.prim[js[u]];
               Pv[u] = s.prim2[js[u]].x;
           }
+      }
+      T dx4[4], dy4[4], dz4[4];
+      offsets4(qv, xi, yi, zi, xim1, yim1, zim1, dx4, dy4, dz4);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         if (k0 + u >= cnt) break;
-        const P4<T> qj = qv[u];
-        const T dxT = mi_diff(qj.x, xi, xim1), dyT = mi_diff(qj.y, yi, yim1), dzT = mi_diff(qj.z, zi, zim1);
-        const T r2 = sep2(dxT, dyT, dzT);
-        const T r = psqrt(r2);
-        const T q = r * iH;
-        const T w = kern_w(q), dw = kern_dw(q);
-        const T psi = (T)(norm * kern_w(q));
-        const T dx = dxT, dy = dyT, dz = dzT;
+        const T dx = dx4[u], dy = dy4[u], dz = dz4[u];
+        const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
+        const T ir = rsq_(r2), r = mul_rn(r2, ir);
+        T w, dw;
+        kern_half_d(r, iH, w, dw);
         const P4<T> pj = pv[u];
-        const T Wj[5] = {pj.x, pj.y, pj.z, pj.w, Pv[u]};
-        T psib = ((Eb[0] * dx * dx + Eb[1] * dx * dy) + (Eb[2] * dx * dz + Eb[3] * dy * dy)) +
-                      (Eb[4] * dy * dz + Eb[5] * dz * dz);
-        T db[3] = {psi * (T(2.0) * Eb[0] * dx + Eb[1] * dy + Eb[2] * dz),
-                        psi * (Eb[1] * dx + T(2.0) * Eb[3] * dy + Eb[4] * dz),
-                        psi * (Eb[2] * dx + Eb[4] * dy + T(2.0) * Eb[5] * dz)};
-        for (int f = 0; f < 5; ++f) {
-            const T df = Wj[f] - (T)Wi[f];
-            const T t = (Sb[3 * f] * dx + Sb[3 * f + 1] * dy) + Sb[3 * f + 2] * dz;
-            fbi[f] -= psi * t;
-            psib += df * t;
-            db[0] += df * psi * Sb[3 * f];
-            db[1] += df * psi * Sb[3 * f + 1];
-            db[2] += df * psi * Sb[3 * f + 2];
-        }
-        normb += psib * w;
-        const T qb = psib * (T)norm * dw;
-        Hbi -= qb * q * iH;
-        if (r > T(0)) {
-            const T rb = qb * iH * pdiv(T(1), r);
-            db[0] += rb * dx;
-            db[1] += rb * dy;
-            db[2] += rb * dz;
-        }
+        const T df[5] = {pj.x - Wi[0], pj.y - Wi[1], pj.z - Wi[2], pj.w - Wi[3], Pv[u] - Wi[4]};
+        T psi, t[5], psib, db[3];
+        pair_grad_adj(Sb, Eb, norm2, w, dw, ir, iH, dx, dy, dz, df, psi, t, psib, db);
+#pragma unroll
+        for (int f = 0; f < 5; ++f) fbi[f] = fma(-psi, t[f], fbi[f]);
+        normb = fma(psib, w, normb);
+        Hq = fma(psib * dw, r, Hq);
         xbi[0] -= db[0];
         xbi[1] -= db[1];
         xbi[2] -= db[2];
       }
     }
+    normb *= T(2);
+    Hbi -= Hq * norm2 * iH * iH;
     Hbi += normb * (-T(3.0) * (T)norm / (T)Hi);
     nbi += normb * (-(T)norm / (T)ni);
     a[AX] += xbi[0];
@@ -681,38 +627,19 @@ __global__ void __launch_bounds__(128)
             const T dx = mi_diff(mj.x, mi.x, mi.x - T(1)), dy = mi_diff(mj.y, mi.y, mi.y - T(1)),
                     dz = mi_diff(mj.z, mi.z, mi.z - T(1));
             const T r2 = sep2(dx, dy, dz);
-            if (!(r2 < Hi * Hi)) continue;  // j is not in N_i
+            if (!less_(r2, Hi * Hi)) continue;  // j is not in N_i
             const T* R = seeds + (size_t)i * kSeed;
             T sd[32];  // record 0-27 (and 4 limiter values, unused here)
             load_row32<32>(R, sd);
-            const T r = psqrt(r2);
-            const T iH = T(1) / Hi;
-            const T q = r * iH;
-            const T norm = sd[21];
-            const T psi = (T)(norm * kern_w(q));
-            const T dw = kern_dw(q);
-            const T* Eb = sd + 15;
-            T psib = ((Eb[0] * dx * dx + Eb[1] * dx * dy) + (Eb[2] * dx * dz + Eb[3] * dy * dy)) +
-                     (Eb[4] * dy * dz + Eb[5] * dz * dz);
-            T db[3] = {psi * (T(2.0) * Eb[0] * dx + Eb[1] * dy + Eb[2] * dz),
-                       psi * (Eb[1] * dx + T(2.0) * Eb[3] * dy + Eb[4] * dz),
-                       psi * (Eb[2] * dx + Eb[4] * dy + T(2.0) * Eb[5] * dz)};
+            const T r2m = max_(r2, Tiny<T>::sq);
+            const T ir = rsq_(r2m), iH = rcp_(Hi);
+            T w, dw;
+            kern_half_d(mul_rn(r2m, ir), iH, w, dw);
+            const T df[5] = {Wj[0] - sd[22], Wj[1] - sd[23], Wj[2] - sd[24], Wj[3] - sd[25], Wj[4] - sd[26]};
+            T psi, t[5], psib, db[3];
+            pair_grad_adj(sd, sd + 15, T(2) * sd[21], w, dw, ir, iH, dx, dy, dz, df, psi, t, psib, db);
 #pragma unroll
-            for (int f = 0; f < 5; ++f) {
-                const T df = Wj[f] - sd[22 + f];
-                const T t = (sd[3 * f] * dx + sd[3 * f + 1] * dy) + sd[3 * f + 2] * dz;
-                fb[f] += psi * t;
-                psib += df * t;
-                db[0] += df * psi * sd[3 * f];
-                db[1] += df * psi * sd[3 * f + 1];
-                db[2] += df * psi * sd[3 * f + 2];
-            }
-            if (r > T(0)) {
-                const T rb = psib * norm * dw * iH * pdiv(T(1), r);
-                db[0] += rb * dx;
-                db[1] += rb * dy;
-                db[2] += rb * dz;
-            }
+            for (int f = 0; f < 5; ++f) fb[f] = fma(psi, t[f], fb[f]);
             xb[0] += db[0];
             xb[1] += db[1];
             xb[2] += db[2];
@@ -779,6 +706,7 @@ __global__ void __launch_bounds__(128)
     const T lam = fH != T(0.0) ? -Hbt / fH : T(0.0);
     const T kappa = (nb * c8 + lam * T(32.0) / T(3.0)) / H;
     kap[i] = kappa;
+    const T kappa2 = T(2) * kappa;  // (kern_half_d: half the kernel's derivative)
     T xb[3] = {0, 0, 0};
     for (int k0 = 0; k0 < cnt; k0 += 4) {  // four neighbours' loads in flight at a time
         const uint4 jj = col4(L, k0, N);
@@ -792,9 +720,10 @@ __global__ void __launch_bounds__(128)
             if (k0 + u >= cnt) break;
             const P4<T> qj = qv[u];
             const T dx = mi_diff(qj.x, xi, xim1), dy = mi_diff(qj.y, yi, yim1), dz = mi_diff(qj.z, zi, zim1);
-            const T r = psqrt(sep2(dx, dy, dz));
-            if (!(r > T(0))) continue;
-            const T c = kappa * (T)kern_dw(r * iH) * pdiv(T(1), r);
+            const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq), ir = rsq_(r2);
+            T w, dw;
+            kern_half_d(mul_rn(r2, ir), iH, w, dw);
+            const T c = kappa2 * dw * ir;
             xb[0] -= c * dx;
             xb[1] -= c * dy;
             xb[2] -= c * dz;
@@ -831,11 +760,13 @@ __global__ void __launch_bounds__(128)
                 const P4<T> mi = mv[u];
                 const T dx = mi_diff(mj.x, mi.x, mi.x - T(1)), dy = mi_diff(mj.y, mi.y, mi.y - T(1)),
                         dz = mi_diff(mj.z, mi.z, mi.z - T(1));
-                const T r2 = sep2(dx, dy, dz);
-                if (!(r2 < mi.w * mi.w)) continue;
-                const T r = psqrt(r2);
-                if (!(r > T(0))) continue;
-                const T c = kap[i] * kern_dw(r * pdiv(T(1), mi.w)) * pdiv(T(1), r);
+                T r2 = sep2(dx, dy, dz);
+                if (!less_(r2, mi.w * mi.w)) continue;
+                r2 = max_(r2, Tiny<T>::sq);
+                const T ir = rsq_(r2);
+                T w, dw;
+                kern_half_d(mul_rn(r2, ir), rcp_(mi.w), w, dw);
+                const T c = T(2) * kap[i] * dw * ir;
                 xb[0] += c * dx;
                 xb[1] += c * dy;
                 xb[2] += c * dz;

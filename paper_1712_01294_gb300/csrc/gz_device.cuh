@@ -110,6 +110,27 @@ __device__ __forceinline__ double kern_half(double r, double iH) {
     return h >= 0x3FF00000 ? 0.0 : w;
 }
 
+// W(q)/2 and W'(q)/2 at q = r/H.
+__device__ __forceinline__ void kern_half_d(float r, float iH, float& w, float& d) {
+    const float t = __saturatef(fmaf(-r, iH, 1.f)), v = __saturatef(fmaf(-r, iH, 0.5f));
+    const float t2 = t * t, v2 = v * v;
+    w = fmaf(-4.f * v2, v, t2 * t);
+    d = fmaf(12.f, v2, -3.f * t2);
+}
+__device__ __forceinline__ void kern_half_d(double r, double iH, double& w, double& d) {
+    const double q = __dmul_rn(r, iH);
+    const int h = __double2hiint(q);
+    const bool in = h < 0x3FE00000, out = h >= 0x3FF00000;
+    const double x = in ? q : 1.0 - q;
+    const double ww = fma(fma(in ? 3.0 : 1.0, x, in ? -3.0 : 0.0), x * x, in ? 0.5 : 0.0);
+    const double dd = x * fma(in ? 9.0 : -3.0, x, in ? -6.0 : 0.0);
+    w = out ? 0.0 : ww;
+    d = out ? 0.0 : dd;
+}
+// a < b, FP64 compared as integers.
+__device__ __forceinline__ bool less_(float a, float b) { return a < b; }
+__device__ __forceinline__ bool less_(double a, double b) { return order_(a) < order_(b); }
+
 // x . y, fused the same way wherever it is formed.
 template <typename T>
 __device__ __forceinline__ T dot3(T x0, T x1, T x2, T y0, T y1, T y2) {
@@ -195,40 +216,6 @@ __device__ __forceinline__ void load_rec(const double* __restrict__ rec, int i, 
         asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
             : "=d"(v[4 * k]), "=d"(v[4 * k + 1]), "=d"(v[4 * k + 2]), "=d"(v[4 * k + 3])
             : "l"(rec + rec_at<double>(i, 4 * k)));
-}
-
-// Face state of particle a toward the face at a + s o (o = offset to the
-// partner): linear reconstruction with a's limited gradients plus the Hancock
-// half step (dt/2) (-rho div v, -grad P / rho, -gamma P div v).
-// Hancock half-step increments of a particle's primitives (O11):
-// (dt/2)(-rho div v, -grad P / rho, -gamma P div v), each product rounded
-// once so that every pass that forms them gets the same bits.
-template <typename T>
-__device__ __forceinline__ void hancock_inc(const T (&a)[kRecord], T hdt, T gam, bool hancock, T (&inc)[5]) {
-    if (!hancock) {
-#pragma unroll
-        for (int f = 0; f < 5; ++f) inc[f] = T(0);
-        return;
-    }
-    const T div = (a[11 + 3] + a[11 + 7]) + a[11 + 11];
-    const T ir = pdiv(T(1), a[6]);
-    inc[0] = mul_rn(hdt, -a[6] * div);
-    inc[1] = mul_rn(hdt, -a[11 + 12] * ir);
-    inc[2] = mul_rn(hdt, -a[11 + 13] * ir);
-    inc[3] = mul_rn(hdt, -a[11 + 14] * ir);
-    inc[4] = mul_rn(hdt, -gam * a[7] * div);
-}
-
-// Face state of a record at offset s (dx, dy, dz) from the particle:
-// W + g . (s d) + the Hancock increments.
-template <typename T>
-__device__ __forceinline__ void face_state(const T (&a)[kRecord], T s, T dx, T dy, T dz, const T (&inc)[5],
-                                           T (&F)[5]) {
-    const T ox = s * dx, oy = s * dy, oz = s * dz;
-    const T W[5] = {a[6], a[8], a[9], a[10], a[7]};
-#pragma unroll
-    for (int f = 0; f < 5; ++f)
-        F[f] = add_rn(W[f] + ((a[11 + 3 * f] * ox + a[12 + 3 * f] * oy) + a[13 + 3 * f] * oz), inc[f]);
 }
 
 // n values (a multiple of 32 bytes) from 32-byte-aligned global memory with
