@@ -658,7 +658,8 @@ gz_status create_ctx(const gz_params* params, int32_t nboxes, const int64_t* cou
         {(void**)&c.ssd, sz * Nz},
         {(void**)&c.srho, sz * Nz},       {(void**)&c.sP, sz * Nz},
         {(void**)&c.sc, sz * Nz},         {(void**)&c.sid, 8 * Nz},
-        {(void**)&c.spos, 4 * sz * Nz},   {(void**)&c.sprim, 4 * sz * Nz},
+        {(void**)&c.spos, 4 * sz * (Nz + 4)},  // (scans read whole groups of four)
+        {(void**)&c.sprim, 4 * sz * Nz},
         {(void**)&c.sprim2, 2 * sz * Nz},
         {(void**)&c.sbox, 4 * Nz},        {(void**)&c.iters, 4 * Nz},
         {(void**)&c.ncount, 4 * Nz},      {(void**)&c.nbr, 4 * Nz * (size_t)c.cap},

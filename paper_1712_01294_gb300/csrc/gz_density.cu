@@ -39,6 +39,10 @@ constexpr int kWideLanes = 16;  // ... and in FP32 launches too small for those
 // (1397).  FP64 keeps four: its sums are the lanes' sums.
 constexpr int kWideMax = 12000;
 constexpr int kThreadMin = 45000;
+// Cells per axis from which k_density_one looks for warps whose windows lie
+// inside the box (dens_fill_inside): most warps of a large box (128^3: 984 us
+// without, 944 with), few of an ensemble's small ones (784 without, 799 with).
+constexpr int kInsideMin = 24;
 
 // Radius of the candidate cache for a support Ht: 5% headroom so that small
 // growth of H during the iteration needs no rescan, never past h_lim.
@@ -346,7 +350,70 @@ __device__ __noinline__ int dens_fill(const Grid& g, const BoxInfo& bx, const P4
     return n;
 }
 
+// The same scan for a window that does not reach the box's faces (lo..hi the
+// cells of [x - R, x + R]): the same candidates, distances and order without
+// any periodic shift, and the particle itself told apart once per four
+// candidates.  pos is readable up to three records past its last.
 template <int kCache>
+__device__ __forceinline__ int dens_fill_inside(const int2* __restrict__ cells, int nc, const int (&lo)[3],
+                                                const int (&hi)[3], const P4<float>* __restrict__ pos, int self,
+                                                float xi, float yi, float zi, float R, float (*c_r2)[kOneBlock],
+                                                unsigned (*c_j)[kOneBlock], int t) {
+    const float R2 = R * R, cl = 1.f / (float)nc, R2m = R2 * 1.0001f;
+    int n = 0;
+    for (int cz = lo[2]; cz <= hi[2]; ++cz) {
+        const float gz = fmaxf(fmaxf((float)cz * cl - zi, zi - (float)(cz + 1) * cl), 0.f);
+        const float gz2 = gz * gz;
+        if (gz2 > R2m) continue;
+        for (int cy = lo[1]; cy <= hi[1]; ++cy) {
+            const float gy = fmaxf(fmaxf((float)cy * cl - yi, yi - (float)(cy + 1) * cl), 0.f);
+            const float gzy2 = gz2 + gy * gy;
+            if (gzy2 > R2m) continue;
+            const int2* __restrict__ row = cells + (cz * nc + cy) * nc;
+            // the ranges of up to three cells of the row in flight together
+            for (int x0 = lo[0]; x0 <= hi[0]; x0 += 3) {
+                int2 ses[3];
+#pragma unroll
+                for (int u = 0; u < 3; ++u) {
+                    const int cx = x0 + u;
+                    const float gx = fmaxf(fmaxf((float)cx * cl - xi, xi - (float)(cx + 1) * cl), 0.f);
+                    ses[u] = make_int2(0, 0);
+                    if (cx <= hi[0] && !(gzy2 + gx * gx > R2m)) ses[u] = row[cx];
+                }
+#pragma unroll 1
+                for (int c = 0; c < 3; ++c) {
+                    const int2 se = c == 0 ? ses[0] : (c == 1 ? ses[1] : ses[2]);
+                    for (int j0 = se.x; j0 < se.y; j0 += 4) {
+                        P4<float> q[4];
+                        float r2[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) q[u] = pos[j0 + u];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) r2[u] = sep2(q[u].x - xi, q[u].y - yi, q[u].z - zi);
+                        if ((unsigned)(self - j0) < 4u) {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (j0 + u == self) r2[u] = 1e30f;
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            if (r2[u] < R2 && j0 + u < se.y) {
+                                if (n < kCache) {
+                                    c_r2[n][t] = r2[u];
+                                    c_j[n][t] = (unsigned)(j0 + u);
+                                }
+                                ++n;
+                            }
+                        }
+                    }
+                }
+            }
+        }
+    }
+    return n;
+}
+
+template <int kCache, bool kInside>
 __global__ void __launch_bounds__(kOneBlock, 10)
     k_density_one(int N, Sorted<float> s, Grid g, KParams p, unsigned* __restrict__ nbr,
                   int* __restrict__ ncount, int* __restrict__ iters, DevStatus* st,
@@ -369,9 +436,29 @@ __global__ void __launch_bounds__(kOneBlock, 10)
     if (bad) set_status(st, GZ_S_NONFINITE, GZ_C_NONFINITE, s.id[i]);
     float Rc = dens_cache_radius<float>(H, p);
     int ncache = 0;
-    if (wide(Rc, bx.nc)) {
+    // the cache of the starting H, scanned before the iteration (few live values
+    // here).  kInside: a warp with every window inside the box takes the plain
+    // scan.
+    bool in = kInside && Rc >= 0.f && !wide(Rc, bx.nc) && 2.f * Rc + 2.f / (float)bx.nc < 0.5f;
+    int lo[3], hi[3];
+    if constexpr (kInside) {
+        const float c3[3] = {me.x, me.y, me.z};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = (int)floorf((c3[a] - Rc) * (float)bx.nc - 1e-3f);
+            hi[a] = (int)floorf((c3[a] + Rc) * (float)bx.nc + 1e-3f);
+            in = in && c3[a] >= 0.f && c3[a] <= 1.f && lo[a] >= 0 && hi[a] < bx.nc;
+        }
+        in = __all_sync(__activemask(), in);
+    }
+    if (in) {
+        ncache = dens_fill_inside<kCache>(g.cells + bx.cell_off, bx.nc, lo, hi, s.pos, i, me.x, me.y, me.z, Rc, c_r2,
+                                          c_j, t);
+    } else if (wide(Rc, bx.nc)) {
         ncache = kCache + 1;
-    } else {  // the cache of the starting H, scanned before the iteration (few live values here)
+    } else if constexpr (kInside) {
+        ncache = dens_fill<kCache>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, c_r2, c_j, t);
+    } else {
         const float R2 = Rc * Rc;
         for_candidates<float>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, [&](int j, float, float, float, float r2) {
             if (r2 < R2) {
@@ -727,7 +814,11 @@ cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
     // seen on the workloads with N_ngb = 32) for boxes of 32^3 particles or
     // more, 48 for smaller ones, whose strong contrasts overflow 40 more often
     long long min_count = c.N;
-    for (const BoxInfo& b : c.hboxes) min_count = std::min(min_count, (long long)b.count);
+    int min_nc = 1 << 30;
+    for (const BoxInfo& b : c.hboxes) {
+        min_count = std::min(min_count, (long long)b.count);
+        min_nc = std::min(min_nc, b.nc);
+    }
     const int asked = c.params.density_cache, ccap = asked > 0 ? asked : kDensCache;
     const int tcap = asked > 0 ? asked : (min_count >= 32 * 32 * 32 ? 40 : 48);
     c.launches += 2;
@@ -740,10 +831,11 @@ cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
     bool done = false;
     if constexpr (std::is_same<T, float>::value) {
         if (n >= kThreadMin) {
+            const bool inside = min_nc >= kInsideMin;
             if (tcap == 40)
-                one(k_density_one<40>);
+                inside ? one(k_density_one<40, true>) : one(k_density_one<40, false>);
             else
-                one(k_density_one<48>);
+                inside ? one(k_density_one<48, true>) : one(k_density_one<48, false>);
             done = true;
         }
     }

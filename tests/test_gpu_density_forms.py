@@ -86,3 +86,19 @@ def test_prefilter_bound_covers_every_pair_inside():
         r2 = (e * e).sum(0, dtype=f)
         b = (f(R) + f(4e-7)) * f(1 + 1e-6)
         assert (r2[inside] < b * b).all(), R
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("make", [lambda: I.turbulence(49, seed=9), lambda: _random(49, 10), lambda: _random(50, 11, clump=0.1)])
+def test_windows_inside_the_box_give_the_same_bits(make):
+    # alone, a large box's inner warps scan without periodic shifts; beside a
+    # small box the launch keeps the general scan
+    import paper_1712_01294_gb300 as m
+    q, tiny = cast_state(make(), 1), cast_state(I.turbulence(8, seed=1), 1)
+    alone = _run(m, [q.N], q, 1)
+    both = q.copy()
+    for k in I.FIELDS + ("id",):
+        setattr(both, k, np.concatenate([getattr(q, k), getattr(tiny, k)]))
+    mixed = _run(m, [q.N, tiny.N], both, 1)
+    for a, b in zip(alone, mixed):
+        assert np.array_equal(a, b[..., :q.N])
