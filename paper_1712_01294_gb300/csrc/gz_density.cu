@@ -822,7 +822,6 @@ cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
     const int asked = c.params.density_cache, ccap = asked > 0 ? asked : kDensCache;
     const int tcap = asked > 0 ? asked : (min_count >= 32 * 32 * 32 ? 40 : 48);
     c.launches += 2;
-    cudaMemsetAsync(c.ndefer, 0, sizeof(int), c.stream);
     auto one = [&](auto kernel) {
         kernel<<<blocks(n, kOneBlock), kOneBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
                                                                  c.iters, c.status, list, nlist, c.defer,

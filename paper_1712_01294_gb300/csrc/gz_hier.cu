@@ -705,7 +705,6 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             if (e == cudaSuccess) e = compact(c, c.aflag, c.alist, c.hcount + 1);
             timer.end(GZ_PASS_SORT);
             cudaMemsetAsync(c.ncount, 0, sizeof(int) * (size_t)N, st);
-            cudaMemsetAsync(c.rcount, 0, sizeof(int) * (size_t)N, st);
             timer.begin(GZ_PASS_DENSITY);
             if (e == cudaSuccess) e = run_density<T>(c, c.alist, c.hcount + 1, nA);
             timer.end(GZ_PASS_DENSITY);
@@ -769,7 +768,6 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             launch_exchange<T>(c, kp, N, nA);
             timer.end(GZ_PASS_FLUX);
             timer.begin(GZ_PASS_UPDATE);
-            cudaMemsetAsync(c.box_hits, 0, sizeof(int) * (size_t)c.nboxes, st);
             c.launches += 1;
             k_h_kick<T><<<nblk(N, 256), 256, 0, st>>>(c.tlist, c.hcount + 2, N, sv, c.sbin, c.dpdt, c.dEdt,
                                                        c.params.scheme == GZ_MFV ? c.dmdt : nullptr, c.dt_use,

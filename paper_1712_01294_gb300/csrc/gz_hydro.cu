@@ -20,7 +20,24 @@ namespace {
 inline int blocks(int n, int t) { return (n + t - 1) / t; }
 
 // Reverse pairs (O10): j in N_i with r_ij >= H_j is appended to j's list.
-// Reads the packed positions, whose w component is the converged H.
+// Reads the packed positions, whose w component is the converged H.  Launches
+// under kRevSplit particles have eight threads a particle (k_reverse_split),
+// larger ones one (k_reverse, 32 registers: with the four positions of a group
+// in flight it takes 55, and 178 us at 128^3 instead of 132).  Reverse lists
+// with their sort, eight threads / one, us: Sod 16^3 13 / 28, Sod 32^3 15 / 29,
+// KH 41^3 19 / 27, Sedov 64^3 39 / 35, turbulence 128^3 252 / 132.
+constexpr int kRevGroups = 8, kRevSplit = 150000;
+template <typename T>
+__device__ __forceinline__ void append_reverse(int i, int j, int N, int rcap, int* __restrict__ rcount,
+                                               unsigned* __restrict__ rnbr, const long long* __restrict__ id,
+                                               DevStatus* st) {
+    const int slot = atomicAdd(&rcount[j], 1);
+    if (slot < rcap)
+        rnbr[lslot(slot, j, N)] = (unsigned)i;
+    else
+        set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, id[j]);
+}
+
 template <typename T>
 __global__ void k_reverse(int N, Sorted<T> s, KParams p, const unsigned* __restrict__ nbr,
                           const int* __restrict__ ncount, int* __restrict__ rcount,
@@ -41,15 +58,39 @@ __global__ void k_reverse(int N, Sorted<T> s, KParams p, const unsigned* __restr
             const P4<T> q = s.pos[j];
             const T dx = mi_diff(q.x, me.x, xim1), dy = mi_diff(q.y, me.y, yim1),
                     dz = mi_diff(q.z, me.z, zim1);
-            const T r2 = sep2(dx, dy, dz);
-            if (!(r2 < q.w * q.w)) {
-                const int slot = atomicAdd(&rcount[j], 1);
-                if (slot < p.rcap)
-                    rnbr[lslot(slot, j, N)] = (unsigned)i;
-                else
-                    set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[j]);
-            }
+            if (!less_(sep2(dx, dy, dz), q.w * q.w)) append_reverse<T>(i, j, N, p.rcap, rcount, rnbr, s.id, st);
         }
+    }
+}
+
+// Thread (i, y) takes list groups y, y + kRevGroups, ... of particle i, the four
+// partners' positions in flight together; most threads do one group.
+template <typename T>
+__global__ void __launch_bounds__(32 * kRevGroups)
+    k_reverse_split(int N, Sorted<T> s, KParams p, const unsigned* __restrict__ nbr,
+                    const int* __restrict__ ncount, int* __restrict__ rcount, unsigned* __restrict__ rnbr,
+                    DevStatus* st) {
+    const int i = blockIdx.x * 32 + threadIdx.x;
+    if (i >= N) return;
+    const int cnt = min(ncount[i], p.cap);
+    if (4 * (int)threadIdx.y >= cnt) return;
+    const P4<T> me = s.pos[i];
+    const unsigned* L = nbr + 4 * (size_t)i;
+    for (int k0 = 4 * threadIdx.y; k0 < cnt; k0 += 4 * kRevGroups) {
+        const uint4 jj = col4_once(L, k0, N);
+        const unsigned js[4] = {jj.x, jj.y, jj.z, jj.w};
+        P4<T> q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            q[u] = me;
+            if (k0 + u < cnt) q[u] = s.pos[js[u]];
+        }
+        T dx[4], dy[4], dz[4];
+        offsets4(q, me.x, me.y, me.z, me.x - T(1), me.y - T(1), me.z - T(1), dx, dy, dz);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (k0 + u < cnt && !less_(sep2(dx[u], dy[u], dz[u]), q[u].w * q[u].w))
+                append_reverse<T>(i, (int)js[u], N, p.rcap, rcount, rnbr, s.id, st);
     }
 }
 
@@ -80,12 +121,28 @@ __global__ void k_sort_rev(int N, const int* __restrict__ rcount, unsigned* __re
     }
     insert_sort(L, n, N);
 }
+// The same with eight lanes a list, for launches under kRevSplit particles (Sod
+// 16^3, late in the run: one thread a list took 11 us, half of it waiting on
+// the few lists of more than eight).
+__global__ void __launch_bounds__(kListBlock) k_sort_rev_lanes(int N, const int* __restrict__ rcount,
+                                                               unsigned* __restrict__ rnbr, int rcap) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / kListLanes;
+    if (i < N) sort_list(rnbr + 4 * (size_t)i, min(rcount[i], rcap), N);
+}
 
-// O5 primitives: rho = m n, P = (gamma - 1) rho u, c = sqrt(gamma P / rho).
+// O5 primitives: rho = m n, P = (gamma - 1) rho u, c = sqrt(gamma P / rho); and
+// what the passes after it count from zero (every one of them follows a
+// k_prim): reverse-list counts, CFL minima, u-floor hits.
 template <typename T>
-__global__ void k_prim(int N, Sorted<T> s, KParams p, DevStatus* st) {
+__global__ void k_prim(int N, Sorted<T> s, KParams p, DevStatus* st, int* __restrict__ rcount, int nb,
+                       unsigned long long* __restrict__ dtmin, int* __restrict__ box_hits) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int b = i; b < nb; b += gridDim.x * blockDim.x) {
+        dtmin[b] = dbits(INFINITY);
+        box_hits[b] = 0;
+    }
     if (i >= N) return;
+    rcount[i] = 0;
     const T g = (T)p.gamma;
     const T rho = s.m[i] * s.n[i];
     const T P = (g - T(1)) * rho * s.u[i];
@@ -653,10 +710,6 @@ __global__ void k_ufloor(Sorted<T> s, const BoxInfo* __restrict__ boxes,
     }
 }
 
-__global__ void k_dt_init(int nb, unsigned long long* dtmin) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nb) dtmin[b] = dbits(INFINITY);
-}
 __global__ void k_dt_final(int nb, const unsigned long long* __restrict__ dtmin, double cfl,
                            double dt_fixed, double* __restrict__ dt_use, double* __restrict__ out) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -749,25 +802,32 @@ KParams kparams(const Ctx& c) {
 template <typename T>
 cudaError_t run_reverse(Ctx& c) {
     c.launches += 2;
-    cudaMemsetAsync(c.rcount, 0, sizeof(int) * (size_t)c.N, c.stream);
-    k_reverse<T><<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, sorted_view<T>(c), kparams(c), c.nbr,
-                                                          c.ncount, c.rcount, c.rnbr, c.status);
-    k_sort_rev<<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, c.rcount, c.rnbr, c.rcap);
+    if (c.N < kRevSplit)
+        k_reverse_split<T><<<blocks(c.N, 32), dim3(32, kRevGroups), 0, c.stream>>>(
+            c.N, sorted_view<T>(c), kparams(c), c.nbr, c.ncount, c.rcount, c.rnbr, c.status);
+    else
+        k_reverse<T><<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, sorted_view<T>(c), kparams(c), c.nbr, c.ncount,
+                                                              c.rcount, c.rnbr, c.status);
+    if (c.N < kRevSplit)
+        k_sort_rev_lanes<<<blocks(c.N, kListBlock / kListLanes), kListBlock, 0, c.stream>>>(c.N, c.rcount, c.rnbr,
+                                                                                            c.rcap);
+    else
+        k_sort_rev<<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, c.rcount, c.rnbr, c.rcap);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t run_prim(Ctx& c) {
     c.launches += 1;
-    k_prim<T><<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, sorted_view<T>(c), kparams(c), c.status);
+    k_prim<T><<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, sorted_view<T>(c), kparams(c), c.status, c.rcount,
+                                                       c.nboxes, (unsigned long long*)c.dt_box, c.box_hits);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t run_gradients(Ctx& c, bool want_dt, bool with_info, const int* list, const int* nlist, int n) {
-    c.launches += want_dt ? 2 : 1;
+    c.launches += 1;
     if (!list) n = c.N;
-    if (want_dt) k_dt_init<<<blocks(c.nboxes, 256), 256, 0, c.stream>>>(c.nboxes, (unsigned long long*)c.dt_box);
     if (n < 1) return cudaGetLastError();
     if (with_info)
         k_gradients<T, true><<<blocks(n, 128), 128, 0, c.stream>>>(
@@ -828,7 +888,6 @@ template <typename T>
 cudaError_t run_update(Ctx& c, gz_particles& p, double* rates_out) {
     c.launches += 2;
     int* hits = c.box_hits;
-    cudaMemsetAsync(hits, 0, sizeof(int) * (size_t)c.nboxes, c.stream);
     k_update<T><<<blocks(c.N, 256), 256, 0, c.stream>>>(
         c.N, sorted_view<T>(c), c.dpdt, c.dEdt, c.params.scheme == GZ_MFV ? c.dmdt : nullptr, c.dt_use, p,
         hits, c.status, rates_out);
@@ -861,12 +920,6 @@ __global__ void k_rates_in(int N, const unsigned* __restrict__ orig, const doubl
 cudaError_t run_rates_in(Ctx& c, const double* rates) {
     c.launches += 1;
     k_rates_in<<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, c.vals, rates, c.dpdt, c.dEdt);
-    return cudaGetLastError();
-}
-
-cudaError_t run_dt_init(Ctx& c) {
-    c.launches += 1;
-    k_dt_init<<<blocks(c.nboxes, 256), 256, 0, c.stream>>>(c.nboxes, (unsigned long long*)c.dt_box);
     return cudaGetLastError();
 }
 

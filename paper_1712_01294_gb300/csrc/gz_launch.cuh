@@ -73,7 +73,6 @@ cudaError_t run_ufloor(Ctx& c, gz_particles& p);
 template <typename T>
 cudaError_t run_grad_out(Ctx& c, T* grad_out, T* B_out);
 
-cudaError_t run_dt_init(Ctx& c);
 cudaError_t run_dt_finalize(Ctx& c, double dt_fixed, double* dt_used_dev);
 cudaError_t run_dt_set(Ctx& c, double dt);
 cudaError_t run_dt_out(Ctx& c, double* out);

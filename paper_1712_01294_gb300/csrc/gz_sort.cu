@@ -329,9 +329,11 @@ __global__ void k_permute(int N, unsigned* __restrict__ skeys, unsigned* __restr
                           const unsigned* __restrict__ order, const unsigned* __restrict__ key_in,
                           const unsigned* __restrict__ count, const unsigned* __restrict__ start, gz_particles p,
                           const void* __restrict__ n_in, const int* __restrict__ box_of,
-                          const BoxInfo* __restrict__ boxes, Sorted<T> s, int2* __restrict__ cells) {
+                          const BoxInfo* __restrict__ boxes, Sorted<T> s, int2* __restrict__ cells,
+                          int* __restrict__ ndefer) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= N) return;
+    if (q == 0) *ndefer = 0;  // (the density pass after it counts from zero)
     unsigned src, key;
     int i = q;
     if constexpr (kCounted) {
@@ -434,7 +436,7 @@ static cudaError_t counting_sort(Ctx& c, const gz_particles& p, const void* n_in
                                               c.cells);
     k_cs_place<<<blocks(N, 256), 256, 0, st>>>(N, c.keys_alt, c.vals_alt, c.kstart, order);
     k_permute<T, true><<<blocks(N, 256), 256, 0, st>>>(N, c.keys, c.vals, order, c.keys_alt, c.kcount, c.kstart, p,
-                                                        n_in, c.box_of, c.boxes, sorted_view<T>(c), c.cells);
+                                                        n_in, c.box_of, c.boxes, sorted_view<T>(c), c.cells, c.ndefer);
     c.launches += direct ? 4 : 5;
     return cudaGetLastError();
 }
@@ -485,7 +487,7 @@ cudaError_t permute_and_bin(Ctx& c, const gz_particles& p, const void* n_in) {
     c.launches += 1;
     cudaMemsetAsync(c.cells, 0, sizeof(int2) * (size_t)c.total_cells, st);
     k_permute<T, false><<<blocks(N, 256), 256, 0, st>>>(N, c.keys, c.vals, nullptr, nullptr, nullptr, nullptr, p,
-                                                         n_in, c.box_of, c.boxes, sorted_view<T>(c), c.cells);
+                                                         n_in, c.box_of, c.boxes, sorted_view<T>(c), c.cells, c.ndefer);
     return cudaGetLastError();
 }
 template cudaError_t sort_and_bin<float>(Ctx&, const gz_particles&, const void*);
