@@ -349,10 +349,9 @@ __device__ __forceinline__ void mfv_flux(const T (&FL)[5], const T (&FR)[5], T u
     FE = fma(T(0.5) * dot3(vfx, vfy, vfz, vfx, vfy, vfz), fr, fe + dot3(vfx, vfy, vfz, fx, fy, fz));
 }
 
-// x^y for x > 0: FP32 as 2^(y log2 x) from the hardware base-2 logarithm
-// (relative error about 1e-7 (1 + |y log2 x|)); FP64 the library pow.
+// x^y for x > 0 in FP32, 2^(y log2 x) from the hardware base-2 logarithm
+// (relative error about 1e-7 (1 + |y log2 x|)).
 __device__ __forceinline__ float ppow(float x, float y) { return exp2f(y * __log2f(x)); }
-__device__ __forceinline__ double ppow(double x, double y) { return pow(x, y); }
 
 // Exact Riemann problem of the face (option of O12).  Pressure function of one
 // side at the trial star pressure p: shock branch (p > P_K)
@@ -360,18 +359,18 @@ __device__ __forceinline__ double ppow(double x, double y) { return pow(x, y); }
 // B_K = (gamma-1)/(gamma+1) P_K; rarefaction branch
 // 2 c_K/(gamma-1) ((p/P_K)^e - 1), e = (gamma-1)/(2 gamma), whose derivative
 // (p/P_K)^(e-1)/(rho_K c_K) is formed from the same power.  f and df/dp.
-template <typename T>
-__device__ __forceinline__ void pres_side(T p, T rho, T P, T c, T gam, T& f, T& fd) {
+__device__ __forceinline__ void pres_side(double p, double rho, double P, double c, double gam, double& f,
+                                          double& fd) {
     if (p > P) {
-        const T A = pdiv(T(2), (gam + T(1)) * rho), Bk = pdiv(gam - T(1), gam + T(1)) * P;
-        const T q = psqrt(pdiv(A, p + Bk));
+        const double A = 2.0 / ((gam + 1.0) * rho), Bk = (gam - 1.0) / (gam + 1.0) * P;
+        const double q = sqrt(A / (p + Bk));
         f = (p - P) * q;
-        fd = q * (T(1) - T(0.5) * pdiv(p - P, p + Bk));
+        fd = q * (1.0 - 0.5 * ((p - P) / (p + Bk)));
     } else {
-        const T r = pdiv(p, P);
-        const T pe = ppow(r, pdiv(gam - T(1), T(2) * gam));
-        f = pdiv(T(2) * c, gam - T(1)) * (pe - T(1));
-        fd = pdiv(pe, r * rho * c);
+        const double r = p / P;
+        const double pe = pow(r, (gam - 1.0) / (2.0 * gam));
+        f = 2.0 * c / (gam - 1.0) * (pe - 1.0);
+        fd = pe / (r * rho * c);
     }
 }
 
@@ -386,62 +385,130 @@ __device__ __forceinline__ void pres_side(T p, T rho, T P, T c, T gam, T& f, T& 
 // (g_L P_L + g_R P_R - (u_R - u_L))/(g_L + g_R), g_K = sqrt(A_K/(p_PV + B_K));
 // at least 1e-12 (P_L + P_R).  Newton steps kept inside the bracket the signs
 // of F have established (bisection, or doubling while no upper end is known)
-// until two iterates agree to 1e-15 (FP64) or 1e-6 (FP32) relative, or F is at
-// the rounding level of its terms (FP32: 4e-7 of |f_L| + |f_R| + |u_R - u_L|,
-// where a strong rarefaction's F cannot resolve p to 1e-6); at most 200 (FP64)
+// until two iterates agree to 1e-15 (FP64) or 1e-6 (FP32) relative, or (FP32)
+// F is at the rounding level of its terms, 4e-7 of |f_L| + |f_R| + |u_R - u_L|,
+// where a strong rarefaction's F cannot resolve p to 1e-6; at most 200 (FP64)
 // or 20 (FP32) steps.  u* = (u_L + u_R)/2 + (f_R - f_L)/2.  Returns false when
 // the two fans open a vacuum (2 (c_L + c_R)/(gamma-1) <= u_R - u_L).
-template <typename T>
-__device__ __forceinline__ bool exact_star(T rL, T uL, T PL, T rR, T uR, T PR, T gam, T& ps, T& us) {
-    const T cL = psqrt(pdiv(gam * PL, rL)), cR = psqrt(pdiv(gam * PR, rR));
-    const T du = uR - uL;
-    if (pdiv(T(2) * (cL + cR), gam - T(1)) <= du) return false;
-    const T plo = min(PL, PR), phi = max(PL, PR);
-    T p = T(0.5) * (PL + PR) - T(0.125) * du * (rL + rR) * (cL + cR);
-    if (!(phi <= T(2) * plo && p >= plo && p <= phi)) {
+__device__ __forceinline__ bool exact_star(double rL, double uL, double PL, double rR, double uR, double PR, double gam,
+                                           double& ps, double& us) {
+    const double cL = sqrt(gam * PL / rL), cR = sqrt(gam * PR / rR);
+    const double du = uR - uL;
+    if (2.0 * (cL + cR) / (gam - 1.0) <= du) return false;
+    const double plo = min(PL, PR), phi = max(PL, PR);
+    double p = 0.5 * (PL + PR) - 0.125 * du * (rL + rR) * (cL + cR);
+    if (!(phi <= 2.0 * plo && p >= plo && p <= phi)) {
         if (p < plo) {
-            const T e = pdiv(gam - T(1), T(2) * gam);
-            const T num = (cL + cR) - T(0.5) * (gam - T(1)) * du;
-            const T den = cL * ppow(PL, -e) + cR * ppow(PR, -e);
-            p = ppow(pdiv(num, den), pdiv(T(1), e));
+            const double e = (gam - 1.0) / (2.0 * gam);
+            const double num = (cL + cR) - 0.5 * (gam - 1.0) * du;
+            const double den = cL * pow(PL, -e) + cR * pow(PR, -e);
+            p = pow(num / den, 1.0 / e);
         } else {
-            const T p0 = max(p, T(0));
-            const T gp1 = gam + T(1), gm1 = gam - T(1);
-            const T gL = psqrt(pdiv(pdiv(T(2), gp1 * rL), p0 + pdiv(gm1, gp1) * PL));
-            const T gR = psqrt(pdiv(pdiv(T(2), gp1 * rR), p0 + pdiv(gm1, gp1) * PR));
-            p = pdiv((gL * PL + gR * PR) - du, gL + gR);
+            const double p0 = max(p, 0.0);
+            const double gp1 = gam + 1.0, gm1 = gam - 1.0;
+            const double gL = sqrt(2.0 / (gp1 * rL) / (p0 + gm1 / gp1 * PL));
+            const double gR = sqrt(2.0 / (gp1 * rR) / (p0 + gm1 / gp1 * PR));
+            p = ((gL * PL + gR * PR) - du) / (gL + gR);
         }
     }
-    const T pmin = T(1e-12) * (PL + PR);
+    const double pmin = 1e-12 * (PL + PR);
     if (!(p >= pmin)) p = pmin;
-    constexpr bool f32 = sizeof(T) == 4;
-    const T tol = f32 ? T(1e-6) : T(1e-15);
-    const int cap = f32 ? 20 : 200;
-    T lo = T(0), hi = T(0);
+    double lo = 0.0, hi = 0.0;
     bool has_hi = false;
-    for (int it = 0; it < cap; ++it) {
-        T fL, dL, fR, dR;
+    for (int it = 0; it < 200; ++it) {
+        double fL, dL, fR, dR;
         pres_side(p, rL, PL, cL, gam, fL, dL);
         pres_side(p, rR, PR, cR, gam, fR, dR);
-        const T F = (fL + fR) + du;
-        if (f32 && fabs(F) <= T(4e-7) * ((fabs(fL) + fabs(fR)) + fabs(du))) break;
-        if (F > T(0)) {
+        const double F = (fL + fR) + du;
+        if (F > 0.0) {
             hi = p;
             has_hi = true;
         } else {
             lo = p;
         }
-        T pn = p - pdiv(F, dL + dR);
-        if (!(pn > lo) || (has_hi && !(pn < hi))) pn = has_hi ? T(0.5) * (lo + hi) : T(2) * p;
-        const bool done = fabs(pn - p) <= tol * (pn + p);
+        double pn = p - F / (dL + dR);
+        if (!(pn > lo) || (has_hi && !(pn < hi))) pn = has_hi ? 0.5 * (lo + hi) : 2.0 * p;
+        const bool done = fabs(pn - p) <= 1e-15 * (pn + p);
         p = pn;
         if (done) break;
     }
-    T fL, dL, fR, dR;
+    double fL, dL, fR, dR;
     pres_side(p, rL, PL, cL, gam, fL, dL);
     pres_side(p, rR, PR, cR, gam, fR, dR);
     ps = p;
-    us = T(0.5) * (uL + uR) + T(0.5) * (fR - fL);
+    us = 0.5 * (uL + uR) + 0.5 * (fR - fL);
+    return true;
+}
+
+// The same in FP32, written for warps whose lanes hold different waves: both
+// branches of the two pressure functions are formed and selected (three
+// special-function results a side, against four divergent combinations of
+// branches: the form above ran 8 of 32 lanes, 616 us for Sod 50^3's flux pass,
+// this one 282), and the primitive-variable
+// estimate starts the iteration wherever the pressures are within 2x and it is
+// not below half the lower one, where Newton's step from it needs one or two
+// rounds.  Elsewhere the same two-rarefaction and two-shock estimates.  Stops
+// as above; u* takes the two functions at the last pressure, carried there by
+// their derivatives.
+__device__ __forceinline__ bool exact_star(float rL, float uL, float PL, float rR, float uR, float PR, float gam,
+                                           float& ps, float& us) {
+    const float qL = gam * PL * rcp_(rL), qR = gam * PR * rcp_(rR);
+    const float cL = qL * rsq_(fmaxf(qL, 1e-37f)), cR = qR * rsq_(fmaxf(qR, 1e-37f));
+    const float gm1 = gam - 1.f, gp1 = gam + 1.f, i1 = rcp_(gm1), e = 0.5f * gm1 * rcp_(gam);
+    const float du = uR - uL;
+    if (2.f * (cL + cR) * i1 <= du) return false;
+    const float plo = fminf(PL, PR), phi = fmaxf(PL, PR);
+    const float iAL = 0.5f * gp1 * rL, iAR = 0.5f * gp1 * rR;  // 1/A_K
+    const float mu = gm1 * rcp_(gp1), BL = mu * PL, BR = mu * PR;
+    float p = 0.5f * (PL + PR) - 0.125f * du * (rL + rR) * (cL + cR);
+    if (!(phi <= 2.f * plo && p >= 0.5f * plo && p <= phi)) {
+        if (p < plo) {
+            const float num = (cL + cR) - 0.5f * gm1 * du;
+            const float den = cL * ppow(PL, -e) + cR * ppow(PR, -e);
+            p = ppow(num * rcp_(den), rcp_(e));
+        } else {
+            const float p0 = fmaxf(p, 0.f);
+            const float gL = rsq_((p0 + BL) * iAL), gR = rsq_((p0 + BR) * iAR);
+            p = ((gL * PL + gR * PR) - du) * rcp_(gL + gR);
+        }
+    }
+    const float pmin = 1e-12f * (PL + PR);
+    if (!(p >= pmin)) p = pmin;
+    const float iPL = rcp_(PL), iPR = rcp_(PR), kL = 2.f * cL * i1, kR = 2.f * cR * i1;
+    const float jL = PL * rcp_(rL * cL), jR = PR * rcp_(rR * cR);  // P/(rho c)
+    float lo = 0.f, hi = 0.f, fL = 0.f, fR = 0.f, dL = 0.f, dR = 0.f, dp = 0.f;
+    bool has_hi = false;
+    auto side = [&](float P, float iP, float B, float iA, float k, float j, float ip, float& f, float& d) {
+        const float q = rsq_((p + B) * iA), dP = p - P;
+        const float pe = ppow(p * iP, e);
+        const bool shock = p > P;
+        f = shock ? dP * q : k * (pe - 1.f);
+        d = shock ? fmaf(-0.5f * dP * iA, q * q * q, q) : pe * j * ip;
+    };
+#pragma unroll 1
+    for (int it = 0; it < 20; ++it) {
+        const float ip = rcp_(p);
+        side(PL, iPL, BL, iAL, kL, jL, ip, fL, dL);
+        side(PR, iPR, BR, iAR, kR, jR, ip, fR, dR);
+        const float F = (fL + fR) + du;
+        dp = 0.f;
+        if (fabsf(F) <= 4e-7f * ((fabsf(fL) + fabsf(fR)) + fabsf(du))) break;
+        if (F > 0.f) {
+            hi = p;
+            has_hi = true;
+        } else {
+            lo = p;
+        }
+        float pn = p - F * rcp_(dL + dR);
+        if (!(pn > lo) || (has_hi && !(pn < hi))) pn = has_hi ? 0.5f * (lo + hi) : 2.f * p;
+        dp = pn - p;
+        const bool done = fabsf(dp) <= 1e-6f * (pn + p);
+        p = pn;
+        if (done) break;
+        dp = 0.f;
+    }
+    ps = p;
+    us = 0.5f * (uL + uR) + 0.5f * ((fR - fL) + (dR - dL) * dp);
     return true;
 }
 
@@ -633,14 +700,33 @@ struct Totals {
 };
 template <typename T, bool kMFV, int kRiem>
 constexpr bool kLoadAhead = sizeof(T) == 4 && !kMFV && kRiem == 0;
+template <int kRiem>
+constexpr int kPairUnroll = kRiem == 0 ? 4 : 1;
+
+// f(j) for the first min(n, 4) slots of a list group, in kUnroll copies.
+template <int kUnroll, typename F>
+__device__ __forceinline__ void for_slots(const uint4& jj, int n, F&& f) {
+    if constexpr (kUnroll == 4) {
+        const unsigned js[4] = {jj.x, jj.y, jj.z, jj.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (u >= n) break;
+            f((int)js[u]);
+        }
+    } else {
+#pragma unroll 1
+        for (int u = 0; u < min(n, 4); ++u) f((int)(u == 0 ? jj.x : (u == 1 ? jj.y : (u == 2 ? jj.z : jj.w))));
+    }
+}
 
 // pair(rec, j, dst) adds the pair with record rec of partner j to dst[nq].
 // kAhead: the next partner's record is loaded while the current pair is
 // evaluated (two record buffers, so the loop is written for two pairs at a
 // time; 165 registers, 12 warps an SM).  The pass waits on its gathers: FP32
 // MFM at 128^3 856 us without, 803 with.  The forms with more arithmetic a
-// pair (MFV, the exact solver, FP64) need the registers themselves.
-template <typename T, int nq, bool kAhead, typename P>
+// pair (MFV, the exact solver, FP64) need the registers themselves.  kUnroll:
+// copies of the pair's code (the exact solver's is long: one).
+template <typename T, int nq, bool kAhead, int kUnroll, typename P>
 __device__ __forceinline__ Totals<nq> sum_runs(int i, int N, const T* __restrict__ rec,
                                                const unsigned* __restrict__ nbr, int cnt,
                                                const unsigned* __restrict__ rnbr, int rcnt, P&& pair) {
@@ -680,13 +766,10 @@ __device__ __forceinline__ Totals<nq> sum_runs(int i, int N, const T* __restrict
                     }
                 }
             } else {
-                const unsigned js[4] = {jj.x, jj.y, jj.z, jj.w};
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (k0 + u >= n) break;
-                    load_rec(rec, (int)js[u], A);
-                    pair(A, (int)js[u], run);
-                }
+                for_slots<kUnroll>(jj, n - k0, [&](int j) {
+                    load_rec(rec, j, A);
+                    pair(A, j, run);
+                });
             }
             jj = nn;
             if ((k0 & 4) || k0 + 4 >= n) {
@@ -700,7 +783,7 @@ __device__ __forceinline__ Totals<nq> sum_runs(int i, int N, const T* __restrict
 
 // Four warps: warp c forms runs c, c + 4, ...; v[0] becomes quantity c's total
 // (v[1], in warp 0, the fifth's).  Every thread of the block must get here.
-template <typename T, int nq, typename P>
+template <typename T, int nq, int kUnroll, typename P>
 __device__ __forceinline__ Totals<2> sum_runs_split(int i, int N, const T* __restrict__ rec,
                                                     const unsigned* __restrict__ nbr, int cnt,
                                                     const unsigned* __restrict__ rnbr, int rcnt, P&& pair) {
@@ -720,14 +803,11 @@ __device__ __forceinline__ Totals<2> sum_runs_split(int i, int N, const T* __res
 #pragma unroll 1
             for (int k0 = k1; k0 < min(n, k1 + 8); k0 += 4) {
                 const uint4 jj = col4_once(L, k0, N);
-                const unsigned js[4] = {jj.x, jj.y, jj.z, jj.w};
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (k0 + u >= n) break;
+                for_slots<kUnroll>(jj, n - k0, [&](int j) {
                     T b[kRecord];
-                    load_rec(rec, (int)js[u], b);
-                    pair(b, (int)js[u], run);
-                }
+                    load_rec(rec, j, b);
+                    pair(b, j, run);
+                });
             }
         }
 #pragma unroll

@@ -504,10 +504,10 @@ __global__ void __launch_bounds__(kXBlock)
         nneg += (fl >> 1) & 1;
     };
     if constexpr (kSplit) {
-        const Totals<2> s = sum_runs_split<T, nq>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
+        const Totals<2> s = sum_runs_split<T, nq, kPairUnroll<kRiem>>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
         if (t < n) store_rates_split<nq>(s.v, i, N, dpdt, dEdt, dmdt);
     } else {
-        const Totals<nq> s = sum_runs<T, nq, false>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
+        const Totals<nq> s = sum_runs<T, nq, false, kPairUnroll<kRiem>>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
         store_rates<nq>(s.v, i, N, dpdt, dEdt, dmdt);
     }
     count_flags(st, nfall, nneg);

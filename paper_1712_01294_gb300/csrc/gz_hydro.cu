@@ -589,10 +589,10 @@ __global__ void __launch_bounds__(kFluxBlock, kLoadAhead<T, kMFV, kRiem> ? 3 : 1
         nneg += (fl >> 1) & 1;
     };
     if constexpr (kSplit) {
-        const Totals<2> t = sum_runs_split<T, nq>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
+        const Totals<2> t = sum_runs_split<T, nq, kPairUnroll<kRiem>>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
         if (it < N) store_rates_split<nq>(t.v, i, N, dpdt, dEdt, dmdt);
     } else {
-        const Totals<nq> t = sum_runs<T, nq, kLoadAhead<T, kMFV, kRiem>>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
+        const Totals<nq> t = sum_runs<T, nq, kLoadAhead<T, kMFV, kRiem>, kPairUnroll<kRiem>>(i, N, rec, nbr, cnt, rnbr, rcnt, pair);
         store_rates<nq>(t.v, i, N, dpdt, dEdt, dmdt);
     }
     count_flags(st, nfall, nneg);
