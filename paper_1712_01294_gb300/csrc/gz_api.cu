@@ -151,7 +151,7 @@ gz_status prepare_given(gz_ctx* ctx, const gz_particles* p, const void* n, bool 
     }
     if (e == cudaSuccess) {
         Pass t(c, GZ_PASS_LISTS);
-        e = run_build_lists<T>(c);
+        e = run_build_lists<T>(c, 0);
     }
     if (e == cudaSuccess) {
         Pass t(c, GZ_PASS_PRIM);
@@ -352,7 +352,7 @@ cudaError_t fork_side(Ctx& c) {
 // The backward pass's sort and density pass from a GZ_CKPT_LISTS checkpoint:
 // the sorted order and cells from the saved keys, the saved H, n, sums,
 // counts and list slots, and a scan for the lists longer than the saved
-// slots; the same values the sort and k_dens_given give.
+// slots; the same values the sort and k_lists give.
 template <typename T>
 cudaError_t restore_lists(Ctx& c, const gz_particles& p, const Ckpt& k) {
     const size_t N = (size_t)c.N;
@@ -365,7 +365,7 @@ cudaError_t restore_lists(Ctx& c, const gz_particles& p, const Ckpt& k) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(c.ssd, k.sd, sizeof(T) * N, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c.ncount, k.ncount, 4 * N, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = copy_lists(c, c.ncount, k.nbr, c.nbr, k.slots, st);
-    if (e == cudaSuccess && k.slots < c.cap) e = run_lists_over<T>(c, k.slots);
+    if (e == cudaSuccess && k.slots < c.cap) e = run_build_lists<T>(c, k.slots);
     return e;
 }
 
@@ -412,7 +412,7 @@ gz_status do_step_backward(gz_ctx* ctx, const gz_particles* p, double dt, const 
         if (ck.H) {  // the forward's converged H: no h-iteration; its n and sums
             const size_t bytes = sizeof(T) * (size_t)c.N;
             e = cudaMemcpyAsync(c.sh, ck.H, bytes, cudaMemcpyDeviceToDevice, c.stream);
-            if (e == cudaSuccess) e = run_density_given<T>(c);
+            if (e == cudaSuccess) e = run_build_lists<T>(c, 0);
             if (e == cudaSuccess) e = cudaMemcpyAsync(c.sn, ck.n, bytes, cudaMemcpyDeviceToDevice, c.stream);
             if (e == cudaSuccess) e = cudaMemcpyAsync(c.ssd, ck.sd, bytes, cudaMemcpyDeviceToDevice, c.stream);
         } else {

@@ -354,13 +354,11 @@ __device__ __noinline__ int dens_fill(const Grid& g, const BoxInfo& bx, const P4
 // cells of [x - R, x + R]): the same candidates, distances and order without
 // any periodic shift, and the particle itself told apart once per four
 // candidates.  pos is readable up to three records past its last.
-template <int kCache>
-__device__ __forceinline__ int dens_fill_inside(const int2* __restrict__ cells, int nc, const int (&lo)[3],
-                                                const int (&hi)[3], const P4<float>* __restrict__ pos, int self,
-                                                float xi, float yi, float zi, float R, float (*c_r2)[kOneBlock],
-                                                unsigned (*c_j)[kOneBlock], int t) {
+template <typename E>
+__device__ __forceinline__ void scan_inside(const int2* __restrict__ cells, int nc, const int (&lo)[3],
+                                            const int (&hi)[3], const P4<float>* __restrict__ pos, int self,
+                                            float xi, float yi, float zi, float R, E&& hit) {
     const float R2 = R * R, cl = 1.f / (float)nc, R2m = R2 * 1.0001f;
-    int n = 0;
     for (int cz = lo[2]; cz <= hi[2]; ++cz) {
         const float gz = fmaxf(fmaxf((float)cz * cl - zi, zi - (float)(cz + 1) * cl), 0.f);
         const float gz2 = gz * gz;
@@ -397,20 +395,28 @@ __device__ __forceinline__ int dens_fill_inside(const int2* __restrict__ cells, 
                         }
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            if (r2[u] < R2 && j0 + u < se.y) {
-                                if (n < kCache) {
-                                    c_r2[n][t] = r2[u];
-                                    c_j[n][t] = (unsigned)(j0 + u);
-                                }
-                                ++n;
-                            }
+                            if (r2[u] < R2 && j0 + u < se.y) hit(j0 + u, r2[u]);
                         }
                     }
                 }
             }
         }
     }
-    return n;
+}
+
+// Cells lo..hi of the window [x - R, x + R]; true when every lane's lies
+// inside its box (what scan_inside asks for).
+__device__ __forceinline__ bool warp_inside(const BoxInfo& bx, const P4<float>& me, float R, int (&lo)[3],
+                                            int (&hi)[3]) {
+    bool in = R >= 0.f && !wide(R, bx.nc) && 2.f * R + 2.f / (float)bx.nc < 0.5f;
+    const float c3[3] = {me.x, me.y, me.z};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = (int)floorf((c3[a] - R) * (float)bx.nc - 1e-3f);
+        hi[a] = (int)floorf((c3[a] + R) * (float)bx.nc + 1e-3f);
+        in = in && c3[a] >= 0.f && c3[a] <= 1.f && lo[a] >= 0 && hi[a] < bx.nc;
+    }
+    return __all_sync(__activemask(), in);
 }
 
 template <int kCache, bool kInside>
@@ -439,21 +445,17 @@ __global__ void __launch_bounds__(kOneBlock, 10)
     // the cache of the starting H, scanned before the iteration (few live values
     // here).  kInside: a warp with every window inside the box takes the plain
     // scan.
-    bool in = kInside && Rc >= 0.f && !wide(Rc, bx.nc) && 2.f * Rc + 2.f / (float)bx.nc < 0.5f;
     int lo[3], hi[3];
-    if constexpr (kInside) {
-        const float c3[3] = {me.x, me.y, me.z};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = (int)floorf((c3[a] - Rc) * (float)bx.nc - 1e-3f);
-            hi[a] = (int)floorf((c3[a] + Rc) * (float)bx.nc + 1e-3f);
-            in = in && c3[a] >= 0.f && c3[a] <= 1.f && lo[a] >= 0 && hi[a] < bx.nc;
-        }
-        in = __all_sync(__activemask(), in);
-    }
+    bool in = false;
+    if constexpr (kInside) in = warp_inside(bx, me, Rc, lo, hi);
     if (in) {
-        ncache = dens_fill_inside<kCache>(g.cells + bx.cell_off, bx.nc, lo, hi, s.pos, i, me.x, me.y, me.z, Rc, c_r2,
-                                          c_j, t);
+        scan_inside(g.cells + bx.cell_off, bx.nc, lo, hi, s.pos, i, me.x, me.y, me.z, Rc, [&](int j, float r2) {
+            if (ncache < kCache) {
+                c_r2[ncache][t] = r2;
+                c_j[ncache][t] = (unsigned)j;
+            }
+            ++ncache;
+        });
     } else if (wide(Rc, bx.nc)) {
         ncache = kCache + 1;
     } else if constexpr (kInside) {
@@ -511,12 +513,18 @@ __global__ void __launch_bounds__(kOneBlock, 10)
     if (it > p.max_iter) it = p.max_iter;
     const float H2 = Hev * Hev;
     int cnt = 0;
-    for (int k = 0; k < ncache; ++k) {  // list of the returned H, in scan order
+    // list of the returned H, in scan order, gathered at the cache's front and
+    // written four slots at a time (512 contiguous bytes a warp; slot by slot:
+    // 949 us for the pass at 128^3 instead of 919)
+    for (int k = 0; k < ncache; ++k) {
         if (c_r2[k][t] < H2) {
-            if (cnt < p.cap) store_slot(nbr + lslot(cnt, i, N), c_j[k][t]);
+            c_j[cnt][t] = c_j[k][t];
             ++cnt;
         }
     }
+    for (int k = 0; k < min(cnt, p.cap); k += 4)
+        *reinterpret_cast<uint4*>(nbr + lslot(k, i, N)) =
+            make_uint4(c_j[k][t], c_j[k + 1][t], c_j[k + 2][t], c_j[k + 3][t]);
     s.h[i] = Hev;
     s.n[i] = n_of(Sv, Hev);
     if (s.sd) s.sd[i] = sdv;
@@ -696,73 +704,68 @@ __global__ void __launch_bounds__(kWarpDensBlock)
 // Neighbour lists N_i = {j : r_ij < H_i} for given H (O3).  only_over > 0:
 // only the particles whose count exceeds it (lists a checkpoint kept up to
 // that many slots; the others are restored from it).
-template <typename T>
-__global__ void __launch_bounds__(128)
-    k_lists(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
-            int* __restrict__ ncount, DevStatus* st, int only_over) {
+// FP32, large launches: one thread per particle with the density pass's scan.
+// Bound like it by the chain range -> candidates through L1 and L2, and by its
+// own scattered stores: the first kStage neighbours are gathered in shared
+// memory and written four slots at a time.  75^3 particles: 124 us (slot by
+// slot 138, and 150 with the periodic shifts in every window); kStage = 40
+// leaves less of L1 (127), 16 and 24 send more to the slow stores (130..137).
+// Four lanes a particle take 201 there, so the line to the form below is the
+// density pass's.
+constexpr int kGivenBlock = 128, kStage = 32;
+template <bool kInside>
+__global__ void __launch_bounds__(kGivenBlock, 8)
+    k_lists_one(int N, Sorted<float> s, Grid g, KParams p, unsigned* __restrict__ nbr, int* __restrict__ ncount,
+                DevStatus* st, int only_over) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     if (only_over > 0 && ncount[i] <= only_over) return;
     const BoxInfo bx = g.boxes[s.box[i]];
-    const T Hi = s.h[i];
-    const T H2 = Hi * Hi;
+    const float H = s.h[i], H2 = H * H;
+    const P4<float> me = s.pos[i];
+    unsigned* L = nbr + lslot(0, i, N);
     int c = 0;
-    const P4<T> me = s.pos[i];
-    for_candidates<T>(g, bx, s.pos, i, me.x, me.y, me.z, Hi,
-                      [&](int j, T, T, T, T r2) {
-                          if (r2 < H2) {
-                              if (c < p.cap) store_slot(nbr + lslot(c, i, N), (unsigned)j);
-                              ++c;
-                          }
-                      });
+    const int t = threadIdx.x;
+    __shared__ unsigned c_j[kStage][kGivenBlock];
+    auto hit = [&](int j, float) {
+        if (c < kStage)
+            c_j[c][t] = (unsigned)j;
+        else if (c < p.cap)
+            store_slot(L + lcol(c, N), (unsigned)j);
+        ++c;
+    };
+    int lo[3], hi[3];
+    bool in = false;
+    if constexpr (kInside) in = warp_inside(bx, me, H, lo, hi);
+    if (in)
+        scan_inside(g.cells + bx.cell_off, bx.nc, lo, hi, s.pos, i, me.x, me.y, me.z, H, hit);
+    else
+        for_candidates<float>(g, bx, s.pos, i, me.x, me.y, me.z, H, [&](int j, float, float, float, float r2) {
+            if (r2 < H2) hit(j, r2);
+        });
+    const int most = min(min(c, kStage), p.cap);
+    for (int k = 0; k < most; k += 4)
+        *reinterpret_cast<uint4*>(L + lcol(k, N)) = make_uint4(c_j[k][t], c_j[k + 1][t], c_j[k + 2][t], c_j[k + 3][t]);
     ncount[i] = c;
     if (c > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
 }
 
-// Density pass for a known converged H (a step checkpoint's): the neighbour
-// list of H, n and the sum of -w'(q) q in one cell scan of radius H.  The
-// candidates inside H come in the h-iteration's scan order and are summed the
-// same way, so n and the sums equal the h-iteration's last evaluation bit
-// for bit.
+// Small launches and FP64: four lanes per particle.
 template <typename T>
-__global__ void __launch_bounds__(128)
-    k_dens_given(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
-                 int* __restrict__ ncount, DevStatus* st) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kDensBlock)
+    k_lists(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr, int* __restrict__ ncount,
+            DevStatus* st, int only_over) {
+    const int gl = threadIdx.x % kLanes, i = (blockIdx.x * kDensBlock + threadIdx.x) / kLanes;
+    const unsigned gm = group_mask<kLanes>();
     if (i >= N) return;
-    const BoxInfo bx = g.boxes[s.box[i]];
-    const T Ht = s.h[i];
-    const T H2 = Ht * Ht;
-    const T iH = T(1) / Ht;
+    if (only_over > 0 && ncount[i] <= only_over) return;
     const P4<T> me = s.pos[i];
-    Acc<T> sw;
-    T sd = T(0);
-    int c = 0;
-    for_candidates<T>(g, bx, s.pos, i, me.x, me.y, me.z, Ht,
-                      [&](int j, T, T, T, T r2) {
-                          if (r2 < H2) {
-                              const T q = psqrt(r2) * iH;
-                              T w, qdw;
-                              dens_terms(q, w, qdw);
-                              sw.add(w);
-                              sd += qdw;
-                              if (c < p.cap) store_slot(nbr + lslot(c, i, N), (unsigned)j);
-                              ++c;
-                          }
-                      });
-    double S;
-    if constexpr (std::is_same<T, float>::value)
-        S = (double)sw.fvalue();  // as the h-iteration forms it
-    else
-        S = sw.value();
-    const double Hev = (double)Ht;
-    if (std::is_same<T, float>::value) {
-        const float Hf = (float)Hev;
-        s.n[i] = (T)(8.f * (float)(1.0 + S) / ((float)kPi * Hf * Hf * Hf));
-    } else {
-        s.n[i] = (T)(8.0 * (1.0 + S) / (kPi * Hev * Hev * Hev));
-    }
-    s.sd[i] = sd;
+    unsigned* L = nbr + lslot(0, i, N);
+    const int c = group_scan<T, kLanes, true>(g, g.boxes[s.box[i]], s.pos, i, me.x, me.y, me.z, s.h[i], gl, gm, 1 << 30,
+                                              [&](int k, int j) {
+                                                  if (k < p.cap) store_slot(L + lcol(k, N), (unsigned)j);
+                                              });
+    if (gl != 0) return;
     ncount[i] = c;
     if (c > p.cap) set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
 }
@@ -856,30 +859,27 @@ cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
     return cudaGetLastError();
 }
 
+// kept > 0: only the lists longer than that (their first slots are there already).
 template <typename T>
-cudaError_t run_density_given(Ctx& c) {
+cudaError_t run_build_lists(Ctx& c, int kept) {
     c.launches += 1;
-    k_dens_given<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
-                                                             c.nbr, c.ncount, c.status);
+    const Sorted<T> sv = sorted_view<T>(c);
+    if constexpr (std::is_same<T, float>::value) {
+        if (c.N >= kThreadMin) {
+            int min_nc = 1 << 30;
+            for (const BoxInfo& b : c.hboxes) min_nc = std::min(min_nc, b.nc);
+            auto one = [&](auto kernel) {
+                kernel<<<blocks(c.N, kGivenBlock), kGivenBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
+                                                               c.status, kept);
+            };
+            min_nc >= kInsideMin ? one(k_lists_one<true>) : one(k_lists_one<false>);
+            return cudaGetLastError();
+        }
+    }
+    k_lists<T><<<blocks(c.N, kDensBlock / kLanes), kDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr,
+                                                                              c.ncount, c.status, kept);
     return cudaGetLastError();
 }
-
-template <typename T>
-cudaError_t run_build_lists(Ctx& c) {
-    c.launches += 1;
-    k_lists<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
-                                                        c.nbr, c.ncount, c.status, 0);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t run_lists_over(Ctx& c, int kept) {
-    c.launches += 1;
-    k_lists<T><<<blocks(c.N, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), grid_of(c), kparams(c),
-                                                        c.nbr, c.ncount, c.status, kept);
-    return cudaGetLastError();
-}
-
 
 template <typename T>
 cudaError_t run_scan_stats(Ctx& c, long long* out_dev) {
@@ -896,9 +896,7 @@ template cudaError_t run_scan_stats<double>(Ctx&, long long*);
 
 #define GZ_INST(T)                                                            \
     template cudaError_t run_density<T>(Ctx&, const int*, const int*, int);   \
-    template cudaError_t run_density_given<T>(Ctx&);                          \
-    template cudaError_t run_build_lists<T>(Ctx&);                            \
-    template cudaError_t run_lists_over<T>(Ctx&, int);
+    template cudaError_t run_build_lists<T>(Ctx&, int);
 GZ_INST(float)
 GZ_INST(double)
 #undef GZ_INST

@@ -651,8 +651,9 @@ __device__ __forceinline__ void sort_list(unsigned* __restrict__ L, int n, int N
 // hits, where every lane is busy).  Returns the number of hits (the same for
 // every lane); stops early once there are more than `most`.
 // FP64: the mask comes from FP32 distances with a margin, so the FP64 pipe
-// sees only the hits; candidates up to 5e-7 outside R are handed over too.
-template <typename T, int G, typename E>
+// sees only the hits; candidates up to 5e-7 outside R are handed over
+// too, unless kExact asks for the FP64 test of each.
+template <typename T, int G, bool kExact = false, typename E>
 __device__ __forceinline__ int group_scan(const Grid& g, const BoxInfo& bx, const P4<T>* __restrict__ pos,
                                           int self, T xi, T yi, T zi, T R, int gl, unsigned gm, int most,
                                           E&& emit) {
@@ -681,10 +682,14 @@ __device__ __forceinline__ int group_scan(const Grid& g, const BoxInfo& bx, cons
                 bzz = cz >= w.nc ? zim1 : zi;
             }
         }
-        auto near = [&](const P4<T>& q) {
-            if constexpr (sizeof(T) == 8) return r2_chop(q.x, q.y, q.z, xf, yf, zf) < R2f;
-            if (w.percell) return sep2((q.x + ax) - bxx, (q.y + ay) - byy, (q.z + az) - bzz) < R2;
+        auto within = [&](const P4<T>& q) {
             return sep2(mi_diff(q.x, xi, xim1), mi_diff(q.y, yi, yim1), mi_diff(q.z, zi, zim1)) < R2;
+        };
+        auto near = [&](const P4<T>& q) {
+            if constexpr (sizeof(T) == 8)
+                return r2_chop(q.x, q.y, q.z, xf, yf, zf) < R2f && (!kExact || within(q));
+            if (w.percell) return sep2((q.x + ax) - bxx, (q.y + ay) - byy, (q.z + az) - bzz) < R2;
+            return within(q);
         };
         unsigned m = 0;  // hits among the cell's first 32 candidates
         const int end = min(se.y, se.x + 32), last = se.y - 1;
@@ -701,7 +706,7 @@ __device__ __forceinline__ int group_scan(const Grid& g, const BoxInfo& bx, cons
             }
         };
         if constexpr (sizeof(T) == 8)
-            test4(near);
+            test4([&](const P4<T>& q) { return r2_chop(q.x, q.y, q.z, xf, yf, zf) < R2f; });
         else if (w.percell)
             test4([&](const P4<T>& q) { return sep2((q.x + ax) - bxx, (q.y + ay) - byy, (q.z + az) - bzz) < R2; });
         else
@@ -709,6 +714,9 @@ __device__ __forceinline__ int group_scan(const Grid& g, const BoxInfo& bx, cons
         const int nj = se.y - se.x;
         if (nj < 32) m &= (1u << nj) - 1u;  // (the last group of four repeats the last candidate)
         if (self >= se.x && self < end) m &= ~(1u << (self - se.x));
+        if constexpr (sizeof(T) == 8 && kExact)
+            for (unsigned b = m; b; b &= b - 1)
+                if (!within(pos[se.x + __ffs(b) - 1])) m &= ~(b & (0u - b));
         int more = 0;  // hits past the cell's first 32 candidates
         for (int j = se.x + 32; j < se.y; ++j)
             if (j != self && near(pos[j])) ++more;

@@ -43,14 +43,10 @@ constexpr int kFluxSplit = 30000;
 // those particles only.
 template <typename T>
 cudaError_t run_density(Ctx& c, const int* list = nullptr, const int* nlist = nullptr, int n = 0);
+// The lists of the H at hand.  kept > 0: only those of the particles with more
+// than `kept` neighbours (the others' lists and counts restored from a checkpoint).
 template <typename T>
-cudaError_t run_density_given(Ctx& c);
-template <typename T>
-cudaError_t run_build_lists(Ctx& c);
-// Rebuilds the lists of the particles with more than `kept` neighbours (the
-// others' lists and counts restored from a checkpoint).
-template <typename T>
-cudaError_t run_lists_over(Ctx& c, int kept);
+cudaError_t run_build_lists(Ctx& c, int kept);
 template <typename T>
 cudaError_t run_reverse(Ctx& c);
 template <typename T>

@@ -102,3 +102,27 @@ def test_windows_inside_the_box_give_the_same_bits(make):
     mixed = _run(m, [q.N, tiny.N], both, 1)
     for a, b in zip(alone, mixed):
         assert np.array_equal(a, b[..., :q.N])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("name,make,copies", [(n, mk, 1) for n, mk in CASES] + [
+    ("lattice 12, many", CASES[0][1], 30), ("clump, many", CASES[5][1], 12), ("wide start, many", CASES[3][1], 18),
+    ("large box", lambda: _random(38, 12, clump=0.05), 1), ("large lattice", lambda: I.turbulence(49, seed=9), 1)])
+def test_lists_of_a_given_support_are_the_density_pass_s(name, make, copies, prec):
+    # the lists of the frozen-input calls (four lanes, one thread, inner
+    # windows of a large box) against those the density pass left, in order
+    import torch
+    import paper_1712_01294_gb300 as m
+    q = cast_state(make(), prec)
+    ctx = m.Context([q.N] * copies, m.default_params(precision=prec))
+    d = {k: v.repeat(copies).contiguous() for k, v in device(q, prec).items()}
+    d["id"] = torch.arange(d["id"].numel(), device="cuda")
+    n, _ = ctx.density(d)
+    ref = [t.cpu().numpy() for t in ctx.neighbours(96)]
+    ctx.gradients(d, n)
+    got = [t.cpu().numpy() for t in ctx.neighbours(96)]
+    ctx.status(reset=True)
+    ctx.close()
+    for a, b in zip(ref, got):
+        assert np.array_equal(a, b), name
