@@ -34,14 +34,14 @@ constexpr int kWideLanes = 16;  // ... and in FP32 launches too small for those
 // four, and from there on one thread each (k_density_one), which fills the
 // chip with fewer instructions a particle.  Measured, us a launch on the first
 // steps (late in the run): Sod 16^3 sixteen lanes 24 (27), eight 28 (35), four
-// 40 (53); Sod 32^3 sixteen 69 (81), eight 58 (68), four 50 (67), one 51 (93);
-// KH 41^3 four 105 (99), one 76 (77); Sedov 64^3 one 121 (532); 128^3 one 984
-// (1397).  FP64 keeps four: its sums are the lanes' sums.
+// 40 (53); Sod 32^3 sixteen 69 (81), eight 58 (68), four 50 (67), one 42 (81);
+// KH 41^3 four 105 (99), one 66 (69); Sedov 64^3 one 102 (506); 128^3 one 803
+// (1175).  FP64 keeps four: its sums are the lanes' sums.
 constexpr int kWideMax = 12000;
 constexpr int kThreadMin = 45000;
 // Cells per axis from which k_density_one looks for warps whose windows lie
-// inside the box (dens_fill_inside): most warps of a large box (128^3: 984 us
-// without, 944 with), few of an ensemble's small ones (784 without, 799 with).
+// inside the box (scan_inside): most warps of a large box (128^3: 865 us
+// without, 803 with), few of an ensemble's small ones (703 without, 705 with).
 constexpr int kInsideMin = 24;
 
 // Radius of the candidate cache for a support Ht: 5% headroom so that small
@@ -338,14 +338,11 @@ __device__ __noinline__ int dens_fill(const Grid& g, const BoxInfo& bx, const P4
                                       unsigned (*c_j)[kOneBlock], int t) {
     const float R2 = R * R;
     int n = 0;
-    for_candidates<float>(g, bx, pos, i, xi, yi, zi, R, [&](int j, float, float, float, float r2) {
-        if (r2 < R2) {
-            if (n < kCache) {
-                c_r2[n][t] = r2;
-                c_j[n][t] = (unsigned)j;
-            }
-            ++n;
-        }
+    for_candidates<float>(g, bx, pos, i, xi, yi, zi, R, [&](int j, float r2, bool ok) {
+        const int k = min(n, kCache);
+        c_r2[k][t] = r2;
+        c_j[k][t] = (unsigned)j;
+        n += ok && r2 < R2;
     });
     return n;
 }
@@ -388,14 +385,9 @@ __device__ __forceinline__ void scan_inside(const int2* __restrict__ cells, int 
                         for (int u = 0; u < 4; ++u) q[u] = pos[j0 + u];
 #pragma unroll
                         for (int u = 0; u < 4; ++u) r2[u] = sep2(q[u].x - xi, q[u].y - yi, q[u].z - zi);
-                        if ((unsigned)(self - j0) < 4u) {
-#pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                if (j0 + u == self) r2[u] = 1e30f;
-                        }
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            if (r2[u] < R2 && j0 + u < se.y) hit(j0 + u, r2[u]);
+                            hit(j0 + u, r2[u], r2[u] < R2 && j0 + u < se.y && j0 + u != self);
                         }
                     }
                 }
@@ -419,14 +411,22 @@ __device__ __forceinline__ bool warp_inside(const BoxInfo& bx, const P4<float>& 
     return __all_sync(__activemask(), in);
 }
 
+// The loops have no branch a candidate, an entry or a neighbour: a candidate
+// is written at the cache's end and overwritten by the next unless it counts,
+// and the sums advance by selection.  Some lane of a warp takes nearly every
+// such branch, so it saved nothing and cost its reconvergence: 128^3 919 us
+// with the branches, 871 without those of the scan, 855 of the list, 820 of
+// the sums, 803 with the last group's unused entries filled up.  Neither
+// fewer steps (two neighbouring cells as one range: 853) nor the next
+// candidates loaded ahead (925 against 919) gave anything.
 template <int kCache, bool kInside>
 __global__ void __launch_bounds__(kOneBlock, 10)
     k_density_one(int N, Sorted<float> s, Grid g, KParams p, unsigned* __restrict__ nbr,
                   int* __restrict__ ncount, int* __restrict__ iters, DevStatus* st,
                   const int* __restrict__ list, const int* __restrict__ nlist, int* __restrict__ defer,
                   int* __restrict__ ndefer) {
-    __shared__ float c_r2[kCache][kOneBlock];
-    __shared__ unsigned c_j[kCache][kOneBlock];
+    __shared__ float c_r2[kCache + 1][kOneBlock];
+    __shared__ unsigned c_j[kCache + 1][kOneBlock];
     const int t = threadIdx.x;
     int i = blockIdx.x * kOneBlock + t;
     if (list) {  // the particles of an index list only (hierarchical steps)
@@ -449,12 +449,11 @@ __global__ void __launch_bounds__(kOneBlock, 10)
     bool in = false;
     if constexpr (kInside) in = warp_inside(bx, me, Rc, lo, hi);
     if (in) {
-        scan_inside(g.cells + bx.cell_off, bx.nc, lo, hi, s.pos, i, me.x, me.y, me.z, Rc, [&](int j, float r2) {
-            if (ncache < kCache) {
-                c_r2[ncache][t] = r2;
-                c_j[ncache][t] = (unsigned)j;
-            }
-            ++ncache;
+        scan_inside(g.cells + bx.cell_off, bx.nc, lo, hi, s.pos, i, me.x, me.y, me.z, Rc, [&](int j, float r2, bool h) {
+            const int k = min(ncache, kCache);
+            c_r2[k][t] = r2;
+            c_j[k][t] = (unsigned)j;
+            ncache += h;
         });
     } else if (wide(Rc, bx.nc)) {
         ncache = kCache + 1;
@@ -462,14 +461,11 @@ __global__ void __launch_bounds__(kOneBlock, 10)
         ncache = dens_fill<kCache>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, c_r2, c_j, t);
     } else {
         const float R2 = Rc * Rc;
-        for_candidates<float>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, [&](int j, float, float, float, float r2) {
-            if (r2 < R2) {
-                if (ncache < kCache) {
-                    c_r2[ncache][t] = r2;
-                    c_j[ncache][t] = (unsigned)j;
-                }
-                ++ncache;
-            }
+        for_candidates<float>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, [&](int j, float r2, bool ok) {
+            const int k = min(ncache, kCache);
+            c_r2[k][t] = r2;
+            c_j[k][t] = (unsigned)j;
+            ncache += ok && r2 < R2;
         });
     }
     float Hev = H, Sv = 0.f, sdv = 0.f;
@@ -488,19 +484,24 @@ __global__ void __launch_bounds__(kOneBlock, 10)
         const float H2 = H * H, iH = 1.f / H;
         Acc<float> sw;
         sdv = 0.f;
+#pragma unroll
+        for (int u = 0; u < 3; ++u) c_r2[min(ncache + u, kCache)][t] = 1e30f;  // (fills up the last four)
         for (int k0 = 0; k0 < ncache; k0 += 4) {  // four entries' terms at a time, added in order
             float r2[4], w[4], x[4], y[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                r2[u] = k0 + u < ncache ? c_r2[k0 + u][t] : 1e30f;
+                r2[u] = c_r2[k0 + u][t];
                 dens_terms2(dist(r2[u]) * iH, w[u], x[u], y[u]);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (r2[u] < H2) {
-                    sw.add(w[u]);
-                    sdv = fmaf(y[u], x[u], sdv);
-                }
+                const bool h = r2[u] < H2;
+                Acc<float> a = sw;
+                a.add(w[u]);
+                const float d = fmaf(y[u], x[u], sdv);
+                sw.s = h ? a.s : sw.s;
+                sw.c = h ? a.c : sw.c;
+                sdv = h ? d : sdv;
             }
         }
         Sv = sw.fvalue();
@@ -514,13 +515,11 @@ __global__ void __launch_bounds__(kOneBlock, 10)
     const float H2 = Hev * Hev;
     int cnt = 0;
     // list of the returned H, in scan order, gathered at the cache's front and
-    // written four slots at a time (512 contiguous bytes a warp; slot by slot:
-    // 949 us for the pass at 128^3 instead of 919)
+    // written four slots at a time (512 contiguous bytes a warp; slot by slot
+    // the pass took 30 us more at 128^3)
     for (int k = 0; k < ncache; ++k) {
-        if (c_r2[k][t] < H2) {
-            c_j[cnt][t] = c_j[k][t];
-            ++cnt;
-        }
+        c_j[cnt][t] = c_j[k][t];  // (overwritten unless it counts)
+        cnt += c_r2[k][t] < H2;
     }
     for (int k = 0; k < min(cnt, p.cap); k += 4)
         *reinterpret_cast<uint4*>(nbr + lslot(k, i, N)) =
@@ -727,7 +726,8 @@ __global__ void __launch_bounds__(kGivenBlock, 8)
     int c = 0;
     const int t = threadIdx.x;
     __shared__ unsigned c_j[kStage][kGivenBlock];
-    auto hit = [&](int j, float) {
+    auto hit = [&](int j, float, bool h) {
+        if (!h) return;
         if (c < kStage)
             c_j[c][t] = (unsigned)j;
         else if (c < p.cap)
@@ -740,8 +740,8 @@ __global__ void __launch_bounds__(kGivenBlock, 8)
     if (in)
         scan_inside(g.cells + bx.cell_off, bx.nc, lo, hi, s.pos, i, me.x, me.y, me.z, H, hit);
     else
-        for_candidates<float>(g, bx, s.pos, i, me.x, me.y, me.z, H, [&](int j, float, float, float, float r2) {
-            if (r2 < H2) hit(j, r2);
+        for_candidates<float>(g, bx, s.pos, i, me.x, me.y, me.z, H, [&](int j, float r2, bool ok) {
+            hit(j, r2, ok && r2 < H2);
         });
     const int most = min(min(c, kStage), p.cap);
     for (int k = 0; k < most; k += 4)
@@ -784,10 +784,10 @@ __global__ void __launch_bounds__(128)
         const T Ht = s.h[i];
         const T R = dens_cache_radius<T>(Ht, p);
         const T R2 = R * R, H2 = Ht * Ht;
-        for_candidates<T>(g, bx, s.pos, i, me.x, me.y, me.z, R, [&](int, T, T, T, T r2) {
-            if (r2 < T(1e29)) ++v[0];  // (slots past a cell's range read a far point)
-            if (r2 < R2) ++v[1];
-            if (r2 < H2) ++v[2];
+        for_candidates<T>(g, bx, s.pos, i, me.x, me.y, me.z, R, [&](int, T r2, bool ok) {
+            v[0] += ok;
+            v[1] += ok && r2 < R2;
+            v[2] += ok && r2 < H2;
         });
     }
 #pragma unroll

@@ -298,25 +298,22 @@ __device__ __forceinline__ unsigned long long dbits(double v) {
     return (unsigned long long)__double_as_longlong(v);
 }
 
-// Loop over all candidates j != self in the cells that overlap the cube
-// [x - R, x + R] of particle self's box, calling fn(j, dx, dy, dz, r2).
+// Loop over all candidates in the cells that overlap the cube [x - R, x + R]
+// of particle self's box, calling fn(j, r2, ok): ok is false for the particle
+// itself and for the slots of a cell's last group of four that lie past its
+// range (j and r2 then mean nothing).  The callers act on ok and r2 by
+// selection: a branch a candidate, which some lane of the warp nearly always
+// takes, costs more than the two stores it would save.
 // FP32 with a range well inside half the box: the periodic shift is chosen
 // per cell row instead of per candidate, d = (x_j + a) - b with
 // (a, b) = (0, x_i), (-1, x_i) for cells wrapped below 0 (x_j - 1 is exact
 // there) or (0, x_i - 1) for cells wrapped above 1 (x_i - 1 is exact): the
 // same correctly rounded offsets mi_diff gives, at a third of the cost.
-// On that path fn is also called for the slots of the last group of four
-// that lie past a cell's range, with r2 = +inf (j then names no candidate):
-// every fn tests r2 against a finite radius before it uses j, so those calls
-// do nothing, and the loop needs no per-candidate bounds test.  Candidates
-// arrive in ascending j within each cell, as on the other path.
-struct AllCells {
-    __device__ __forceinline__ bool operator()(int) const { return true; }
-};
-template <typename T, typename F, typename CellOk = AllCells>
+// Candidates arrive in ascending j within each cell.
+template <typename T, typename F>
 __device__ __forceinline__ void for_candidates(const Grid& g, const BoxInfo& bx,
                                                const P4<T>* __restrict__ pos, int self, T xi, T yi,
-                                               T zi, T R, F&& fn, CellOk cell_ok = CellOk()) {
+                                               T zi, T R, F&& fn) {
     const int nc = bx.nc;
     const int2* __restrict__ cells = g.cells + bx.cell_off;
     // positions outside [0, 1] (flagged by the binning pass) see no candidates
@@ -361,51 +358,26 @@ __device__ __forceinline__ void for_candidates(const Grid& g, const BoxInfo& bx,
                 const T ax = cx < 0 ? T(-1) : T(0), bxx = cx >= nc ? xim1 : xi;
                 const T gx = wraps_all ? T(0) : max(max((T)cx * cl - xi, xi - (T)(cx + 1) * cl), T(0));
                 if (gzy2 + gx * gx > R2m) continue;
-                if (!cell_ok(row + wx)) continue;  // (cell index within the box)
                 const int2 se = cells[row + wx];
-                if (percell) {
-                    // four candidates' positions in flight at a time, their
-                    // offsets formed before any is used (independent chains);
-                    // slots past the range read a far-away point (r2 = +inf)
-                    for (int j0 = se.x; j0 < se.y; j0 += 4) {
-                        P4<T> q[4];
-                        T dxs[4], dys[4], dzs[4], r2s[4];
+                // four candidates at a time, their distances formed together
+                // (pos is readable up to three records past its last), and
+                // handed over without a branch
+                for (int j0 = se.x; j0 < se.y; j0 += 4) {
+                    P4<T> q[4];
+                    T r2s[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) q[u] = pos[j0 + u];
+                    if (percell) {
 #pragma unroll
                         for (int u = 0; u < 4; ++u)
-                            q[u] = j0 + u < se.y ? pos[j0 + u] : P4<T>{T(1e30), T(1e30), T(1e30), T(0)};
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            dxs[u] = (q[u].x + ax) - bxx;
-                            dys[u] = (q[u].y + ay) - by;
-                            dzs[u] = (q[u].z + az) - bz;
-                            r2s[u] = sep2(dxs[u], dys[u], dzs[u]);
-                        }
+                            r2s[u] = sep2((q[u].x + ax) - bxx, (q[u].y + ay) - by, (q[u].z + az) - bz);
+                    } else {
 #pragma unroll
                         for (int u = 0; u < 4; ++u)
-                            if (j0 + u != self) fn(j0 + u, dxs[u], dys[u], dzs[u], r2s[u]);
+                            r2s[u] = sep2(mi_diff(q[u].x, xi, xim1), mi_diff(q[u].y, yi, yim1), mi_diff(q[u].z, zi, zim1));
                     }
-                } else {
-                    for (int j0 = se.x; j0 < se.y; j0 += 4) {
-                        P4<T> q[4];
-                        T dxs[4], dys[4], dzs[4], r2s[4];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (j0 + u < se.y) q[u] = pos[j0 + u];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            dxs[u] = mi_diff(q[u].x, xi, xim1);
-                            dys[u] = mi_diff(q[u].y, yi, yim1);
-                            dzs[u] = mi_diff(q[u].z, zi, zim1);
-                            r2s[u] = sep2(dxs[u], dys[u], dzs[u]);
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int j = j0 + u;
-                            if (j >= se.y) break;
-                            if (j == self) continue;
-                            fn(j, dxs[u], dys[u], dzs[u], r2s[u]);
-                        }
-                    }
+                    for (int u = 0; u < 4; ++u) fn(j0 + u, r2s[u], j0 + u < se.y && j0 + u != self);
                 }
             }
         }
