@@ -168,18 +168,19 @@ __global__ void k_prim(int N, Sorted<T> s, KParams p, DevStatus* st, int* __rest
 // together.  The pass waits on them half the time and issues the other half;
 // instructions a neighbour (one boundary test for four offsets, the kernel
 // without its two pieces, the pair weight's constant applied after the loop,
-// min/max as such) took it from 624 to 488 us at 128^3, FP64 at 48^3 894 to
+// min/max as such) took it from 624 to 494 us at 128^3, FP64 at 48^3 894 to
 // 627.  Held to 128 registers (4 blocks per SM); at 5 blocks it spills (570 us),
 // and with the next group's records loaded ahead (162 registers) it took 598.
 // kInfo: also track which particles the limiter's bounds came from and write
 // what the adjoint reads (ginfo, lim); without it (a plain forward step) that
 // bookkeeping takes no registers or instructions.
-template <typename T, bool kInfo>
+// kDt: also the signal-speed step.
+template <typename T, bool kInfo, bool kDt>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
     k_gradients(int N, Sorted<T> s, const unsigned* __restrict__ nbr, const int* __restrict__ ncount,
                 const unsigned* __restrict__ rnbr, const int* __restrict__ rcount, KParams p,
                 T* __restrict__ rec, double* __restrict__ dti, unsigned long long* __restrict__ dtmin,
-                DevStatus* st, int want_dt, T* __restrict__ ginfo, int* __restrict__ lim,
+                DevStatus* st, T* __restrict__ ginfo, int* __restrict__ lim,
                 const int* __restrict__ list, const int* __restrict__ nlist,
                 const unsigned char* __restrict__ owned) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -204,6 +205,11 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
         const T ci = pm2.y;
         const T iH = T(1) / Hi;
         const T norm = T(8.0 / kPi) * iH * iH * iH / ni;
+        // FP32 steps: the spare slots of a list's last group run through with no
+        // weight instead of a branch a slot, 494 -> 473 us at 128^3 (late in
+        // the run 549 -> 519); gradients alone (90 us at 75^3) and
+        // FP64, bound by its arithmetic (48^3 625 against 645), skip them
+        constexpr bool kFlat = sizeof(T) == 4 && kDt && !kInfo;
         T E[6] = {0, 0, 0, 0, 0, 0};
         T Sg[15];
         T fmax[5], fmin[5];
@@ -227,18 +233,17 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
             P2<T> w2[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                q[u] = me;
-                if (k0 + u < cnt) {
-                    q[u] = s.pos[js[u]];
-                    w[u] = s.prim[js[u]];
-                    w2[u] = s.prim2[js[u]];
-                }
+                // (a spare slot reads the particle itself: no weight, no extreme)
+                const unsigned j = k0 + u < cnt ? js[u] : (unsigned)i;
+                q[u] = s.pos[j];
+                w[u] = s.prim[j];
+                w2[u] = s.prim2[j];
             }
             T dx4[4], dy4[4], dz4[4];
             offsets4(q, xi, yi, zi, xim1, yim1, zim1, dx4, dy4, dz4);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (k0 + u >= cnt) break;
+                if (!kFlat && k0 + u >= cnt) break;
                 const T dx = dx4[u], dy = dy4[u], dz = dz4[u];
                 const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
                 const T ir = rsq_(r2);
@@ -273,14 +278,14 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
                         fmin[f] = min_(fmin[f], Wj[f]);
                     }
                 }
-                if (want_dt) {
+                if constexpr (kDt) {
                     const T vd = dot3(df[1], df[2], df[3], dx, dy, dz);
                     const T vs = ci + w2[u].y - min_(vd * ir, T(0));
-                    vmax = any ? max_(vmax, vs) : vs;
-                    any = true;
+                    vmax = k0 + u == 0 ? vs : (k0 + u < cnt ? max_(vmax, vs) : vmax);
                 }
             }
         }
+        any = cnt > 0;
 #pragma unroll
         for (int q = 0; q < 6; ++q) E[q] *= T(2) * norm;
 #pragma unroll
@@ -354,8 +359,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
             P4<T> q[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                q[u] = me;  // (a spare slot: D = 0, no constraint)
-                if (k0 + u < cnt) q[u] = s.pos[js[u]];
+                q[u] = s.pos[k0 + u < cnt ? js[u] : (unsigned)i];  // (a spare slot: D = 0, no constraint)
             }
             T dx4[4], dy4[4], dz4[4];
             offsets4(q, xi, yi, zi, xim1, yim1, zim1, dx4, dy4, dz4);
@@ -411,20 +415,32 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
             }
             al[f] = a;
         }
-        if (want_dt) {
+        if constexpr (kDt) {
             const int rc = min(rcount[i], p.rcap);
             const unsigned* RL = rnbr + 4 * (size_t)i;
-            for (int k = 0; k < rc; ++k) {
-                const int j = (int)RL[lcol(k, N)];
-                const P4<T> q = s.pos[j];
-                const P4<T> w = s.prim[j];
-                const T dx = mi_diff(q.x, xi, xim1), dy = mi_diff(q.y, yi, yim1),
-                        dz = mi_diff(q.z, zi, zim1);
-                const T ir = rsq_(max_(sep2(dx, dy, dz), Tiny<T>::sq));
-                const T vd = dot3(w.y - Wi[1], w.z - Wi[2], w.w - Wi[3], dx, dy, dz);
-                const T vs = ci + s.prim2[j].y - min_(vd * ir, T(0));
-                vmax = any ? max_(vmax, vs) : vs;
-                any = true;
+            for (int k0 = 0; k0 < rc; k0 += 4) {
+                const uint4 rr = col4(RL, k0, N);
+                const unsigned js[4] = {rr.x, rr.y, rr.z, rr.w};
+                P4<T> q[4], w[4];
+                P2<T> w2[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const unsigned j = k0 + u < rc ? js[u] : js[0];
+                    q[u] = s.pos[j];
+                    w[u] = s.prim[j];
+                    w2[u] = s.prim2[j];
+                }
+                T dx4[4], dy4[4], dz4[4];
+                offsets4(q, xi, yi, zi, xim1, yim1, zim1, dx4, dy4, dz4);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {  // (a spare slot repeats the first)
+                    if (!kFlat && k0 + u >= rc) break;
+                    const T ir = rsq_(max_(sep2(dx4[u], dy4[u], dz4[u]), Tiny<T>::sq));
+                    const T vd = dot3(w[u].y - Wi[1], w[u].z - Wi[2], w[u].w - Wi[3], dx4[u], dy4[u], dz4[u]);
+                    const T vs = ci + w2[u].y - min_(vd * ir, T(0));
+                    vmax = any ? max_(vmax, vs) : vs;
+                    any = true;
+                }
             }
             if (std::is_same<T, float>::value)  // FP32 path: no FP64 cbrt / division per particle
                 dt_i = (any && vmax > T(0)) ? (double)(2.f * cbrtf(1.f / (float)ni) / (float)vmax) : INFINITY;
@@ -472,7 +488,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
         for (int q = 0; q < 6; ++q) R[26 + q] = B[q];
         store_rec(rec, i, R);
     }
-    if (want_dt) {
+    if constexpr (kDt) {
         // warp-level minimum per box, one atomic per warp when the warp is in one box;
         // in a subdomain only its owned particles take part
         const unsigned full = 0xffffffffu;
@@ -829,14 +845,16 @@ cudaError_t run_gradients(Ctx& c, bool want_dt, bool with_info, const int* list,
     c.launches += 1;
     if (!list) n = c.N;
     if (n < 1) return cudaGetLastError();
+    auto go = [&](auto kernel) {
+        kernel<<<blocks(n, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), c.nbr, c.ncount, c.rnbr, c.rcount,
+                                                     kparams(c), (T*)c.rec, c.dti, (unsigned long long*)c.dt_box,
+                                                     c.status, with_info ? (T*)c.ginfo : nullptr,
+                                                     with_info ? c.lim : nullptr, list, nlist, c.owned);
+    };
     if (with_info)
-        k_gradients<T, true><<<blocks(n, 128), 128, 0, c.stream>>>(
-            c.N, sorted_view<T>(c), c.nbr, c.ncount, c.rnbr, c.rcount, kparams(c), (T*)c.rec, c.dti,
-            (unsigned long long*)c.dt_box, c.status, want_dt ? 1 : 0, (T*)c.ginfo, c.lim, list, nlist, c.owned);
+        want_dt ? go(k_gradients<T, true, true>) : go(k_gradients<T, true, false>);
     else
-        k_gradients<T, false><<<blocks(n, 128), 128, 0, c.stream>>>(
-            c.N, sorted_view<T>(c), c.nbr, c.ncount, c.rnbr, c.rcount, kparams(c), (T*)c.rec, c.dti,
-            (unsigned long long*)c.dt_box, c.status, want_dt ? 1 : 0, nullptr, nullptr, list, nlist, c.owned);
+        want_dt ? go(k_gradients<T, false, true>) : go(k_gradients<T, false, false>);
     return cudaGetLastError();
 }
 
