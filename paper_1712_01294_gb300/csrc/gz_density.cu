@@ -218,10 +218,12 @@ __device__ __forceinline__ bool h_step(HIter<double>& b, double& H, double S, do
 // Whether a support spans so many cells that scanning its window is left to a
 // warp from the start (a blast's emptied centre: up to thousands of mostly
 // empty cells, which one thread or a group of four would walk while the rest
-// of the block waits).
+// of the block waits).  In cells: 1.7 (2.1: ensemble late in the run 1318 us
+// instead of 1292, Sedov 64^3 370 instead of 364; 1.4: 1304 and 387); the mean
+// support is one.
 template <typename T>
 __device__ __forceinline__ bool wide(T R, int nc) {
-    return (float)R * (float)nc > 2.1f;
+    return (float)R * (float)nc > 1.7f;
 }
 
 // Starting H of particle i: its guess, or (flagged by the caller) the box's
@@ -853,7 +855,9 @@ cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
         }
     }
     if (!done) group(k_density<T, kLanes>, kLanes);
-    const int wb = std::max(1, std::min(blocks(n, kWarpDensBlock / 32), 152 * 4));
+    // as many warps as fit: each waits on its own loads (Sedov 64^3 late in the
+    // run, the whole pass: 4 blocks an SM 509 us, 8 409, 24 395)
+    const int wb = std::max(1, std::min(blocks(n, kWarpDensBlock / 32), 152 * 24));
     k_density_warp<T><<<wb, kWarpDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
                                                             c.iters, c.status, c.defer, c.ndefer);
     return cudaGetLastError();
