@@ -250,22 +250,55 @@ __device__ __forceinline__ int cell_of(T v, int nc) {
 // the list of each active i there with r >= H_i; the lists are put in index
 // order by k_h_sort.  r^2 is the bit pattern the density pass forms for the
 // pair, so these lists and N_i split the flux pairs exactly.  Cells whose
-// active particles all have H >= H_j hold no such pair and are skipped.  Sixteen
-// lanes share a particle's cells: a blast's emptied centre spans up to
-// thousands of them, and with one thread each the launch waited for those
-// (Sedov 64^3, an interval's lists of 16 substeps, late in the run: one thread
-// 9.6 ms, 4 lanes 6.2, 8 lanes 5.1, 16 lanes 4.7).
+// active particles all have H >= H_j hold no such pair and are skipped.  An
+// active j needs no scan: its N_j, which the density pass has just listed,
+// holds every such i.  Sixteen lanes share a particle's cells, or its list: a
+// blast's emptied centre spans up to thousands of cells, and with one thread
+// each the launch waited for those (Sedov 64^3, an interval's lists of 16
+// substeps, late in the run: one thread 9.6 ms, 4 lanes 6.2, 8 lanes 5.1, 16
+// lanes 4.7; active particles by their lists 2.75).
 constexpr int kScatterLanes = 16;
 template <typename T>
 __global__ void __launch_bounds__(128)
-    k_h_rscatter(int N, Sorted<T> s, Grid g, KParams p, const unsigned char* __restrict__ aflag,
+    k_h_rscatter(int N, Sorted<T> s, Grid g, KParams p, const unsigned* __restrict__ nbr,
+                 const int* __restrict__ ncount, const unsigned char* __restrict__ aflag,
                  const float* __restrict__ cellmin, const unsigned char* __restrict__ near,
                  unsigned* __restrict__ rnbr, int* __restrict__ rcount, DevStatus* st) {
     const int gl = threadIdx.x % kScatterLanes;
     const int j = (blockIdx.x * blockDim.x + threadIdx.x) / kScatterLanes;
     if (j >= N) return;
-    const BoxInfo bx = g.boxes[s.box[j]];
     const P4<T> me = s.pos[j];
+    const T xm1 = me.x - T(1), ym1 = me.y - T(1), zm1 = me.z - T(1);
+    auto append = [&](int i) {
+        const int slot = atomicAdd(&rcount[i], 1);
+        if (slot < p.rcap)
+            rnbr[lslot(slot, i, N)] = (unsigned)j;
+        else
+            set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
+    };
+    if (aflag[j]) {  // its N_j holds every such i
+        const int cnt = min(ncount[j], p.cap);
+        const unsigned* L = nbr + 4 * (size_t)j;
+        for (int k0 = 4 * gl; k0 < cnt; k0 += 4 * kScatterLanes) {
+            const uint4 jj = col4(L, k0, N);
+            const unsigned is[4] = {jj.x, jj.y, jj.z, jj.w};
+            P4<T> q[4];
+            bool in[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const unsigned i = k0 + u < cnt ? is[u] : (unsigned)j;
+                q[u] = s.pos[i];
+                in[u] = k0 + u < cnt && aflag[i];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const T r2 = sep2(mi_diff(q[u].x, me.x, xm1), mi_diff(q[u].y, me.y, ym1), mi_diff(q[u].z, me.z, zm1));
+                if (in[u] && !(r2 < q[u].w * q[u].w)) append((int)is[u]);
+            }
+        }
+        return;
+    }
+    const BoxInfo bx = g.boxes[s.box[j]];
     const T Hj = me.w;
     // a support spanning under two cells lies within two cells of its own
     // (the scan's range floor((x -+ H) nc -+ 1e-3)): without an active cell
@@ -276,7 +309,6 @@ __global__ void __launch_bounds__(128)
     }
     const T H2 = Hj * Hj;
     const float Hf = (float)Hj * (1.f + 1e-6f);  // (not below H_j)
-    const T xm1 = me.x - T(1), ym1 = me.y - T(1), zm1 = me.z - T(1);
     const float xf = chop(me.x), yf = chop(me.y), zf = chop(me.z);
     const Window<T> w(bx.nc, me.x, me.y, me.z, Hj);
     for (int f = gl; f < w.ncube; f += kScatterLanes) {
@@ -299,11 +331,7 @@ __global__ void __launch_bounds__(128)
                 const int i = i0 + u;
                 const T r2 = sep2(mi_diff(q[u].x, me.x, xm1), mi_diff(q[u].y, me.y, ym1), mi_diff(q[u].z, me.z, zm1));
                 if (i >= se.y || i == j || !act[u] || !(r2 < H2) || r2 < q[u].w * q[u].w) continue;
-                const int slot = atomicAdd(&rcount[i], 1);
-                if (slot < p.rcap)
-                    rnbr[lslot(slot, i, N)] = (unsigned)j;
-                else
-                    set_status(st, GZ_S_NBR_OVERFLOW, GZ_C_NBR_OVERFLOW, s.id[i]);
+                append(i);
             }
         }
     }
@@ -719,8 +747,9 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             cudaMemsetAsync(c.cellnear, 0, (size_t)c.total_cells, st);
             k_h_dilate<<<nblk(c.total_cells, 256), 256, 0, st>>>(c.total_cells, c.boxes, c.nboxes, c.cellmin,
                                                                   c.cellnear);
-            k_h_rscatter<T><<<nblk(N, 128 / kScatterLanes), 128, 0, st>>>(N, sv, g, kp, c.aflag, c.cellmin, c.cellnear,
-                                                                           c.rnbr, c.rcount, c.status);
+            k_h_rscatter<T><<<nblk(N, 128 / kScatterLanes), 128, 0, st>>>(N, sv, g, kp, c.nbr, c.ncount, c.aflag,
+                                                                           c.cellmin, c.cellnear, c.rnbr, c.rcount,
+                                                                           c.status);
             k_h_inlist<<<nblk(nA, 32), dim3(32, kInGroups), 0, st>>>(c.alist, c.hcount + 1, c.aflag, c.nbr, c.ncount,
                                                                      c.rnbr, c.rcount, c.cap, c.rcap, c.sid, c.N,
                                                                      c.status);
