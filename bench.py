@@ -389,7 +389,7 @@ def run_ours(a, world, rank, local):
              "gradients": (work["neighbours"], "particle-neighbour terms (+60 FLOP per particle)",
                            FLOPS_PER_GRAD_NEIGHBOUR),
              "fluxes": (pairs // 2, "unordered flux pairs", FLOPS_PER_PAIR)}
-    kern = {"density": "k_density", "gradients": "k_gradients", "fluxes": "k_fluxes"}
+    kern = {"density": "k_density_one", "gradients": "k_gradients", "fluxes": "k_fluxes"}
     kernels = []
     for name in ("density", "gradients", "fluxes"):
         ms_k = prof[name][0] / max(prof[name][1], 1)

@@ -138,9 +138,10 @@ typedef struct {
     int32_t riemann;     /* MFM face solver: GZ_RIEMANN_HLLC, _EXACT or _FALLBACK     */
                          /* (GZ_RIEMANN_HLLC); GZ_MFV takes GZ_RIEMANN_HLLC only      */
     int32_t density_cache; /* h-iteration candidate cache per particle: 40 or 48      */
-                           /* entries, or 0 (40 when every box holds >= 32^3          */
-                           /* particles, else 48); a particle with more candidates    */
-                           /* within 1.05 H is iterated by a whole warp (0)            */
+                           /* entries, or 0 (the density pass's own choice: 64 where  */
+                           /* lanes share a particle; else 40 when every box holds    */
+                           /* >= 32^3 particles, 48 otherwise); a particle with more  */
+                           /* candidates within 1.05 H is iterated by a whole warp (0) */
 } gz_params;
 
 /* Structure-of-arrays particle set; every pointer is device memory with N
@@ -323,7 +324,7 @@ gz_status gz_graph_launch(gz_ctx* ctx);
  * particle in FP32) so the backward pass skips that pass too;
  * GZ_CKPT_LISTS also keeps the sort's order and the neighbour lists
  * (their first 64 slots: about 270 bytes a particle more in FP32) so the
- * backward pass skips the radix sort and the density rescan that rebuilds
+ * backward pass skips the sort and the density rescan that rebuilds
  * them (lists longer than 64 are rebuilt by a scan).  No pair quantity is
  * ever stored: the backward pass recomputes every one.  Every level gives
  * the same backward result bit for bit. */
@@ -381,7 +382,7 @@ gz_status gz_get_status(gz_ctx* ctx, uint32_t* bits, int64_t* first_bad_id, int6
                         int32_t reset);
 
 /* Pass indices of the per-pass profile. */
-#define GZ_PASS_SORT 0      /* S1 binning, radix sort, permutation            */
+#define GZ_PASS_SORT 0      /* S1 binning, sort, permutation                  */
 #define GZ_PASS_DENSITY 1   /* S2 h-iteration and neighbour lists             */
 #define GZ_PASS_LISTS 2     /* neighbour lists for a given H                  */
 #define GZ_PASS_REVERSE 3   /* reverse flux pairs                             */

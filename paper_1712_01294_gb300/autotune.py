@@ -6,10 +6,10 @@ Two knobs decide how the density pass maps particles to lanes:
   a warp are filled; the best value depends on the particle distribution (a
   lattice-aligned grid can be twice as fast as a misaligned one);
 * the candidate cache per particle (``density_cache``, 40 or 48 entries)
-  decides which particles get one lane and which a whole warp: a particle
-  with more candidates within 1.05 H than its cache holds is iterated by a
-  warp (a blast cavity, the smallest boxes of an ensemble), and the larger
-  cache costs occupancy.
+  decides which particles get one lane (in launches too small for that, a
+  group of lanes) and which a whole warp: a particle with more candidates
+  within 1.05 H than its cache holds is iterated by a warp (a blast cavity,
+  the smallest boxes of an ensemble), and the larger cache costs occupancy.
 The tuner times full steps for each combination on a copy of the caller's
 particles (through the C ABI, CUDA-event timed) and keeps the fastest.  The
 steps timed should cover the run being tuned for: the best cache size moves
@@ -17,9 +17,9 @@ as the run evolves (in the 256-box Sod/Sedov ensemble the 40-entry cache is
 fastest over steps 2-3 and the 48-entry one over the 20 steps of the run,
 by 8 %, once the blast cavities form), so `tune(..., steps=20, warmup=0)`
 tunes a 20-step run from its initial state.  Results are cached by
-(particle counts, precision, distribution signature, steps) in a JSON file.  The other kernels' block shapes are fixed by
-design (one thread per particle, sized for occupancy at their register
-counts).
+(particle counts, precision, distribution signature, steps) in a JSON file.
+The other kernels' shapes follow from the launch's size and their register
+counts.
 """
 from __future__ import annotations
 

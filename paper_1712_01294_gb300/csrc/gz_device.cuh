@@ -32,13 +32,10 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 
-// Pair-pass division and square roots: the FP32 path uses the hardware
-// reciprocal / reciprocal square root (about 2 ulp; deterministic, so both
-// particles of a pair still compute identical values); FP64 stays IEEE.
+// Division of the gradient limiter and the adjoint: the FP32 path uses the
+// hardware reciprocal (about 2 ulp, deterministic); FP64 stays IEEE.
 __device__ __forceinline__ float pdiv(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double pdiv(double a, double b) { return a / b; }
-__device__ __forceinline__ float psqrt(float x) { return x > 0.f ? x * rsqrtf(x) : 0.f; }
-__device__ __forceinline__ double psqrt(double x) { return sqrt(x); }
 
 // Reciprocal and reciprocal square root of the flux pass, for normal positive
 // arguments.  FP32: the hardware approximations (2 ulp), without the range

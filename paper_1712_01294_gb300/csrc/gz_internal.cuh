@@ -221,33 +221,6 @@ __device__ __forceinline__ T kern_w(T q) {
     T b = T(2) * t * t * t;
     return q <= T(0.5) ? a : (q < T(1) ? b : T(0));
 }
-template <typename T>
-__device__ __forceinline__ T kern_dw(T q) {
-    T t = T(1) - q;
-    T a = q * (T(-12) + T(18) * q);
-    T b = T(-6) * t * t;
-    return q <= T(0.5) ? a : (q < T(1) ? b : T(0));
-}
-
-// The two terms of the density sum at q = r / H (Eq. O2's kernel): W(q) and
-// -q W'(q).  FP64: the pieces as above.  FP32: one cubic in x = q (q <= 1/2)
-// or x = 1 - q (beyond), whose coefficients are selected, not both pieces
-// evaluated:  W = 1 - 6x^2 + 6x^3 | 2x^3,  -q W' = 12x^2 - 18x^3 | 6x^2 - 6x^3
-// (the outer piece in 1 - q, as in kern_w, so no cancellation near q = 1).
-// Callers pass q < 1 up to rounding (entries with r^2 < H^2).
-template <typename T>
-__device__ __forceinline__ void dens_terms(T q, T& w, T& qdw) {
-    w = kern_w(q);
-    qdw = -kern_dw(q) * q;
-}
-template <>
-__device__ __forceinline__ void dens_terms<float>(float q, float& w, float& qdw) {
-    const bool in = q <= 0.5f;
-    const float x = in ? q : 1.f - q;
-    const float x2 = x * x;
-    w = fmaf(fmaf(in ? 6.f : 2.f, x, in ? -6.f : 0.f), x2, in ? 1.f : 0.f);
-    qdw = fmaf(in ? -18.f : -6.f, x, in ? 12.f : 6.f) * x2;
-}
 
 __device__ __forceinline__ bool finite_(float v) { return isfinite(v); }
 __device__ __forceinline__ bool finite_(double v) { return isfinite(v); }
