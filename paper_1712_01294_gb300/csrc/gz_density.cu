@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
     k_density(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr, int* __restrict__ ncount,
               int* __restrict__ iters, DevStatus* st, const int* __restrict__ list,
               const int* __restrict__ nlist, int* __restrict__ defer, int* __restrict__ ndefer, int ccap) {
+    after_previous();
     constexpr int P = kDensBlock / G, E = kDensCache / G;
     constexpr int S = kDensCache + G;  // (the groups of a warp start on different banks)
     __shared__ T c_r2[P][S];
@@ -427,6 +428,7 @@ __global__ void __launch_bounds__(kOneBlock, 10)
                   int* __restrict__ ncount, int* __restrict__ iters, DevStatus* st,
                   const int* __restrict__ list, const int* __restrict__ nlist, int* __restrict__ defer,
                   int* __restrict__ ndefer) {
+    after_previous();
     __shared__ float c_r2[kCache + 1][kOneBlock];
     __shared__ unsigned c_j[kCache + 1][kOneBlock];
     const int t = threadIdx.x;
@@ -625,6 +627,7 @@ __global__ void __launch_bounds__(kWarpDensBlock)
     k_density_warp(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
                    int* __restrict__ ncount, int* __restrict__ iters, DevStatus* st,
                    const int* __restrict__ defer, const int* __restrict__ ndefer) {
+    after_previous();
     constexpr unsigned full = 0xffffffffu;
     __shared__ T w_r2[kWarpDensBlock / 32][kWarpCache];
     __shared__ unsigned w_j[kWarpDensBlock / 32][kWarpCache];
@@ -718,6 +721,7 @@ template <bool kInside>
 __global__ void __launch_bounds__(kGivenBlock, 8)
     k_lists_one(int N, Sorted<float> s, Grid g, KParams p, unsigned* __restrict__ nbr, int* __restrict__ ncount,
                 DevStatus* st, int only_over) {
+    after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     if (only_over > 0 && ncount[i] <= only_over) return;
@@ -757,6 +761,7 @@ template <typename T>
 __global__ void __launch_bounds__(kDensBlock)
     k_lists(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr, int* __restrict__ ncount,
             DevStatus* st, int only_over) {
+    after_previous();
     const int gl = threadIdx.x % kLanes, i = (blockIdx.x * kDensBlock + threadIdx.x) / kLanes;
     const unsigned gm = group_mask<kLanes>();
     if (i >= N) return;
@@ -828,9 +833,9 @@ cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
     const int tcap = asked > 0 ? asked : (min_count >= 32 * 32 * 32 ? 40 : 48);
     c.launches += 2;
     auto one = [&](auto kernel) {
-        kernel<<<blocks(n, kOneBlock), kOneBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
-                                                                 c.iters, c.status, list, nlist, c.defer,
-                                                                 c.ndefer);
+        launch_next(c, kernel, blocks(n, kOneBlock), kOneBlock, c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
+                    c.iters, c.status, list, nlist, c.defer,
+                    c.ndefer);
     };
     bool done = false;
     if constexpr (std::is_same<T, float>::value) {
@@ -844,9 +849,9 @@ cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
         }
     }
     auto group = [&](auto kernel, int lanes) {
-        kernel<<<blocks(n, kDensBlock / lanes), kDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr,
-                                                                           c.ncount, c.iters, c.status, list, nlist,
-                                                                           c.defer, c.ndefer, ccap);
+        launch_next(c, kernel, blocks(n, kDensBlock / lanes), kDensBlock, c.N, sv, grid_of(c), kparams(c), c.nbr,
+                    c.ncount, c.iters, c.status, list, nlist,
+                    c.defer, c.ndefer, ccap);
     };
     if constexpr (std::is_same<T, float>::value) {
         if (!done && n < kWideMax) {
@@ -858,8 +863,8 @@ cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
     // as many warps as fit: each waits on its own loads (Sedov 64^3 late in the
     // run, the whole pass: 4 blocks an SM 509 us, 8 409, 24 395)
     const int wb = std::max(1, std::min(blocks(n, kWarpDensBlock / 32), 152 * 24));
-    k_density_warp<T><<<wb, kWarpDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
-                                                            c.iters, c.status, c.defer, c.ndefer);
+    launch_next(c, k_density_warp<T>, wb, kWarpDensBlock, c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
+                c.iters, c.status, c.defer, c.ndefer);
     return cudaGetLastError();
 }
 
@@ -873,15 +878,15 @@ cudaError_t run_build_lists(Ctx& c, int kept) {
             int min_nc = 1 << 30;
             for (const BoxInfo& b : c.hboxes) min_nc = std::min(min_nc, b.nc);
             auto one = [&](auto kernel) {
-                kernel<<<blocks(c.N, kGivenBlock), kGivenBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr, c.ncount,
-                                                               c.status, kept);
+                launch_next(c, kernel, blocks(c.N, kGivenBlock), kGivenBlock, c.N, sv, grid_of(c), kparams(c), c.nbr,
+                            c.ncount, c.status, kept);
             };
             min_nc >= kInsideMin ? one(k_lists_one<true>) : one(k_lists_one<false>);
             return cudaGetLastError();
         }
     }
-    k_lists<T><<<blocks(c.N, kDensBlock / kLanes), kDensBlock, 0, c.stream>>>(c.N, sv, grid_of(c), kparams(c), c.nbr,
-                                                                              c.ncount, c.status, kept);
+    launch_next(c, k_lists<T>, blocks(c.N, kDensBlock / kLanes), kDensBlock, c.N, sv, grid_of(c), kparams(c), c.nbr,
+                c.ncount, c.status, kept);
     return cudaGetLastError();
 }
 

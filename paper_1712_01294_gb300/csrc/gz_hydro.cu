@@ -42,6 +42,7 @@ template <typename T>
 __global__ void k_reverse(int N, Sorted<T> s, KParams p, const unsigned* __restrict__ nbr,
                           const int* __restrict__ ncount, int* __restrict__ rcount,
                           unsigned* __restrict__ rnbr, DevStatus* st) {
+    after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const P4<T> me = s.pos[i];
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(32 * kRevGroups)
     k_reverse_split(int N, Sorted<T> s, KParams p, const unsigned* __restrict__ nbr,
                     const int* __restrict__ ncount, int* __restrict__ rcount, unsigned* __restrict__ rnbr,
                     DevStatus* st) {
+    after_previous();
     const int i = blockIdx.x * 32 + threadIdx.x;
     if (i >= N) return;
     const int cnt = min(ncount[i], p.cap);
@@ -99,6 +101,7 @@ __global__ void __launch_bounds__(32 * kRevGroups)
 // smaller ones; longer ones by insertion.
 __global__ void k_sort_rev(int N, const int* __restrict__ rcount, unsigned* __restrict__ rnbr,
                            int rcap) {
+    after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const int n = min(rcount[i], rcap);
@@ -126,6 +129,7 @@ __global__ void k_sort_rev(int N, const int* __restrict__ rcount, unsigned* __re
 // the few lists of more than eight).
 __global__ void __launch_bounds__(kListBlock) k_sort_rev_lanes(int N, const int* __restrict__ rcount,
                                                                unsigned* __restrict__ rnbr, int rcap) {
+    after_previous();
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) / kListLanes;
     if (i < N) sort_list(rnbr + 4 * (size_t)i, min(rcount[i], rcap), N);
 }
@@ -136,6 +140,7 @@ __global__ void __launch_bounds__(kListBlock) k_sort_rev_lanes(int N, const int*
 template <typename T>
 __global__ void k_prim(int N, Sorted<T> s, KParams p, DevStatus* st, int* __restrict__ rcount, int nb,
                        unsigned long long* __restrict__ dtmin, int* __restrict__ box_hits) {
+    after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     for (int b = i; b < nb; b += gridDim.x * blockDim.x) {
         dtmin[b] = dbits(INFINITY);
@@ -183,6 +188,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
                 DevStatus* st, T* __restrict__ ginfo, int* __restrict__ lim,
                 const int* __restrict__ list, const int* __restrict__ nlist,
                 const unsigned char* __restrict__ owned) {
+    after_previous();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     bool active;
     if (list) {  // the particles of an index list only (hierarchical steps)
@@ -578,6 +584,7 @@ __global__ void __launch_bounds__(kFluxBlock, kLoadAhead<T, kMFV, kRiem> ? 3 : 1
              const int* __restrict__ rcount, KParams p, const double* __restrict__ dt_use,
              double* __restrict__ dpdt, double* __restrict__ dEdt, double* __restrict__ dmdt,
              DevStatus* st) {
+    after_previous();
     constexpr int nq = kMFV ? 5 : 4;
     const int it = flux_item<kSplit>();
     if (!kSplit && it >= N) return;
@@ -620,6 +627,7 @@ __global__ void k_update(int N, Sorted<T> s, const double* __restrict__ dpdt,
                          const double* __restrict__ dEdt, const double* __restrict__ dmdt,
                          const double* __restrict__ dt_use, gz_particles out,
                          int* __restrict__ box_hits, DevStatus* st, double* __restrict__ rates_out) {
+    after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const unsigned o = s.orig[i];
@@ -683,6 +691,7 @@ template <typename T>
 __global__ void k_ufloor(Sorted<T> s, const BoxInfo* __restrict__ boxes,
                          const int* __restrict__ box_hits, gz_particles out, double frac,
                          const unsigned char* __restrict__ owned, int nown) {
+    after_previous();
     typedef typename Bits<T>::U U;
     const int b = blockIdx.x;
     if (box_hits[b] == 0) return;
@@ -728,6 +737,7 @@ __global__ void k_ufloor(Sorted<T> s, const BoxInfo* __restrict__ boxes,
 
 __global__ void k_dt_final(int nb, const unsigned long long* __restrict__ dtmin, double cfl,
                            double dt_fixed, double* __restrict__ dt_use, double* __restrict__ out) {
+    after_previous();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nb) return;
     const double raw = __longlong_as_double((long long)dtmin[b]);
@@ -819,24 +829,24 @@ template <typename T>
 cudaError_t run_reverse(Ctx& c) {
     c.launches += 2;
     if (c.N < kRevSplit)
-        k_reverse_split<T><<<blocks(c.N, 32), dim3(32, kRevGroups), 0, c.stream>>>(
-            c.N, sorted_view<T>(c), kparams(c), c.nbr, c.ncount, c.rcount, c.rnbr, c.status);
+        launch_next(c, k_reverse_split<T>, blocks(c.N, 32), dim3(32, kRevGroups), c.N, sorted_view<T>(c), kparams(c),
+                    c.nbr, c.ncount, c.rcount, c.rnbr, c.status);
     else
-        k_reverse<T><<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, sorted_view<T>(c), kparams(c), c.nbr, c.ncount,
-                                                              c.rcount, c.rnbr, c.status);
+        launch_next(c, k_reverse<T>, blocks(c.N, 256), 256, c.N, sorted_view<T>(c), kparams(c), c.nbr, c.ncount,
+                    c.rcount, c.rnbr, c.status);
     if (c.N < kRevSplit)
-        k_sort_rev_lanes<<<blocks(c.N, kListBlock / kListLanes), kListBlock, 0, c.stream>>>(c.N, c.rcount, c.rnbr,
-                                                                                            c.rcap);
+        launch_next(c, k_sort_rev_lanes, blocks(c.N, kListBlock / kListLanes), kListBlock, c.N, c.rcount, c.rnbr,
+                    c.rcap);
     else
-        k_sort_rev<<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, c.rcount, c.rnbr, c.rcap);
+        launch_next(c, k_sort_rev, blocks(c.N, 256), 256, c.N, c.rcount, c.rnbr, c.rcap);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t run_prim(Ctx& c) {
     c.launches += 1;
-    k_prim<T><<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, sorted_view<T>(c), kparams(c), c.status, c.rcount,
-                                                       c.nboxes, (unsigned long long*)c.dt_box, c.box_hits);
+    launch_next(c, k_prim<T>, blocks(c.N, 256), 256, c.N, sorted_view<T>(c), kparams(c), c.status, c.rcount,
+                c.nboxes, (unsigned long long*)c.dt_box, c.box_hits);
     return cudaGetLastError();
 }
 
@@ -846,10 +856,10 @@ cudaError_t run_gradients(Ctx& c, bool want_dt, bool with_info, const int* list,
     if (!list) n = c.N;
     if (n < 1) return cudaGetLastError();
     auto go = [&](auto kernel) {
-        kernel<<<blocks(n, 128), 128, 0, c.stream>>>(c.N, sorted_view<T>(c), c.nbr, c.ncount, c.rnbr, c.rcount,
-                                                     kparams(c), (T*)c.rec, c.dti, (unsigned long long*)c.dt_box,
-                                                     c.status, with_info ? (T*)c.ginfo : nullptr,
-                                                     with_info ? c.lim : nullptr, list, nlist, c.owned);
+        launch_next(c, kernel, blocks(n, 128), 128, c.N, sorted_view<T>(c), c.nbr, c.ncount, c.rnbr, c.rcount,
+                    kparams(c), (T*)c.rec, c.dti, (unsigned long long*)c.dt_box,
+                    c.status, with_info ? (T*)c.ginfo : nullptr,
+                    with_info ? c.lim : nullptr, list, nlist, c.owned);
     };
     if (with_info)
         want_dt ? go(k_gradients<T, true, true>) : go(k_gradients<T, true, false>);
@@ -878,9 +888,9 @@ cudaError_t run_grad_out(Ctx& c, T* grad, T* B) {
 template <typename T, bool kMFV, int kRiem>
 static void launch_fluxes(Ctx& c) {
     auto go = [&](auto kernel, int items) {
-        kernel<<<blocks(c.N, items), kFluxBlock, 0, c.stream>>>(c.N, (const T*)c.rec, c.sid, c.sbox, c.nbr, c.ncount,
-                                                                c.rnbr, c.rcount, kparams(c), c.dt_use, c.dpdt,
-                                                                c.dEdt, kMFV ? c.dmdt : nullptr, c.status);
+        launch_next(c, kernel, blocks(c.N, items), kFluxBlock, c.N, (const T*)c.rec, c.sid, c.sbox, c.nbr, c.ncount,
+                    c.rnbr, c.rcount, kparams(c), c.dt_use, c.dpdt,
+                    c.dEdt, kMFV ? c.dmdt : nullptr, c.status);
     };
     if (c.N < kFluxSplit)
         go(k_fluxes<T, kMFV, kRiem, true>, 32);
@@ -906,11 +916,11 @@ template <typename T>
 cudaError_t run_update(Ctx& c, gz_particles& p, double* rates_out) {
     c.launches += 2;
     int* hits = c.box_hits;
-    k_update<T><<<blocks(c.N, 256), 256, 0, c.stream>>>(
-        c.N, sorted_view<T>(c), c.dpdt, c.dEdt, c.params.scheme == GZ_MFV ? c.dmdt : nullptr, c.dt_use, p,
-        hits, c.status, rates_out);
-    k_ufloor<T><<<c.nboxes, 1024, 0, c.stream>>>(sorted_view<T>(c), c.boxes, hits, p,
-                                                  c.params.u_floor_frac, c.owned, c.n_owned);
+    launch_next(c, k_update<T>, blocks(c.N, 256), 256, c.N, sorted_view<T>(c), c.dpdt, c.dEdt,
+                c.params.scheme == GZ_MFV ? c.dmdt : nullptr, c.dt_use, p,
+                hits, c.status, rates_out);
+    launch_next(c, k_ufloor<T>, c.nboxes, 1024, sorted_view<T>(c), c.boxes, hits, p,
+                c.params.u_floor_frac, c.owned, c.n_owned);
     return cudaGetLastError();
 }
 
@@ -918,8 +928,8 @@ cudaError_t run_update(Ctx& c, gz_particles& p, double* rates_out) {
 template <typename T>
 cudaError_t run_ufloor(Ctx& c, gz_particles& p) {
     c.launches += 1;
-    k_ufloor<T><<<c.nboxes, 1024, 0, c.stream>>>(sorted_view<T>(c), c.boxes, c.box_hits, p,
-                                                  c.params.u_floor_frac, c.owned, c.n_owned);
+    launch_next(c, k_ufloor<T>, c.nboxes, 1024, sorted_view<T>(c), c.boxes, c.box_hits, p,
+                c.params.u_floor_frac, c.owned, c.n_owned);
     return cudaGetLastError();
 }
 
@@ -943,8 +953,8 @@ cudaError_t run_rates_in(Ctx& c, const double* rates) {
 
 cudaError_t run_dt_finalize(Ctx& c, double dt_fixed, double* dt_used_dev) {
     c.launches += 1;
-    k_dt_final<<<blocks(c.nboxes, 256), 256, 0, c.stream>>>(
-        c.nboxes, (const unsigned long long*)c.dt_box, c.params.cfl, dt_fixed, c.dt_use, dt_used_dev);
+    launch_next(c, k_dt_final, blocks(c.nboxes, 256), 256, c.nboxes, (const unsigned long long*)c.dt_box, c.params.cfl,
+                dt_fixed, c.dt_use, dt_used_dev);
     return cudaGetLastError();
 }
 

@@ -116,6 +116,7 @@ __device__ __forceinline__ unsigned block_sum(unsigned v, unsigned* sh) {
 
 __global__ void __launch_bounds__(kScanThreads)
     k_cs_sums(long long K, const unsigned* __restrict__ count, unsigned* __restrict__ sums) {
+    after_previous();
     __shared__ unsigned sh[kScanThreads / 32];
     const uint4 v = count4(count, (long long)blockIdx.x * kScanTile + 4 * threadIdx.x, K);
     const unsigned t = block_sum(v.x + v.y + v.z + v.w, sh);
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(kScanThreads)
     k_cs_scan(long long K, const unsigned* __restrict__ count, const unsigned* __restrict__ sums,
               const BoxInfo* __restrict__ boxes, int nboxes, unsigned* __restrict__ start,
               int2* __restrict__ cells) {
+    after_previous();
     __shared__ unsigned sh[kScanThreads / 32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     unsigned before = 0;
@@ -185,6 +187,7 @@ __global__ void __launch_bounds__(kScanThreads)
 
 __global__ void k_cs_place(int N, const unsigned* __restrict__ key, const unsigned* __restrict__ slot,
                            const unsigned* __restrict__ start, unsigned* __restrict__ order) {
+    after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < N) order[start[key[i]] + slot[i]] = (unsigned)i;
 }
@@ -331,6 +334,7 @@ __global__ void k_permute(int N, unsigned* __restrict__ skeys, unsigned* __restr
                           const void* __restrict__ n_in, const int* __restrict__ box_of,
                           const BoxInfo* __restrict__ boxes, Sorted<T> s, int2* __restrict__ cells,
                           int* __restrict__ ndefer) {
+    after_previous();
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= N) return;
     if (q == 0) *ndefer = 0;  // (the density pass after it counts from zero)
@@ -431,12 +435,12 @@ static cudaError_t counting_sort(Ctx& c, const gz_particles& p, const void* n_in
                                                    c.boxes, c.kcount, c.keys_alt, c.vals_alt, c.status);
     const int tiles = (int)((K + kScanTile - 1) / kScanTile);
     const bool direct = tiles <= kScanDirect;
-    if (!direct) k_cs_sums<<<tiles, kScanThreads, 0, st>>>(K, c.kcount, c.hist);
-    k_cs_scan<<<tiles, kScanThreads, 0, st>>>(K, c.kcount, direct ? nullptr : c.hist, c.boxes, c.nboxes, c.kstart,
-                                              c.cells);
-    k_cs_place<<<blocks(N, 256), 256, 0, st>>>(N, c.keys_alt, c.vals_alt, c.kstart, order);
-    k_permute<T, true><<<blocks(N, 256), 256, 0, st>>>(N, c.keys, c.vals, order, c.keys_alt, c.kcount, c.kstart, p,
-                                                        n_in, c.box_of, c.boxes, sorted_view<T>(c), c.cells, c.ndefer);
+    if (!direct) launch_next(c, k_cs_sums, tiles, kScanThreads, K, c.kcount, c.hist);
+    launch_next(c, k_cs_scan, tiles, kScanThreads, K, c.kcount, direct ? nullptr : c.hist, c.boxes, c.nboxes, c.kstart,
+                c.cells);
+    launch_next(c, k_cs_place, blocks(N, 256), 256, N, c.keys_alt, c.vals_alt, c.kstart, order);
+    launch_next(c, k_permute<T, true>, blocks(N, 256), 256, N, c.keys, c.vals, order, c.keys_alt, c.kcount, c.kstart, p,
+                n_in, c.box_of, c.boxes, sorted_view<T>(c), c.cells, c.ndefer);
     c.launches += direct ? 4 : 5;
     return cudaGetLastError();
 }
