@@ -51,6 +51,7 @@ __device__ __forceinline__ T wrap_pos(T v) {
 template <typename T>
 __global__ void k_h_init(int N, gz_particles p, T* __restrict__ hva, T* __restrict__ hdvs,
                          int* __restrict__ hsa, int* __restrict__ hbin) {
+    after_previous();
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= N) return;
     hva[o] = ((const T*)p.vx)[o];
@@ -76,6 +77,7 @@ template <typename T>
 __global__ void k_h_predict(int N, int s, int K, gz_particles p, const T* __restrict__ hva,
                             const T* __restrict__ hdvs, const int* __restrict__ hsa,
                             const int* __restrict__ box_of, const double* __restrict__ D, T* __restrict__ xp) {
+    after_previous();
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o < N) {
         const int steps = s - hsa[o];
@@ -97,6 +99,7 @@ __global__ void k_h_predict(int N, int s, int K, gz_particles p, const T* __rest
 
 // Number of particles active at substep s, once the bins up to it are final.
 __global__ void k_h_count(int N, int s, int K, const int* __restrict__ hbin, int* __restrict__ count) {
+    after_previous();
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     const int c = __syncthreads_count(o < N && s % (1 << (K - hbin[o])) == 0);
     if (threadIdx.x == 0 && c) atomicAdd(count, c);
@@ -106,6 +109,7 @@ __global__ void k_h_count(int N, int s, int K, const int* __restrict__ hbin, int
 __global__ void __launch_bounds__(kCmpBlock)
     k_h_flags(int N, int s, int K, const unsigned* __restrict__ orig, const int* __restrict__ hbin,
               int* __restrict__ sbin, unsigned char* __restrict__ aflag, int* __restrict__ bcount) {
+    after_previous();
     const int i = blockIdx.x * kCmpBlock + threadIdx.x;
     bool act = false;
     if (i < N) {
@@ -126,6 +130,7 @@ __global__ void __launch_bounds__(kCmpBlock)
 constexpr int kCmpDirect = 4096;
 
 __global__ void __launch_bounds__(kCmpBlock) k_cmp_scan(int nb, int* __restrict__ bcount, int* __restrict__ total) {
+    after_previous();
     __shared__ int part[kCmpBlock];
     const int t = threadIdx.x;
     const int chunk = (nb + kCmpBlock - 1) / kCmpBlock;
@@ -153,6 +158,7 @@ __global__ void __launch_bounds__(kCmpBlock) k_cmp_scan(int nb, int* __restrict_
 __global__ void __launch_bounds__(kCmpBlock)
     k_cmp_write(int N, const unsigned char* __restrict__ flag, const int* __restrict__ boff,
                 int* __restrict__ list, int* __restrict__ total) {
+    after_previous();
     __shared__ int wsum[kCmpBlock / 32];
     int base = 0;
     if (total) {
@@ -194,6 +200,7 @@ __global__ void __launch_bounds__(kCmpBlock)
 template <typename T>
 __global__ void k_h_cellmin(int ncells, const int2* __restrict__ cells, const unsigned char* __restrict__ aflag,
                             const P4<T>* __restrict__ pos, float* __restrict__ cellmin) {
+    after_previous();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncells) return;
     const int2 se = cells[c];
@@ -212,6 +219,7 @@ __global__ void k_h_cellmin(int ncells, const int2* __restrict__ cells, const un
 // particle, marked by the active cells themselves (near must start zeroed).
 __global__ void k_h_dilate(int ncells, const BoxInfo* __restrict__ boxes, int nboxes,
                            const float* __restrict__ cellmin, unsigned char* __restrict__ near) {
+    after_previous();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncells || cellmin[c] == INFINITY) return;
     int lo = 0, hi = nboxes - 1;  // box of the cell: last box with cell_off <= c
@@ -264,6 +272,7 @@ __global__ void __launch_bounds__(128)
                  const int* __restrict__ ncount, const unsigned char* __restrict__ aflag,
                  const float* __restrict__ cellmin, const unsigned char* __restrict__ near,
                  unsigned* __restrict__ rnbr, int* __restrict__ rcount, DevStatus* st) {
+    after_previous();
     const int gl = threadIdx.x % kScatterLanes;
     const int j = (blockIdx.x * blockDim.x + threadIdx.x) / kScatterLanes;
     if (j >= N) return;
@@ -345,6 +354,7 @@ __global__ void k_h_inlist(const int* __restrict__ alist, const int* __restrict_
                            int* __restrict__ ncount, const unsigned* __restrict__ rnbr,
                            const int* __restrict__ rcount, int cap, int rcap,
                            const long long* __restrict__ sid, int N, DevStatus* st) {
+    after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= *nA) return;
     const int i = alist[t];
@@ -377,6 +387,7 @@ __global__ void __launch_bounds__(kListBlock)
     k_h_sort(int N, const unsigned char* __restrict__ aflag, int* __restrict__ ncount,
              unsigned* __restrict__ nbr, int cap, const int* __restrict__ rcount,
              unsigned* __restrict__ rnbr, int rcap) {
+    after_previous();
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) / kListLanes;
     if (i >= N) return;
     unsigned* L;
@@ -397,6 +408,7 @@ __global__ void __launch_bounds__(kListBlock)
 __global__ void __launch_bounds__(kCmpBlock)
     k_h_tflags(int N, const unsigned char* __restrict__ aflag, const int* __restrict__ ncount,
                unsigned char* __restrict__ tflag, int* __restrict__ bcount) {
+    after_previous();
     const int i = blockIdx.x * kCmpBlock + threadIdx.x;
     const bool t = i < N && (aflag[i] || ncount[i] > 0);
     if (i < N) tflag[i] = (unsigned char)t;
@@ -411,6 +423,7 @@ template <typename T>
 __global__ void k_h_persist(int N, const int* __restrict__ alist, const int* __restrict__ nA,
                             Sorted<T> s, const T* __restrict__ rec, gz_particles p, T* __restrict__ hn,
                             T* __restrict__ hgrad, T* __restrict__ hB) {
+    after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= *nA) return;
     const int i = alist[t];
@@ -431,6 +444,7 @@ __global__ void k_h_persist(int N, const int* __restrict__ alist, const int* __r
 __global__ void k_h_dtmax(const int* __restrict__ alist, const int* __restrict__ nA,
                           const int* __restrict__ box, const double* __restrict__ dti,
                           unsigned long long* __restrict__ dtmax) {
+    after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = t < *nA;
     const int i = in ? alist[t] : 0;
@@ -455,6 +469,7 @@ __global__ void k_h_dtmax(const int* __restrict__ alist, const int* __restrict__
 __global__ void k_h_interval(int nb, const unsigned long long* __restrict__ dtmin,
                              const unsigned long long* __restrict__ dtmax, double cfl, int K,
                              double* __restrict__ D) {
+    after_previous();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nb) return;
     const double lo = __longlong_as_double((long long)dtmin[b]);
@@ -474,6 +489,7 @@ __global__ void k_h_bins(const int* __restrict__ alist, const int* __restrict__ 
                          const unsigned* __restrict__ orig, const int* __restrict__ box,
                          const double* __restrict__ dti, const double* __restrict__ D, double cfl, int K,
                          int first, int* __restrict__ hbin, int* __restrict__ sbin) {
+    after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= *nA) return;
     const int i = alist[t];
@@ -513,6 +529,7 @@ __global__ void __launch_bounds__(kXBlock, kLoadAhead<T, kMFV, kRiem> ? 3 : 1)
                  const int* __restrict__ rcount, KParams p, const double* __restrict__ D,
                  double* __restrict__ dpdt, double* __restrict__ dEdt, double* __restrict__ dmdt, int N,
                  DevStatus* st) {
+    after_previous();
     constexpr int nq = kMFV ? 5 : 4;
     const int t = flux_item<kSplit>(), n = *nT;
     if (kSplit ? (int)blockIdx.x * 32 >= n : t >= n) return;
@@ -563,6 +580,7 @@ __global__ void k_h_kick(const int* __restrict__ tlist, const int* __restrict__ 
                          const double* __restrict__ dEdt, const double* __restrict__ dmdt,
                          const double* __restrict__ D, gz_particles out, T* __restrict__ hdvs,
                          int* __restrict__ box_hits, DevStatus* st) {
+    after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= *nT) return;
     const int i = tlist[t];
@@ -606,6 +624,7 @@ template <typename T>
 __global__ void k_h_finalize(int N, int s, int K, gz_particles p, T* __restrict__ hva, T* __restrict__ hdvs,
                              int* __restrict__ hsa, const int* __restrict__ hbin,
                              const int* __restrict__ box_of, const double* __restrict__ D, DevStatus* st) {
+    after_previous();
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= N) return;
     const int k = hbin[o];
@@ -637,9 +656,9 @@ void launch_exchange(Ctx& c, const KParams& kp, int N, int nA) {
     const bool split = nA < kFluxSplit;
     auto go = [&](auto one, auto four) {
         auto kernel = split ? four : one;
-        kernel<<<nblk(N, split ? 32 : kXBlock), kXBlock, 0, c.stream>>>(c.tlist, c.hcount + 2, (const T*)c.rec, c.sid, c.sbox,
-                                                           c.sbin, c.nbr, c.ncount, c.rnbr, c.rcount, kp, c.dt_use,
-                                                           c.dpdt, c.dEdt, c.dmdt, N, c.status);
+        launch_next(c, kernel, nblk(N, split ? 32 : kXBlock), kXBlock, c.tlist, c.hcount + 2, (const T*)c.rec, c.sid, c.sbox,
+                    c.sbin, c.nbr, c.ncount, c.rnbr, c.rcount, kp, c.dt_use,
+                    c.dpdt, c.dEdt, c.dmdt, N, c.status);
     };
     if (c.params.scheme == GZ_MFV)
         go(k_h_exchange<T, GZ_RIEMANN_HLLC, true, false>, k_h_exchange<T, GZ_RIEMANN_HLLC, true, true>);
@@ -701,8 +720,8 @@ static cudaError_t compact(Ctx& c, const unsigned char* flag, int* list, int* co
     const int nb = nblk(c.N, kCmpBlock);
     const bool direct = nb <= kCmpDirect;
     c.launches += direct ? 1 : 2;
-    if (!direct) k_cmp_scan<<<1, kCmpBlock, 0, c.stream>>>(nb, c.bcount, count);
-    k_cmp_write<<<nb, kCmpBlock, 0, c.stream>>>(c.N, flag, c.bcount, list, direct ? count : nullptr);
+    if (!direct) launch_next(c, k_cmp_scan, 1, kCmpBlock, nb, c.bcount, count);
+    launch_next(c, k_cmp_write, nb, kCmpBlock, c.N, flag, c.bcount, list, direct ? count : nullptr);
     return cudaGetLastError();
 }
 
@@ -723,7 +742,7 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
     pp.y = hxp + N;
     pp.z = hxp + 2 * (size_t)N;
     c.launches += 1;
-    k_h_init<T><<<nblk(N, 256), 256, 0, st>>>(N, p, (T*)c.hva, (T*)c.hdvs, c.hsa, c.hbin);
+    launch_next(c, k_h_init<T>, nblk(N, 256), 256, N, p, (T*)c.hva, (T*)c.hdvs, c.hsa, c.hbin);
     long long active = 0;
     const int S = 1 << K;
     int nA = N;  // (substep 0: every particle)
@@ -734,15 +753,15 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             nA = c.hcount_host[s & 1];
         }
         c.launches += 1;
-        k_h_predict<T><<<nblk(N, 256), 256, 0, st>>>(N, s, K, p, (const T*)c.hva, (const T*)c.hdvs, c.hsa,
-                                                      c.box_of, c.dt_use, hxp);
+        launch_next(c, k_h_predict<T>, nblk(N, 256), 256, N, s, K, p, (const T*)c.hva, (const T*)c.hdvs, c.hsa,
+                    c.box_of, c.dt_use, hxp);
         active += nA;
         if (nA > 0) {
             Sorted<T> sv = sorted_view<T>(c);
             timer.begin(GZ_PASS_SORT);
             e = sort_and_bin<T>(c, pp, c.hn);
             c.launches += 1;
-            k_h_flags<<<nblk(N, kCmpBlock), kCmpBlock, 0, st>>>(N, s, K, c.vals, c.hbin, c.sbin, c.aflag, c.bcount);
+            launch_next(c, k_h_flags, nblk(N, kCmpBlock), kCmpBlock, N, s, K, c.vals, c.hbin, c.sbin, c.aflag, c.bcount);
             if (e == cudaSuccess) e = compact(c, c.aflag, c.alist, c.hcount + 1);
             timer.end(GZ_PASS_SORT);
             cudaMemsetAsync(c.ncount, 0, sizeof(int) * (size_t)N, st);
@@ -755,20 +774,18 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             timer.begin(GZ_PASS_REVERSE);
             c.launches += 6;
             c.launches += 1;
-            k_h_cellmin<T><<<nblk(c.total_cells, 256), 256, 0, st>>>(c.total_cells, c.cells, c.aflag, sv.pos,
-                                                                      c.cellmin);
+            launch_next(c, k_h_cellmin<T>, nblk(c.total_cells, 256), 256, c.total_cells, c.cells, c.aflag, sv.pos,
+                        c.cellmin);
             cudaMemsetAsync(c.cellnear, 0, (size_t)c.total_cells, st);
-            k_h_dilate<<<nblk(c.total_cells, 256), 256, 0, st>>>(c.total_cells, c.boxes, c.nboxes, c.cellmin,
-                                                                  c.cellnear);
-            k_h_rscatter<T><<<nblk(N, 128 / kScatterLanes), 128, 0, st>>>(N, sv, g, kp, c.nbr, c.ncount, c.aflag,
-                                                                           c.cellmin, c.cellnear, c.rnbr, c.rcount,
-                                                                           c.status);
-            k_h_inlist<<<nblk(nA, 32), dim3(32, kInGroups), 0, st>>>(c.alist, c.hcount + 1, c.aflag, c.nbr, c.ncount,
-                                                                     c.rnbr, c.rcount, c.cap, c.rcap, c.sid, c.N,
-                                                                     c.status);
-            k_h_sort<<<nblk(N, kListBlock / kListLanes), kListBlock, 0, st>>>(N, c.aflag, c.ncount, c.nbr, c.cap,
-                                                                              c.rcount, c.rnbr, c.rcap);
-            k_h_tflags<<<nblk(N, kCmpBlock), kCmpBlock, 0, st>>>(N, c.aflag, c.ncount, c.tflag, c.bcount);
+            launch_next(c, k_h_dilate, nblk(c.total_cells, 256), 256, c.total_cells, c.boxes, c.nboxes, c.cellmin,
+                        c.cellnear);
+            launch_next(c, k_h_rscatter<T>, nblk(N, 128 / kScatterLanes), 128, N, sv, g, kp, c.nbr, c.ncount, c.aflag,
+                        c.cellmin, c.cellnear, c.rnbr, c.rcount, c.status);
+            launch_next(c, k_h_inlist, nblk(nA, 32), dim3(32, kInGroups), c.alist, c.hcount + 1, c.aflag, c.nbr, c.ncount,
+                        c.rnbr, c.rcount, c.cap, c.rcap, c.sid, c.N, c.status);
+            launch_next(c, k_h_sort, nblk(N, kListBlock / kListLanes), kListBlock, N, c.aflag, c.ncount, c.nbr, c.cap,
+                        c.rcount, c.rnbr, c.rcap);
+            launch_next(c, k_h_tflags, nblk(N, kCmpBlock), kCmpBlock, N, c.aflag, c.ncount, c.tflag, c.bcount);
             if (e == cudaSuccess) e = compact(c, c.tflag, c.tlist, c.hcount + 2);
             timer.end(GZ_PASS_REVERSE);
             timer.begin(GZ_PASS_GRAD);
@@ -776,22 +793,22 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             if (e == cudaSuccess)
                 e = run_pack_given<T>(c, (const T*)c.hgrad, (const T*)c.hB, c.tlist, c.hcount + 2, N, c.aflag);
             c.launches += 1;
-            k_h_persist<T><<<nblk(nA, 256), 256, 0, st>>>(N, c.alist, c.hcount + 1, sv, (const T*)c.rec, p,
-                                                           (T*)c.hn, (T*)c.hgrad, (T*)c.hB);
+            launch_next(c, k_h_persist<T>, nblk(nA, 256), 256, N, c.alist, c.hcount + 1, sv, (const T*)c.rec, p,
+                        (T*)c.hn, (T*)c.hgrad, (T*)c.hB);
             if (s == 0) {
                 if (dt_fixed > 0.0) {
                     if (e == cudaSuccess) e = run_dt_set(c, dt_fixed);
                 } else {
                     cudaMemsetAsync(c.dtmax, 0, 8 * (size_t)c.nboxes, st);
                     c.launches += 2;
-                    k_h_dtmax<<<nblk(nA, 256), 256, 0, st>>>(c.alist, c.hcount + 1, c.sbox, c.dti, c.dtmax);
-                    k_h_interval<<<nblk(c.nboxes, 256), 256, 0, st>>>(
-                        c.nboxes, (const unsigned long long*)c.dt_box, c.dtmax, c.params.cfl, K, c.dt_use);
+                    launch_next(c, k_h_dtmax, nblk(nA, 256), 256, c.alist, c.hcount + 1, c.sbox, c.dti, c.dtmax);
+                    launch_next(c, k_h_interval, nblk(c.nboxes, 256), 256, c.nboxes,
+                                (const unsigned long long*)c.dt_box, c.dtmax, c.params.cfl, K, c.dt_use);
                 }
             }
             c.launches += 1;
-            k_h_bins<<<nblk(nA, 256), 256, 0, st>>>(c.alist, c.hcount + 1, c.vals, c.sbox, c.dti, c.dt_use,
-                                                     c.params.cfl, K, s == 0 ? 1 : 0, c.hbin, c.sbin);
+            launch_next(c, k_h_bins, nblk(nA, 256), 256, c.alist, c.hcount + 1, c.vals, c.sbox, c.dti, c.dt_use,
+                        c.params.cfl, K, s == 0 ? 1 : 0, c.hbin, c.sbin);
             timer.end(GZ_PASS_GRAD);
         }
         if (s + 1 < S) {
@@ -799,7 +816,7 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             // while the exchange runs
             c.launches += 1;
             cudaMemsetAsync(c.hcount + 3, 0, sizeof(int), st);
-            k_h_count<<<nblk(N, 256), 256, 0, st>>>(N, s + 1, K, c.hbin, c.hcount + 3);
+            launch_next(c, k_h_count, nblk(N, 256), 256, N, s + 1, K, c.hbin, c.hcount + 3);
             cudaMemcpyAsync(c.hcount_host + ((s + 1) & 1), c.hcount + 3, sizeof(int), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaEventRecord(c.hier_counted, st);
         }
@@ -811,15 +828,15 @@ cudaError_t run_step_hier(Ctx& c, gz_particles& p, int K, double dt_fixed, doubl
             timer.end(GZ_PASS_FLUX);
             timer.begin(GZ_PASS_UPDATE);
             c.launches += 1;
-            k_h_kick<T><<<nblk(N, 256), 256, 0, st>>>(c.tlist, c.hcount + 2, N, sv, c.sbin, c.dpdt, c.dEdt,
-                                                       c.params.scheme == GZ_MFV ? c.dmdt : nullptr, c.dt_use,
-                                                       p, (T*)c.hdvs, c.box_hits, c.status);
+            launch_next(c, k_h_kick<T>, nblk(N, 256), 256, c.tlist, c.hcount + 2, N, sv, c.sbin, c.dpdt, c.dEdt,
+                        c.params.scheme == GZ_MFV ? c.dmdt : nullptr, c.dt_use,
+                        p, (T*)c.hdvs, c.box_hits, c.status);
             if (e == cudaSuccess) e = run_ufloor<T>(c, p);
             timer.end(GZ_PASS_UPDATE);
         }
         c.launches += 1;
-        k_h_finalize<T><<<nblk(N, 256), 256, 0, st>>>(N, s, K, p, (T*)c.hva, (T*)c.hdvs, c.hsa, c.hbin,
-                                                       c.box_of, c.dt_use, c.status);
+        launch_next(c, k_h_finalize<T>, nblk(N, 256), 256, N, s, K, p, (T*)c.hva, (T*)c.hdvs, c.hsa, c.hbin,
+                    c.box_of, c.dt_use, c.status);
         if (e == cudaSuccess) e = cudaGetLastError();
     }
     if (e == cudaSuccess && dt_used_dev)

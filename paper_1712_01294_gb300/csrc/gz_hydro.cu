@@ -523,6 +523,7 @@ template <typename T>
 __global__ void k_pack_given(int N, Sorted<T> s, const T* __restrict__ grad, const T* __restrict__ B,
                              T* __restrict__ rec, const int* __restrict__ list,
                              const int* __restrict__ nlist, const unsigned char* __restrict__ skip) {
+    after_previous();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (list) {
         if (i >= *nlist) return;
@@ -556,6 +557,7 @@ __global__ void k_pack_given(int N, Sorted<T> s, const T* __restrict__ grad, con
 template <typename T>
 __global__ void k_grad_out(int N, const unsigned* __restrict__ orig, const T* __restrict__ rec,
                            T* __restrict__ grad, T* __restrict__ B) {
+    after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const unsigned o = orig[i];
@@ -746,6 +748,7 @@ __global__ void k_dt_final(int nb, const unsigned long long* __restrict__ dtmin,
     if (out) out[b] = dt;
 }
 __global__ void k_dt_set(int nb, double dt, double* __restrict__ dt_use) {
+    after_previous();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b < nb) dt_use[b] = dt;
 }
@@ -873,15 +876,15 @@ cudaError_t run_pack_given(Ctx& c, const T* grad, const T* B, const int* list, c
                            const unsigned char* skip) {
     c.launches += 1;
     if (list && n < 1) return cudaSuccess;
-    k_pack_given<T><<<blocks(list ? n : c.N, 256), 256, 0, c.stream>>>(c.N, sorted_view<T>(c), grad, B,
-                                                                     (T*)c.rec, list, nlist, skip);
+    launch_next(c, k_pack_given<T>, blocks(list ? n : c.N, 256), 256, c.N, sorted_view<T>(c), grad, B,
+                (T*)c.rec, list, nlist, skip);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t run_grad_out(Ctx& c, T* grad, T* B) {
     c.launches += 1;
-    k_grad_out<T><<<blocks(c.N, 256), 256, 0, c.stream>>>(c.N, c.vals, (const T*)c.rec, grad, B);
+    launch_next(c, k_grad_out<T>, blocks(c.N, 256), 256, c.N, c.vals, (const T*)c.rec, grad, B);
     return cudaGetLastError();
 }
 
@@ -960,7 +963,7 @@ cudaError_t run_dt_finalize(Ctx& c, double dt_fixed, double* dt_used_dev) {
 
 cudaError_t run_dt_set(Ctx& c, double dt) {
     c.launches += 1;
-    k_dt_set<<<blocks(c.nboxes, 256), 256, 0, c.stream>>>(c.nboxes, dt, c.dt_use);
+    launch_next(c, k_dt_set, blocks(c.nboxes, 256), 256, c.nboxes, dt, c.dt_use);
     return cudaGetLastError();
 }
 

@@ -268,13 +268,8 @@ __device__ __forceinline__ void store_slot(unsigned* p, unsigned v) {
 
 // First statement of every kernel that launch_next starts: waits until the
 // kernel before it (and so everything before that) has completed and its writes
-// are visible, then lets the kernel after it be set up (in that order, so at
-// most two kernels of the chain are on the chip).  Without effect in a kernel
-// launched the ordinary way.
-__device__ __forceinline__ void after_previous() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
-}
+// are visible.  Without effect in a kernel launched the ordinary way.
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ordered-integer image of a non-negative double (for atomicMin)
 __device__ __forceinline__ unsigned long long dbits(double v) {

@@ -7,13 +7,13 @@
 
 namespace gz {
 
-// Launches a kernel of the step's chain (each begins with after_previous).
-// Under kChainMax particles its blocks are set up while the kernel before it
-// runs, instead of after it: fifteen short launches wait for each other in a
-// small box (step of Sod 16^3 96 -> 69 us, Sod 32^3 155 -> 135, KH 41^3 188 ->
-// 169, Sod 50^3 with exact faces 631 -> 614); large launches lose by it (Sedov
-// 64^3 689 -> 703, turbulence 80^3 937 -> 969, 128^3 2920 -> 3010).
-constexpr int kChainMax = 200000;
+// Launches a kernel that begins with after_previous: the chip sets it up as the
+// kernel before it ends, instead of after that kernel's writes are flushed.  A
+// step is fifteen launches in a row: Sod 16^3 96 -> 68 us, Sod 32^3 155 -> 129,
+// KH 41^3 188 -> 159, Sedov 64^3 689 -> 661, 128^3 2930 -> 2894.  Kernels do not
+// let the next one start any earlier (griddepcontrol.launch_dependents): its
+// blocks then take slots from the kernel that still runs (KH 41^3 167, 128^3
+// 3010).
 template <typename... P, typename... A>
 inline void launch_next(const Ctx& c, void (*kernel)(P...), dim3 grid, dim3 block, A&&... args) {
     cudaLaunchAttribute at{};
@@ -24,7 +24,7 @@ inline void launch_next(const Ctx& c, void (*kernel)(P...), dim3 grid, dim3 bloc
     cfg.blockDim = block;
     cfg.stream = c.stream;
     cfg.attrs = &at;
-    cfg.numAttrs = c.N < kChainMax ? 1 : 0;
+    cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 

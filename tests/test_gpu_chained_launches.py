@@ -1,6 +1,5 @@
-"""Launches under 200000 particles overlap a kernel's set-up with the kernel
-before it; larger ones do not.  The same boxes stepped either way, and stepped
-again, give the same bits."""
+"""A kernel's set-up overlaps the end of the kernel before it.  The same boxes
+stepped again, alone and beside others, give the same bits."""
 import pytest
 
 from gpu_common import cast_state, device
@@ -23,8 +22,7 @@ def _steps(m, q, prec, copies, steps=4):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("prec,copies", [(1, 24), (1, 25), (0, 25)])
-def test_chained_and_separate_launches_give_the_same_bits(prec, copies):
-    # 24 boxes of 20^3: the largest launch still chained; 25: the smallest that is not
+def test_chained_launches_give_the_same_bits(prec, copies):
     import torch
     import paper_1712_01294_gb300 as m
     q = cast_state(I.turbulence(20, seed=21), prec)
