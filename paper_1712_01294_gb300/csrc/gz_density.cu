@@ -244,9 +244,9 @@ __device__ __forceinline__ double n_of(double S, double H) { return 8.0 * (1.0 +
 
 template <typename T, int G>
 __global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
-    k_density(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr, int* __restrict__ ncount,
-              int* __restrict__ iters, DevStatus* st, const int* __restrict__ list,
-              const int* __restrict__ nlist, int* __restrict__ defer, int* __restrict__ ndefer, int ccap) {
+    k_density(int N, Sorted<T> s, Grid g, KParams p, unsigned* nbr, int* ncount,
+              int* iters, DevStatus* st, const int* list,
+              const int* nlist, int* defer, int* ndefer, int ccap) {
     after_previous();
     constexpr int P = kDensBlock / G, E = kDensCache / G;
     constexpr int S = kDensCache + G;  // (the groups of a warp start on different banks)
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
 // memory.  Held to 96 registers (10 blocks of 64 per SM).
 constexpr int kOneBlock = 64;
 template <int kCache>
-__device__ __noinline__ int dens_fill(const Grid& g, const BoxInfo& bx, const P4<float>* __restrict__ pos, int i,
+__device__ __noinline__ int dens_fill(const Grid& g, const BoxInfo& bx, const P4<float>* pos, int i,
                                       float xi, float yi, float zi, float R, float (*c_r2)[kOneBlock],
                                       unsigned (*c_j)[kOneBlock], int t) {
     const float R2 = R * R;
@@ -355,8 +355,8 @@ __device__ __noinline__ int dens_fill(const Grid& g, const BoxInfo& bx, const P4
 // any periodic shift, and the particle itself told apart once per four
 // candidates.  pos is readable up to three records past its last.
 template <typename E>
-__device__ __forceinline__ void scan_inside(const int2* __restrict__ cells, int nc, const int (&lo)[3],
-                                            const int (&hi)[3], const P4<float>* __restrict__ pos, int self,
+__device__ __forceinline__ void scan_inside(const int2* cells, int nc, const int (&lo)[3],
+                                            const int (&hi)[3], const P4<float>* pos, int self,
                                             float xi, float yi, float zi, float R, E&& hit) {
     const float R2 = R * R, cl = 1.f / (float)nc, R2m = R2 * 1.0001f;
     for (int cz = lo[2]; cz <= hi[2]; ++cz) {
@@ -367,7 +367,7 @@ __device__ __forceinline__ void scan_inside(const int2* __restrict__ cells, int 
             const float gy = fmaxf(fmaxf((float)cy * cl - yi, yi - (float)(cy + 1) * cl), 0.f);
             const float gzy2 = gz2 + gy * gy;
             if (gzy2 > R2m) continue;
-            const int2* __restrict__ row = cells + (cz * nc + cy) * nc;
+            const int2* row = cells + (cz * nc + cy) * nc;
             // the ranges of up to three cells of the row in flight together
             for (int x0 = lo[0]; x0 <= hi[0]; x0 += 3) {
                 int2 ses[3];
@@ -424,10 +424,10 @@ __device__ __forceinline__ bool warp_inside(const BoxInfo& bx, const P4<float>& 
 // candidates loaded ahead (925 against 919) gave anything.
 template <int kCache, bool kInside>
 __global__ void __launch_bounds__(kOneBlock, 10)
-    k_density_one(int N, Sorted<float> s, Grid g, KParams p, unsigned* __restrict__ nbr,
-                  int* __restrict__ ncount, int* __restrict__ iters, DevStatus* st,
-                  const int* __restrict__ list, const int* __restrict__ nlist, int* __restrict__ defer,
-                  int* __restrict__ ndefer) {
+    k_density_one(int N, Sorted<float> s, Grid g, KParams p, unsigned* nbr,
+                  int* ncount, int* iters, DevStatus* st,
+                  const int* list, const int* nlist, int* defer,
+                  int* ndefer) {
     after_previous();
     __shared__ float c_r2[kCache + 1][kOneBlock];
     __shared__ unsigned c_j[kCache + 1][kOneBlock];
@@ -599,7 +599,7 @@ __device__ __forceinline__ void warp_eval(int lane, int n, const double* r2, dou
 // An evaluation straight from the cells (more candidates than the warp's cache
 // holds), the lanes' sums added up.
 template <typename T>
-__device__ __noinline__ void warp_eval_cells(const Grid& g, const BoxInfo& bx, const P4<T>* __restrict__ pos, int i,
+__device__ __noinline__ void warp_eval_cells(const Grid& g, const BoxInfo& bx, const P4<T>* pos, int i,
                                              const P4<T>& me, int lane, T H, T& S, T& sd) {
     const T H2 = H * H, iH = T(1) / H;
     double a = 0.0, b = 0.0;
@@ -624,9 +624,9 @@ __device__ __noinline__ void warp_eval_cells(const Grid& g, const BoxInfo& bx, c
 
 template <typename T>
 __global__ void __launch_bounds__(kWarpDensBlock)
-    k_density_warp(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr,
-                   int* __restrict__ ncount, int* __restrict__ iters, DevStatus* st,
-                   const int* __restrict__ defer, const int* __restrict__ ndefer) {
+    k_density_warp(int N, Sorted<T> s, Grid g, KParams p, unsigned* nbr,
+                   int* ncount, int* iters, DevStatus* st,
+                   const int* defer, const int* ndefer) {
     after_previous();
     constexpr unsigned full = 0xffffffffu;
     __shared__ T w_r2[kWarpDensBlock / 32][kWarpCache];
@@ -719,7 +719,7 @@ __global__ void __launch_bounds__(kWarpDensBlock)
 constexpr int kGivenBlock = 128, kStage = 32;
 template <bool kInside>
 __global__ void __launch_bounds__(kGivenBlock, 8)
-    k_lists_one(int N, Sorted<float> s, Grid g, KParams p, unsigned* __restrict__ nbr, int* __restrict__ ncount,
+    k_lists_one(int N, Sorted<float> s, Grid g, KParams p, unsigned* nbr, int* ncount,
                 DevStatus* st, int only_over) {
     after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -759,7 +759,7 @@ __global__ void __launch_bounds__(kGivenBlock, 8)
 // Small launches and FP64: four lanes per particle.
 template <typename T>
 __global__ void __launch_bounds__(kDensBlock)
-    k_lists(int N, Sorted<T> s, Grid g, KParams p, unsigned* __restrict__ nbr, int* __restrict__ ncount,
+    k_lists(int N, Sorted<T> s, Grid g, KParams p, unsigned* nbr, int* ncount,
             DevStatus* st, int only_over) {
     after_previous();
     const int gl = threadIdx.x % kLanes, i = (blockIdx.x * kDensBlock + threadIdx.x) / kLanes;
@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(kDensBlock)
 // those inside H; summed over the particles (out[0..2]).
 template <typename T>
 __global__ void __launch_bounds__(128)
-    k_scan_stats(int N, Sorted<T> s, Grid g, KParams p, unsigned long long* __restrict__ out) {
+    k_scan_stats(int N, Sorted<T> s, Grid g, KParams p, unsigned long long* out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long v[3] = {0, 0, 0};
     if (i < N) {

@@ -199,25 +199,33 @@ __device__ __forceinline__ size_t rec_at(int i, int q) {  // place of value q of
     constexpr int per = 32 / sizeof(T), ns = kRecord / per;
     return (size_t)i * kRecord + (((q / per + i) & (ns - 1)) * per + q % per);
 }
-__device__ __forceinline__ void load_rec(const float* __restrict__ rec, int i, float (&v)[kRecord]) {
+// The record passes may be set up while the pass that writes the records still
+// runs (launch_next), so the loads are coherent ones, not of the read-only path
+// (.nc: memory nobody writes while the kernel lives), and volatile with a
+// memory clobber: they stay behind after_previous.  They take the same time
+// (128^3: 2.90 ms a step with the read-only loads, 2.89 with these).
+__device__ __forceinline__ void load_rec(const float* rec, int i, float (&v)[kRecord]) {
 #pragma unroll
     for (int k = 0; k < kRecord / 8; ++k)
-        asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
             : "=f"(v[8 * k]), "=f"(v[8 * k + 1]), "=f"(v[8 * k + 2]), "=f"(v[8 * k + 3]), "=f"(v[8 * k + 4]),
               "=f"(v[8 * k + 5]), "=f"(v[8 * k + 6]), "=f"(v[8 * k + 7])
-            : "l"(rec + rec_at<float>(i, 8 * k)));
+            : "l"(rec + rec_at<float>(i, 8 * k))
+            : "memory");
 }
-__device__ __forceinline__ void load_rec(const double* __restrict__ rec, int i, double (&v)[kRecord]) {
+__device__ __forceinline__ void load_rec(const double* rec, int i, double (&v)[kRecord]) {
 #pragma unroll
     for (int k = 0; k < kRecord / 4; ++k)
-        asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
+        asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
             : "=d"(v[4 * k]), "=d"(v[4 * k + 1]), "=d"(v[4 * k + 2]), "=d"(v[4 * k + 3])
-            : "l"(rec + rec_at<double>(i, 4 * k)));
+            : "l"(rec + rec_at<double>(i, 4 * k))
+            : "memory");
 }
 
 // n values (a multiple of 32 bytes) from 32-byte-aligned global memory with
 // 32-byte vector loads, for per-particle rows read by other particles'
-// threads (scattered rows: whole sectors per L1 wavefront).
+// threads (scattered rows: whole sectors per L1 wavefront).  Read-only path: for
+// kernels launched the ordinary way (the adjoint passes) only.
 template <int n>
 __device__ __forceinline__ void load_row32(const float* __restrict__ p, float* v) {
     static_assert(n % 8 == 0, "rows of whole 32-byte vectors");
@@ -516,7 +524,7 @@ __device__ __forceinline__ bool exact_star(float rL, float uL, float PL, float r
 // compute the same canonical flux and get bitwise-opposite contributions
 // (the adjoint orients by id: its tie rule at the clamp names L).
 template <bool kById>
-__device__ __forceinline__ bool pair_order(int i, int j, long long idi, const long long* __restrict__ sid) {
+__device__ __forceinline__ bool pair_order(int i, int j, long long idi, const long long* sid) {
     if constexpr (kById)
         return idi < sid[j];
     else
@@ -746,9 +754,9 @@ __device__ __forceinline__ void for_slots(const uint4& jj, int n, F&& f) {
 // pair (MFV, the exact solver, FP64) need the registers themselves.  kUnroll:
 // copies of the pair's code (the exact solver's is long: one).
 template <typename T, int nq, bool kAhead, int kUnroll, typename P>
-__device__ __forceinline__ Totals<nq> sum_runs(int i, int N, const T* __restrict__ rec,
-                                               const unsigned* __restrict__ nbr, int cnt,
-                                               const unsigned* __restrict__ rnbr, int rcnt, P&& pair) {
+__device__ __forceinline__ Totals<nq> sum_runs(int i, int N, const T* rec,
+                                               const unsigned* nbr, int cnt,
+                                               const unsigned* rnbr, int rcnt, P&& pair) {
     Total<T> sum[nq];
     T A[kRecord], B[kRecord];
 #pragma unroll 1
@@ -804,9 +812,9 @@ __device__ __forceinline__ Totals<nq> sum_runs(int i, int N, const T* __restrict
 // Four warps: warp c forms runs c, c + 4, ...; v[0] becomes quantity c's total
 // (v[1], in warp 0, the fifth's).  Every thread of the block must get here.
 template <typename T, int nq, int kUnroll, typename P>
-__device__ __forceinline__ Totals<2> sum_runs_split(int i, int N, const T* __restrict__ rec,
-                                                    const unsigned* __restrict__ nbr, int cnt,
-                                                    const unsigned* __restrict__ rnbr, int rcnt, P&& pair) {
+__device__ __forceinline__ Totals<2> sum_runs_split(int i, int N, const T* rec,
+                                                    const unsigned* nbr, int cnt,
+                                                    const unsigned* rnbr, int rcnt, P&& pair) {
     __shared__ T sh[4][nq][32];
     const int c = threadIdx.x >> 5, l = threadIdx.x & 31;
     const int runs = (cnt + 7) / 8, all = runs + (rcnt + 7) / 8;
@@ -852,8 +860,8 @@ __device__ __forceinline__ int flux_item() {
 }
 // The rates of a thread's particle: all of them, or (four warps) quantity c.
 template <int nq>
-__device__ __forceinline__ void store_rates(const double (&v)[nq], int i, int N, double* __restrict__ dpdt,
-                                            double* __restrict__ dEdt, double* __restrict__ dmdt) {
+__device__ __forceinline__ void store_rates(const double (&v)[nq], int i, int N, double* dpdt,
+                                            double* dEdt, double* dmdt) {
     dpdt[i] = v[0];
     dpdt[(size_t)N + i] = v[1];
     dpdt[2 * (size_t)N + i] = v[2];
@@ -861,8 +869,8 @@ __device__ __forceinline__ void store_rates(const double (&v)[nq], int i, int N,
     if constexpr (nq == 5) dmdt[i] = v[4];
 }
 template <int nq>
-__device__ __forceinline__ void store_rates_split(const double (&v)[2], int i, int N, double* __restrict__ dpdt,
-                                                  double* __restrict__ dEdt, double* __restrict__ dmdt) {
+__device__ __forceinline__ void store_rates_split(const double (&v)[2], int i, int N, double* dpdt,
+                                                  double* dEdt, double* dmdt) {
     const int c = threadIdx.x >> 5;
     if (c < 3)
         dpdt[(size_t)c * N + i] = v[0];

@@ -49,8 +49,8 @@ __device__ __forceinline__ T wrap_pos(T v) {
 
 // ------------------------------------------------------ interval start
 template <typename T>
-__global__ void k_h_init(int N, gz_particles p, T* __restrict__ hva, T* __restrict__ hdvs,
-                         int* __restrict__ hsa, int* __restrict__ hbin) {
+__global__ void k_h_init(int N, gz_particles p, T* hva, T* hdvs,
+                         int* hsa, int* hbin) {
     after_previous();
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= N) return;
@@ -74,9 +74,9 @@ __device__ __forceinline__ T vbar(T va, T v, T dvs) {
 
 // Predicted positions of every particle at substep s (caller order).
 template <typename T>
-__global__ void k_h_predict(int N, int s, int K, gz_particles p, const T* __restrict__ hva,
-                            const T* __restrict__ hdvs, const int* __restrict__ hsa,
-                            const int* __restrict__ box_of, const double* __restrict__ D, T* __restrict__ xp) {
+__global__ void k_h_predict(int N, int s, int K, gz_particles p, const T* hva,
+                            const T* hdvs, const int* hsa,
+                            const int* box_of, const double* D, T* xp) {
     after_previous();
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o < N) {
@@ -98,7 +98,7 @@ __global__ void k_h_predict(int N, int s, int K, gz_particles p, const T* __rest
 }
 
 // Number of particles active at substep s, once the bins up to it are final.
-__global__ void k_h_count(int N, int s, int K, const int* __restrict__ hbin, int* __restrict__ count) {
+__global__ void k_h_count(int N, int s, int K, const int* hbin, int* count) {
     after_previous();
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     const int c = __syncthreads_count(o < N && s % (1 << (K - hbin[o])) == 0);
@@ -107,8 +107,8 @@ __global__ void k_h_count(int N, int s, int K, const int* __restrict__ hbin, int
 
 // Sorted bins and active flags, and the flags' counts per compaction block.
 __global__ void __launch_bounds__(kCmpBlock)
-    k_h_flags(int N, int s, int K, const unsigned* __restrict__ orig, const int* __restrict__ hbin,
-              int* __restrict__ sbin, unsigned char* __restrict__ aflag, int* __restrict__ bcount) {
+    k_h_flags(int N, int s, int K, const unsigned* orig, const int* hbin,
+              int* sbin, unsigned char* aflag, int* bcount) {
     after_previous();
     const int i = blockIdx.x * kCmpBlock + threadIdx.x;
     bool act = false;
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kCmpBlock)
 // ballots within a block).
 constexpr int kCmpDirect = 4096;
 
-__global__ void __launch_bounds__(kCmpBlock) k_cmp_scan(int nb, int* __restrict__ bcount, int* __restrict__ total) {
+__global__ void __launch_bounds__(kCmpBlock) k_cmp_scan(int nb, int* bcount, int* total) {
     after_previous();
     __shared__ int part[kCmpBlock];
     const int t = threadIdx.x;
@@ -156,8 +156,8 @@ __global__ void __launch_bounds__(kCmpBlock) k_cmp_scan(int nb, int* __restrict_
 
 // total non-null: boff holds the counts, and the last block writes their sum.
 __global__ void __launch_bounds__(kCmpBlock)
-    k_cmp_write(int N, const unsigned char* __restrict__ flag, const int* __restrict__ boff,
-                int* __restrict__ list, int* __restrict__ total) {
+    k_cmp_write(int N, const unsigned char* flag, const int* boff,
+                int* list, int* total) {
     after_previous();
     __shared__ int wsum[kCmpBlock / 32];
     int base = 0;
@@ -198,8 +198,8 @@ __global__ void __launch_bounds__(kCmpBlock)
 // Smallest support radius among every cell's active particles (+inf without
 // any), rounded down.
 template <typename T>
-__global__ void k_h_cellmin(int ncells, const int2* __restrict__ cells, const unsigned char* __restrict__ aflag,
-                            const P4<T>* __restrict__ pos, float* __restrict__ cellmin) {
+__global__ void k_h_cellmin(int ncells, const int2* cells, const unsigned char* aflag,
+                            const P4<T>* pos, float* cellmin) {
     after_previous();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncells) return;
@@ -217,8 +217,8 @@ __global__ void k_h_cellmin(int ncells, const int2* __restrict__ cells, const un
 
 // Cells within two cells (per axis, periodic) of a cell holding an active
 // particle, marked by the active cells themselves (near must start zeroed).
-__global__ void k_h_dilate(int ncells, const BoxInfo* __restrict__ boxes, int nboxes,
-                           const float* __restrict__ cellmin, unsigned char* __restrict__ near) {
+__global__ void k_h_dilate(int ncells, const BoxInfo* boxes, int nboxes,
+                           const float* cellmin, unsigned char* near) {
     after_previous();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncells || cellmin[c] == INFINITY) return;
@@ -268,10 +268,10 @@ __device__ __forceinline__ int cell_of(T v, int nc) {
 constexpr int kScatterLanes = 16;
 template <typename T>
 __global__ void __launch_bounds__(128)
-    k_h_rscatter(int N, Sorted<T> s, Grid g, KParams p, const unsigned* __restrict__ nbr,
-                 const int* __restrict__ ncount, const unsigned char* __restrict__ aflag,
-                 const float* __restrict__ cellmin, const unsigned char* __restrict__ near,
-                 unsigned* __restrict__ rnbr, int* __restrict__ rcount, DevStatus* st) {
+    k_h_rscatter(int N, Sorted<T> s, Grid g, KParams p, const unsigned* nbr,
+                 const int* ncount, const unsigned char* aflag,
+                 const float* cellmin, const unsigned char* near,
+                 unsigned* rnbr, int* rcount, DevStatus* st) {
     after_previous();
     const int gl = threadIdx.x % kScatterLanes;
     const int j = (blockIdx.x * blockDim.x + threadIdx.x) / kScatterLanes;
@@ -349,11 +349,11 @@ __global__ void __launch_bounds__(128)
 // Active i appends itself to the list of each inactive partner: thread (t, y)
 // takes list groups y, y + kInGroups, ... (four slots each) of active particle t.
 constexpr int kInGroups = 8;
-__global__ void k_h_inlist(const int* __restrict__ alist, const int* __restrict__ nA,
-                           const unsigned char* __restrict__ aflag, unsigned* __restrict__ nbr,
-                           int* __restrict__ ncount, const unsigned* __restrict__ rnbr,
-                           const int* __restrict__ rcount, int cap, int rcap,
-                           const long long* __restrict__ sid, int N, DevStatus* st) {
+__global__ void k_h_inlist(const int* alist, const int* nA,
+                           const unsigned char* aflag, unsigned* nbr,
+                           int* ncount, const unsigned* rnbr,
+                           const int* rcount, int cap, int rcap,
+                           const long long* sid, int N, DevStatus* st) {
     after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= *nA) return;
@@ -384,9 +384,9 @@ __global__ void k_h_inlist(const int* __restrict__ alist, const int* __restrict_
 // Index order for the lists written by other threads: the inactive
 // particles' partner lists and the active particles' r >= H_i pairs.
 __global__ void __launch_bounds__(kListBlock)
-    k_h_sort(int N, const unsigned char* __restrict__ aflag, int* __restrict__ ncount,
-             unsigned* __restrict__ nbr, int cap, const int* __restrict__ rcount,
-             unsigned* __restrict__ rnbr, int rcap) {
+    k_h_sort(int N, const unsigned char* aflag, int* ncount,
+             unsigned* nbr, int cap, const int* rcount,
+             unsigned* rnbr, int rcap) {
     after_previous();
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) / kListLanes;
     if (i >= N) return;
@@ -406,8 +406,8 @@ __global__ void __launch_bounds__(kListBlock)
 // Touched particles (active, or with an active partner), and their counts per
 // compaction block.
 __global__ void __launch_bounds__(kCmpBlock)
-    k_h_tflags(int N, const unsigned char* __restrict__ aflag, const int* __restrict__ ncount,
-               unsigned char* __restrict__ tflag, int* __restrict__ bcount) {
+    k_h_tflags(int N, const unsigned char* aflag, const int* ncount,
+               unsigned char* tflag, int* bcount) {
     after_previous();
     const int i = blockIdx.x * kCmpBlock + threadIdx.x;
     const bool t = i < N && (aflag[i] || ncount[i] > 0);
@@ -420,9 +420,9 @@ __global__ void __launch_bounds__(kCmpBlock)
 // Active particles keep what the inactive ones will read later: H (into the
 // caller's h), n, the limited gradients and B (from the flux record).
 template <typename T>
-__global__ void k_h_persist(int N, const int* __restrict__ alist, const int* __restrict__ nA,
-                            Sorted<T> s, const T* __restrict__ rec, gz_particles p, T* __restrict__ hn,
-                            T* __restrict__ hgrad, T* __restrict__ hB) {
+__global__ void k_h_persist(int N, const int* alist, const int* nA,
+                            Sorted<T> s, const T* rec, gz_particles p, T* hn,
+                            T* hgrad, T* hB) {
     after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= *nA) return;
@@ -441,9 +441,9 @@ __global__ void k_h_persist(int N, const int* __restrict__ alist, const int* __r
 // Largest finite criterion of every box (substep 0): a warp's maximum in one
 // atomic when the warp lies in one box (positive doubles order like their
 // bit patterns).
-__global__ void k_h_dtmax(const int* __restrict__ alist, const int* __restrict__ nA,
-                          const int* __restrict__ box, const double* __restrict__ dti,
-                          unsigned long long* __restrict__ dtmax) {
+__global__ void k_h_dtmax(const int* alist, const int* nA,
+                          const int* box, const double* dti,
+                          unsigned long long* dtmax) {
     after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = t < *nA;
@@ -466,9 +466,9 @@ __global__ void k_h_dtmax(const int* __restrict__ alist, const int* __restrict__
 }
 
 // Interval per box: min(cfl max dtc, 2^K cfl min dtc).
-__global__ void k_h_interval(int nb, const unsigned long long* __restrict__ dtmin,
-                             const unsigned long long* __restrict__ dtmax, double cfl, int K,
-                             double* __restrict__ D) {
+__global__ void k_h_interval(int nb, const unsigned long long* dtmin,
+                             const unsigned long long* dtmax, double cfl, int K,
+                             double* D) {
     after_previous();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nb) return;
@@ -485,10 +485,10 @@ __device__ __forceinline__ int bin_for(double D, double cfl_dtc, int K) {
 }
 
 // Bins of the active particles: assigned at substep 0, deepened later.
-__global__ void k_h_bins(const int* __restrict__ alist, const int* __restrict__ nA,
-                         const unsigned* __restrict__ orig, const int* __restrict__ box,
-                         const double* __restrict__ dti, const double* __restrict__ D, double cfl, int K,
-                         int first, int* __restrict__ hbin, int* __restrict__ sbin) {
+__global__ void k_h_bins(const int* alist, const int* nA,
+                         const unsigned* orig, const int* box,
+                         const double* dti, const double* D, double cfl, int K,
+                         int first, int* hbin, int* sbin) {
     after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= *nA) return;
@@ -522,12 +522,12 @@ __device__ __forceinline__ T pow2_(int e) {
 // 2.86 ms with them, 1.61 without, 1.59 with the next record ahead).
 template <typename T, int kRiem, bool kMFV, bool kSplit>
 __global__ void __launch_bounds__(kXBlock, kLoadAhead<T, kMFV, kRiem> ? 3 : 1)
-    k_h_exchange(const int* __restrict__ tlist, const int* __restrict__ nT, const T* __restrict__ rec,
-                 const long long* __restrict__ sid, const int* __restrict__ sbox,
-                 const int* __restrict__ sbin, const unsigned* __restrict__ nbr,
-                 const int* __restrict__ ncount, const unsigned* __restrict__ rnbr,
-                 const int* __restrict__ rcount, KParams p, const double* __restrict__ D,
-                 double* __restrict__ dpdt, double* __restrict__ dEdt, double* __restrict__ dmdt, int N,
+    k_h_exchange(const int* tlist, const int* nT, const T* rec,
+                 const long long* sid, const int* sbox,
+                 const int* sbin, const unsigned* nbr,
+                 const int* ncount, const unsigned* rnbr,
+                 const int* rcount, KParams p, const double* D,
+                 double* dpdt, double* dEdt, double* dmdt, int N,
                  DevStatus* st) {
     after_previous();
     constexpr int nq = kMFV ? 5 : 4;
@@ -575,11 +575,11 @@ __global__ void __launch_bounds__(kXBlock, kLoadAhead<T, kMFV, kRiem> ? 3 : 1)
 // and energy update without the drift (FP64 literal form; FP32 increments,
 // which also accumulate the step's velocity change for the drift).
 template <typename T>
-__global__ void k_h_kick(const int* __restrict__ tlist, const int* __restrict__ nT, int N, Sorted<T> s,
-                         const int* __restrict__ sbin, const double* __restrict__ dpdt,
-                         const double* __restrict__ dEdt, const double* __restrict__ dmdt,
-                         const double* __restrict__ D, gz_particles out, T* __restrict__ hdvs,
-                         int* __restrict__ box_hits, DevStatus* st) {
+__global__ void k_h_kick(const int* tlist, const int* nT, int N, Sorted<T> s,
+                         const int* sbin, const double* dpdt,
+                         const double* dEdt, const double* dmdt,
+                         const double* D, gz_particles out, T* hdvs,
+                         int* box_hits, DevStatus* st) {
     after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= *nT) return;
@@ -621,9 +621,9 @@ __global__ void k_h_kick(const int* __restrict__ tlist, const int* __restrict__ 
 // End of the steps that finish after substep s: drift by dt_i v_bar, new
 // step start (caller order).
 template <typename T>
-__global__ void k_h_finalize(int N, int s, int K, gz_particles p, T* __restrict__ hva, T* __restrict__ hdvs,
-                             int* __restrict__ hsa, const int* __restrict__ hbin,
-                             const int* __restrict__ box_of, const double* __restrict__ D, DevStatus* st) {
+__global__ void k_h_finalize(int N, int s, int K, gz_particles p, T* hva, T* hdvs,
+                             int* hsa, const int* hbin,
+                             const int* box_of, const double* D, DevStatus* st) {
     after_previous();
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= N) return;

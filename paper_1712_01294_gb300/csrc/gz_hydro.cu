@@ -28,8 +28,8 @@ inline int blocks(int n, int t) { return (n + t - 1) / t; }
 // KH 41^3 19 / 27, Sedov 64^3 39 / 35, turbulence 128^3 252 / 132.
 constexpr int kRevGroups = 8, kRevSplit = 150000;
 template <typename T>
-__device__ __forceinline__ void append_reverse(int i, int j, int N, int rcap, int* __restrict__ rcount,
-                                               unsigned* __restrict__ rnbr, const long long* __restrict__ id,
+__device__ __forceinline__ void append_reverse(int i, int j, int N, int rcap, int* rcount,
+                                               unsigned* rnbr, const long long* id,
                                                DevStatus* st) {
     const int slot = atomicAdd(&rcount[j], 1);
     if (slot < rcap)
@@ -39,9 +39,9 @@ __device__ __forceinline__ void append_reverse(int i, int j, int N, int rcap, in
 }
 
 template <typename T>
-__global__ void k_reverse(int N, Sorted<T> s, KParams p, const unsigned* __restrict__ nbr,
-                          const int* __restrict__ ncount, int* __restrict__ rcount,
-                          unsigned* __restrict__ rnbr, DevStatus* st) {
+__global__ void k_reverse(int N, Sorted<T> s, KParams p, const unsigned* nbr,
+                          const int* ncount, int* rcount,
+                          unsigned* rnbr, DevStatus* st) {
     after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -68,8 +68,8 @@ __global__ void k_reverse(int N, Sorted<T> s, KParams p, const unsigned* __restr
 // partners' positions in flight together; most threads do one group.
 template <typename T>
 __global__ void __launch_bounds__(32 * kRevGroups)
-    k_reverse_split(int N, Sorted<T> s, KParams p, const unsigned* __restrict__ nbr,
-                    const int* __restrict__ ncount, int* __restrict__ rcount, unsigned* __restrict__ rnbr,
+    k_reverse_split(int N, Sorted<T> s, KParams p, const unsigned* nbr,
+                    const int* ncount, int* rcount, unsigned* rnbr,
                     DevStatus* st) {
     after_previous();
     const int i = blockIdx.x * 32 + threadIdx.x;
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(32 * kRevGroups)
 // Orders each reverse list by sorted index so the flux sums are deterministic:
 // up to eight entries (most lists) in registers, each placed by the number of
 // smaller ones; longer ones by insertion.
-__global__ void k_sort_rev(int N, const int* __restrict__ rcount, unsigned* __restrict__ rnbr,
+__global__ void k_sort_rev(int N, const int* rcount, unsigned* rnbr,
                            int rcap) {
     after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -127,8 +127,8 @@ __global__ void k_sort_rev(int N, const int* __restrict__ rcount, unsigned* __re
 // The same with eight lanes a list, for launches under kRevSplit particles (Sod
 // 16^3, late in the run: one thread a list took 11 us, half of it waiting on
 // the few lists of more than eight).
-__global__ void __launch_bounds__(kListBlock) k_sort_rev_lanes(int N, const int* __restrict__ rcount,
-                                                               unsigned* __restrict__ rnbr, int rcap) {
+__global__ void __launch_bounds__(kListBlock) k_sort_rev_lanes(int N, const int* rcount,
+                                                               unsigned* rnbr, int rcap) {
     after_previous();
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) / kListLanes;
     if (i < N) sort_list(rnbr + 4 * (size_t)i, min(rcount[i], rcap), N);
@@ -138,8 +138,8 @@ __global__ void __launch_bounds__(kListBlock) k_sort_rev_lanes(int N, const int*
 // what the passes after it count from zero (every one of them follows a
 // k_prim): reverse-list counts, CFL minima, u-floor hits.
 template <typename T>
-__global__ void k_prim(int N, Sorted<T> s, KParams p, DevStatus* st, int* __restrict__ rcount, int nb,
-                       unsigned long long* __restrict__ dtmin, int* __restrict__ box_hits) {
+__global__ void k_prim(int N, Sorted<T> s, KParams p, DevStatus* st, int* rcount, int nb,
+                       unsigned long long* dtmin, int* box_hits) {
     after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     for (int b = i; b < nb; b += gridDim.x * blockDim.x) {
@@ -182,12 +182,12 @@ __global__ void k_prim(int N, Sorted<T> s, KParams p, DevStatus* st, int* __rest
 // kDt: also the signal-speed step.
 template <typename T, bool kInfo, bool kDt>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
-    k_gradients(int N, Sorted<T> s, const unsigned* __restrict__ nbr, const int* __restrict__ ncount,
-                const unsigned* __restrict__ rnbr, const int* __restrict__ rcount, KParams p,
-                T* __restrict__ rec, double* __restrict__ dti, unsigned long long* __restrict__ dtmin,
-                DevStatus* st, T* __restrict__ ginfo, int* __restrict__ lim,
-                const int* __restrict__ list, const int* __restrict__ nlist,
-                const unsigned char* __restrict__ owned) {
+    k_gradients(int N, Sorted<T> s, const unsigned* nbr, const int* ncount,
+                const unsigned* rnbr, const int* rcount, KParams p,
+                T* rec, double* dti, unsigned long long* dtmin,
+                DevStatus* st, T* ginfo, int* lim,
+                const int* list, const int* nlist,
+                const unsigned char* owned) {
     after_previous();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     bool active;
@@ -520,9 +520,9 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
 // inactive partners of a hierarchical substep, whose gradients and B are
 // those of their last active time).
 template <typename T>
-__global__ void k_pack_given(int N, Sorted<T> s, const T* __restrict__ grad, const T* __restrict__ B,
-                             T* __restrict__ rec, const int* __restrict__ list,
-                             const int* __restrict__ nlist, const unsigned char* __restrict__ skip) {
+__global__ void k_pack_given(int N, Sorted<T> s, const T* grad, const T* B,
+                             T* rec, const int* list,
+                             const int* nlist, const unsigned char* skip) {
     after_previous();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (list) {
@@ -555,8 +555,8 @@ __global__ void k_pack_given(int N, Sorted<T> s, const T* __restrict__ grad, con
 }
 
 template <typename T>
-__global__ void k_grad_out(int N, const unsigned* __restrict__ orig, const T* __restrict__ rec,
-                           T* __restrict__ grad, T* __restrict__ B) {
+__global__ void k_grad_out(int N, const unsigned* orig, const T* rec,
+                           T* grad, T* B) {
     after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -580,11 +580,11 @@ constexpr int kFluxBlock = 128;
 
 template <typename T, bool kMFV, int kRiem, bool kSplit>
 __global__ void __launch_bounds__(kFluxBlock, kLoadAhead<T, kMFV, kRiem> ? 3 : 1)
-    k_fluxes(int N, const T* __restrict__ rec, const long long* __restrict__ sid,
-             const int* __restrict__ sbox, const unsigned* __restrict__ nbr,
-             const int* __restrict__ ncount, const unsigned* __restrict__ rnbr,
-             const int* __restrict__ rcount, KParams p, const double* __restrict__ dt_use,
-             double* __restrict__ dpdt, double* __restrict__ dEdt, double* __restrict__ dmdt,
+    k_fluxes(int N, const T* rec, const long long* sid,
+             const int* sbox, const unsigned* nbr,
+             const int* ncount, const unsigned* rnbr,
+             const int* rcount, KParams p, const double* dt_use,
+             double* dpdt, double* dEdt, double* dmdt,
              DevStatus* st) {
     after_previous();
     constexpr int nq = kMFV ? 5 : 4;
@@ -625,10 +625,10 @@ __global__ void __launch_bounds__(kFluxBlock, kLoadAhead<T, kMFV, kRiem> ? 3 : 1
 
 // dmdt (MFV, O15) non-null: the mass advances too and is written back.
 template <typename T>
-__global__ void k_update(int N, Sorted<T> s, const double* __restrict__ dpdt,
-                         const double* __restrict__ dEdt, const double* __restrict__ dmdt,
-                         const double* __restrict__ dt_use, gz_particles out,
-                         int* __restrict__ box_hits, DevStatus* st, double* __restrict__ rates_out) {
+__global__ void k_update(int N, Sorted<T> s, const double* dpdt,
+                         const double* dEdt, const double* dmdt,
+                         const double* dt_use, gz_particles out,
+                         int* box_hits, DevStatus* st, double* rates_out) {
     after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -690,9 +690,9 @@ struct Bits<double> {
 // (radix select on the bit patterns of positive values), then every
 // non-positive updated u of the box is set to u_floor_frac * median.
 template <typename T>
-__global__ void k_ufloor(Sorted<T> s, const BoxInfo* __restrict__ boxes,
-                         const int* __restrict__ box_hits, gz_particles out, double frac,
-                         const unsigned char* __restrict__ owned, int nown) {
+__global__ void k_ufloor(Sorted<T> s, const BoxInfo* boxes,
+                         const int* box_hits, gz_particles out, double frac,
+                         const unsigned char* owned, int nown) {
     after_previous();
     typedef typename Bits<T>::U U;
     const int b = blockIdx.x;
@@ -737,8 +737,8 @@ __global__ void k_ufloor(Sorted<T> s, const BoxInfo* __restrict__ boxes,
     }
 }
 
-__global__ void k_dt_final(int nb, const unsigned long long* __restrict__ dtmin, double cfl,
-                           double dt_fixed, double* __restrict__ dt_use, double* __restrict__ out) {
+__global__ void k_dt_final(int nb, const unsigned long long* dtmin, double cfl,
+                           double dt_fixed, double* dt_use, double* out) {
     after_previous();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nb) return;
@@ -747,7 +747,7 @@ __global__ void k_dt_final(int nb, const unsigned long long* __restrict__ dtmin,
     dt_use[b] = dt;
     if (out) out[b] = dt;
 }
-__global__ void k_dt_set(int nb, double dt, double* __restrict__ dt_use) {
+__global__ void k_dt_set(int nb, double dt, double* dt_use) {
     after_previous();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b < nb) dt_use[b] = dt;

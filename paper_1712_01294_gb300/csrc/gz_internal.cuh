@@ -246,17 +246,19 @@ __device__ __forceinline__ size_t lcol(int k, int N) { return (size_t)(k >> 2) *
 __device__ __forceinline__ size_t lslot(int k, int i, int N) { return 4 * (size_t)i + lcol(k, N); }
 // Slots k0..k0+3 (k0 a multiple of four) of the list column L; those at or
 // past the list's count hold no particle.
-__device__ __forceinline__ uint4 col4(const unsigned* __restrict__ L, int k0, int N) {
+__device__ __forceinline__ uint4 col4(const unsigned* L, int k0, int N) {
     return *reinterpret_cast<const uint4*>(L + lcol(k0, N));
 }
 // The same slots for a pass that reads each list once: not kept in L1, which
 // stays for the records and positions the pass gathers (a pass that reads
-// its lists twice, like the gradient pass, keeps col4).
-__device__ __forceinline__ uint4 col4_once(const unsigned* __restrict__ L, int k0, int N) {
+// its lists twice, like the gradient pass, keeps col4).  A coherent load that
+// stays behind after_previous.
+__device__ __forceinline__ uint4 col4_once(const unsigned* L, int k0, int N) {
     uint4 r;
-    asm("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-        : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-        : "l"(L + lcol(k0, N)));
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+                 : "l"(L + lcol(k0, N))
+                 : "memory");
     return r;
 }
 
@@ -268,7 +270,10 @@ __device__ __forceinline__ void store_slot(unsigned* p, unsigned v) {
 
 // First statement of every kernel that launch_next starts: waits until the
 // kernel before it (and so everything before that) has completed and its writes
-// are visible.  Without effect in a kernel launched the ordinary way.
+// are visible.  Without effect in a kernel launched the ordinary way.  What the
+// kernel before it writes must not be read through the read-only path: such a
+// kernel and what it calls take no __restrict__ pointers (the compiler may then
+// use that path, or move a load above the wait) and no .nc loads.
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ordered-integer image of a non-negative double (for atomicMin)
@@ -290,10 +295,10 @@ __device__ __forceinline__ unsigned long long dbits(double v) {
 // Candidates arrive in ascending j within each cell.
 template <typename T, typename F>
 __device__ __forceinline__ void for_candidates(const Grid& g, const BoxInfo& bx,
-                                               const P4<T>* __restrict__ pos, int self, T xi, T yi,
+                                               const P4<T>* pos, int self, T xi, T yi,
                                                T zi, T R, F&& fn) {
     const int nc = bx.nc;
-    const int2* __restrict__ cells = g.cells + bx.cell_off;
+    const int2* cells = g.cells + bx.cell_off;
     // positions outside [0, 1] (flagged by the binning pass) see no candidates
     if (!(xi >= T(0) && xi <= T(1) && yi >= T(0) && yi <= T(1) && zi >= T(0) && zi <= T(1) &&
           R >= T(0)))
@@ -378,10 +383,10 @@ constexpr int kLaneCells = 16;
 // combined in a fixed order are deterministic.  Offsets from mi_diff.
 template <typename T, typename F>
 __device__ __forceinline__ void for_candidates_lanes(const Grid& g, const BoxInfo& bx,
-                                                     const P4<T>* __restrict__ pos, int self, T xi, T yi,
+                                                     const P4<T>* pos, int self, T xi, T yi,
                                                      T zi, T R, int lane, F&& fn) {
     const int nc = bx.nc;
-    const int2* __restrict__ cells = g.cells + bx.cell_off;
+    const int2* cells = g.cells + bx.cell_off;
     if (!(xi >= T(0) && xi <= T(1) && yi >= T(0) && yi <= T(1) && zi >= T(0) && zi <= T(1) &&
           R >= T(0)))
         return;
@@ -512,7 +517,7 @@ struct Window {
     // Candidates of cell (cx, cy, cz): none when its nearest point lies beyond R.
     // In FP32 for both precisions: the margin on R^2 covers the rounding of the
     // cell bounds and of the FP32 copies of x and R.
-    __device__ __forceinline__ int2 range(const int2* __restrict__ cells, int cx, int cy, int cz, float xi, float yi,
+    __device__ __forceinline__ int2 range(const int2* cells, int cx, int cy, int cz, float xi, float yi,
                                           float zi) const {
         auto gap = [&](int c, float v) {
             return wraps_all ? 0.f : max(max((float)c * cl - v, v - (float)(c + 1) * cl), 0.f);
@@ -552,7 +557,7 @@ __device__ __forceinline__ float r2_chop_bound(double R) {
 }
 
 // The n entries of the list column L put in increasing order by insertion.
-__device__ __forceinline__ void insert_sort(unsigned* __restrict__ L, int n, int N) {
+__device__ __forceinline__ void insert_sort(unsigned* L, int n, int N) {
     for (int a = 1; a < n; ++a) {
         const unsigned x = L[lcol(a, N)];
         int b = a - 1;
@@ -570,7 +575,7 @@ __device__ __forceinline__ void insert_sort(unsigned* __restrict__ L, int n, int
 // thread's insertion through global memory is a chain of dependent accesses
 // (hierarchical Sedov 64^3: 26 us a substep, 15 so).
 constexpr int kListLanes = 8, kListBlock = 128, kListMax = 64;
-__device__ __forceinline__ void sort_list(unsigned* __restrict__ L, int n, int N) {
+__device__ __forceinline__ void sort_list(unsigned* L, int n, int N) {
     __shared__ unsigned sh[kListBlock / kListLanes][kListMax + kListLanes];
     if (n < 2) return;
     const int gl = threadIdx.x % kListLanes;
@@ -604,11 +609,11 @@ __device__ __forceinline__ void sort_list(unsigned* __restrict__ L, int n, int N
 // sees only the hits; candidates up to 5e-7 outside R are handed over
 // too, unless kExact asks for the FP64 test of each.
 template <typename T, int G, bool kExact = false, typename E>
-__device__ __forceinline__ int group_scan(const Grid& g, const BoxInfo& bx, const P4<T>* __restrict__ pos,
+__device__ __forceinline__ int group_scan(const Grid& g, const BoxInfo& bx, const P4<T>* pos,
                                           int self, T xi, T yi, T zi, T R, int gl, unsigned gm, int most,
                                           E&& emit) {
     const Window<T> w(bx.nc, xi, yi, zi, R);
-    const int2* __restrict__ cells = g.cells + bx.cell_off;
+    const int2* cells = g.cells + bx.cell_off;
     const T xim1 = xi - T(1), yim1 = yi - T(1), zim1 = zi - T(1);
     const T R2 = R * R;
     const float xf = chop(xi), yf = chop(yi), zf = chop(zi);
@@ -708,10 +713,10 @@ __device__ __forceinline__ int group_scan(const Grid& g, const BoxInfo& bx, cons
 constexpr int kAhead = 4;
 template <typename T, typename E>
 __device__ __forceinline__ int for_hits_lanes_ordered(const Grid& g, const BoxInfo& bx,
-                                                      const P4<T>* __restrict__ pos, int self, T xi, T yi,
+                                                      const P4<T>* pos, int self, T xi, T yi,
                                                       T zi, T R, T R2, int lane, E&& emit) {
     const Window<T> w(bx.nc, xi, yi, zi, R);
-    const int2* __restrict__ cells = g.cells + bx.cell_off;
+    const int2* cells = g.cells + bx.cell_off;
     const T xim1 = xi - T(1), yim1 = yi - T(1), zim1 = zi - T(1);
     const float xf = chop(xi), yf = chop(yi), zf = chop(zi);
     auto r2_of = [&](int j) {

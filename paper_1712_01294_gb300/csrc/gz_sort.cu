@@ -93,7 +93,7 @@ constexpr int kScanThreads = 1024;
 constexpr int kScanTile = 4 * kScanThreads;
 constexpr int kScanDirect = 8;  // up to this many tiles, a block sums the counts before its own itself
 
-__device__ __forceinline__ uint4 count4(const unsigned* __restrict__ count, long long k, long long K) {
+__device__ __forceinline__ uint4 count4(const unsigned* count, long long k, long long K) {
     if (k + 3 < K) return *reinterpret_cast<const uint4*>(count + k);
     uint4 v = make_uint4(0, 0, 0, 0);
     if (k < K) v.x = count[k];
@@ -115,7 +115,7 @@ __device__ __forceinline__ unsigned block_sum(unsigned v, unsigned* sh) {
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-    k_cs_sums(long long K, const unsigned* __restrict__ count, unsigned* __restrict__ sums) {
+    k_cs_sums(long long K, const unsigned* count, unsigned* sums) {
     after_previous();
     __shared__ unsigned sh[kScanThreads / 32];
     const uint4 v = count4(count, (long long)blockIdx.x * kScanTile + 4 * threadIdx.x, K);
@@ -127,9 +127,9 @@ __global__ void __launch_bounds__(kScanThreads)
 // included).  sums: the tiles' sums, or null when every block adds the counts
 // before its tile itself.
 __global__ void __launch_bounds__(kScanThreads)
-    k_cs_scan(long long K, const unsigned* __restrict__ count, const unsigned* __restrict__ sums,
-              const BoxInfo* __restrict__ boxes, int nboxes, unsigned* __restrict__ start,
-              int2* __restrict__ cells) {
+    k_cs_scan(long long K, const unsigned* count, const unsigned* sums,
+              const BoxInfo* boxes, int nboxes, unsigned* start,
+              int2* cells) {
     after_previous();
     __shared__ unsigned sh[kScanThreads / 32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -185,8 +185,8 @@ __global__ void __launch_bounds__(kScanThreads)
     }
 }
 
-__global__ void k_cs_place(int N, const unsigned* __restrict__ key, const unsigned* __restrict__ slot,
-                           const unsigned* __restrict__ start, unsigned* __restrict__ order) {
+__global__ void k_cs_place(int N, const unsigned* key, const unsigned* slot,
+                           const unsigned* start, unsigned* order) {
     after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < N) order[start[key[i]] + slot[i]] = (unsigned)i;
@@ -328,12 +328,12 @@ __global__ void k_rs_scatter(const unsigned* __restrict__ kin, const unsigned* _
 // and indices are written.  Else they are given, and the cells' ranges
 // are written from the keys' boundaries (cells zeroed before).
 template <typename T, bool kCounted>
-__global__ void k_permute(int N, unsigned* __restrict__ skeys, unsigned* __restrict__ svals,
-                          const unsigned* __restrict__ order, const unsigned* __restrict__ key_in,
-                          const unsigned* __restrict__ count, const unsigned* __restrict__ start, gz_particles p,
-                          const void* __restrict__ n_in, const int* __restrict__ box_of,
-                          const BoxInfo* __restrict__ boxes, Sorted<T> s, int2* __restrict__ cells,
-                          int* __restrict__ ndefer) {
+__global__ void k_permute(int N, unsigned* skeys, unsigned* svals,
+                          const unsigned* order, const unsigned* key_in,
+                          const unsigned* count, const unsigned* start, gz_particles p,
+                          const void* n_in, const int* box_of,
+                          const BoxInfo* boxes, Sorted<T> s, int2* cells,
+                          int* ndefer) {
     after_previous();
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= N) return;
