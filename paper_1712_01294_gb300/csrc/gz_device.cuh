@@ -695,32 +695,14 @@ __device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[k
 
 // Sums of one particle's pair contributions, shared by the flux pass and the
 // hierarchical exchange: over N_i then R_i, in the working precision over runs
-// of 8 list slots, the runs added up in list order (Total).  One thread forms
+// of 8 list slots, the runs added up in list order.  One thread forms
 // the runs one after another (sum_runs), or the block's four warps, which then
 // hold the same 32 particles, form four of them at a time (sum_runs_split):
 // the same bits.
-// A quantity's total.  FP32: an unevaluated sum hi + lo (Knuth's two-sum, 48
-// bits), an FP64 number only when it is stored: conversions and additions of
-// every run in FP64, at 1/64 of the FP32 rate, took 5 % of the pass (128^3 797
-// -> 758 us, ensemble 551 -> 521, MFV at 80^3 284 -> 277).  The rates' error
-// against the FP64 pass on the same inputs is the pairs' own (turbulence 48^3
-// 1.6065119e-6 of rms either way).
-template <typename T>
-struct Total {
-    T s = T(0);
-    __device__ __forceinline__ void add(T v) { s += v; }
-    __device__ __forceinline__ double value() const { return s; }
-};
-template <>
-struct Total<float> {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float v) {
-        const float s = __fadd_rn(hi, v), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b)));
-        hi = s;
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
+// Totals are FP64 in both precisions (the FP32 mode's rates are accumulated in
+// double).  Two FP32 words instead (48 bits) took 5 % less of the pass, 128^3 797
+// -> 758 us, but the low word loses its bits below 1e-38 and an infinite term
+// turns the total into NaN.
 template <int nq>
 struct Totals {
     double v[nq];
@@ -750,14 +732,16 @@ __device__ __forceinline__ void for_slots(const uint4& jj, int n, F&& f) {
 // kAhead: the next partner's record is loaded while the current pair is
 // evaluated (two record buffers, so the loop is written for two pairs at a
 // time; 165 registers, 12 warps an SM).  The pass waits on its gathers: FP32
-// MFM at 128^3 856 us without, 803 with (FP64 totals; see Total).  The forms with more arithmetic a
+// MFM at 128^3 856 us without, 803 with.  The forms with more arithmetic a
 // pair (MFV, the exact solver, FP64) need the registers themselves.  kUnroll:
 // copies of the pair's code (the exact solver's is long: one).
 template <typename T, int nq, bool kAhead, int kUnroll, typename P>
 __device__ __forceinline__ Totals<nq> sum_runs(int i, int N, const T* rec,
                                                const unsigned* nbr, int cnt,
                                                const unsigned* rnbr, int rcnt, P&& pair) {
-    Total<T> sum[nq];
+    double sum[nq];
+#pragma unroll
+    for (int q = 0; q < nq; ++q) sum[q] = 0.0;
     T A[kRecord], B[kRecord];
 #pragma unroll 1
     for (int list = 0; list < 2; ++list) {
@@ -799,13 +783,13 @@ __device__ __forceinline__ Totals<nq> sum_runs(int i, int N, const T* rec,
             jj = nn;
             if ((k0 & 4) || k0 + 4 >= n) {
 #pragma unroll
-                for (int q = 0; q < nq; ++q) sum[q].add(run[q]);
+                for (int q = 0; q < nq; ++q) sum[q] += (double)run[q];
             }
         }
     }
     Totals<nq> t;
 #pragma unroll
-    for (int q = 0; q < nq; ++q) t.v[q] = sum[q].value();
+    for (int q = 0; q < nq; ++q) t.v[q] = sum[q];
     return t;
 }
 
@@ -818,7 +802,7 @@ __device__ __forceinline__ Totals<2> sum_runs_split(int i, int N, const T* rec,
     __shared__ T sh[4][nq][32];
     const int c = threadIdx.x >> 5, l = threadIdx.x & 31;
     const int runs = (cnt + 7) / 8, all = runs + (rcnt + 7) / 8;
-    Total<T> sum[2];
+    double sum[2] = {0.0, 0.0};
     for (int r0 = 0; __syncthreads_or(r0 < all); r0 += 4) {
         const int r = r0 + c;
         T run[nq];
@@ -843,13 +827,13 @@ __device__ __forceinline__ Totals<2> sum_runs_split(int i, int N, const T* rec,
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
             if (r0 + w >= all) break;
-            sum[0].add(sh[w][c][l]);
-            if constexpr (nq == 5) sum[1].add(sh[w][4][l]);
+            sum[0] += (double)sh[w][c][l];
+            if constexpr (nq == 5) sum[1] += (double)sh[w][4][l];
         }
     }
     Totals<2> t;
-    t.v[0] = sum[0].value();
-    t.v[1] = sum[1].value();
+    t.v[0] = sum[0];
+    t.v[1] = sum[1];
     return t;
 }
 
