@@ -112,8 +112,11 @@ __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)
     const T e1 = du - ccb, e2 = cca - du;
     const T al = min_(-cca, e1), be = max_(ccb, e2);
     const T ma = mul_rn(Ga[0], al), mb = mul_rn(Gb[0], be);
-    const T iden = rcp_(ma - mb), msum = ma + mb;
-    const T psr = fma(-(ma * mb), du, add_rn(mul_rn(ma, Gb[4]), -mul_rn(mb, Ga[4]))) * iden;
+    const T den = ma - mb, iden = rcp_(den), msum = ma + mb;
+    T sc, isc;  // (the scaling of pair_rates)
+    pow2_near(den, sc, isc);
+    const T mas = ma * sc, mbs = mb * sc, idens = iden * isc;
+    const T psr = fma(-(mas * mb), du, add_rn(mul_rn(mas, Gb[4]), -mul_rn(mbs, Ga[4]))) * idens;
     const T X = fma(-msum, du, T(2) * (Gb[4] - Ga[4])) * iden;
     const T S = T(0.5) * (us + X);
     const bool neg = psr < T(0);
@@ -124,13 +127,15 @@ __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)
     const T wS = wE * S;
     const T b_psr = neg ? T(0) : -fma(wS, Am, wA);
     const T b_h = T(-0.5) * (ps * wE) * Am;  // of us and of X
-    // X = num2 iden, psr = num1 iden, iden = 1 / (ma - mb)
-    const T b_2 = b_h * iden, b_1 = b_psr * iden;
-    const T b_den = -fma(b_2, X, b_1 * psr);
-    T b_Pa = -fma(b_1, mb, T(2) * b_2), b_Pb = fma(b_1, ma, T(2) * b_2);
-    const T b_ma = fma(b_1, fma(-mb, du, Gb[4]), fma(-du, b_2, b_den));
-    const T b_mb = -fma(b_1, fma(ma, du, Ga[4]), fma(du, b_2, b_den));
-    T b_du = -fma(msum, b_2, b_1 * (ma * mb));
+    // X = num2 iden, psr = num1 idens with num1 = sc (ma Pb - mb Pa - ma mb du),
+    // iden = 1 / (ma - mb); b_1 the adjoint of num1, of order b_psr like every
+    // product formed with it
+    const T b_2 = b_h * iden, b_1 = b_psr * idens;
+    const T b_den = -fma(b_2, X, b_1 * (sc * psr));
+    T b_Pa = -fma(b_1, mbs, T(2) * b_2), b_Pb = fma(b_1, mas, T(2) * b_2);
+    const T b_ma = fma(b_1, fma(-mbs, du, sc * Gb[4]), fma(-du, b_2, b_den));
+    const T b_mb = -fma(b_1, fma(mas, du, sc * Ga[4]), fma(du, b_2, b_den));
+    T b_du = -fma(msum, b_2, b_1 * (mas * mb));
     // ma = rho_a min(-c_a, du - c_b), mb = rho_b max(c_b, c_a - du); a tie goes to
     // the particle that is L (the derivative oracle's rule)
     T b_ra = b_ma * al, b_rb = b_mb * be;
@@ -281,7 +286,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 1)
     for (int q = 0; q < 15; ++q) bg[q] = s.g[q];
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-        bW[0] -= k * irho * a[11 + 12 + q] * s.F[1 + q];
+        bW[0] -= (k * s.F[1 + q]) * (irho * a[11 + 12 + q]);  // (1/rho^2 alone could leave the range)
         bg[12 + q] += k * s.F[1 + q];
     }
     const T b_div = -hdt * (a[6] * s.F[0] + gam * a[7] * s.F[4]);

@@ -80,6 +80,18 @@ __device__ __forceinline__ bool pos_(double a) {  // a > 0 (false for NaN)
     const long long i = __double_as_longlong(a);
     return i > 0 && i <= 0x7ff0000000000000ll;
 }
+// s, a power of two near 1/|D|, and is = 1/s (D normal; clamped where one of the
+// two would not be): scaling by them is exact.
+__device__ __forceinline__ void pow2_near(float D, float& s, float& is) {
+    const unsigned e = min(max(__float_as_uint(D) & 0x7f800000u, 0x00800000u), 0x7e800000u);
+    s = __uint_as_float(0x7f000000u - e);
+    is = __uint_as_float(e);
+}
+__device__ __forceinline__ void pow2_near(double D, double& s, double& is) {
+    const int e = min(max(__double2hiint(D) & 0x7ff00000, 0x00100000), 0x7fd00000);
+    s = __hiloint2double(0x7fe00000 - e, 0);
+    is = __hiloint2double(e, 0);
+}
 // Smallest squares the pair geometry takes (below them rsq_ has no normal
 // argument): a face this small (area 3e-19) carries nothing.
 template <typename T>
@@ -562,7 +574,11 @@ __device__ __forceinline__ void half_state(const T (&a)[kRecord], T hdt, T gam, 
 //   P* = (m_a P_b - m_b P_a - m_a m_b du) / (m_a - m_b),
 //   S* = ((v_a + v_b).n + (2 (P_b - P_a) - (m_a + m_b) du) / (m_a - m_b)) / 2,
 // the contact speed in the lab frame, S*_face + v_f.n whatever v_f is.  Only
-// velocity differences enter P*, so nothing cancels at high Mach number.
+// velocity differences enter P*, so nothing cancels at high Mach number.  P*'s
+// products of an impedance with a pressure or another impedance would leave the
+// range long before the states do (FP32: rho c below 1e-19 or above 1e19), so
+// one of the two impedances is scaled to about 1 by an exact power of two, and
+// 1/(m_a - m_b) back by it: the same bits, and P* has the states' own range.
 template <typename T, bool kMFV, int kRiem>
 __device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[kRecord], const T (&Wh)[5], bool aL,
                                            T hdt, T gam, T (&dp)[3], T& dE, T& dm, int& fl) {
@@ -613,8 +629,11 @@ __device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[k
     const T cca = mul_rn(qa, rsq_(max_(qa, Tiny<T>::sq))), ccb = mul_rn(qb, rsq_(max_(qb, Tiny<T>::sq)));
     const T du = dot3(Fb[1] - Fa[1], Fb[2] - Fa[2], Fb[3] - Fa[3], n0, n1, n2);
     const T ma = mul_rn(Fa[0], min_(-cca, du - ccb)), mb = mul_rn(Fb[0], max_(ccb, cca - du));
-    const T iden = rcp_(ma - mb);
-    T ps = fma(-(ma * mb), du, add_rn(mul_rn(ma, Fb[4]), -mul_rn(mb, Fa[4]))) * iden;
+    const T den = ma - mb, iden = rcp_(den);
+    T sc, isc;
+    pow2_near(den, sc, isc);
+    const T mas = ma * sc, mbs = mb * sc;  // (of order one)
+    T ps = fma(-(mas * mb), du, add_rn(mul_rn(mas, Fb[4]), -mul_rn(mbs, Fa[4]))) * (iden * isc);
     bool neg = ps < T(0);
     const T Am = T(2) * (Aq * iA);
     if constexpr (!kMFV && kRiem == 0) {
