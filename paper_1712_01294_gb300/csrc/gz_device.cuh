@@ -500,7 +500,8 @@ __device__ __forceinline__ bool exact_star(float rL, float uL, float PL, float r
         const float pe = ppow(p * iP, e);
         const bool shock = p > P;
         f = shock ? dP * q : k * (pe - 1.f);
-        d = shock ? fmaf(-0.5f * dP * iA, q * q * q, q) : pe * j * ip;
+        // (iA q q = 1/(p + B): q^3 would overflow at rho P below 1e-26)
+        d = shock ? fmaf(-0.5f * dP * (iA * q * q), q, q) : pe * j * ip;
     };
 #pragma unroll 1
     for (int it = 0; it < 20; ++it) {
