@@ -65,13 +65,14 @@ __device__ __forceinline__ double rsq_(double x) {
     const double e = fma(-(x * y), y, 1.0);
     return fma(y * e, fma(e, 0.375, 0.5), y);
 }
-// min and max of two numbers.  FP64: compared as integers (a negative number's
-// magnitude bits flipped), which leaves the FP64 pipe alone.
+// min and max of two numbers.  FP64: compared as integers, which leaves the FP64
+// pipe alone; a negative number's integer is mirrored, so that -0 and +0 are one
+// number.
 __device__ __forceinline__ float min_(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ float max_(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ long long order_(double a) {
     const long long i = __double_as_longlong(a);
-    return i ^ ((i >> 63) & 0x7fffffffffffffffll);
+    return i < 0 ? (long long)(0x8000000000000000ull - (unsigned long long)i) : i;
 }
 __device__ __forceinline__ double min_(double a, double b) { return order_(a) < order_(b) ? a : b; }
 __device__ __forceinline__ double max_(double a, double b) { return order_(a) < order_(b) ? b : a; }
@@ -136,7 +137,7 @@ __device__ __forceinline__ void kern_half_d(double r, double iH, double& w, doub
     w = out ? 0.0 : ww;
     d = out ? 0.0 : dd;
 }
-// a < b, FP64 compared as integers.
+// a < b (of numbers, not NaN), FP64 compared as integers.
 __device__ __forceinline__ bool less_(float a, float b) { return a < b; }
 __device__ __forceinline__ bool less_(double a, double b) { return order_(a) < order_(b); }
 
