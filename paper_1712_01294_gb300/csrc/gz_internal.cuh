@@ -443,12 +443,16 @@ __device__ __forceinline__ void for_candidates_lanes(const Grid& g, const BoxInf
     }
 }
 
-// The FP32 number below a position x in [0, 1] (its leading 24 bits), formed
+// The FP32 number next to a position x towards 0 (its leading 24 bits), formed
 // from its words: a conversion would go through the FP64 pipe, whose rate is
-// 1/64 of FP32's.  (Numbers below 2^-126 give 0 or a denormal.)
+// 1/64 of FP32's.  (Numbers below 2^-126 give 0 or a denormal.)  Positions that
+// are no numbers, or out of FP32's range, give an infinity or NaN, whose
+// distance to anything is no number, so they are near nothing; those outside
+// [0, 1] keep their sign.
 __device__ __forceinline__ float chop(double x) {
-    const int h = max(__double2hiint(x), 0x38000000);
-    return __int_as_float(((h - 0x38000000) << 3) | (int)((unsigned)__double2loint(x) >> 29));
+    const int h = __double2hiint(x);
+    const int m = min(max(h & 0x7fffffff, 0x38000000) - 0x38000000, 0x0ff00000);
+    return __int_as_float((h & 0x80000000) | (m << 3) | (int)((unsigned)__double2loint(x) >> 29));
 }
 __device__ __forceinline__ float chop(float x) { return x; }
 
