@@ -286,6 +286,8 @@ __global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
                 return;
             }
             __syncwarp(gm);
+            bool outside = false;  // (FP64: the prefilter lets candidates just outside through)
+            const T Rc2 = Rc * Rc;
 #pragma unroll
             for (int u = 0; u < E; ++u) {
                 const int k = u * G + gl;
@@ -296,6 +298,28 @@ __global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
                                       mi_diff(q.z, me.z, me.z - T(1)));
                     c_r2[gp][k] = r2;
                     r[u] = dist(r2);
+                    if constexpr (sizeof(T) == 8) outside |= !(r2 < Rc2);
+                }
+            }
+            if constexpr (sizeof(T) == 8) {
+                // taken out (one particle in a thousand), so that every entry's
+                // place, and with it the order of the sums, is the warp form's
+                if (__any_sync(gm, outside)) {
+                    __syncwarp(gm);
+                    if (gl == 0) {
+                        int kept = 0;
+                        for (int k = 0; k < ncache; ++k) {
+                            const T r2 = c_r2[gp][k];
+                            if (!(r2 < Rc2)) continue;
+                            c_r2[gp][kept] = r2;
+                            c_j[gp][kept++] = c_j[gp][k];
+                        }
+                        ncache = kept;
+                    }
+                    ncache = __shfl_sync(gm, ncache, 0, G);
+                    __syncwarp(gm);
+#pragma unroll
+                    for (int u = 0; u < E; ++u) r[u] = u * G + gl < ncache ? dist(c_r2[gp][u * G + gl]) : T(8);
                 }
             }
         }
