@@ -292,7 +292,8 @@ gz_status gz_set_subdomain(gz_ctx* ctx, int64_t n, int64_t n_owned, const uint8_
  * order, may be NULL) the final bins, *active_out (host, may be NULL) the
  * number of active particle-substeps.  Host synchronisation: one per substep
  * (the number of active particles sizes the launches; substeps without one
- * only drift), so the call cannot be captured in a CUDA graph.  Scratch of
+ * only drift), so the call cannot be captured in a CUDA graph: on a stream
+ * that is capturing it fails with GZ_E_CUDA, whatever K.  Scratch of
  * about 150 bytes a particle (FP32) is allocated on the first call.  Every
  * Riemann option of the MFM face applies, and GZ_MFV (O15: the mass shares are
  * exchanged with momentum and energy, m is updated too).  Errors: GZ_E_INVAL

@@ -872,6 +872,13 @@ gz_status gz_step_hier(gz_ctx* ctx, gz_particles* p, int32_t K, double dt_fixed,
     if (K < 0 || K > 20) return fail(ctx, GZ_E_INVAL, "K must be in [0, 20]");
     if (ctx->c.owned) return refuse_subdomain(ctx, "gz_step_hier");
     Ctx& c = ctx->c;
+    // (the host reads counts between substeps; refused before anything is launched)
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    const cudaError_t ec = cudaStreamIsCapturing(c.stream, &capturing);
+    if (ec != cudaSuccess || capturing != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return cuda_check(ctx, ec != cudaSuccess ? ec : cudaErrorStreamCaptureUnsupported, "gz_step_hier");
+    }
     const PassTimer timer{&c};
     long long act = 0;
     cudaError_t e = c.precision == GZ_FP64
