@@ -853,6 +853,7 @@ cudaError_t run_density(Ctx& c, const int* list, const int* nlist, int n) {
         min_count = std::min(min_count, (long long)b.count);
         min_nc = std::min(min_nc, b.nc);
     }
+    if (c.grid_count > 0) min_count = c.grid_count;  // a subdomain: as the whole box
     const int asked = c.params.density_cache, ccap = asked > 0 ? asked : kDensCache;
     const int tcap = asked > 0 ? asked : (min_count >= 32 * 32 * 32 ? 40 : 48);
     c.launches += 2;
