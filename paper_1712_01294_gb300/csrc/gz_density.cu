@@ -570,16 +570,35 @@ __global__ void __launch_bounds__(kOneBlock, 10)
 // (in scan order); later evaluations and the list read only that.  A particle
 // with more of them scans the cells at every evaluation.  Grid-stride over
 // the deferred list, whose length only the device knows.
-// The sums run as in group_eval (FP32: the lanes form the terms of 32 entries,
-// then every lane adds those with r < H in order), so which form iterates a
-// particle does not change its bits.
+// FP32: up to kDensCache entries, which another form could hold, the sums run as
+// in group_eval (the lanes form the terms of 32 entries, then every lane adds
+// those with r < H in order), so which form iterates a particle does not change
+// its H and n; the derivative sum kept for the adjoint is a compensated one.
+// More entries are nobody else's: each lane sums its own and the lanes' sums are
+// added up in FP64 (one chain of 400 terms leaves 2.6e-7 of the derivative sum,
+// the lanes 3e-8).  FP64: the lanes' sums of group_eval.
 constexpr int kWarpDensBlock = 64;
 constexpr int kWarpCache = 512;
 
+// sd: for the iteration; sdk: to keep.
 __device__ __forceinline__ void warp_eval(int lane, int n, const float* r2, float* tw, float* tx, float* ty, float H,
-                                          float& S, float& sd) {
+                                          float& S, float& sd, float& sdk) {
     const float H2 = H * H, iH = 1.f / H;
-    Acc<float> sw;
+    if (n > kDensCache) {
+        Acc<float> w;
+        float d = 0.f;
+        for (int k = lane; k < n; k += 32)
+            if (r2[k] < H2) {
+                float t, x, y;
+                dens_terms2(dist(r2[k]) * iH, t, x, y);
+                w.add(t);
+                d = fmaf(y, x, d);
+            }
+        S = (float)group_add<32>(0xffffffffu, (double)w.s - (double)w.c);
+        sd = sdk = (float)group_add<32>(0xffffffffu, (double)d);
+        return;
+    }
+    Acc<float> sw, sk;
     sd = 0.f;
     for (int k0 = 0; k0 < n; k0 += 32) {
         const int k = k0 + lane;
@@ -596,13 +615,15 @@ __device__ __forceinline__ void warp_eval(int lane, int n, const float* r2, floa
         for (int s = 0; s < hits; ++s) {
             sw.add(tw[s]);
             sd = fmaf(ty[s], tx[s], sd);
+            sk.add(__fmul_rn(ty[s], tx[s]));
         }
         __syncwarp();
     }
     S = sw.fvalue();
+    sdk = sk.fvalue();
 }
 __device__ __forceinline__ void warp_eval(int lane, int n, const double* r2, double*, double*, double*, double H,
-                                          double& S, double& sd) {
+                                          double& S, double& sd, double& sdk) {
     // (lane l's four-entry stride as in group_eval: lanes 4 m + c add class c)
     const double iH = 1.0 / H;
     double a = 0.0, b = 0.0;
@@ -617,7 +638,7 @@ __device__ __forceinline__ void warp_eval(int lane, int n, const double* r2, dou
     a = group_add<kLanes>(0xffffffffu, a);
     b = group_add<kLanes>(0xffffffffu, b);
     S = 2.0 * __shfl_sync(0xffffffffu, a, 0);
-    sd = 6.0 * __shfl_sync(0xffffffffu, b, 0);
+    sd = sdk = 6.0 * __shfl_sync(0xffffffffu, b, 0);
 }
 
 // An evaluation straight from the cells (more candidates than the warp's cache
@@ -668,7 +689,7 @@ __global__ void __launch_bounds__(kWarpDensBlock)
         const P4<T> me = s.pos[i];
         bool bad;  // (flagged by k_density)
         T H = h_start<T>(s.h[i], bx, p, bad);
-        T Rc = T(-1), Hev = H, Sv = T(0), sdv = T(0);
+        T Rc = T(-1), Hev = H, Sv = T(0), sdv = T(0), sdk = T(0);
         int ncache = 0, it;
         HIter<T> b;
         bool conv = false;
@@ -686,9 +707,11 @@ __global__ void __launch_bounds__(kWarpDensBlock)
                 __syncwarp();
             }
             if (ncache <= kWarpCache)
-                warp_eval(lane, ncache, c_r2, t_w, t_x, t_y, H, Sv, sdv);
-            else
+                warp_eval(lane, ncache, c_r2, t_w, t_x, t_y, H, Sv, sdv, sdk);
+            else {
                 warp_eval_cells(g, bx, s.pos, i, me, lane, H, Sv, sdv);
+                sdk = sdv;
+            }
             Hev = H;
             if (h_step(b, H, Sv, sdv, p, it == p.max_iter)) {
                 conv = true;
@@ -716,7 +739,7 @@ __global__ void __launch_bounds__(kWarpDensBlock)
         if (lane == 0) {
             s.h[i] = Hev;
             s.n[i] = n_of(Sv, Hev);
-            if (s.sd) s.sd[i] = sdv;
+            if (s.sd) s.sd[i] = sdk;
             iters[i] = it;
             ncount[i] = cnt;
             if (!conv) {
