@@ -619,6 +619,7 @@ gz_status create_ctx(const gz_params* params, int32_t nboxes, const int64_t* cou
         c.hboxes[b].first = first;
         c.hboxes[b].count = (int)counts[b];
         c.hboxes[b].key_off = (unsigned)keys;
+        c.hboxes[b].wide = wide_cells(H0, nc);
         first += (int)counts[b];
         cells += (long long)nc * nc * nc;
         keys += 1ll << (3 * ceil_log2(nc));

@@ -215,15 +215,10 @@ __device__ __forceinline__ bool h_step(HIter<double>& b, double& H, double S, do
     return false;
 }
 
-// Whether a support spans so many cells that scanning its window is left to a
-// warp from the start (a blast's emptied centre: up to thousands of mostly
-// empty cells, which one thread or a group of four would walk while the rest
-// of the block waits).  In cells: 1.7 (2.1: ensemble late in the run 1318 us
-// instead of 1292, Sedov 64^3 370 instead of 364; 1.4: 1304 and 387); the mean
-// support is one.
+// Whether a particle's scan is left to a warp from the start (wide_cells).
 template <typename T>
-__device__ __forceinline__ bool wide(T R, int nc) {
-    return (float)R * (float)nc > 1.7f;
+__device__ __forceinline__ bool wide(T R, const BoxInfo& bx) {
+    return (float)R * (float)bx.nc > bx.wide;
 }
 
 // Starting H of particle i: its guess, or (flagged by the caller) the box's
@@ -275,7 +270,7 @@ __global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
         if (!(H <= Rc)) {  // first evaluation, or grown past the cache radius
             Rc = dens_cache_radius<T>(H, p);
             __syncwarp(gm);
-            ncache = wide(Rc, bx.nc) ? ccap + 1 : group_scan<T, G>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, gl, gm, ccap,
+            ncache = wide(Rc, bx) ? ccap + 1 : group_scan<T, G>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, gl, gm, ccap,
                                             [&](int k, int j) {
                                                 if (k < kDensCache) c_j[gp][k] = (unsigned)j;
                                             });
@@ -427,7 +422,7 @@ __device__ __forceinline__ void scan_inside(const int2* cells, int nc, const int
 // inside its box (what scan_inside asks for).
 __device__ __forceinline__ bool warp_inside(const BoxInfo& bx, const P4<float>& me, float R, int (&lo)[3],
                                             int (&hi)[3]) {
-    bool in = R >= 0.f && !wide(R, bx.nc) && 2.f * R + 2.f / (float)bx.nc < 0.5f;
+    bool in = R >= 0.f && !wide(R, bx) && 2.f * R + 2.f / (float)bx.nc < 0.5f;
     const float c3[3] = {me.x, me.y, me.z};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -483,7 +478,7 @@ __global__ void __launch_bounds__(kOneBlock, 10)
             c_j[k][t] = (unsigned)j;
             ncache += h;
         });
-    } else if (wide(Rc, bx.nc)) {
+    } else if (wide(Rc, bx)) {
         ncache = kCache + 1;
     } else if constexpr (kInside) {
         ncache = dens_fill<kCache>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, c_r2, c_j, t);
@@ -503,7 +498,7 @@ __global__ void __launch_bounds__(kOneBlock, 10)
     for (it = 1; it <= p.max_iter; ++it) {
         if (H > Rc) {  // grown past the cache radius: rescan
             Rc = dens_cache_radius<float>(H, p);
-            ncache = wide(Rc, bx.nc) ? kCache + 1 : dens_fill<kCache>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, c_r2, c_j, t);
+            ncache = wide(Rc, bx) ? kCache + 1 : dens_fill<kCache>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, c_r2, c_j, t);
         }
         if (ncache > kCache) {  // left to k_density_warp
             defer[atomicAdd(ndefer, 1)] = i;

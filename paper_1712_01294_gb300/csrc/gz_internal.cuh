@@ -35,7 +35,18 @@ struct BoxInfo {
     int first;       // first particle (sorted order == caller order per box)
     int count;       // particles in the box
     unsigned key_off;  // first sort key of this box (keys: Morton index of the cell + key_off)
+    float wide;        // cells from which a support counts as wide (wide_cells)
 };
+
+// A support spanning more cells than this is left to a warp by the density
+// pass: its scan is mostly of empty cells (a blast's emptied centre: up to
+// thousands, which one thread or a group of four would walk while the rest of
+// the block waits).  In cells of the mean support radius H0 or larger: 1.7 (2.1:
+// ensemble late in the run 1318 us instead of 1292, Sedov 64^3 370 instead of
+// 364; 1.4: 1304 and 387).  Finer cells hold fewer particles each, and a support
+// of H0 then spans H0 nc of them: 1.7 H0 (1.7 cells sent every particle there
+// once cells were under 0.6 H0, 64^3 at 0.5: 946 us instead of 296).
+inline float wide_cells(double H0, int nc) { return (float)(1.7 * (H0 * nc > 1.0 ? H0 * nc : 1.0)); }
 
 // Scalar parameters passed by value to kernels.
 struct KParams {

@@ -68,8 +68,8 @@ cudaError_t scratch_on_current_device(void** out) {
 
 // The one-box table, written on the device from values passed by value (no
 // host buffer is referenced by the enqueued work).
-__global__ void k_noalloc_box(BoxInfo* boxes, int nc, int count) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) boxes[0] = BoxInfo{nc, 0, 0, count, 0u};
+__global__ void k_noalloc_box(BoxInfo* boxes, int nc, int count, float wide) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) boxes[0] = BoxInfo{nc, 0, 0, count, 0u, wide};
 }
 
 // Copies the status bits of this call to the caller's word.  The lists are
@@ -157,7 +157,7 @@ gz_status run(const gz_params* prm, int N, gz_particles* p, void* n_out, int32_t
     // deferred count is reset by the density launcher)
     cudaError_t e = cudaMemsetAsync(c.box_of, 0, 4 * (size_t)N, stream);
     if (e == cudaSuccess) {
-        k_noalloc_box<<<1, 32, 0, stream>>>(c.boxes, nc, N);
+        k_noalloc_box<<<1, 32, 0, stream>>>(c.boxes, nc, N, wide_cells(H0, nc));
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(c.status, 0, sizeof(DevStatus), stream);
