@@ -647,7 +647,7 @@ gz_status create_ctx(const gz_params* params, int32_t nboxes, const int64_t* cou
         {(void**)&c.keys, 4 * Nz},        {(void**)&c.keys_alt, 4 * Nz},
         {(void**)&c.vals, 4 * Nz},        {(void**)&c.vals_alt, 4 * Nz},
         {(void**)&c.hist, 4 * sort_sums_len(N, keys, counted)},
-        {(void**)&c.kcount, counted ? 4 * (size_t)keys : 0},
+        {(void**)&c.kcount, counted ? 4 * (size_t)(keys + kCountExtra) : 0},
         {(void**)&c.kstart, counted ? 4 * (size_t)keys : 0},
         {(void**)&c.box_of, 4 * Nz},      {(void**)&c.boxes, sizeof(BoxInfo) * (size_t)nboxes},
         {(void**)&c.cells, sizeof(int2) * (size_t)cells},

@@ -37,6 +37,8 @@ Sorted<T> sorted_view(Ctx& c);
 // particles has more).
 constexpr long long kKeysPerParticle = 8;
 inline bool counting_sort_fits(long long N, long long keys) { return keys <= kKeysPerParticle * N + 65536; }
+// Words behind the counting sort's keys counts (k_cs_count).
+constexpr int kCountExtra = 2;
 // Partial sums (32-bit words) the sort needs.
 size_t sort_sums_len(long long N, long long keys, bool counted);
 

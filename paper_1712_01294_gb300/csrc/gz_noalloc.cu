@@ -29,7 +29,7 @@ constexpr size_t kSumsLen = 64;     // partial sums of the counting sort's scan
 // Worst case (FP64) of every slice the density pass touches.
 constexpr size_t kScratchBytes =
     4 * al(4 * (size_t)kMaxN)                          // keys, keys_alt, vals, vals_alt
-    + al(4 * kSumsLen) + 2 * al(4 * kMaxKeys)          // counting sort
+    + al(4 * kSumsLen) + al(4 * (kMaxKeys + kCountExtra)) + al(4 * kMaxKeys)  // counting sort
     + al(4 * (size_t)kMaxN)                            // box of each particle
     + al(sizeof(BoxInfo))                              // box table
     + al(sizeof(int2) * (size_t)kMaxCells)             // cell ranges
@@ -42,7 +42,7 @@ constexpr size_t kScratchBytes =
     + al(sizeof(DevStatus));
 
 // The scratch itself: every GPU that loads the library holds these bytes
-// (8,520,704 B, about 8.5 MB) until the process exits.  All calls share it.
+// (8,520,960 B, about 8.5 MB) until the process exits.  All calls share it.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 std::mutex g_mu;
@@ -120,7 +120,7 @@ gz_status run(const gz_params* prm, int N, gz_particles* p, void* n_out, int32_t
     c.vals = (unsigned*)take(4 * Nz);
     c.vals_alt = (unsigned*)take(4 * Nz);
     c.hist = (unsigned*)take(4 * kSumsLen);
-    c.kcount = (unsigned*)take(4 * kMaxKeys);
+    c.kcount = (unsigned*)take(4 * (kMaxKeys + kCountExtra));
     c.kstart = (unsigned*)take(4 * kMaxKeys);
     c.box_of = (int*)take(4 * Nz);
     c.boxes = (BoxInfo*)take(sizeof(BoxInfo));
@@ -154,7 +154,7 @@ gz_status run(const gz_params* prm, int N, gz_particles* p, void* n_out, int32_t
 
     // the scratch keeps the previous call's contents: reset what must start
     // clean (the box of every particle, the box table, the status word; the
-    // deferred count is reset by the density launcher)
+    // deferred count is reset by the permutation)
     cudaError_t e = cudaMemsetAsync(c.box_of, 0, 4 * (size_t)N, stream);
     if (e == cudaSuccess) {
         k_noalloc_box<<<1, 32, 0, stream>>>(c.boxes, nc, N, wide_cells(H0, nc));

@@ -74,7 +74,8 @@ __global__ void k_keys(int N, const T* __restrict__ x, const T* __restrict__ y,
 
 // ------------------------------------------------------- counting sort
 // Key of every particle and its arrival number in its key's count (any order:
-// k_permute puts the particles of a cell in caller order).
+// k_permute puts the particles of a cell in caller order).  Behind the keys'
+// counts: the number of crowded keys and of k_cs_place's finished blocks.
 template <typename T>
 __global__ void k_cs_count(int N, const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z,
                            const int64_t* __restrict__ id, const int* __restrict__ box_of,
@@ -123,13 +124,18 @@ __global__ void __launch_bounds__(kScanThreads)
     if (threadIdx.x == 0) sums[blockIdx.x] = t;
 }
 
-// First sorted index of every key, and the range of every cell (empty ones
-// included).  sums: the tiles' sums, or null when every block adds the counts
-// before its tile itself.
+// Particles of one key beyond which k_permute's walk of the cell (its number of
+// steps squared) costs more than k_cs_place's last block sorting the cell.  The
+// whole sort with every particle in one cell, walked / sorted: 32^3 584 / 153 us,
+// 64^3 10314 / 507, 128^3 - / 6257 (a lattice: 19, 25 and 100).
+constexpr int kCrowd = 16384;
+
+// First sorted index of every key, the range of every cell (empty ones
+// included) and the list of the crowded keys.  sums: the tiles' sums, or null
+// when every block adds the counts before its tile itself.
 __global__ void __launch_bounds__(kScanThreads)
-    k_cs_scan(long long K, const unsigned* count, const unsigned* sums,
-              const BoxInfo* boxes, int nboxes, unsigned* start,
-              int2* cells) {
+    k_cs_scan(long long K, unsigned* count, const unsigned* sums, const BoxInfo* boxes, int nboxes,
+              unsigned* start, int2* cells, unsigned* crowd) {
     after_previous();
     __shared__ unsigned sh[kScanThreads / 32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -177,6 +183,7 @@ __global__ void __launch_bounds__(kScanThreads)
             next = b + 1 < nboxes ? boxes[b + 1].key_off : 0xffffffffu;
         }
         start[k] = s;
+        if (c[u] > kCrowd) crowd[atomicAdd(count + K, 1u)] = (unsigned)k;
         const unsigned mort = (unsigned)k - bx.key_off;
         const int cx = compact3(mort), cy = compact3(mort >> 1), cz = compact3(mort >> 2);
         if (cx < bx.nc && cy < bx.nc && cz < bx.nc)
@@ -185,11 +192,69 @@ __global__ void __launch_bounds__(kScanThreads)
     }
 }
 
-__global__ void k_cs_place(int N, const unsigned* key, const unsigned* slot,
-                           const unsigned* start, unsigned* order) {
+// The n distinct caller indices (below N) of a crowded cell in increasing order,
+// by one block: a bitmap of a window of indices after another, whose set bits
+// come out in order.
+constexpr int kCrowdWords = 8192;
+__device__ __forceinline__ void sort_crowd(unsigned* seg, unsigned* tmp, int n, int N) {
+    __shared__ unsigned bits[kCrowdWords];
+    __shared__ int wsum[32];
+    const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5;
+    const int per = kCrowdWords / T;
+    int done = 0;
+    for (unsigned base = 0; base < (unsigned)N; base += 32 * kCrowdWords) {
+        for (int w = t; w < kCrowdWords; w += T) bits[w] = 0;
+        __syncthreads();
+        for (int e = t; e < n; e += T) {
+            const unsigned v = __ldcg(seg + e) - base;  // (written by other blocks)
+            if (v < 32u * kCrowdWords) atomicOr(&bits[v >> 5], 1u << (v & 31));
+        }
+        __syncthreads();
+        int mine = 0;
+        for (int w = t * per; w < (t + 1) * per; ++w) mine += __popc(bits[w]);
+        int x = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
+        __syncthreads();
+        int at = done + x - mine;
+        for (int w = 0; w < T / 32; ++w) {
+            if (w < warp) at += wsum[w];
+            done += wsum[w];
+        }
+        for (int w = t * per; w < (t + 1) * per; ++w)
+            for (unsigned b = bits[w]; b; b &= b - 1) tmp[at++] = base + 32u * w + (unsigned)(__ffs(b) - 1);
+        __syncthreads();
+    }
+    for (int e = t; e < n; e += T) seg[e] = tmp[e];
+    __syncthreads();
+}
+
+// Particles by key, in any order within a cell, except in crowded cells (a
+// state that went to NaN is binned in one): once every block has placed its
+// particles, the last one puts those in caller order (tmp: N words).  Without
+// crowded cells a block reads one word more.
+__global__ void k_cs_place(int N, const unsigned* key, const unsigned* slot, const unsigned* start, unsigned* order,
+                           unsigned* count, long long K, const unsigned* crowd, unsigned* tmp) {
     after_previous();
+    __shared__ bool last;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int crowds = (int)count[K];
     if (i < N) order[start[key[i]] + slot[i]] = (unsigned)i;
+    if (crowds == 0) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(count + K + 1, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int c = 0; c < crowds; ++c) {
+        const unsigned k = crowd[c], a = start[k];
+        sort_crowd(order + a, tmp + a, (int)count[k], N);
+    }
 }
 
 // ----------------------------------------------------------- radix sort
@@ -324,7 +389,7 @@ __global__ void k_rs_scatter(const unsigned* __restrict__ kin, const unsigned* _
 // The state in sorted order.  kCounted: p walks k_cs_place's order, a cell's
 // particles in any order; a particle's place is its cell's start plus the
 // number of the cell's particles before it in caller order (a loop over the
-// cell, fewer steps than the density pass's scan of it), and the sorted keys
+// cell; a crowded one is in order already), and the sorted keys
 // and indices are written.  Else they are given, and the cells' ranges
 // are written from the keys' boundaries (cells zeroed before).
 template <typename T, bool kCounted>
@@ -343,9 +408,11 @@ __global__ void k_permute(int N, unsigned* skeys, unsigned* svals,
     if constexpr (kCounted) {
         src = order[q];
         key = key_in[src];
-        const int a = (int)start[key], e = a + (int)count[key];
-        i = a;
-        for (int k = a; k < e; ++k) i += order[k] < src;
+        const int n = (int)count[key], a = (int)start[key], e = a + n;
+        if (n <= kCrowd) {
+            i = a;
+            for (int k = a; k < e; ++k) i += order[k] < src;
+        }
         skeys[i] = key;
         svals[i] = src;
     } else {
@@ -430,15 +497,19 @@ static cudaError_t counting_sort(Ctx& c, const gz_particles& p, const void* n_in
     const long long K = c.total_keys;
     cudaStream_t st = c.stream;
     unsigned* order = (unsigned*)c.defer;  // (free until the density pass)
-    cudaMemsetAsync(c.kcount, 0, 4 * (size_t)K, st);
+    cudaMemsetAsync(c.kcount, 0, 4 * (size_t)(K + kCountExtra), st);
     k_cs_count<T><<<blocks(N, 256), 256, 0, st>>>(N, (const T*)p.x, (const T*)p.y, (const T*)p.z, p.id, c.box_of,
                                                    c.boxes, c.kcount, c.keys_alt, c.vals_alt, c.status);
     const int tiles = (int)((K + kScanTile - 1) / kScanTile);
     const bool direct = tiles <= kScanDirect;
     if (!direct) launch_next(c, k_cs_sums, tiles, kScanThreads, K, c.kcount, c.hist);
     launch_next(c, k_cs_scan, tiles, kScanThreads, K, c.kcount, direct ? nullptr : c.hist, c.boxes, c.nboxes, c.kstart,
-                c.cells);
-    launch_next(c, k_cs_place, blocks(N, 256), 256, N, c.keys_alt, c.vals_alt, c.kstart, order);
+                c.cells, c.keys);
+    // (c.keys and c.vals are k_permute's to write: room for the crowded keys and
+    // their sort; large launches have blocks that sort faster)
+    const int pt = N < (1 << 17) ? 256 : 1024;
+    launch_next(c, k_cs_place, blocks(N, pt), pt, N, c.keys_alt, c.vals_alt, c.kstart, order, c.kcount, K, c.keys,
+                c.vals);
     launch_next(c, k_permute<T, true>, blocks(N, 256), 256, N, c.keys, c.vals, order, c.keys_alt, c.kcount, c.kstart, p,
                 n_in, c.box_of, c.boxes, sorted_view<T>(c), c.cells, c.ndefer);
     c.launches += direct ? 4 : 5;
