@@ -215,10 +215,17 @@ __device__ __forceinline__ bool h_step(HIter<double>& b, double& H, double S, do
     return false;
 }
 
-// Whether a particle's scan is left to a warp from the start (wide_cells).
+// Whether a support is wide (wide_cells).
 template <typename T>
 __device__ __forceinline__ bool wide(T R, const BoxInfo& bx) {
     return (float)R * (float)bx.nc > bx.wide;
+}
+// Whether a particle's scan is left to a warp from the start.  A position outside
+// the box (or none) sees no candidates: nothing to share.
+template <typename T>
+__device__ __forceinline__ bool to_warp(T R, const BoxInfo& bx, const P4<T>& me) {
+    return wide(R, bx) && me.x >= T(0) && me.x <= T(1) && me.y >= T(0) && me.y <= T(1) && me.z >= T(0) &&
+           me.z <= T(1);
 }
 
 // Starting H of particle i: its guess, or (flagged by the caller) the box's
@@ -270,7 +277,7 @@ __global__ void __launch_bounds__(kDensBlock, sizeof(T) == 4 ? 7 : 1)
         if (!(H <= Rc)) {  // first evaluation, or grown past the cache radius
             Rc = dens_cache_radius<T>(H, p);
             __syncwarp(gm);
-            ncache = wide(Rc, bx) ? ccap + 1 : group_scan<T, G>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, gl, gm, ccap,
+            ncache = to_warp(Rc, bx, me) ? ccap + 1 : group_scan<T, G>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, gl, gm, ccap,
                                             [&](int k, int j) {
                                                 if (k < kDensCache) c_j[gp][k] = (unsigned)j;
                                             });
@@ -478,7 +485,7 @@ __global__ void __launch_bounds__(kOneBlock, 10)
             c_j[k][t] = (unsigned)j;
             ncache += h;
         });
-    } else if (wide(Rc, bx)) {
+    } else if (to_warp(Rc, bx, me)) {
         ncache = kCache + 1;
     } else if constexpr (kInside) {
         ncache = dens_fill<kCache>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, c_r2, c_j, t);
@@ -498,7 +505,7 @@ __global__ void __launch_bounds__(kOneBlock, 10)
     for (it = 1; it <= p.max_iter; ++it) {
         if (H > Rc) {  // grown past the cache radius: rescan
             Rc = dens_cache_radius<float>(H, p);
-            ncache = wide(Rc, bx) ? kCache + 1 : dens_fill<kCache>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, c_r2, c_j, t);
+            ncache = to_warp(Rc, bx, me) ? kCache + 1 : dens_fill<kCache>(g, bx, s.pos, i, me.x, me.y, me.z, Rc, c_r2, c_j, t);
         }
         if (ncache > kCache) {  // left to k_density_warp
             defer[atomicAdd(ndefer, 1)] = i;

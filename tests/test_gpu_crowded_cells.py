@@ -6,12 +6,13 @@ from gpu_common import cast_state, device
 from paper_1712_01294_gb300 import inputs as I
 
 
-def _time(m, n):
+def _time(m, n, bad=True):
     import torch
     q = cast_state(I.sod(n, seed=3), 1)
     d = device(q, 1)
-    for k in ("x", "y", "z"):
-        d[k].fill_(float("nan"))
+    if bad:
+        for k in ("x", "y", "z"):
+            d[k].fill_(float("nan"))
     ctx = m.Context([q.N], m.default_params())
     best = 1e9
     for _ in range(4):
@@ -73,3 +74,14 @@ def test_crowded_cells_keep_caller_order(n):
     for c in cell:
         assert (np.diff(c)[same] == 0).all()  # one key, one cell
     assert np.bincount(keys).max() > 16384
+
+
+@pytest.mark.gpu
+def test_positions_that_are_no_numbers_keep_to_one_thread():
+    # they see no candidates, so their supports grow to the limit; a warp for
+    # each took the pass 4.6 ms at 64^3, where a lattice takes 0.15
+    import paper_1712_01294_gb300 as m
+    _time(m, 64)
+    nan, lattice = _time(m, 64), _time(m, 64, bad=False)
+    print(f"64^3: no positions {nan:.3f} ms, lattice {lattice:.3f} ms")
+    assert nan < 8 * lattice
