@@ -43,21 +43,21 @@ struct AdjSums {
 // Adjoint of particle a's share of the pair (a, b).  wp = dpbar_a - dpbar_b
 // and wE = dEbar_a - dEbar_b weight the pair's rate contributions.  The
 // forward is re-evaluated as pair_rates forms it (its symmetric star state,
-// in which v_f drops out), so every branch matches; Wh: half_state of a.
+// in which v_f drops out), so every branch matches; ia: half_inc of a.
 // Divisions are products with the reciprocals the forward takes anyway: FP64
 // is bound by its pipe (977 operations a pair where the canonical L/R order,
 // v_f and a's own terms were carried through each pair, 3.88 ms at 40^3; 486
 // here, 1.93 ms).
 template <typename T>
-__device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)[kRecord], const T (&Wh)[5], bool aL,
+__device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)[kRecord], const T (&ia)[5], bool aL,
                                              T hdt, T gam, const T* wp, T wE, AdjSums<T>& s) {
     // ---- forward (same operations as pair_rates)
     const T dx = mi_diff(b[0], a[0], a[0] - T(1));
     const T dy = mi_diff(b[1], a[1], a[1] - T(1));
     const T dz = mi_diff(b[2], a[2], a[2] - T(1));
     const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
-    const T ir = rsq_(r2);
-    const T r = mul_rn(r2, ir);
+    T r, ir;
+    roots_(r2, r, ir);
     T wa, wb, da, db;
     kern_half_d(r, a[4], wa, da);
     kern_half_d(r, b[4], wb, db);
@@ -73,13 +73,14 @@ __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)
     for (int k = 0; k < 3; ++k) A[k] = add_rn(mul_rn(ca, ua[k]), mul_rn(cb, ub[k]));
     const T Aq = sep2(A[0], A[1], A[2]);
     if (!pos_(Aq - Tiny<T>::sq)) return;
-    const T iA = rsq_(Aq);
+    T Ah, iA;
+    roots_(Aq, Ah, iA);
     const T n[3] = {A[0] * iA, A[1] * iA, A[2] * iA};
     const T iHs = rcp_(a[3] + b[3]);
     const T sa = a[3] * iHs, sb = b[3] * iHs;
-    T Ga[5], Gb[5], Da[5], Db[5], Wb[5];
+    T Ga[5], Gb[5], Da[5], Db[5], ib[5];
     int ka[5], kb[5];  // clamp sides: 0 inside, -1 at the lower bound, +1 at the upper
-    half_state(b, hdt, gam, Wb);
+    half_inc(b, hdt, gam, ib);
     const T Wa0[5] = {a[6], a[8], a[9], a[10], a[7]};
     const T Wb0[5] = {b[6], b[8], b[9], b[10], b[7]};
 #pragma unroll
@@ -87,7 +88,7 @@ __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)
         Da[f] = dot3(a[11 + 3 * f], a[12 + 3 * f], a[13 + 3 * f], dx, dy, dz);
         Db[f] = dot3(b[11 + 3 * f], b[12 + 3 * f], b[13 + 3 * f], dx, dy, dz);
         const T lo = min_(Wa0[f], Wb0[f]), hi = max_(Wa0[f], Wb0[f]);
-        const T Fa = fma(sa, Da[f], Wh[f]), Fb = fma(-sb, Db[f], Wb[f]);
+        const T Fa = face_value(Wa0[f], sa, Da[f], ia[f]), Fb = face_value(Wb0[f], -sb, Db[f], ib[f]);
         ka[f] = less_(Fa, lo) ? -1 : (less_(hi, Fa) ? 1 : 0);
         kb[f] = less_(Fb, lo) ? -1 : (less_(hi, Fb) ? 1 : 0);
         Ga[f] = ka[f] < 0 ? lo : (ka[f] > 0 ? hi : Fa);
@@ -116,12 +117,14 @@ __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)
     T sc, isc;  // (the scaling of pair_rates)
     pow2_near(den, sc, isc);
     const T mas = ma * sc, mbs = mb * sc, idens = iden * isc;
-    const T psr = fma(-(mas * mb), du, add_rn(mul_rn(mas, Gb[4]), -mul_rn(mbs, Ga[4]))) * idens;
-    const T X = fma(-msum, du, T(2) * (Gb[4] - Ga[4])) * iden;
+    const T dP = Gb[4] - Ga[4];
+    T num;
+    const T psr = star_pressure(Ga[4], Gb[4], dP, du, mas, mbs, mb, idens, num);
+    const T X = fma(-msum, du, T(2) * dP) * iden;
     const T S = T(0.5) * (us + X);
     const bool neg = psr < T(0);
     const T ps = neg ? T(0) : psr;
-    const T Am = T(2) * (Aq * iA);
+    const T Am = T(2) * Ah;
     // ---- reverse: J = -ps (wp . A + wE S |A|)
     const T wA = T(2) * dot3(wp[0], wp[1], wp[2], A[0], A[1], A[2]);
     const T wS = wE * S;
@@ -193,7 +196,7 @@ __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)
             }
         }
     }
-    // face states: F_a = Wh_a + s_a g_a . d ; F_b = Wh_b - s_b g_b . d
+    // face states: F_a = W_a + s_a g_a . d + inc_a ; F_b = W_b - s_b g_b . d + inc_b
     T bd[3] = {T(0), T(0), T(0)}, b_sa = T(0), b_sb = T(0);
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
@@ -248,8 +251,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 1)
     const long long idi = sid[i];
     const T hdt = p.hancock ? (T)(0.5 * dt_use[sbox[i]]) : T(0);
     const T gam = (T)p.gamma;
-    T Wh[5];
-    half_state(a, hdt, gam, Wh);
+    T ia[5];
+    half_inc(a, hdt, gam, ia);
     T wi[4];
     load4(wgt + 4 * (size_t)i, wi);
     AdjSums<T> s;
@@ -270,10 +273,10 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 1)
             T wj[4];
             load4(wgt + 4 * (size_t)j, wj);
             const T wp[3] = {wi[0] - wj[0], wi[1] - wj[1], wi[2] - wj[2]};
-            pair_adjoint(a, b, Wh, idi < sid[j], hdt, gam, wp, wi[3] - wj[3], s);
+            pair_adjoint(a, b, ia, idi < sid[j], hdt, gam, wp, wi[3] - wj[3], s);
         }
     }
-    // the half-step primitives: Wh = W + (dt/2)(-rho div v, -grad P/rho, -gamma P div v)
+    // the half-step primitives: W + (dt/2)(-rho div v, -grad P/rho, -gamma P div v)
     const T div = (a[11 + 3] + a[11 + 7]) + a[11 + 11];
     const T irho = pdiv(T(1), a[6]);
     const T e = -hdt * div, k = -hdt * irho;
@@ -562,8 +565,8 @@ __global__ void __launch_bounds__(128)
         if (k0 + u >= cnt) break;
         const T dx = dx4[u], dy = dy4[u], dz = dz4[u];
         const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
-        const T ir = rsq_(r2), r = mul_rn(r2, ir);
-        T w, dw;
+        T r, ir, w, dw;
+        roots_(r2, r, ir);
         kern_half_d(r, iH, w, dw);
         const P4<T> pj = pv[u];
         const T df[5] = {pj.x - Wi[0], pj.y - Wi[1], pj.z - Wi[2], pj.w - Wi[3], Pv[u] - Wi[4]};
@@ -637,9 +640,10 @@ __global__ void __launch_bounds__(128)
             T sd[32];  // record 0-27 (and 4 limiter values, unused here)
             load_row32<32>(R, sd);
             const T r2m = max_(r2, Tiny<T>::sq);
-            const T ir = rsq_(r2m), iH = rcp_(Hi);
-            T w, dw;
-            kern_half_d(mul_rn(r2m, ir), iH, w, dw);
+            const T iH = rcp_(Hi);
+            T r, ir, w, dw;
+            roots_(r2m, r, ir);
+            kern_half_d(r, iH, w, dw);
             const T df[5] = {Wj[0] - sd[22], Wj[1] - sd[23], Wj[2] - sd[24], Wj[3] - sd[25], Wj[4] - sd[26]};
             T psi, t[5], psib, db[3];
             pair_grad_adj(sd, sd + 15, T(2) * sd[21], w, dw, ir, iH, dx, dy, dz, df, psi, t, psib, db);
@@ -725,9 +729,10 @@ __global__ void __launch_bounds__(128)
             if (k0 + u >= cnt) break;
             const P4<T> qj = qv[u];
             const T dx = mi_diff(qj.x, xi, xim1), dy = mi_diff(qj.y, yi, yim1), dz = mi_diff(qj.z, zi, zim1);
-            const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq), ir = rsq_(r2);
-            T w, dw;
-            kern_half_d(mul_rn(r2, ir), iH, w, dw);
+            const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
+            T r, ir, w, dw;
+            roots_(r2, r, ir);
+            kern_half_d(r, iH, w, dw);
             const T c = kappa2 * dw * ir;
             xb[0] -= c * dx;
             xb[1] -= c * dy;
@@ -768,9 +773,9 @@ __global__ void __launch_bounds__(128)
                 T r2 = sep2(dx, dy, dz);
                 if (!less_(r2, mi.w * mi.w)) continue;
                 r2 = max_(r2, Tiny<T>::sq);
-                const T ir = rsq_(r2);
-                T w, dw;
-                kern_half_d(mul_rn(r2, ir), rcp_(mi.w), w, dw);
+                T r, ir, w, dw;
+                roots_(r2, r, ir);
+                kern_half_d(r, rcp_(mi.w), w, dw);
                 const T c = T(2) * kap[i] * dw * ir;
                 xb[0] += c * dx;
                 xb[1] += c * dy;

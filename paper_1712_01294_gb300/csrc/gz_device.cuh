@@ -37,12 +37,16 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 __device__ __forceinline__ float pdiv(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double pdiv(double a, double b) { return a / b; }
 
-// Reciprocal and reciprocal square root of the flux pass, for normal positive
-// arguments.  FP32: the hardware approximations (2 ulp), without the range
-// scaling the library forms add around them.  FP64: the hardware's 20-bit
+// Reciprocal, reciprocal square root and both roots for the pair passes.
+// FP32: the hardware approximations (2 ulp), without the range scaling the
+// library forms add around them; normal arguments.  FP64: the hardware's 20-bit
 // start and one step of third order, y (1 + e + e^2) with e = 1 - x y, and
-// y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 (the binomial series of 1/(1 - e)
-// and (1 - e)^(-1/2)): 3 and 5 FP64 operations, to the last place or two.
+// y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 (the binomial series of 1/(1 - e) and
+// (1 - e)^(-1/2)), e formed to more than 53 bits: within 0.51 ulp, for |x| in
+// [2^-1000, 2^1000], negative x too for the reciprocal.  The square root is
+// x y with one correction (x - s^2) y / 2, as accurate: pairs' distances enter
+// every face, and x y alone (1 ulp) made FP64 rates 10 % less accurate than
+// CUDA's sqrt does.
 __device__ __forceinline__ float rcp_(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -62,8 +66,26 @@ __device__ __forceinline__ double rcp_(double x) {
 __device__ __forceinline__ double rsq_(double x) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-(x * y), y, 1.0);
+    const double h = __dmul_rn(x, y);
+    const double e = fma(-fma(x, y, -h), y, fma(-h, y, 1.0));
     return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+// s = sqrt(x), y = 1/s.
+__device__ __forceinline__ void roots_(float x, float& s, float& y) {
+    y = rsq_(x);
+    s = __fmul_rn(x, y);
+}
+__device__ __forceinline__ void roots_(double x, double& s, double& y) {
+    y = rsq_(x);
+    const double r = __dmul_rn(x, y);
+    s = fma(fma(-r, r, x), 0.5 * y, r);
+}
+// a / b with y = rcp_(b).  FP64: one correction, so that the quotient rounds
+// about once, like a division.
+__device__ __forceinline__ float quot_(float a, float, float y) { return __fmul_rn(a, y); }
+__device__ __forceinline__ double quot_(double a, double b, double y) {
+    const double q = __dmul_rn(a, y);
+    return fma(fma(-q, b, a), y, q);
 }
 // min and max of two numbers.  FP64: compared as integers, which leaves the FP64
 // pipe alone; a negative number's integer is mirrored, so that -0 and +0 are one
@@ -545,24 +567,43 @@ __device__ __forceinline__ bool pair_order(int i, int j, long long idi, const lo
         return i < j;
 }
 
-// Primitives of a record (rho, v, P) at the half step: W plus the Hancock
-// increments of O11, (dt/2)(-rho div v, -grad P / rho, -gamma P div v); hdt = 0
-// without them.  Both particles of a pair form a particle's values with these
-// same operations.
+// Hancock increments of a record's primitives (rho, v, P) to the half step (O11),
+// (dt/2)(-rho div v, -grad P / rho, -gamma P div v); hdt = 0 without them.  Both
+// particles of a pair form a particle's values with these same operations.
 template <typename T>
-__device__ __forceinline__ void half_state(const T (&a)[kRecord], T hdt, T gam, T (&W)[5]) {
+__device__ __forceinline__ void half_inc(const T (&a)[kRecord], T hdt, T gam, T (&inc)[5]) {
     const T div = (a[11 + 3] + a[11 + 7]) + a[11 + 11];
     const T e = -hdt * div;
     const T k = -hdt * rcp_(a[6]);
-    W[0] = fma(e, a[6], a[6]);
-    W[1] = fma(k, a[11 + 12], a[8]);
-    W[2] = fma(k, a[11 + 13], a[9]);
-    W[3] = fma(k, a[11 + 14], a[10]);
-    W[4] = fma(gam * e, a[7], a[7]);
+    inc[0] = e * a[6];
+    inc[1] = k * a[11 + 12];
+    inc[2] = k * a[11 + 13];
+    inc[3] = k * a[11 + 14];
+    inc[4] = gam * e * a[7];
+}
+// Face value of a field: w + (s g.d + inc), the small terms first, so that it is
+// rounded once at the field's size.  (With w + inc formed before: one operation
+// a field less, and energy and mass fluxes of quiet gas 3 to 6 % less accurate.)
+template <typename T>
+__device__ __forceinline__ T face_value(T w, T s, T gd, T inc) {
+    return add_rn(w, fma(s, gd, inc));
+}
+
+// HLLC star pressure from the face pressures, dP = P_b - P_a, du and the
+// impedances (mas, mbs scaled to order one, idens 1/(m_a - m_b) scaled back):
+// the lower pressure plus (m dP - m_a m_b du)/(m_a - m_b), m its side's impedance.
+// One rounding at the pressure's size where waves are weak (the quotient of
+// pressure terms has three, and rates are differences of pressures over the
+// neighbours), and no cancellation where they are strong.
+template <typename T>
+__device__ __forceinline__ T star_pressure(T Pa, T Pb, T dP, T du, T mas, T mbs, T mb, T idens, T& num) {
+    const bool lower = less_(Pa, Pb);
+    num = fma(-(mas * mb), du, mul_rn(lower ? mas : mbs, dP));
+    return fma(num, idens, lower ? Pa : Pb);
 }
 
 // Contribution of the pair (a, b) to particle a's rates: dp (3), dE and,
-// under MFV (O15), dm.  Wh: half_state of a.  kRiem: the MFM face's star from
+// under MFV (O15), dm.  ia: half_inc of a.  kRiem: the MFM face's star from
 // HLLC (0), the exact solver (1), or HLLC with the exact star where HLLC's
 // P* < 0 (2).  Returns false when the face area vanishes.  flags: 1 fallback,
 // 2 P* < 0 (or vacuum).
@@ -573,7 +614,7 @@ __device__ __forceinline__ void half_state(const T (&a)[kRecord], T hdt, T gam, 
 // du = (v_b - v_a).n of the face states, m_a = rho_a min(-c_a, du - c_b) and
 // m_b = rho_b max(c_b, c_a - du) (the Davis speeds relative to the face
 // states; their exchange is -m_b, -m_a),
-//   P* = (m_a P_b - m_b P_a - m_a m_b du) / (m_a - m_b),
+//   P* = (m_a P_b - m_b P_a - m_a m_b du) / (m_a - m_b) (star_pressure),
 //   S* = ((v_a + v_b).n + (2 (P_b - P_a) - (m_a + m_b) du) / (m_a - m_b)) / 2,
 // the contact speed in the lab frame, S*_face + v_f.n whatever v_f is.  Only
 // velocity differences enter P*, so nothing cancels at high Mach number.  P*'s
@@ -582,13 +623,16 @@ __device__ __forceinline__ void half_state(const T (&a)[kRecord], T hdt, T gam, 
 // one of the two impedances is scaled to about 1 by an exact power of two, and
 // 1/(m_a - m_b) back by it: the same bits, and P* has the states' own range.
 template <typename T, bool kMFV, int kRiem>
-__device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[kRecord], const T (&Wh)[5], bool aL,
+__device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[kRecord], const T (&ia)[5], bool aL,
                                            T hdt, T gam, T (&dp)[3], T& dE, T& dm, int& fl) {
     const T dx = mi_diff(b[0], a[0], a[0] - T(1));
     const T dy = mi_diff(b[1], a[1], a[1] - T(1));
     const T dz = mi_diff(b[2], a[2], a[2] - T(1));
     const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
-    const T r = mul_rn(r2, rsq_(r2));
+    T r, ir;
+    roots_(r2, r, ir);
+    // (the approximate root is most of the FP32 rates' error; MFV pays for a correction)
+    if constexpr (kMFV && sizeof(T) == 4) r = fma(fma(-r, r, r2), T(0.5) * ir, r);
     const T ca = a[5] * kern_half(r, a[4]);  // (half of V psi; doubled in A)
     const T cb = b[5] * kern_half(r, b[4]);
     const T Bax = dot3(a[26], a[27], a[28], dx, dy, dz), Bay = dot3(a[27], a[29], a[30], dx, dy, dz),
@@ -600,14 +644,16 @@ __device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[k
     const T A2 = add_rn(mul_rn(ca, Baz), mul_rn(cb, Bbz));
     const T Aq = sep2(A0, A1, A2);
     if (!pos_(Aq - Tiny<T>::sq)) return false;
-    const T iA = rsq_(Aq);
+    T Ah, iA;
+    roots_(Aq, Ah, iA);
     const T n0 = A0 * iA, n1 = A1 * iA, n2 = A2 * iA;
-    const T iH = rcp_(a[3] + b[3]);
-    const T sa = a[3] * iH, sb = b[3] * iH;
-    // face states: half-step primitives + g . (s d), clamped between the
+    const T Hs = a[3] + b[3], iH = rcp_(Hs);
+    // (MFV: the face's velocity, which the mass flux is measured from, hangs on them)
+    const T sa = kMFV ? quot_(a[3], Hs, iH) : a[3] * iH, sb = kMFV ? quot_(b[3], Hs, iH) : b[3] * iH;
+    // face states: primitives + g . (s d) + Hancock increments, clamped between the
     // particles' primitives
-    T Fa[5], Fb[5], Wb[5];
-    half_state(b, hdt, gam, Wb);
+    T Fa[5], Fb[5], ib[5];
+    half_inc(b, hdt, gam, ib);
     const T Wa0[5] = {a[6], a[8], a[9], a[10], a[7]};
     const T Wb0[5] = {b[6], b[8], b[9], b[10], b[7]};
 #pragma unroll
@@ -615,8 +661,8 @@ __device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[k
         const T ga = dot3(a[11 + 3 * f], a[12 + 3 * f], a[13 + 3 * f], dx, dy, dz);
         const T gb = dot3(b[11 + 3 * f], b[12 + 3 * f], b[13 + 3 * f], dx, dy, dz);
         const T lo = min_(Wa0[f], Wb0[f]), hi = max_(Wa0[f], Wb0[f]);
-        Fa[f] = min_(max_(fma(sa, ga, Wh[f]), lo), hi);
-        Fb[f] = min_(max_(fma(-sb, gb, Wb[f]), lo), hi);
+        Fa[f] = min_(max_(face_value(Wa0[f], sa, ga, ia[f]), lo), hi);
+        Fb[f] = min_(max_(face_value(Wb0[f], -sb, gb, ib[f]), lo), hi);
     }
     if (!(pos_(Fa[0]) && pos_(Fa[4]) && pos_(Fb[0]) && pos_(Fb[4]))) {
 #pragma unroll
@@ -635,24 +681,25 @@ __device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[k
     T sc, isc;
     pow2_near(den, sc, isc);
     const T mas = ma * sc, mbs = mb * sc;  // (of order one)
-    T ps = fma(-(mas * mb), du, add_rn(mul_rn(mas, Fb[4]), -mul_rn(mbs, Fa[4]))) * (iden * isc);
+    const T dP = Fb[4] - Fa[4];
+    T num, ps = star_pressure(Fa[4], Fb[4], dP, du, mas, mbs, mb, iden * isc, num);
     bool neg = ps < T(0);
-    const T Am = T(2) * (Aq * iA);
     if constexpr (!kMFV && kRiem == 0) {
         if (neg) {
             fl |= 2;
             ps = T(0);
         }
-        const T us = dot3(Fa[1] + Fb[1], Fa[2] + Fb[2], Fa[3] + Fb[3], n0, n1, n2);
-        const T ss = add_rn(us, mul_rn(fma(-(ma + mb), du, T(2) * (Fb[4] - Fa[4])), iden));
+        const T X = quot_(fma(-(ma + mb), du, T(2) * dP), den, iden);
         const T p2 = T(-2) * ps;
         dp[0] = mul_rn(p2, A0);  // (rounded here: every caller adds the same bits)
         dp[1] = mul_rn(p2, A1);
         dp[2] = mul_rn(p2, A2);
-        dE = mul_rn(T(-0.5) * ps, ss * Am);
+        // S* |A|, the velocities' part straight from the area vector (A0.. are half of it)
+        dE = mul_rn(-ps, fma(X, Ah, dot3(Fa[1] + Fb[1], Fa[2] + Fb[2], Fa[3] + Fb[3], A0, A1, A2)));
         dm = T(0);
         return true;
     } else {
+        const T Am = T(2) * Ah;
         // canonical order: L = a when aL (pair_order); face frame v_f
         T FL[5], FR[5];
 #pragma unroll
@@ -668,7 +715,7 @@ __device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[k
         const T uL = dot3(FL[1] - vfx, FL[2] - vfy, FL[3] - vfz, nx, ny, nz);
         const T uR = dot3(FR[1] - vfx, FR[2] - vfy, FR[3] - vfz, nx, ny, nz);
         const T mL = aL ? ma : -mb, mR = aL ? mb : -ma;
-        const T s0 = mul_rn(fma(-mR, uR, fma(mL, uL, FR[4] - FL[4])), iden);  // S* in the face frame
+        const T s0 = quot_(fma(-mR, uR, fma(mL, uL, FR[4] - FL[4])), den, iden);  // S* in the face frame
         if constexpr (kMFV) {
             // both particles of the pair form the same canonical flux bits; L
             // loses what R gains

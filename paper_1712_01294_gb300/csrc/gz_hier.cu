@@ -545,12 +545,12 @@ __global__ void __launch_bounds__(kXBlock, kLoadAhead<T, kMFV, kRiem> ? 3 : 1)
     auto pair = [&](const T(&b)[kRecord], int j, T(&run)[nq]) {
         const int kab = max(ka, sbin[j]);
         const T hdt = hD * pow2_<T>(-kab);
-        T Wh[5];
-        half_state(a, hdt, gam, Wh);
+        T ia[5];
+        half_inc(a, hdt, gam, ia);
         T dp[3], dE, dm;
         int fl = 0;
         const bool aL = pair_order<kMFV>(i, j, idi, sid);
-        if (pair_rates<T, kMFV, kRiem>(a, b, Wh, aL, hdt, gam, dp, dE, dm, fl)) {
+        if (pair_rates<T, kMFV, kRiem>(a, b, ia, aL, hdt, gam, dp, dE, dm, fl)) {
             const T sc = pow2_<T>(ka - kab);
             run[0] += dp[0] * sc;
             run[1] += dp[1] * sc;

@@ -252,9 +252,12 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
                 if (!kFlat && k0 + u >= cnt) break;
                 const T dx = dx4[u], dy = dy4[u], dz = dz4[u];
                 const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
-                const T ir = rsq_(r2);
-                // (half of W(r/H); the pair's weight is psi = norm W, applied after the loop)
-                const T kh = kern_half(mul_rn(r2, ir), iH);
+                T r, ir;
+                roots_(r2, r, ir);
+                // (half of W(r/H); the pair's weight is psi = norm W, in FP32 applied after
+                // the loop; in FP64 that rounding of the sums shows, 2 % of B's error)
+                T kh = kern_half(r, iH);
+                if constexpr (sizeof(T) == 8) kh *= T(2) * norm;
                 const T pdx = kh * dx, pdy = kh * dy, pdz = kh * dz;
                 E[0] += pdx * dx;
                 E[1] += pdx * dy;
@@ -292,10 +295,12 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
             }
         }
         any = cnt > 0;
+        if constexpr (sizeof(T) == 4) {
 #pragma unroll
-        for (int q = 0; q < 6; ++q) E[q] *= T(2) * norm;
+            for (int q = 0; q < 6; ++q) E[q] *= T(2) * norm;
 #pragma unroll
-        for (int q = 0; q < 15; ++q) Sg[q] *= T(2) * norm;
+            for (int q = 0; q < 15; ++q) Sg[q] *= T(2) * norm;
+        }
         // O7: B = E^-1; FP64 re-do of E and its inverse when kappa > kappa_max
         T B[6], det, kap;
         invert_sym<T>(E, B, det, kap);
@@ -371,7 +376,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
             offsets4(q, xi, yi, zi, xim1, yim1, zim1, dx4, dy4, dz4);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const T sij = Hi * rcp_(Hi + q[u].w);
+                const T Hs = Hi + q[u].w, sij = quot_(Hi, Hs, rcp_(Hs));
                 const T ox = sij * dx4[u], oy = sij * dy4[u], oz = sij * dz4[u];
 #pragma unroll
                 for (int f = 0; f < 5; ++f) {
@@ -596,14 +601,14 @@ __global__ void __launch_bounds__(kFluxBlock, kLoadAhead<T, kMFV, kRiem> ? 3 : 1
     const long long idi = kMFV ? sid[i] : 0;  // (MFV pairs are oriented by id)
     const T hdt = p.hancock ? (T)(0.5 * dt_use[sbox[i]]) : T(0);
     const T gam = (T)p.gamma;
-    T Wh[5];
-    half_state(a, hdt, gam, Wh);
+    T ia[5];
+    half_inc(a, hdt, gam, ia);
     const int cnt = it < N ? min(ncount[i], p.cap) : 0, rcnt = it < N ? min(rcount[i], p.rcap) : 0;
     int nfall = 0, nneg = 0;
     auto pair = [&](const T(&b)[kRecord], int j, T(&run)[nq]) {
         T dp[3], dE, dm;
         int fl = 0;
-        if (pair_rates<T, kMFV, kRiem>(a, b, Wh, pair_order<kMFV>(i, j, idi, sid), hdt, gam, dp, dE, dm, fl)) {
+        if (pair_rates<T, kMFV, kRiem>(a, b, ia, pair_order<kMFV>(i, j, idi, sid), hdt, gam, dp, dE, dm, fl)) {
             run[0] += dp[0];
             run[1] += dp[1];
             run[2] += dp[2];
