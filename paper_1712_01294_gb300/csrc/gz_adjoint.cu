@@ -36,7 +36,7 @@ struct AdjSums {
     T g[15];  // F_a's gradients
     T B[6];
     T k;      // knorm_a
-    T q;      // sum of (dJ/dq_a) q_a, q_a = r / H_a
+    T q;      // sum of dJ/dln(1/H_a) through knorm_a w(r/H_a), over knorm_a
     T h;      // H_a through the face position
 };
 
@@ -120,6 +120,10 @@ __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)
     const T dP = Gb[4] - Ga[4];
     T num;
     const T psr = star_pressure(Ga[4], Gb[4], dP, du, mas, mbs, mb, idens, num);
+    // P_a - P*, P_b - P* without the rounding of P*
+    const T cor = num * idens;
+    const bool lower = less_(Ga[4], Gb[4]);
+    const T Pas = lower ? -cor : -(dP + cor), Pbs = lower ? dP - cor : -cor;
     const T X = fma(-msum, du, T(2) * dP) * iden;
     const T S = T(0.5) * (us + X);
     const bool neg = psr < T(0);
@@ -132,33 +136,36 @@ __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)
     const T b_h = T(-0.5) * (ps * wE) * Am;  // of us and of X
     // X = num2 iden, psr = num1 idens with num1 = sc (ma Pb - mb Pa - ma mb du),
     // iden = 1 / (ma - mb); b_1 the adjoint of num1, of order b_psr like every
-    // product formed with it
+    // product formed with it.  The pressures enter as differences from psr.
     const T b_2 = b_h * iden, b_1 = b_psr * idens;
-    const T b_den = -fma(b_2, X, b_1 * (sc * psr));
     T b_Pa = -fma(b_1, mbs, T(2) * b_2), b_Pb = fma(b_1, mas, T(2) * b_2);
-    const T b_ma = fma(b_1, fma(-mbs, du, sc * Gb[4]), fma(-du, b_2, b_den));
-    const T b_mb = -fma(b_1, fma(mas, du, sc * Ga[4]), fma(du, b_2, b_den));
+    const T b_ma = fma(b_1, fma(-mbs, du, sc * Pbs), -(b_2 * (du + X)));
+    const T b_mb = -fma(b_1, fma(mas, du, sc * Pas), b_2 * (du - X));
     T b_du = -fma(msum, b_2, b_1 * (mas * mb));
     // ma = rho_a min(-c_a, du - c_b), mb = rho_b max(c_b, c_a - du); a tie goes to
-    // the particle that is L (the derivative oracle's rule)
+    // the particle that is L (the derivative oracle's rule).  rho c is
+    // sqrt(gamma P rho): half of its logarithm's derivative to each
     T b_ra = b_ma * al, b_rb = b_mb * be;
-    const T b_al = b_ma * Ga[0], b_be = b_mb * Gb[0];
     T b_ca = T(0), b_cb = T(0);
     const bool own_a = aL ? !less_(e1, -cca) : less_(-cca, e1);
     const bool own_b = aL ? less_(e2, ccb) : !less_(ccb, e2);
     if (own_a) {
-        b_ca -= b_al;
+        b_ra *= T(0.5);
+        b_Pa = fma(T(-0.5) * gam * ica, b_ma, b_Pa);
     } else {
+        const T b_al = b_ma * Ga[0];
         b_du += b_al;
         b_cb -= b_al;
     }
     if (own_b) {
-        b_cb += b_be;
+        b_rb *= T(0.5);
+        b_Pb = fma(T(0.5) * gam * icb, b_mb, b_Pb);
     } else {
+        const T b_be = b_mb * Gb[0];
         b_ca += b_be;
         b_du -= b_be;
     }
-    // c = sqrt(gamma P / rho)
+    // c = sqrt(gamma P / rho), where the other side bounds
     const T ha = T(0.5) * ira * b_ca, hb = T(0.5) * irb * b_cb;
     b_Pa = fma(ha * gam, ica, b_Pa);
     b_ra = fma(-ha, cca, b_ra);
@@ -228,8 +235,8 @@ __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)
     bd[2] += dot3(Ba[2], Ba[4], Ba[5], va[0], va[1], va[2]) + dot3(Bb[2], Bb[4], Bb[5], vb[0], vb[1], vb[2]);
     // ca = knorm_a w(r / Ha), cb likewise
     s.k = fma(b_cka, wa, s.k);
+    s.q = fma(b_cka, fma(da, r * a[4], T(3) * wa), s.q);  // (the two parts of dJ/dH_a cancel in part)
     const T b_qa = b_cka * a[5] * da;
-    s.q = fma(b_qa, r, s.q);  // (times 1/H_a after the last pair)
     const T br = fma(b_qa, a[4], (b_ckb * b[5] * db) * b[4]) * ir;
     // d = x_b - x_a
     s.x[0] += fma(br, dx, bd[0]);
@@ -297,7 +304,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 1)
     bg[7] += b_div;
     bg[11] += b_div;
     // knorm = 8 / (pi H^3 n^2); q = r / H
-    const T bH = s.h - T(3) * s.k * a[5] * a[4] - s.q * a[4] * a[4];
+    const T bH = s.h - s.q * a[5] * a[4];
     const T bn = T(-2) * s.k * a[5] * pdiv(T(1), sn[i]);
     T* o = adj + (size_t)i * kAdj;
 #pragma unroll

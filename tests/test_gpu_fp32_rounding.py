@@ -12,7 +12,8 @@ from gpu_common import cast_state, device, ostate
 from paper_1712_01294_gb300 import inputs as I
 
 GAM = 5.0 / 3.0
-LIMITS = {"p": 6.56e-7, "E": 6.312e-7}
+LIMITS = {"p": 6.56e-7, "E": 6.312e-7, "x": 2.504e-7, "h": 4.354e-7, "rho": 2.864e-7, "v": 1.837e-7, "P": 1.778e-7,
+          "grad rho": 2.838e-7, "grad v": 2.319e-7, "grad P": 1.965e-7, "B": 2.862e-7}
 
 
 def _errors(m, seed):
