@@ -116,9 +116,10 @@ typedef int32_t gz_status;
 
 /* Precision modes. */
 #define GZ_FP64 0    /* every step in double                                          */
-#define GZ_MIXED32 1 /* float state and pair math; double for the Newton update of H,
-                        the E inversion when kappa > kappa_max, and the per-particle
-                        rate accumulation and update                                 */
+#define GZ_MIXED32 1 /* float state and pair math; double for the Newton update of H
+                        (FP32 operations that give the FP64 update's results), the E
+                        inversion when kappa > kappa_max, and the per-particle rate
+                        accumulation and update                                      */
 
 typedef struct {
     double gamma;        /* adiabatic index (5/3)                                     */

@@ -154,10 +154,12 @@ struct HIter {
 // One step of the bracketed Newton iteration on
 // f(H) = (32/3)(1 + S) - N_ngb, f' = (32/3) sd / H, S = sum w, sd = sum -w' q.
 // Returns true when |f| is within the tolerance, else sets H to the next
-// trial.  FP32: f, the quotient and the bracket are FP32 numbers, and so is
-// the next trial's rounding H - f/f' (the FP64 difference of two FP32 numbers
-// rounded to FP32 is their FP32 difference), so the FP64 update needs no FP64
-// arithmetic except near h_lim.
+// trial.  FP32: f, the quotient and the bracket are FP32 numbers, the update
+// H - f/f' is an FP64 one, whose results FP32 operations give exactly: the FP64
+// difference of two FP32 numbers rounded to FP32 is their FP32 difference, and
+// where that falls on an end of the bracket the sign of its rounding error
+// tells which side the FP64 number lies on.  (The FP64 operations themselves,
+// at 1/64 of the FP32 rate, would be a tenth of the pass.)
 __device__ __forceinline__ bool h_step(HIter<float>& b, float& H, float S, float sd, const KParams& p, bool last) {
     const float C = 32.f / 3.f;
     const float f = C * __fadd_rn(1.f, S) - (float)p.ngb;
@@ -175,8 +177,14 @@ __device__ __forceinline__ bool h_step(HIter<float>& b, float& H, float S, float
     float Hn = 0.f;
     bool ok = false;
     if (fp > 0.f) {
-        Hn = __fsub_rn(H, f / fp);
+        const float q = f / fp;
+        Hn = __fsub_rn(H, q);
         ok = Hn > lo && Hn < hi;
+        if (Hn == lo || Hn == hi) {
+            const float t = __fsub_rn(Hn, H);
+            const float err = __fsub_rn(__fsub_rn(H, __fsub_rn(Hn, t)), __fadd_rn(q, t));  // (H - q) - Hn
+            ok = Hn == lo ? err > 0.f : err < 0.f;
+        }
     }
     if (!ok) Hn = (b.has_lo && b.has_hi) ? 0.5f * __fadd_rn(b.lo, b.hi) : (f < 0.f ? 2.f * H : 0.5f * H);
     if (Hn >= p.hlimf) {
