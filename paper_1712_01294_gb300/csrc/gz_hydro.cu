@@ -172,8 +172,7 @@ __global__ void k_prim(int N, Sorted<T> s, KParams p, DevStatus* st, int* rcount
 // ahead, then the packed records of all four) so their loads are in flight
 // together.  The pass waits on them half the time and issues the other half;
 // instructions a neighbour (one boundary test for four offsets, the kernel
-// without its two pieces, the pair weight's constant applied after the loop,
-// min/max as such) took it from 624 to 494 us at 128^3, FP64 at 48^3 894 to
+// without its two pieces, min/max as such) took it from 624 to 494 us at 128^3, FP64 at 48^3 894 to
 // 627.  Held to 128 registers (4 blocks per SM); at 5 blocks it spills (570 us),
 // and with the next group's records loaded ahead (162 registers) it took 598.
 // kInfo: also track which particles the limiter's bounds came from and write
@@ -210,7 +209,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
         const T Wi[5] = {pm.x, pm.y, pm.z, pm.w, pm2.x};
         const T ci = pm2.y;
         const T iH = T(1) / Hi;
-        const T norm = T(8.0 / kPi) * iH * iH * iH / ni;
+        const T norm = T(8.0 / kPi) * iH * iH * iH / ni, norm2 = T(2) * norm;
         // FP32 steps: the spare slots of a list's last group run through with no
         // weight instead of a branch a slot, 494 -> 473 us at 128^3 (late in
         // the run 549 -> 519); gradients alone (90 us at 75^3) and
@@ -254,10 +253,10 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
                 const T r2 = max_(sep2(dx, dy, dz), Tiny<T>::sq);
                 T r, ir;
                 roots_(r2, r, ir);
-                // (half of W(r/H); the pair's weight is psi = norm W, in FP32 applied after
-                // the loop; in FP64 that rounding of the sums shows, 2 % of B's error)
-                T kh = kern_half(r, iH);
-                if constexpr (sizeof(T) == 8) kh *= T(2) * norm;
+                // psi (norm applied per pair: applied to the sums, its rounding stays whole
+                // in each of them, up to 3 % of the error of B and the gradients, and
+                // nothing is faster)
+                const T kh = kern_half(r, iH) * norm2;
                 const T pdx = kh * dx, pdy = kh * dy, pdz = kh * dz;
                 E[0] += pdx * dx;
                 E[1] += pdx * dy;
@@ -295,12 +294,6 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (kInfo ? 3 : 4) : 1)
             }
         }
         any = cnt > 0;
-        if constexpr (sizeof(T) == 4) {
-#pragma unroll
-            for (int q = 0; q < 6; ++q) E[q] *= T(2) * norm;
-#pragma unroll
-            for (int q = 0; q < 15; ++q) Sg[q] *= T(2) * norm;
-        }
         // O7: B = E^-1; FP64 re-do of E and its inverse when kappa > kappa_max
         T B[6], det, kap;
         invert_sym<T>(E, B, det, kap);

@@ -64,3 +64,29 @@ def test_rates_and_adjoints_are_no_less_precise():
     mean = {k: float(np.sqrt(np.mean([r[k] ** 2 for r in runs]))) for k in LIMITS}
     print({k: float("%.3e" % v) for k, v in mean.items()})
     assert not {k: (v, LIMITS[k]) for k, v in mean.items() if v > LIMITS[k]}
+
+
+# The gradient pass, likewise.  What rounds once a particle and enters all its
+# sums alike averages out over nothing; how much it is hangs on the mantissas of
+# 1/H^3 and n, and with them on the box's size (26^3 is one of the worse).
+GRADIENT_LIMITS = {"B": 1.42e-7, "grad": 1.684e-7}
+
+
+@pytest.mark.gpu
+def test_gradients_are_no_less_precise():
+    import torch
+    import paper_1712_01294_gb300 as m
+    q = cast_state(I.turbulence(26, seed=1), 1)
+    s = ostate(q)
+    H, n, _, _ = O.density(s, O.params())
+    H, n = (a.astype(np.float32).astype(np.float64) for a in (H, n))
+    g = O.gradients(s, H, n, O.params())
+    ctx = m.Context([s.N], m.default_params())
+    got = dict(zip(("grad", "B"), ctx.gradients(device(q, 1, H=H), torch.as_tensor(n).cuda().float())))
+    ctx.status(reset=True)
+    ctx.close()
+    err = {}
+    for k, v in got.items():
+        d = np.sort(np.abs(v.cpu().numpy() - g[k]), axis=None)
+        err[k] = float(np.sqrt(np.mean(d[: int(0.98 * d.size)] ** 2) / np.mean(g[k] ** 2)))
+    assert not {k: (v, GRADIENT_LIMITS[k]) for k, v in err.items() if v > GRADIENT_LIMITS[k]}
