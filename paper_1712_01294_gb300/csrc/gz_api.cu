@@ -237,9 +237,8 @@ gz_status do_fluxes_backward(gz_ctx* ctx, const gz_particles* p, const void* n, 
 // each, the neighbour counts [N] and the first kCkptSlots slots of the
 // neighbour lists (a prefix of their grouped layout); slices start on
 // 256-byte boundaries.  Every level also keeps n and sum(-w'q) at the
-// converged H (sorted order, after H): the density pass of a particle the
-// h-iteration left to the warp kernel sums them in another order than a
-// rescan would.
+// converged H (sorted order, after H), so the backward pass forms neither
+// again.
 // (The backward pass sorts the same start state, so sorted order is the
 // same.)
 constexpr int kCkptSlots = 64;

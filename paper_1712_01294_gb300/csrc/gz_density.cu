@@ -105,7 +105,7 @@ template <int G, int E>
 __device__ __forceinline__ void group_eval(unsigned gm, int gl, int n, const float (&r)[E], const float* r2, float H,
                                            float& S, float& sd) {
     const float H2 = H * H, iH = 1.f / H;
-    Acc<float> sw;
+    Acc sw;
     sd = 0.f;
 #pragma unroll
     for (int u = 0; u < E; ++u) {
@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(kOneBlock, 10)
             return;
         }
         const float H2 = H * H, iH = 1.f / H;
-        Acc<float> sw;
+        Acc sw;
         sdv = 0.f;
 #pragma unroll
         for (int u = 0; u < 3; ++u) c_r2[min(ncache + u, kCache)][t] = 1e30f;  // (fills up the last four)
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(kOneBlock, 10)
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const bool h = r2[u] < H2;
-                Acc<float> a = sw;
+                Acc a = sw;
                 a.add(w[u]);
                 const float d = fmaf(y[u], x[u], sdv);
                 sw.s = h ? a.s : sw.s;
@@ -595,7 +595,7 @@ __device__ __forceinline__ void warp_eval(int lane, int n, const float* r2, floa
                                           float& S, float& sd, float& sdk) {
     const float H2 = H * H, iH = 1.f / H;
     if (n > kDensCache) {
-        Acc<float> w;
+        Acc w;
         float d = 0.f;
         for (int k = lane; k < n; k += 32)
             if (r2[k] < H2) {
@@ -608,7 +608,7 @@ __device__ __forceinline__ void warp_eval(int lane, int n, const float* r2, floa
         sd = sdk = (float)group_add<32>(0xffffffffu, (double)d);
         return;
     }
-    Acc<float> sw, sk;
+    Acc sw, sk;
     sd = 0.f;
     for (int k0 = 0; k0 < n; k0 += 32) {
         const int k = k0 + lane;

@@ -5,16 +5,8 @@
 
 namespace gz {
 
-// Kahan-compensated sum for FP32 neighbour sums; plain sum in FP64.
-template <typename T>
+// Kahan-compensated FP32 sum.
 struct Acc {
-    T s = T(0);
-    __device__ __forceinline__ void add(T v) { s += v; }
-    __device__ __forceinline__ void merge(const Acc& o) { s += o.s; }
-    __device__ __forceinline__ double value() const { return (double)s; }
-};
-template <>
-struct Acc<float> {
     float s = 0.f, c = 0.f;
     __device__ __forceinline__ void add(float v) {
         float y = __fsub_rn(v, c);
@@ -22,8 +14,6 @@ struct Acc<float> {
         c = __fsub_rn(__fsub_rn(t, s), y);
         s = t;
     }
-    __device__ __forceinline__ void merge(const Acc& o) { add(o.fvalue()); }
-    __device__ __forceinline__ double value() const { return (double)s - (double)c; }
     __device__ __forceinline__ float fvalue() const { return __fsub_rn(s, c); }
 };
 

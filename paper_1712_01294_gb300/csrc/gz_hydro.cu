@@ -806,7 +806,6 @@ KParams kparams(const Ctx& c) {
     KParams k;
     k.gamma = c.params.gamma;
     k.ngb = c.params.ngb;
-    k.tol = c.params.tol;
     k.cfl = c.params.cfl;
     k.kappa_max = c.params.kappa_max;
     k.beta = c.params.beta;

@@ -50,7 +50,7 @@ inline float wide_cells(double H0, int nc) { return (float)(1.7 * (H0 * nc > 1.0
 
 // Scalar parameters passed by value to kernels.
 struct KParams {
-    double gamma, ngb, tol, cfl, kappa_max, beta, u_floor_frac, h_lim;
+    double gamma, ngb, cfl, kappa_max, beta, u_floor_frac, h_lim;
     double dtol;        // tol * ngb
     float ftol, hlimf;  // tol * ngb rounded down, h_lim rounded up (the same tests on FP32 numbers)
     int hancock, max_iter, cap, rcap, scheme;

@@ -80,8 +80,6 @@ template <typename T>
 cudaError_t run_gradients(Ctx& c, bool want_dt, bool with_info = false, const int* list = nullptr,
                           const int* nlist = nullptr, int n = 0);
 template <typename T>
-cudaError_t run_timestep_only(Ctx& c);
-template <typename T>
 cudaError_t run_pack_given(Ctx& c, const T* grad, const T* B, const int* list = nullptr,
                            const int* nlist = nullptr, int n = 0, const unsigned char* skip = nullptr);
 template <typename T>
