@@ -228,13 +228,19 @@ template <typename T>
 __device__ __forceinline__ bool wide(T R, const BoxInfo& bx) {
     return (float)R * (float)bx.nc > bx.wide;
 }
+template <typename T>
+__device__ __forceinline__ bool in_box(const P4<T>& p) {
+    return p.x >= T(0) && p.x <= T(1) && p.y >= T(0) && p.y <= T(1) && p.z >= T(0) && p.z <= T(1);
+}
 // Whether a particle's scan is left to a warp from the start.  A position outside
 // the box (or none) sees no candidates: nothing to share.
 template <typename T>
 __device__ __forceinline__ bool to_warp(T R, const BoxInfo& bx, const P4<T>& me) {
-    return wide(R, bx) && me.x >= T(0) && me.x <= T(1) && me.y >= T(0) && me.y <= T(1) && me.z >= T(0) &&
-           me.z <= T(1);
+    return wide(R, bx) && in_box(me);
 }
+
+// Cell coordinate of a position (as the binning forms it).
+__device__ __forceinline__ int cell_at(float v, int nc) { return min(max((int)floorf(v * (float)nc), 0), nc - 1); }
 
 // Starting H of particle i: its guess, or (flagged by the caller) the box's
 // mean when the guess is unusable.
@@ -486,13 +492,21 @@ __global__ void __launch_bounds__(kOneBlock, 10)
     int lo[3], hi[3];
     bool in = false;
     if constexpr (kInside) in = warp_inside(bx, me, Rc, lo, hi);
-    if (in) {
-        scan_inside(g.cells + bx.cell_off, bx.nc, lo, hi, s.pos, i, me.x, me.y, me.z, Rc, [&](int j, float r2, bool h) {
-            const int k = min(ncache, kCache);
-            c_r2[k][t] = r2;
-            c_j[k][t] = (unsigned)j;
-            ncache += h;
-        });
+    // a cell so full that one thread would walk it while its warp waits: its
+    // particles are left to k_density_warp, whose lanes share it (64^3 with 4096
+    // particles in one cell: 6.2 ms one thread each, 1.3 so; 32768 in one: 558 and
+    // 55).  Looking at every cell of the window as well costs 1 to 2 % of the pass.
+    const int2 own = g.cells[bx.cell_off + (cell_at(me.z, bx.nc) * bx.nc + cell_at(me.y, bx.nc)) * bx.nc + cell_at(me.x, bx.nc)];
+    if (own.y - own.x > kCrowdCell && in_box(me)) {
+        ncache = kCache + 1;
+    } else if (in) {
+        scan_inside(g.cells + bx.cell_off, bx.nc, lo, hi, s.pos, i, me.x, me.y, me.z, Rc,
+                                    [&](int j, float r2, bool h) {
+                                        const int k = min(ncache, kCache);
+                                        c_r2[k][t] = r2;
+                                        c_j[k][t] = (unsigned)j;
+                                        ncache += h;
+                                    });
     } else if (to_warp(Rc, bx, me)) {
         ncache = kCache + 1;
     } else if constexpr (kInside) {

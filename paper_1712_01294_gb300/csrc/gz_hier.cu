@@ -196,7 +196,8 @@ __global__ void __launch_bounds__(kCmpBlock)
 
 // --------------------------------------------------------- pair lists
 // Smallest support radius among every cell's active particles (+inf without
-// any), rounded down.
+// any), rounded down; 0 for a crowded cell with one, whose particles one thread
+// would walk (a state that went to NaN, 64^3: 12 ms).
 template <typename T>
 __global__ void k_h_cellmin(int ncells, const int2* cells, const unsigned char* aflag,
                             const P4<T>* pos, float* cellmin) {
@@ -205,13 +206,18 @@ __global__ void k_h_cellmin(int ncells, const int2* cells, const unsigned char* 
     if (c >= ncells) return;
     const int2 se = cells[c];
     float h = INFINITY;
-    for (int i = se.x; i < se.y; ++i)
-        if (aflag[i]) {
-            if constexpr (sizeof(T) == 8)
-                h = fminf(h, __double2float_rd(pos[i].w));
-            else
-                h = fminf(h, pos[i].w);
-        }
+    if (se.y - se.x > kCrowdCell) {  // (0: the cell is only never skipped)
+        for (int i = se.x; i < se.y && h > 0.f; ++i)
+            if (aflag[i]) h = 0.f;
+    } else {
+        for (int i = se.x; i < se.y; ++i)
+            if (aflag[i]) {
+                if constexpr (sizeof(T) == 8)
+                    h = fminf(h, __double2float_rd(pos[i].w));
+                else
+                    h = fminf(h, pos[i].w);
+            }
+    }
     cellmin[c] = h;
 }
 

@@ -379,6 +379,7 @@ __device__ __forceinline__ void for_candidates(const Grid& g, const BoxInfo& bx,
 }
 
 constexpr int kLaneCells = 16;
+constexpr int kCrowdCell = 128;  // particles from which a cell is shared by lanes instead of walked by one thread
 
 // Warp-cooperative candidate scan for one particle per warp (every lane
 // passes the same particle): each lane calls fn(j, dx, dy, dz, r2) for its
@@ -435,10 +436,19 @@ __device__ __forceinline__ void for_candidates_lanes(const Grid& g, const BoxInf
     const int ex = hi[0] - lo[0] + 1, ey = hi[1] - lo[1] + 1, ez = hi[2] - lo[2] + 1;
     const int ncube = ex * ey * ez;
     if (ncube >= kLaneCells) {
-        for (int f = lane; f < ncube; f += 32) {
+        for (int f0 = 0; f0 < ncube; f0 += 32) {
+            const int f = f0 + lane;
             const int cx = lo[0] + f % ex, cy = lo[1] + (f / ex) % ey, cz = lo[2] + f / (ex * ey);
-            int2 se;
-            if (!cell_range(cx, cy, cz, se)) continue;
+            int2 se = make_int2(0, 0);
+            if (f < ncube && !cell_range(cx, cy, cz, se)) se = make_int2(0, 0);
+            // (a crowded cell is shared by the lanes)
+            for (unsigned big = __ballot_sync(0xffffffffu, se.y - se.x > kCrowdCell); big; big &= big - 1) {
+                const int l = __ffs(big) - 1;
+                const int a = __shfl_sync(0xffffffffu, se.x, l), e = __shfl_sync(0xffffffffu, se.y, l);
+                for (int j = a + lane; j < e; j += 32)
+                    if (j != self) visit(j);
+                if (lane == l) se.y = se.x;
+            }
             for (int j = se.x; j < se.y; ++j)
                 if (j != self) visit(j);
         }
@@ -614,8 +624,8 @@ __device__ __forceinline__ void sort_list(unsigned* L, int n, int N) {
 // them pass the same particle): the candidates j != self with r^2 < R^2,
 // handed to emit(k, j) with k = 0, 1, ... in for_candidates' order (cells in
 // its loop order, j ascending within a cell), each by one lane of the group.
-// A round takes G cells, one a lane: the lane tests its cell's candidates
-// into a bit mask, a prefix sum over the group numbers the hits, and the lane
+// A round takes G cells, one a lane (cells of more than 32 candidates one after
+// another, 32 candidates a lane): the lane tests its candidates into a bit mask, a prefix sum over the group numbers the hits, and the lane
 // hands its set bits over (a few instructions each: lanes have unequal hits,
 // so what is done per hit is left to the caller's pass over the numbered
 // hits, where every lane is busy).  Returns the number of hits (the same for
@@ -656,57 +666,56 @@ __device__ __forceinline__ int group_scan(const Grid& g, const BoxInfo& bx, cons
             return sep2(mi_diff(q.x, xi, xim1), mi_diff(q.y, yi, yim1), mi_diff(q.z, zi, zim1)) < R2;
         };
         auto near = [&](const P4<T>& q) {
-            if constexpr (sizeof(T) == 8)
-                return r2_chop(q.x, q.y, q.z, xf, yf, zf) < R2f && (!kExact || within(q));
-            if (w.percell) return sep2((q.x + ax) - bxx, (q.y + ay) - byy, (q.z + az) - bzz) < R2;
+            if constexpr (sizeof(T) == 8) return r2_chop(q.x, q.y, q.z, xf, yf, zf) < R2f;
             return within(q);
         };
-        unsigned m = 0;  // hits among the cell's first 32 candidates
-        const int end = min(se.y, se.x + 32), last = se.y - 1;
-        auto test4 = [&](auto hit) {
-            for (int j0 = se.x; j0 < end; j0 += 4) {
+        // the hits among each lane's candidates a..e-1 (32 at most), numbered and
+        // handed over
+        auto take = [&](int a, int e, auto hit) {
+            unsigned m = 0;
+            for (int j0 = a; j0 < e; j0 += 4) {
                 P4<T> q[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) q[u] = pos[min(j0 + u, last)];
+                for (int u = 0; u < 4; ++u) q[u] = pos[min(j0 + u, e - 1)];
                 unsigned n4 = 0;
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     if (hit(q[u])) n4 |= 1u << u;
-                m |= n4 << (j0 - se.x);
+                m |= n4 << (j0 - a);
             }
-        };
-        if constexpr (sizeof(T) == 8)
-            test4([&](const P4<T>& q) { return r2_chop(q.x, q.y, q.z, xf, yf, zf) < R2f; });
-        else if (w.percell)
-            test4([&](const P4<T>& q) { return sep2((q.x + ax) - bxx, (q.y + ay) - byy, (q.z + az) - bzz) < R2; });
-        else
-            test4(near);
-        const int nj = se.y - se.x;
-        if (nj < 32) m &= (1u << nj) - 1u;  // (the last group of four repeats the last candidate)
-        if (self >= se.x && self < end) m &= ~(1u << (self - se.x));
-        if constexpr (sizeof(T) == 8 && kExact)
-            for (unsigned b = m; b; b &= b - 1)
-                if (!within(pos[se.x + __ffs(b) - 1])) m &= ~(b & (0u - b));
-        int more = 0;  // hits past the cell's first 32 candidates
-        for (int j = se.x + 32; j < se.y; ++j)
-            if (j != self && near(pos[j])) ++more;
-        const int cnt = __popc(m) + more;
-        int pre = cnt;
+            const int nj = max(e - a, 0);
+            if (nj < 32) m &= (1u << nj) - 1u;  // (the last group of four repeats the last candidate)
+            if (self >= a && self < e) m &= ~(1u << (self - a));
+            if constexpr (sizeof(T) == 8 && kExact)
+                for (unsigned b = m; b; b &= b - 1)
+                    if (!within(pos[a + __ffs(b) - 1])) m &= ~(b & (0u - b));
+            const int cnt = __popc(m);
+            int pre = cnt;
 #pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
-            const int y = __shfl_up_sync(gm, pre, o, G);
-            if (gl >= o) pre += y;
+            for (int o = 1; o < G; o <<= 1) {
+                const int y = __shfl_up_sync(gm, pre, o, G);
+                if (gl >= o) pre += y;
+            }
+            const int total = __shfl_sync(gm, pre, G - 1, G);
+            int k = base + pre - cnt;
+            for (; m; m &= m - 1) emit(k++, a + __ffs(m) - 1);
+            base += total;
+        };
+        if (__any_sync(gm, se.y - se.x > 32)) {
+            // a cell of more than 32 candidates: this round's cells one after
+            // another, 32 candidates a lane at a time
+            for (int l = 0; l < G && base <= most; ++l) {
+                const int a = __shfl_sync(gm, se.x, l, G), e = __shfl_sync(gm, se.y, l, G);
+                for (int j0 = a; j0 < e && base <= most; j0 += 32 * G) take(j0 + 32 * gl, min(e, j0 + 32 * gl + 32), near);
+            }
+        } else if constexpr (sizeof(T) == 8) {
+            take(se.x, se.y, near);
+        } else if (w.percell) {
+            take(se.x, se.y,
+                 [&](const P4<T>& q) { return sep2((q.x + ax) - bxx, (q.y + ay) - byy, (q.z + az) - bzz) < R2; });
+        } else {
+            take(se.x, se.y, near);
         }
-        const int total = __shfl_sync(gm, pre, G - 1, G);
-        int k = base + pre - cnt;
-        while (m) {
-            emit(k++, se.x + __ffs(m) - 1);
-            m &= m - 1;
-        }
-        if (more)
-            for (int j = se.x + 32; j < se.y; ++j)
-                if (j != self && near(pos[j])) emit(k++, j);
-        base += total;
         if (base > most) break;
     }
     return base;
@@ -740,6 +749,16 @@ __device__ __forceinline__ int for_hits_lanes_ordered(const Grid& g, const BoxIn
     };
     const unsigned full_mask = 0xffffffffu;
     int base = 0;
+    auto one_cell = [&](int a, int e) {  // the cell's candidates by all lanes, a ballot per 32
+        for (int j0 = a; j0 < e; j0 += 32) {
+            const int j = j0 + lane;
+            const T r2 = j < e ? r2_of(j) : T(0);
+            const bool h = j < e && j != self && r2 < R2;
+            const unsigned m = __ballot_sync(full_mask, h);
+            if (h) emit(base + __popc(m & ((1u << lane) - 1u)), j, r2);
+            base += __popc(m);
+        }
+    };
     if (w.ncube >= kLaneCells) {
         for (int f0 = 0; f0 < w.ncube; f0 += 32 * kAhead) {
             int2 ses[kAhead];
@@ -757,11 +776,15 @@ __device__ __forceinline__ int for_hits_lanes_ordered(const Grid& g, const BoxIn
             for (int u = 0; u < kAhead; ++u) {
                 const int2 se = u == 0 ? ses[0] : (u == 1 ? ses[1] : (u == 2 ? ses[2] : ses[3]));
                 if (!__any_sync(full_mask, se.y > se.x)) continue;
-                // hits among the cell's first 32 candidates, four tested at a
-                // time, and those past them
+                if (__any_sync(full_mask, se.y - se.x > 32)) {  // crowded cells: one after another
+                    for (int l = 0; l < 32; ++l)
+                        one_cell(__shfl_sync(full_mask, se.x, l), __shfl_sync(full_mask, se.y, l));
+                    continue;
+                }
+                // the cell's hits, four candidates tested at a time
                 unsigned m = 0;
-                const int end = min(se.y, se.x + 32), nj = se.y - se.x;
-                for (int j0 = se.x; j0 < end; j0 += 4) {
+                const int nj = se.y - se.x;
+                for (int j0 = se.x; j0 < se.y; j0 += 4) {
                     T r2[4];
 #pragma unroll
                     for (int v = 0; v < 4; ++v) r2[v] = r2_of(min(j0 + v, se.y - 1));
@@ -771,11 +794,8 @@ __device__ __forceinline__ int for_hits_lanes_ordered(const Grid& g, const BoxIn
                     m |= n4 << (j0 - se.x);
                 }
                 if (nj < 32) m &= (1u << nj) - 1u;  // (the last four repeat the last candidate)
-                if (self >= se.x && self < end) m &= ~(1u << (self - se.x));
-                int more = 0;
-                for (int j = se.x + 32; j < se.y; ++j)
-                    if (j != self && r2_of(j) < R2) ++more;
-                const int cnt = __popc(m) + more;
+                if (self >= se.x && self < se.y) m &= ~(1u << (self - se.x));
+                const int cnt = __popc(m);
                 int pre = cnt;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -788,11 +808,6 @@ __device__ __forceinline__ int for_hits_lanes_ordered(const Grid& g, const BoxIn
                     const int j = se.x + __ffs(m) - 1;
                     emit(k++, j, r2_of(j));
                 }
-                if (more)
-                    for (int j = se.x + 32; j < se.y; ++j) {
-                        const T r2 = r2_of(j);
-                        if (j != self && r2 < R2) emit(k++, j, r2);
-                    }
                 base += total;
             }
         }
@@ -801,14 +816,7 @@ __device__ __forceinline__ int for_hits_lanes_ordered(const Grid& g, const BoxIn
             int cx, cy, cz;
             w.coords(f, cx, cy, cz);
             const int2 se = w.range(cells, cx, cy, cz, xf, yf, zf);  // (the same for every lane)
-            for (int j0 = se.x; j0 < se.y; j0 += 32) {
-                const int j = j0 + lane;
-                const T r2 = j < se.y ? r2_of(j) : T(0);
-                const bool h = j < se.y && j != self && r2 < R2;
-                const unsigned m = __ballot_sync(full_mask, h);
-                if (h) emit(base + __popc(m & ((1u << lane) - 1u)), j, r2);
-                base += __popc(m);
-            }
+            one_cell(se.x, se.y);
         }
     }
     return base;
