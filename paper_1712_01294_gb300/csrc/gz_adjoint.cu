@@ -46,8 +46,8 @@ struct AdjSums {
 // in which v_f drops out), so every branch matches; ia: half_inc of a.
 // Divisions are products with the reciprocals the forward takes anyway: FP64
 // is bound by its pipe (977 operations a pair where the canonical L/R order,
-// v_f and a's own terms were carried through each pair, 3.88 ms at 40^3; 486
-// here, 1.93 ms).
+// v_f and a's own terms were carried through each pair, 3.88 ms at 40^3; a good
+// half of that here, 2.20 ms, of which 0.27 ms keep terms from cancelling).
 template <typename T>
 __device__ __forceinline__ void pair_adjoint(const T (&a)[kRecord], const T (&b)[kRecord], const T (&ia)[5], bool aL,
                                              T hdt, T gam, const T* wp, T wE, AdjSums<T>& s) {

@@ -35,8 +35,8 @@ constexpr int kWideLanes = 16;  // ... and in FP32 launches too small for those
 // chip with fewer instructions a particle.  Measured, us a launch on the first
 // steps (late in the run): Sod 16^3 sixteen lanes 24 (27), eight 28 (35), four
 // 40 (53); Sod 32^3 sixteen 69 (81), eight 58 (68), four 50 (67), one 42 (81);
-// KH 41^3 four 105 (99), one 66 (69); Sedov 64^3 one 102 (506); 128^3 one 803
-// (1175).  FP64 keeps four: its sums are the lanes' sums.
+// KH 41^3 four 105 (99), one 66 (66); Sedov 64^3 one 100 (369); 128^3 one 806
+// (1160).  FP64 keeps four: its sums are the lanes' sums.
 constexpr int kWideMax = 12000;
 constexpr int kThreadMin = 45000;
 // Cells per axis from which k_density_one looks for warps whose windows lie

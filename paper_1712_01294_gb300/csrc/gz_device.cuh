@@ -36,7 +36,8 @@ __device__ __forceinline__ double pdiv(double a, double b) { return a / b; }
 // [2^-1000, 2^1000], negative x too for the reciprocal.  The square root is
 // x y with one correction (x - s^2) y / 2, as accurate: pairs' distances enter
 // every face, and x y alone (1 ulp) made FP64 rates 10 % less accurate than
-// CUDA's sqrt does.
+// CUDA's sqrt does.  (CUDA's division and square root in their places would be
+// some 50 more of the 290 FP64 operations a pair.)
 __device__ __forceinline__ float rcp_(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -573,7 +574,8 @@ __device__ __forceinline__ void half_inc(const T (&a)[kRecord], T hdt, T gam, T 
 }
 // Face value of a field: w + (s g.d + inc), the small terms first, so that it is
 // rounded once at the field's size.  (With w + inc formed before: one operation
-// a field less, and energy and mass fluxes of quiet gas 3 to 6 % less accurate.)
+// a field less, FP64 at 48^3 3 % of the step, FP32 nothing measurable, and energy
+// and mass fluxes of quiet gas 3 to 6 % less accurate.)
 template <typename T>
 __device__ __forceinline__ T face_value(T w, T s, T gd, T inc) {
     return add_rn(w, fma(s, gd, inc));
@@ -759,8 +761,8 @@ __device__ __forceinline__ bool pair_rates(const T (&a)[kRecord], const T (&b)[k
 // the same bits.
 // Totals are FP64 in both precisions (the FP32 mode's rates are accumulated in
 // double).  Two FP32 words instead (48 bits) took 5 % less of the pass, 128^3 797
-// -> 758 us, but the low word loses its bits below 1e-38 and an infinite term
-// turns the total into NaN.
+// -> 758 us, but are not what the mode promises, and one infinite term turns
+// such a total into NaN.
 template <int nq>
 struct Totals {
     double v[nq];
@@ -789,8 +791,9 @@ __device__ __forceinline__ void for_slots(const uint4& jj, int n, F&& f) {
 // pair(rec, j, dst) adds the pair with record rec of partner j to dst[nq].
 // kAhead: the next partner's record is loaded while the current pair is
 // evaluated (two record buffers, so the loop is written for two pairs at a
-// time; 165 registers, 12 warps an SM).  The pass waits on its gathers: FP32
-// MFM at 128^3 856 us without, 803 with.  The forms with more arithmetic a
+// time; 164 registers, 12 warps an SM).  The pass waits on its gathers: FP32
+// MFM at 128^3 856 us without, 803 with (821 now, with face values and star
+// pressure rounded once).  The forms with more arithmetic a
 // pair (MFV, the exact solver, FP64) need the registers themselves.  kUnroll:
 // copies of the pair's code (the exact solver's is long: one).
 template <typename T, int nq, bool kAhead, int kUnroll, typename P>
