@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(kScanThreads)
 
 // Particles of one key beyond which k_permute's walk of the cell (its number of
 // steps squared) costs more than k_cs_place's last block sorting the cell.  The
-// whole sort with every particle in one cell, walked / sorted: 32^3 584 / 153 us,
-// 64^3 10314 / 507, 128^3 - / 6257 (a lattice: 19, 25 and 100).
+// whole sort with every particle in one cell, walked / sorted: 32^3 584 / 113 us,
+// 64^3 10314 / 513, 128^3 - / 3869 (a lattice: 19, 26 and 103).
 constexpr int kCrowd = 16384;
 
 // First sorted index of every key, the range of every cell (empty ones
@@ -193,25 +193,23 @@ __global__ void __launch_bounds__(kScanThreads)
 }
 
 // The n distinct caller indices (below N) of a crowded cell in increasing order,
-// by one block: a bitmap of a window of indices after another, whose set bits
-// come out in order.
-constexpr int kCrowdWords = 8192;
-__device__ __forceinline__ void sort_crowd(unsigned* seg, unsigned* tmp, int n, int N) {
-    __shared__ unsigned bits[kCrowdWords];
+// by one block: a bitmap of the N indices, whose set bits come out in order.
+// (Written and read past L1, which does not see the atomics.)
+__device__ __forceinline__ void sort_crowd(unsigned* seg, unsigned* bits, int n, int N) {
     __shared__ int wsum[32];
     const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5;
-    const int per = kCrowdWords / T;
+    const int words = (N - 1) / 32 + 1;
+    for (int w = t; w < words; w += T) __stcg(bits + w, 0u);
+    __syncthreads();
+    for (int e = t; e < n; e += T) {
+        const unsigned v = __ldcg(seg + e);  // (written by other blocks)
+        atomicOr(bits + (v >> 5), 1u << (v & 31));
+    }
+    __syncthreads();
     int done = 0;
-    for (unsigned base = 0; base < (unsigned)N; base += 32 * kCrowdWords) {
-        for (int w = t; w < kCrowdWords; w += T) bits[w] = 0;
-        __syncthreads();
-        for (int e = t; e < n; e += T) {
-            const unsigned v = __ldcg(seg + e) - base;  // (written by other blocks)
-            if (v < 32u * kCrowdWords) atomicOr(&bits[v >> 5], 1u << (v & 31));
-        }
-        __syncthreads();
-        int mine = 0;
-        for (int w = t * per; w < (t + 1) * per; ++w) mine += __popc(bits[w]);
+    for (int w0 = 0; w0 < words; w0 += T) {
+        unsigned b = w0 + t < words ? __ldcg(bits + w0 + t) : 0u;
+        const int mine = __popc(b);
         int x = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -225,20 +223,18 @@ __device__ __forceinline__ void sort_crowd(unsigned* seg, unsigned* tmp, int n, 
             if (w < warp) at += wsum[w];
             done += wsum[w];
         }
-        for (int w = t * per; w < (t + 1) * per; ++w)
-            for (unsigned b = bits[w]; b; b &= b - 1) tmp[at++] = base + 32u * w + (unsigned)(__ffs(b) - 1);
+        for (; b; b &= b - 1) seg[at++] = 32u * (unsigned)(w0 + t) + (unsigned)(__ffs(b) - 1);
         __syncthreads();
     }
-    for (int e = t; e < n; e += T) seg[e] = tmp[e];
-    __syncthreads();
 }
 
 // Particles by key, in any order within a cell, except in crowded cells (a
 // state that went to NaN is binned in one): once every block has placed its
-// particles, the last one puts those in caller order (tmp: N words).  Without
-// crowded cells a block reads one word more.
+// particles, the last one puts those in caller order.  crowd (N words): the
+// crowded keys, then room for a bitmap of the particles.  Without crowded cells
+// a block reads one word more.
 __global__ void k_cs_place(int N, const unsigned* key, const unsigned* slot, const unsigned* start, unsigned* order,
-                           unsigned* count, long long K, const unsigned* crowd, unsigned* tmp) {
+                           unsigned* count, long long K, unsigned* crowd) {
     after_previous();
     __shared__ bool last;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -253,7 +249,7 @@ __global__ void k_cs_place(int N, const unsigned* key, const unsigned* slot, con
     __threadfence();
     for (int c = 0; c < crowds; ++c) {
         const unsigned k = crowd[c], a = start[k];
-        sort_crowd(order + a, tmp + a, (int)count[k], N);
+        sort_crowd(order + a, crowd + crowds, (int)count[k], N);
     }
 }
 
@@ -505,11 +501,11 @@ static cudaError_t counting_sort(Ctx& c, const gz_particles& p, const void* n_in
     if (!direct) launch_next(c, k_cs_sums, tiles, kScanThreads, K, c.kcount, c.hist);
     launch_next(c, k_cs_scan, tiles, kScanThreads, K, c.kcount, direct ? nullptr : c.hist, c.boxes, c.nboxes, c.kstart,
                 c.cells, c.keys);
-    // (c.keys and c.vals are k_permute's to write: room for the crowded keys and
-    // their sort; large launches have blocks that sort faster)
+    // (c.keys is k_permute's to write: room for the crowded keys, at most one in
+    // kCrowd particles, and a bit a particle; large launches have blocks that
+    // sort faster)
     const int pt = N < (1 << 17) ? 256 : 1024;
-    launch_next(c, k_cs_place, blocks(N, pt), pt, N, c.keys_alt, c.vals_alt, c.kstart, order, c.kcount, K, c.keys,
-                c.vals);
+    launch_next(c, k_cs_place, blocks(N, pt), pt, N, c.keys_alt, c.vals_alt, c.kstart, order, c.kcount, K, c.keys);
     launch_next(c, k_permute<T, true>, blocks(N, 256), 256, N, c.keys, c.vals, order, c.keys_alt, c.kcount, c.kstart, p,
                 n_in, c.box_of, c.boxes, sorted_view<T>(c), c.cells, c.ndefer);
     c.launches += direct ? 4 : 5;
