@@ -702,7 +702,7 @@ __device__ __forceinline__ int group_scan(const Grid& g, const BoxInfo& bx, cons
             base += total;
         };
         if (__any_sync(gm, se.y - se.x > 32)) {
-            // a cell of more than 32 candidates: this round's cells one after
+            // a cell of more than 32 candidates: these G cells one after
             // another, 32 candidates a lane at a time
             for (int l = 0; l < G && base <= most; ++l) {
                 const int a = __shfl_sync(gm, se.x, l, G), e = __shfl_sync(gm, se.y, l, G);
