@@ -38,7 +38,7 @@ def test_time_is_linear_in_the_crowd():
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n", [30, 66])  # a bitmap of one word a thread at most, and of several
+@pytest.mark.parametrize("n", [30, 66])  # the cells sorted by a block of 256, of 1024
 def test_crowded_cells_keep_caller_order(n):
     # most particles in two cells (at NaN and beyond the far corner), in any order
     import numpy as np
